@@ -75,12 +75,15 @@ __device__ __forceinline__ void conv_channel(const float* __restrict__ st, const
                                              const float* __restrict__ w2, u64 (&acc)[R], int gl = 0, int gh = 0,
                                              u64 init = 0ull) {
     static_assert(!(WIN && FIRST), "a windowed pass may skip an accumulator's first product");
-    u64 wp[ELL + 1];
+    u64 wp[ELL];
+    {
+        const int lane = threadIdx.x & 31;
+        const float mine = w2[2 * (lane < ELL ? lane : 0)];
 #pragma unroll
-    for (int j = 0; j < ELL; j += 2) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(w2 + 2 * j);
-        wp[j] = v.x;
-        wp[j + 1] = v.y;
+        for (int j = 0; j < ELL; ++j) {
+            const float w = __shfl_sync(kFull, mine, j);
+            wp[j] = pack2(w, w);
+        }
     }
 #pragma unroll
     for (int g = 0; g < (R + ELL - 1 + 3) / 4; ++g) {
