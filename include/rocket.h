@@ -238,9 +238,10 @@ int rocket_transform_u8_host(rocket_params_t* p, const uint8_t* X_u8_host, int N
  * fp32 targets, alpha >= 0 the penalty on the weights.  The intercept is fitted and not penalised:
  * with Fc, yc the column-centred features and targets, w minimises |Fc w - yc|^2 + alpha |w|^2 and
  * b = mean(y) - mean(F) . w.  Solved in its dual form (an N x N system, N <= ROCKET_RIDGE_MAX_EXAMPLES)
- * in double precision; w_dev [P] and b_dev [1] receive the result as fp32.  The call allocates its
- * workspace ((P + N*N + N) doubles) with cudaMalloc, frees it, and returns after the work on
- * cuda_stream has finished.  Errors: ROCKET_EINVAL for NULL pointers, N < 1, P < 1, a negative or
+ * in double precision; w_dev [P] and b_dev [1] receive the result as fp32.  The call returns after the
+ * work on cuda_stream has finished.  Its workspace (about P + N*N doubles and up to 40 MB of partial sums) is
+ * allocated with cudaMalloc; one buffer of up to 64 MiB per device is kept for the next fit until a parameter
+ * handle is destroyed or the library runs short of memory, anything else is freed before the call returns.  Errors: ROCKET_EINVAL for NULL pointers, N < 1, P < 1, a negative or
  * non-finite alpha, or a system that is not positive definite (alpha = 0 with dependent rows);
  * ROCKET_EUNSUPPORTED beyond the size limit; ROCKET_ENOMEM / ROCKET_ECUDA from the runtime.
  *

@@ -258,6 +258,7 @@ void rocket_params_destroy(rocket_params_t* p) {
         if (p->host_stream) cudaStreamDestroy(p->host_stream);
         if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
         for (cudaEvent_t ev : p->copy_events) cudaEventDestroy(ev);
+        release_cached_workspaces();
         cudaGetLastError();
     }
     delete p->fast;

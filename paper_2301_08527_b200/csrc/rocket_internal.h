@@ -40,9 +40,17 @@ inline void count_launch(int n = 1) { g_launch_count.fetch_add(n, std::memory_or
 // Every device allocation of the library goes through here, so that a caller (and the tests) can
 // tell whether a call allocated: rocket_device_alloc_count reports the number made so far.
 extern std::atomic<int64_t> g_alloc_count;
+// Gives back what the library keeps on the current device between calls that own no handle (the regressor's workspace).
+void release_cached_workspaces();
 inline cudaError_t device_malloc(void** ptr, size_t bytes) {
     g_alloc_count.fetch_add(1, std::memory_order_relaxed);
-    return cudaMalloc(ptr, bytes);
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        release_cached_workspaces();
+        e = cudaMalloc(ptr, bytes);
+    }
+    return e;
 }
 
 // Draws K kernels by the rules of Section 3.1 with the counter-based generator.

@@ -5,181 +5,434 @@
 // system (Fc Fc^T + alpha I) a = yc (N x N, N examples << P features), w = Fc^T a,
 // b = mean(y) - mean(F) . w.  The Gram matrix, its Cholesky factor and the two triangular solves are
 // kept in double precision: the features are fp32 data, everything derived from them is not rounded
-// to fp32 before w and b are stored.
+// to fp32 before w and b are stored.  Every sum is taken in an order that depends on the sizes alone, so two fits
+// of the same data are bitwise identical.
+//
+// Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights took
+// 55 / 2,607 / 20,270 / 174 us as one thread per column, 2 x 2 outputs per thread, one block and one thread per
+// column.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstdint>
+#include <mutex>
 
 #include "rocket_internal.h"
 
 namespace rocket {
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kRThreads = 256;
+constexpr int kRWarps = kRThreads / 32;
 
-// mu[p] = mean over the N rows of F[.][p]; one thread per column, rows coalesced across the warp.
+// Column kernels: a block owns 32 columns (a lane each, so that a warp reads 128 contiguous bytes of a row) and its
+// eight warps share the rows; the warps' sums are added in warp order.
+//
+// mu[p] = mean over the N rows of F[.][p]; the block past the last column takes ybar = mean(y) and clears the ticket
+// the weights kernel counts its blocks with.
 __global__ void __launch_bounds__(kRThreads)
-ridge_colmean_kernel(const float* __restrict__ F, int N, int P, double* __restrict__ mu) {
-    const int p = blockIdx.x * kRThreads + threadIdx.x;
-    if (p >= P) return;
+ridge_means_kernel(const float* __restrict__ F, const float* __restrict__ y, int N, int P, double* __restrict__ mu,
+                   double* __restrict__ ybar, unsigned* __restrict__ ticket) {
+    __shared__ double red[kRWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool targets = (int)blockIdx.x * 32 >= P;
+    const int p = blockIdx.x * 32 + lane;
     double s = 0.0;
-    for (int i = 0; i < N; ++i) s += (double)F[(size_t)i * P + p];
-    mu[p] = s / (double)N;
-}
-
-// ybar = mean(y); one block.
-__global__ void __launch_bounds__(kRThreads)
-ridge_ymean_kernel(const float* __restrict__ y, int N, double* __restrict__ ybar) {
-    __shared__ double red[kRThreads];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < N; i += kRThreads) s += (double)y[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = kRThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *ybar = red[0] / (double)N;
-}
-
-// G[i][j] = sum_p (F[i][p] - mu[p]) (F[j][p] - mu[p]) (+ alpha on the diagonal), lower triangle and
-// its mirror.  One block per 32 x 32 tile with bi >= bj; the feature axis goes through shared memory
-// in pieces of 32 (centred on the way in); every thread owns a 2 x 2 piece of the tile.
-constexpr int kGT = 32, kGP = 32;
-__global__ void __launch_bounds__(kRThreads)
-ridge_gram_kernel(const float* __restrict__ F, int N, int P, const double* __restrict__ mu, double alpha,
-                  double* __restrict__ G) {
-    const int bi = blockIdx.y, bj = blockIdx.x;
-    if (bj > bi) return;
-    __shared__ double A[kGT][kGP + 1], B[kGT][kGP + 1];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;   // 16 x 16 threads, 2 x 2 outputs each
-    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-    for (int p0 = 0; p0 < P; p0 += kGP) {
-        for (int e = threadIdx.x; e < kGT * kGP; e += kRThreads) {
-            const int r = e / kGP, c = e % kGP, p = p0 + c;
-            const int ia = bi * kGT + r, ib = bj * kGT + r;
-            const double m = p < P ? mu[p] : 0.0;
-            A[r][c] = (ia < N && p < P) ? (double)F[(size_t)ia * P + p] - m : 0.0;
-            B[r][c] = (ib < N && p < P) ? (double)F[(size_t)ib * P + p] - m : 0.0;
-        }
-        __syncthreads();
+    if (targets) {
+        for (int i = threadIdx.x; i < N; i += kRThreads) s += (double)y[i];
+    } else if (p < P) {
+        const float* __restrict__ f = F + p;
 #pragma unroll 8
-        for (int c = 0; c < kGP; ++c) {
-            const double a0 = A[2 * ty][c], a1 = A[2 * ty + 1][c], b0 = B[2 * tx][c], b1 = B[2 * tx + 1][c];
-            acc[0][0] += a0 * b0; acc[0][1] += a0 * b1; acc[1][0] += a1 * b0; acc[1][1] += a1 * b1;
+        for (int i = warp; i < N; i += kRWarps) s += (double)__ldg(f + (size_t)i * P);
+    }
+    red[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int w = 1; w < kRWarps; ++w) s += red[w][lane];
+        if (targets) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) { *ybar = s / (double)N; *ticket = 0u; }
+        } else if (p < P) {
+            mu[p] = s / (double)N;
+        }
+    }
+}
+
+// One 64 x 64 tile of the lower triangle of G over a slice of the feature axis, as a partial sum.  Bound: the FP64 rate
+// (64 multiply-adds per clock and SM, reached by the FP64 matrix instruction with eight warps per SM; the scalar form
+// reaches 58.7 and loads twelve shared-memory words for 32 products where the fragments below take eight for 128).  A
+// warp owns 32 x 32 outputs as 4 x 4 fragments of m8n8k4; the slice goes through shared memory 32 columns at a time,
+// centred on the way in, the next piece on its way in registers.  A row of the staged piece is 36 doubles, so that the
+// 16 lanes of a fragment load's half warp (4 rows x 4 columns) fall on 16 different bank pairs.
+constexpr int kGT = 64, kGP = 32, kGPitch = kGP + 4, kGThreads = 128;
+constexpr int kGRows = 2 * kGT * kGP / kGThreads;      // staged values per thread and piece (half of them of each operand)
+__global__ void __launch_bounds__(kGThreads, 4)
+ridge_gram_kernel(const float* __restrict__ F, int N, int P, const double* __restrict__ mu, int slice,
+                  double* __restrict__ part) {
+    extern __shared__ double smem[];
+    double (*A)[kGPitch] = reinterpret_cast<double (*)[kGPitch]>(smem);
+    double (*B)[kGPitch] = A + kGT;
+    // tile index -> (bi, bj) with bj <= bi
+    int bi = (int)((sqrtf(8.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+    while (bi * (bi + 1) / 2 > (int)blockIdx.x) --bi;
+    while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
+    const int bj = blockIdx.x - bi * (bi + 1) / 2;
+    const int p_beg = blockIdx.y * slice, p_end = min(P, p_beg + slice);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int col = lane, row0 = warp;                      // staging: thread takes column `col` of rows row0 + 4 i
+    const int wr = (warp >> 1) * 32, wc = (warp & 1) * 32;  // the warp's outputs
+    const int fr = lane >> 2, fk = lane & 3;
+    double acc[4][4][2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[u][v][0] = acc[u][v][1] = 0.0;
+    float x[kGRows];
+    double m = 0.0;
+    auto fetch = [&](int p0) {
+        const int p = p0 + col;
+        const bool ok = p < p_end;
+        m = ok ? mu[p] : 0.0;
+#pragma unroll
+        for (int i = 0; i < kGRows / 2; ++i) {
+            const int ra = bi * kGT + row0 + 4 * i, rb = bj * kGT + row0 + 4 * i;
+            x[i] = ok && ra < N ? __ldg(F + (size_t)ra * P + p) : 0.0f;
+            x[kGRows / 2 + i] = ok && rb < N ? __ldg(F + (size_t)rb * P + p) : 0.0f;
+        }
+    };
+    fetch(p_beg);
+    for (int p0 = p_beg; p0 < p_end; p0 += kGP) {
+        __syncthreads();
+        const bool ok = p0 + col < p_end;
+#pragma unroll
+        for (int i = 0; i < kGRows / 2; ++i) {
+            const int r = row0 + 4 * i;
+            A[r][col] = ok && bi * kGT + r < N ? (double)x[i] - m : 0.0;
+            B[r][col] = ok && bj * kGT + r < N ? (double)x[kGRows / 2 + i] - m : 0.0;
         }
         __syncthreads();
+        if (p0 + kGP < p_end) fetch(p0 + kGP);
+#pragma unroll
+        for (int k = 0; k < kGP; k += 4) {
+            double a[4], b[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a[u] = A[wr + 8 * u + fr][k + fk];
+                b[u] = B[wc + 8 * u + fr][k + fk];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v)
+                    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                                 : "+d"(acc[u][v][0]), "+d"(acc[u][v][1]) : "d"(a[u]), "d"(b[v]));
+        }
     }
-    for (int u = 0; u < 2; ++u)
-        for (int v = 0; v < 2; ++v) {
-            const int i = bi * kGT + 2 * ty + u, j = bj * kGT + 2 * tx + v;
+    double* __restrict__ out = part + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (kGT * kGT);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            *reinterpret_cast<double2*>(out + (wr + 8 * u + fr) * kGT + wc + 8 * v + 2 * fk) =
+                make_double2(acc[u][v][0], acc[u][v][1]);
+}
+
+// ---- Cholesky factor and solves -------------------------------------------------------------------------------
+// G [Np][Np] (Np a multiple of 32 above N) holds the lower triangle of Fc Fc^T + alpha I, row N holds yc^T, rows below are
+// zero: the factorisation then leaves z = L^-1 yc in row N by itself.  Blocks of 32 x 32, right-looking: at step kb every
+// block of the grid factors the diagonal block for itself (one warp, a row per lane), solves the two panel blocks its
+// tile needs and updates the tile, so that a step takes one grid-wide barrier and no panel travels between barriers.
+// Solved panel blocks go transposed into the upper triangle, diagonal factors into Ld.  Bound: the chain of steps (22 of
+// them at N = 677; a diagonal block is 32 dependent pivots), not arithmetic.
+constexpr int kCB = 32, kCThreads = 256, kCPitch = kCB + 1, kDPitch = kCB + 2;
+
+struct CholArgs {
+    const double* part;       // partial Gram tiles [slices][tiles][64][64]
+    int slices, tiles;
+    double alpha;
+    const float* y;
+    const double* ybar;
+    double* G;
+    double* Ld;               // diagonal factors [nb][32][32]
+    double* a;                // solution [N]
+    int* status;              // 0 = ok, 1 = a pivot was not positive
+    int N, Np;
+};
+
+// Factors the leading `ncols` columns of the block whose rows are held by the lanes (s[lane][0 .. lane]); the factor's
+// transpose goes to t (t[j][c] = L[c][j]), the reciprocal pivots to rinv.  One warp.
+__device__ __forceinline__ bool chol_factor_block(const double (*s)[kCPitch], double (*t)[kDPitch], double* rinv, int ncols,
+                                                  int lane) {
+    double a[kCB];
+    bool good = true;
+#pragma unroll
+    for (int c = 0; c < kCB; ++c) a[c] = s[lane][c];
+#pragma unroll
+    for (int j = 0; j < kCB; ++j) {
+        if (j < ncols) {
+            double d = __shfl_sync(0xffffffffu, a[j], j);
+            if (!(d > 0.0)) { good = false; d = 1.0; }
+            const double r = rsqrt(d);
+            const double l = lane == j ? d * r : a[j] * r;
+            t[j][lane] = lane >= j ? l : 0.0;
+            if (lane == 0) rinv[j] = r;
+            __syncwarp();
+#pragma unroll
+            for (int c = j + 1; c < kCB; ++c) a[c] -= l * t[j][c];
+        }
+    }
+    __syncwarp();
+    return good;
+}
+
+// Row `lane` of a panel block: x L^T = g, in place.  One warp.
+__device__ __forceinline__ void chol_solve_row(double (*p)[kCPitch], const double (*t)[kDPitch], const double* rinv, int lane) {
+    double g[kCB];
+#pragma unroll
+    for (int c = 0; c < kCB; ++c) g[c] = p[lane][c];
+#pragma unroll
+    for (int j = 0; j < kCB; ++j) {
+        const double x = g[j] * rinv[j];
+        g[j] = x;
+#pragma unroll
+        for (int c = j + 1; c < kCB; ++c) g[c] -= x * t[j][c];
+    }
+#pragma unroll
+    for (int c = 0; c < kCB; ++c) p[lane][c] = g[c];
+}
+
+__global__ void __launch_bounds__(kCThreads)
+ridge_cholesky_solve_kernel(CholArgs q) {
+    __shared__ double s_t[kCB][kDPitch];
+    __shared__ double s_rinv[kCB];
+    __shared__ double s_raw[ROCKET_RIDGE_MAX_EXAMPLES];      // the panel blocks; in the end the solution
+    static_assert(2 * kCB * kCPitch <= ROCKET_RIDGE_MAX_EXAMPLES, "two panel blocks fit");
+    double (*s_pi)[kCPitch] = reinterpret_cast<double (*)[kCPitch]>(s_raw);
+    double (*s_pj)[kCPitch] = s_pi + kCB;
+    cg::grid_group grid = cg::this_grid();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = q.N, Np = q.Np, nb = Np / kCB;
+    double* __restrict__ G = q.G;
+
+    // lower blocks of G from the partial tiles, in slice order
+    const int blocks = nb * (nb + 1) / 2;
+    for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
+        int ib = (int)((sqrtf(8.0f * (float)b + 1.0f) - 1.0f) * 0.5f);
+        while (ib * (ib + 1) / 2 > b) --ib;
+        while ((ib + 1) * (ib + 2) / 2 <= b) ++ib;
+        const int jb = b - ib * (ib + 1) / 2;
+        for (int e = tid; e < kCB * kCB; e += kCThreads) {
+            const int i = ib * kCB + e / kCB, j = jb * kCB + e % kCB;
+            double g = 0.0;
             if (i < N && j < N) {
-                const double g = acc[u][v] + (i == j ? alpha : 0.0);
-                G[(size_t)i * N + j] = g;
-                G[(size_t)j * N + i] = g;
+                const int ti = i / kGT, tj = j / kGT;
+                const double* __restrict__ src = q.part + (size_t)(ti * (ti + 1) / 2 + tj) * (kGT * kGT) + (i % kGT) * kGT + j % kGT;
+#pragma unroll 4
+                for (int v = 0; v < q.slices; ++v) g += src[(size_t)v * q.tiles * (kGT * kGT)];
+                if (i == j) g += q.alpha;
+            } else if (i == N && j < N) {
+                g = (double)q.y[j] - *q.ybar;
+            }
+            G[(size_t)i * Np + j] = g;
+        }
+    }
+    if (blockIdx.x == 0 && tid == 0) *q.status = 0;
+    grid.sync();
+
+    bool good = true;
+    for (int kb = 0; kb < nb; ++kb) {
+        const int k0 = kb * kCB, ncols = min(kCB, N - k0);
+        const int rest = nb - kb - 1, tiles = rest * (rest + 1) / 2;
+        if (ncols > 0 && ((int)blockIdx.x < tiles || blockIdx.x == 0)) {
+            for (int e = tid; e < kCB * kCB; e += kCThreads) s_pi[e / kCB][e % kCB] = G[(size_t)(k0 + e / kCB) * Np + k0 + e % kCB];
+            __syncthreads();
+            if (warp == 0) good = chol_factor_block(s_pi, s_t, s_rinv, ncols, lane) && good;
+            __syncthreads();
+            if (blockIdx.x == 0)
+                for (int e = tid; e < kCB * kCB; e += kCThreads)
+                    q.Ld[(size_t)kb * kCB * kCB + e] = s_t[e % kCB][e / kCB];    // Ld[r][c] = L[r][c], read below r's diagonal only
+            for (int b = blockIdx.x; b < tiles; b += gridDim.x) {
+                // tile (ib, jb) of the trailing blocks, column by column so that the first ones are the panel's own
+                int x = (int)((sqrtf(8.0f * (float)(tiles - 1 - b) + 1.0f) - 1.0f) * 0.5f);
+                while (x * (x + 1) / 2 > tiles - 1 - b) --x;
+                while ((x + 1) * (x + 2) / 2 <= tiles - 1 - b) ++x;
+                const int jb = nb - 1 - x, ib = nb - 1 - ((tiles - 1 - b) - x * (x + 1) / 2);
+                const int i0 = ib * kCB, j0 = jb * kCB;
+                for (int e = tid; e < kCB * kCB; e += kCThreads) {
+                    const int r = e / kCB, c = e % kCB;
+                    s_pi[r][c] = G[(size_t)(i0 + r) * Np + k0 + c];
+                    if (ib != jb) s_pj[r][c] = G[(size_t)(j0 + r) * Np + k0 + c];
+                }
+                const int ty = tid / 16, tx = tid % 16;
+                double g[2][2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) g[u][v] = G[(size_t)(i0 + ty + 16 * u) * Np + j0 + tx + 16 * v];
+                __syncthreads();
+                if (warp == 0) chol_solve_row(s_pi, s_t, s_rinv, lane);
+                else if (warp == 1 && ib != jb) chol_solve_row(s_pj, s_t, s_rinv, lane);
+                __syncthreads();
+                const double (*pj)[kCPitch] = ib != jb ? s_pj : s_pi;
+#pragma unroll 8
+                for (int k = 0; k < kCB; ++k) {
+                    const double a0 = s_pi[ty][k], a1 = s_pi[ty + 16][k], b0 = pj[tx][k], b1 = pj[tx + 16][k];
+                    g[0][0] -= a0 * b0; g[0][1] -= a0 * b1; g[1][0] -= a1 * b0; g[1][1] -= a1 * b1;
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) G[(size_t)(i0 + ty + 16 * u) * Np + j0 + tx + 16 * v] = g[u][v];
+                if (jb == kb + 1)
+                    for (int e = tid; e < kCB * kCB; e += kCThreads) G[(size_t)(k0 + e / kCB) * Np + i0 + e % kCB] = s_pi[e % kCB][e / kCB];
+                __syncthreads();
             }
         }
+        if (rest > 0) grid.sync();
+    }
+    if (blockIdx.x != 0) return;
+
+    // L^T a = z, from the last block up.  Row k0 + j of the upper triangle holds L's column: a warp per row takes the
+    // part below the diagonal block, one warp solves the diagonal block.
+    if (warp == 0 && lane == 0 && !good) *q.status = 1;
+    __syncthreads();
+    double* s_a = s_raw;
+    const int nblk = (N + kCB - 1) / kCB;
+    for (int kb = nblk - 1; kb >= 0; --kb) {
+        const int k0 = kb * kCB, ncols = min(kCB, N - k0);
+        for (int e = tid; e < kCB * kCB; e += kCThreads) s_t[e / kCB][e % kCB] = q.Ld[(size_t)kb * kCB * kCB + e];   // s_t[r][c] = L[r][c]
+        double sum[kCB / (kCThreads / 32)];
+#pragma unroll
+        for (int u = 0; u < kCB / (kCThreads / 32); ++u) sum[u] = 0.0;
+        for (int i = k0 + kCB + lane; i < N; i += 32) {
+            const double ai = s_a[i];
+#pragma unroll
+            for (int u = 0; u < kCB / (kCThreads / 32); ++u)
+                sum[u] += G[(size_t)(k0 + warp + (kCThreads / 32) * u) * Np + i] * ai;
+        }
+#pragma unroll
+        for (int u = 0; u < kCB / (kCThreads / 32); ++u) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], o);
+            if (lane == 0) s_rinv[warp + (kCThreads / 32) * u] = sum[u];
+        }
+        __syncthreads();
+        if (warp == 0) {
+            double z = 0.0;
+            if (lane < ncols) z = (N / kCB == kb ? q.Ld[(size_t)kb * kCB * kCB + (N - k0) * kCB + lane] : G[(size_t)(k0 + lane) * Np + N]);
+            double v = lane < ncols ? z - s_rinv[lane] : 0.0;
+            const double inv = lane < ncols ? 1.0 / s_t[lane][lane] : 0.0;
+#pragma unroll 4
+            for (int j = ncols - 1; j >= 0; --j) {
+                const double aj = __shfl_sync(0xffffffffu, v * inv, j);
+                if (lane == j) v = aj;
+                else if (lane < j) v -= s_t[j][lane] * aj;
+            }
+            if (lane < ncols) { s_a[k0 + lane] = v; q.a[k0 + lane] = v; }
+        }
+        __syncthreads();
+    }
 }
 
-// In-place Cholesky factor (lower triangle, G = L L^T) and the two triangular solves, one block.
-// Right-looking, column by column; status: 0 = ok, 1 = a pivot was not positive.
-__global__ void __launch_bounds__(1024)
-ridge_cholesky_solve_kernel(double* __restrict__ G, int N, const float* __restrict__ y, const double* __restrict__ ybar,
-                            double* __restrict__ a, int* __restrict__ status) {
-    __shared__ double pivot;
-    __shared__ int bad;
-    __shared__ double col[ROCKET_RIDGE_MAX_EXAMPLES];   // column k of L below the diagonal
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    for (int k = 0; k < N; ++k) {
-        if (threadIdx.x == 0) {
-            const double d = G[(size_t)k * N + k];
-            if (!(d > 0.0)) bad = 1;
-            pivot = d > 0.0 ? sqrt(d) : 1.0;
-            G[(size_t)k * N + k] = pivot;
-        }
-        __syncthreads();
-        const double inv = 1.0 / pivot;
-        for (int i = k + 1 + threadIdx.x; i < N; i += blockDim.x) {
-            const double l = G[(size_t)i * N + k] * inv;
-            G[(size_t)i * N + k] = l;
-            col[i] = l;
-        }
-        __syncthreads();
-        // trailing update of the lower triangle: G[i][j] -= L[i][k] L[j][k], k < j <= i (a warp per row)
-        for (int i = k + 1 + warp; i < N; i += nwarps) {
-            const double li = col[i];
-            double* __restrict__ row = G + (size_t)i * N;
-            for (int j = k + 1 + lane; j <= i; j += 32) row[j] -= li * col[j];
-        }
-        __syncthreads();
-    }
-    // L z = yc (forward), then L^T a = z (backward); a holds z in between
-    for (int i = threadIdx.x; i < N; i += blockDim.x) a[i] = (double)y[i] - *ybar;
-    __syncthreads();
-    for (int k = 0; k < N; ++k) {
-        if (threadIdx.x == 0) a[k] /= G[(size_t)k * N + k];
-        __syncthreads();
-        const double zk = a[k];
-        for (int i = k + 1 + threadIdx.x; i < N; i += blockDim.x) a[i] -= G[(size_t)i * N + k] * zk;
-        __syncthreads();
-    }
-    for (int k = N - 1; k >= 0; --k) {
-        if (threadIdx.x == 0) a[k] /= G[(size_t)k * N + k];
-        __syncthreads();
-        const double ak = a[k];
-        for (int i = threadIdx.x; i < k; i += blockDim.x) a[i] -= G[(size_t)k * N + i] * ak;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *status = bad;
-}
-
-// w[p] = sum_i a[i] (F[i][p] - mu[p]); one thread per feature.  Also part[block] = sum_p mu[p] w[p].
+// w[p] = sum_i a[i] (F[i][p] - mu[p]), and the intercept b = ybar - sum_p mu[p] w[p] (with the stored fp32 weights) by the
+// last block to finish, in block order.
 __global__ void __launch_bounds__(kRThreads)
-ridge_weights_kernel(const float* __restrict__ F, int N, int P, const double* __restrict__ mu,
-                     const double* __restrict__ a, float* __restrict__ w, double* __restrict__ part) {
-    __shared__ double red[kRThreads];
-    const int p = blockIdx.x * kRThreads + threadIdx.x;
+ridge_weights_kernel(const float* __restrict__ F, int N, int P, const double* __restrict__ mu, const double* __restrict__ a,
+                     const double* __restrict__ ybar, float* __restrict__ w, float* __restrict__ b, double* __restrict__ part,
+                     unsigned* __restrict__ ticket) {
+    __shared__ double s_a[ROCKET_RIDGE_MAX_EXAMPLES];
+    __shared__ double red[kRWarps][32];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < N; i += kRThreads) s_a[i] = a[i];
+    __syncthreads();
+    const int p = blockIdx.x * 32 + lane;
     double s = 0.0, m = 0.0;
     if (p < P) {
         m = mu[p];
-        for (int i = 0; i < N; ++i) s += a[i] * ((double)F[(size_t)i * P + p] - m);
-        w[p] = (float)s;
+        const float* __restrict__ f = F + p;
+#pragma unroll 8
+        for (int i = warp; i < N; i += kRWarps) s += s_a[i] * ((double)__ldg(f + (size_t)i * P) - m);
     }
-    red[threadIdx.x] = p < P ? m * (double)(float)s : 0.0;   // the intercept matches the stored fp32 weights
+    red[warp][lane] = s;
     __syncthreads();
-    for (int o = kRThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int v = 1; v < kRWarps; ++v) s += red[v][lane];
+        if (p < P) w[p] = (float)s;
+        double c = p < P ? m * (double)(float)s : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        if (lane == 0) {
+            part[blockIdx.x] = c;
+            __threadfence();
+            s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        }
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double c = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kRThreads) c += __ldcg(part + i);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) red[warp][0] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int v = 1; v < kRWarps; ++v) c += red[v][0];
+        *b = (float)(*ybar - c);
+    }
 }
 
-// b = ybar - sum of the partial dot products, in block order (run-to-run identical).
-__global__ void ridge_intercept_kernel(const double* __restrict__ part, int nparts, const double* __restrict__ ybar,
-                                       float* __restrict__ b) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < nparts; ++i) s += part[i];
-        *b = (float)(*ybar - s);
-    }
-}
-
-// yhat[n] = b + sum_p F[n][p] w[p]; one block per example, products summed in double.
-__global__ void __launch_bounds__(kRThreads)
+// yhat[n] = b + sum_p F[n][p] w[p], products summed in double.  A row is shared by the blocks of a cluster (as many as
+// it takes to put a block on every SM, at most eight): each sums its contiguous part, the first adds the parts in rank
+// order through distributed shared memory.  Bound: the latency of one trip to memory; a block per row and one float
+// per load took 14.7 us for 60 rows of 20,000.
+constexpr int kPThreads = 512;
+template <bool VEC>
+__global__ void __launch_bounds__(kPThreads)
 ridge_predict_kernel(const float* __restrict__ F, int P, const float* __restrict__ w, const float* __restrict__ b,
                      float* __restrict__ yhat) {
-    __shared__ double red[kRThreads];
-    const float* __restrict__ f = F + (size_t)blockIdx.x * P;
+    __shared__ double red[kPThreads / 32];
+    __shared__ double s_part[8];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int parts = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float* __restrict__ f = F + (size_t)blockIdx.y * P;
     double s = 0.0;
-    for (int p = threadIdx.x; p < P; p += kRThreads) s += (double)f[p] * (double)w[p];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = kRThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
+    if (VEC) {
+        const int n4 = P / 4, beg = (int)((long long)n4 * rank / parts), end = (int)((long long)n4 * (rank + 1) / parts);
+        const float4* __restrict__ f4 = reinterpret_cast<const float4*>(f);
+        const float4* __restrict__ w4 = reinterpret_cast<const float4*>(w);
+#pragma unroll 4
+        for (int i = beg + threadIdx.x; i < end; i += kPThreads) {
+            const float4 x = __ldg(f4 + i), v = __ldg(w4 + i);
+            s += (double)x.x * (double)v.x + (double)x.y * (double)v.y + ((double)x.z * (double)v.z + (double)x.w * (double)v.w);
+        }
+    } else {
+        const int beg = (int)((long long)P * rank / parts), end = (int)((long long)P * (rank + 1) / parts);
+#pragma unroll 8
+        for (int i = beg + threadIdx.x; i < end; i += kPThreads) s += (double)__ldg(f + i) * (double)__ldg(w + i);
     }
-    if (threadIdx.x == 0) yhat[blockIdx.x] = (float)(red[0] + (double)*b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) red[warp] = s;
+    __syncthreads();
+    if (warp == 0) {
+        s = lane < kPThreads / 32 ? red[lane] : 0.0;
+#pragma unroll
+        for (int o = kPThreads / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) *cluster.map_shared_rank(&s_part[rank], 0) = s;
+    }
+    cluster.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        s = s_part[0];
+        for (int r = 1; r < parts; ++r) s += s_part[r];
+        yhat[blockIdx.y] = (float)(s + (double)*b);
+    }
 }
 
 int status_of(cudaError_t e) {
@@ -188,7 +441,71 @@ int status_of(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? ROCKET_ENOMEM : ROCKET_ECUDA;
 }
 
+// Workspace of a fit.  cudaMalloc and cudaFree take 0.4 to 5 ms each here, several times the fit itself, so one buffer
+// per device, of at most kKeepBytes, outlives the call: a fit takes it while nobody else has it and puts it back after its
+// stream has finished; a larger or a concurrent fit allocates and frees its own.  The buffer is given back when a handle
+// of the library is destroyed and when a device allocation of the library fails (release_cached_workspaces).
+constexpr size_t kKeepBytes = (size_t)64 << 20;
+constexpr int kMaxDevices = 64;
+struct Kept { void* ptr = nullptr; size_t bytes = 0; bool taken = false; };
+std::mutex g_kept_mu;
+Kept g_kept[kMaxDevices];
+
+struct FitWorkspace {
+    void* ptr = nullptr;
+    int slot = -1;          // >= 0: the device's kept buffer
+    cudaError_t take(size_t bytes) {
+        int dev = -1;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (bytes <= kKeepBytes && dev < kMaxDevices) {
+            std::lock_guard<std::mutex> lk(g_kept_mu);
+            Kept& k = g_kept[dev];
+            if (!k.taken && k.bytes >= bytes) {
+                k.taken = true;
+                slot = dev;
+                ptr = k.ptr;
+                return cudaSuccess;
+            }
+        }
+        return device_malloc(&ptr, bytes);
+    }
+    // the work that used it has finished
+    void put_back(size_t bytes) {
+        void* gone = ptr;
+        int dev = -1;
+        if (slot >= 0) {
+            std::lock_guard<std::mutex> lk(g_kept_mu);
+            g_kept[slot].taken = false;
+            return;
+        }
+        if (bytes <= kKeepBytes && cudaGetDevice(&dev) == cudaSuccess && dev < kMaxDevices) {
+            std::lock_guard<std::mutex> lk(g_kept_mu);
+            Kept& k = g_kept[dev];
+            if (!k.taken && k.bytes < bytes) {       // the larger buffer stays
+                gone = k.ptr;
+                k.ptr = ptr;
+                k.bytes = bytes;
+            }
+        }
+        if (gone) cudaFree(gone);
+    }
+};
+
 }  // namespace
+
+void release_cached_workspaces() {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kMaxDevices) { cudaGetLastError(); return; }
+    void* gone = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_kept_mu);
+        Kept& k = g_kept[dev];
+        if (!k.taken) { gone = k.ptr; k = Kept(); }
+    }
+    if (gone) cudaFree(gone);
+}
+
 }  // namespace rocket
 
 using namespace rocket;
@@ -199,31 +516,48 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     if (!(alpha >= 0.0f) || !(alpha < 3.0e38f)) return ROCKET_EINVAL;
     if (N > ROCKET_RIDGE_MAX_EXAMPLES) return ROCKET_EUNSUPPORTED;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const int nparts = (P + kRThreads - 1) / kRThreads;
-    // workspace: mu[P], G[N][N], a[N], part[nparts], ybar, status
-    const size_t doubles = (size_t)P + (size_t)N * N + (size_t)N + (size_t)nparts + 1;
-    char* ws = nullptr;
-    cudaError_t e = rocket::device_malloc(reinterpret_cast<void**>(&ws), doubles * sizeof(double) + 16);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const size_t gram_smem = (size_t)2 * kGT * kGPitch * sizeof(double);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ridge_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem);
     if (e != cudaSuccess) return status_of(e);
-    double* mu = reinterpret_cast<double*>(ws);
-    double* G = mu + P;
-    double* a = G + (size_t)N * N;
-    double* part = a + N;
-    double* ybar = part + nparts;
-    int* status = reinterpret_cast<int*>(ybar + 1);
-    const int tiles = (N + kGT - 1) / kGT;
-    ridge_colmean_kernel<<<nparts, kRThreads, 0, stream>>>(feat_dev, N, P, mu);
-    ridge_ymean_kernel<<<1, kRThreads, 0, stream>>>(y_dev, N, ybar);
-    ridge_gram_kernel<<<dim3(tiles, tiles), kRThreads, 0, stream>>>(feat_dev, N, P, mu, (double)alpha, G);
-    ridge_cholesky_solve_kernel<<<1, 1024, 0, stream>>>(G, N, y_dev, ybar, a, status);
-    ridge_weights_kernel<<<nparts, kRThreads, 0, stream>>>(feat_dev, N, P, mu, a, w_dev, part);
-    ridge_intercept_kernel<<<1, 32, 0, stream>>>(part, nparts, ybar, b_dev);
-    count_launch(6);
+    const int col_blocks = (P + 31) / 32;
+    // Slices of the feature axis: about two waves of the four blocks an SM holds, at least 128 columns each, and no more
+    // than 40 MB of partial tiles.
+    const int nt = (N + kGT - 1) / kGT, tiles = nt * (nt + 1) / 2;
+    const size_t tile_bytes = (size_t)kGT * kGT * sizeof(double);
+    int slices = std::max(1, std::min({8 * sms / tiles, P / 128, (int)(((size_t)40 << 20) / (tile_bytes * tiles))}));
+    const int slice = ((P + slices - 1) / slices + kGP - 1) / kGP * kGP;
+    slices = (P + slice - 1) / slice;
+    const int nb = (N + 1 + kCB - 1) / kCB, Np = nb * kCB;
+    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Ld[nb][32][32], partial Gram tiles, ticket, status
+    size_t off = 0;
+    auto take = [&](size_t doubles) { const size_t o = off; off += (doubles + 31) / 32 * 32; return o; };
+    const size_t o_mu = take(P), o_a = take(N), o_part = take(col_blocks), o_ybar = take(1), o_G = take((size_t)Np * Np);
+    const size_t o_Ld = take((size_t)nb * kCB * kCB), o_gram = take((size_t)slices * tiles * kGT * kGT), o_int = take(2);
+    const size_t bytes = off * sizeof(double);
+    FitWorkspace ws;
+    if ((e = ws.take(bytes)) != cudaSuccess) return status_of(e);
+    double* d = static_cast<double*>(ws.ptr);
+    unsigned* ticket = reinterpret_cast<unsigned*>(d + o_int);
+    int* status = reinterpret_cast<int*>(d + o_int + 1);
+    ridge_means_kernel<<<col_blocks + 1, kRThreads, 0, stream>>>(feat_dev, y_dev, N, P, d + o_mu, d + o_ybar, ticket);
+    ridge_gram_kernel<<<dim3(tiles, slices), kGThreads, gram_smem, stream>>>(feat_dev, N, P, d + o_mu, slice, d + o_gram);
+    CholArgs q{d + o_gram, slices, tiles, (double)alpha, y_dev, d + o_ybar, d + o_G, d + o_Ld, d + o_a, status, N, Np};
+    void* args[] = {&q};
+    // one block per SM: more would lengthen the grid barriers without shortening the chain
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(ridge_cholesky_solve_kernel),
+                                    dim3((unsigned)std::max(1, std::min(sms, nb * (nb + 1) / 2))), dim3(kCThreads), args, 0, stream);
+    ridge_weights_kernel<<<col_blocks, kRThreads, 0, stream>>>(feat_dev, N, P, d + o_mu, d + o_a, d + o_ybar, w_dev, b_dev,
+                                                               d + o_part, ticket);
+    count_launch(4);
     int host_status = 0;
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(&host_status, status, sizeof(int), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    cudaFree(ws);
+    const cudaError_t done = cudaStreamSynchronize(stream);
+    ws.put_back(bytes);
+    if (e == cudaSuccess) e = done;
     if (e != cudaSuccess) return status_of(e);
     return host_status == 0 ? ROCKET_OK : ROCKET_EINVAL;
 }
@@ -233,8 +567,30 @@ extern "C" int rocket_ridge_predict(const float* feat_dev, int N, int P, const f
     if (N < 0 || P < 1) return ROCKET_EINVAL;
     if (N == 0) return ROCKET_OK;
     if (!feat_dev || !w_dev || !b_dev || !yhat_dev) return ROCKET_EINVAL;
-    ridge_predict_kernel<<<(unsigned)N, kRThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(feat_dev, P, w_dev, b_dev,
-                                                                                              yhat_dev);
-    count_launch();
-    return status_of(cudaGetLastError());
+    const bool vec = P % 4 == 0 && ((reinterpret_cast<uintptr_t>(feat_dev) | reinterpret_cast<uintptr_t>(w_dev)) & 15u) == 0;
+    // grid.y is limited to 65,535 rows
+    for (int n0 = 0; n0 < N; n0 += 65535) {
+        const int n = std::min(N - n0, 65535);
+        cudaLaunchConfig_t cfg = {};
+        // blocks per row: up to two per SM of this GPU's 148, and no fewer than one step of a block's threads each
+        unsigned parts = 1;
+        while (parts < 8 && (long long)n * parts * 2 <= 296 && (int)parts * 2 * kPThreads * 4 <= P) parts *= 2;
+        cfg.gridDim = dim3(parts, (unsigned)n);
+        cfg.blockDim = dim3(kPThreads);
+        cfg.stream = static_cast<cudaStream_t>(cuda_stream);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = parts;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const float* f = feat_dev + (size_t)n0 * P;
+        float* out = yhat_dev + n0;
+        const cudaError_t e = vec ? cudaLaunchKernelEx(&cfg, ridge_predict_kernel<true>, f, P, w_dev, b_dev, out)
+                                  : cudaLaunchKernelEx(&cfg, ridge_predict_kernel<false>, f, P, w_dev, b_dev, out);
+        count_launch();
+        if (e != cudaSuccess) return status_of(e);
+    }
+    return ROCKET_OK;
 }
