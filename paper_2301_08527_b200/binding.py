@@ -128,7 +128,7 @@ def kernel_launch_count():
 
 
 def _np_ptr(a):
-    return a.ctypes.data_as(ctypes.c_void_p)
+    return a.ctypes.data
 
 
 class RocketParams:
@@ -240,29 +240,50 @@ class RocketParams:
             pass
 
 
+_torch = None
+_current_stream = None
+
+
+def _t():
+    """torch, imported at the first call that needs it (importing this module does not)."""
+    global _torch, _current_stream
+    if _torch is None:
+        import torch
+        # the raw handle of the current stream, without building a Stream object (1.5 us) on every call
+        raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and device is not None:
+            _current_stream = lambda: raw(device())  # noqa: E731
+        else:
+            _current_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+        _torch = torch
+    return _torch
+
+
 def _dev_ptr(t, dtype, name):
-    import torch
-    if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype != dtype or not t.is_contiguous():
-        raise TypeError("%s must be a contiguous CUDA tensor of dtype %s" % (name, dtype))
-    return ctypes.c_void_p(t.data_ptr())
+    try:
+        if t.dtype is dtype and t.is_cuda and t.is_contiguous():
+            return t.data_ptr()
+    except AttributeError:   # not a tensor
+        pass
+    raise TypeError("%s must be a contiguous CUDA tensor of dtype %s" % (name, dtype))
 
 
 def _stream():
-    import torch
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _current_stream()
 
 
 def _check_x(params, X):
-    if X.dim() != 3:
+    shape = X.shape
+    if len(shape) != 3:
         raise ValueError("X must be [N, C, L]")
-    return int(X.shape[0]), int(X.shape[1]), int(X.shape[2])
+    return shape
 
 
 def rocket_transform(params, X, out=None):
     """Hard PPV + max.  X: CUDA fp32 [N, C, L] -> features CUDA fp32 [N, 2K] on the current stream."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X)
-    feat = out if out is not None else torch.empty((N, 2 * params.K), dtype=torch.float32, device=X.device)
+    feat = out if out is not None else X.new_empty((N, 2 * params.K), dtype=torch.float32)
     _check(load_library().rocket_transform(params.handle, _dev_ptr(X, torch.float32, "X"), N, C, L,
                                            _dev_ptr(feat, torch.float32, "out"), _stream()), "rocket_transform")
     return feat
@@ -270,9 +291,9 @@ def rocket_transform(params, X, out=None):
 
 def rocket_transform_f16(params, X, out=None):
     """Hard PPV + max in half precision (binary16 samples, weights and biases; one rounding per multiply-add)."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X)
-    feat = out if out is not None else torch.empty((N, 2 * params.K), dtype=torch.float32, device=X.device)
+    feat = out if out is not None else X.new_empty((N, 2 * params.K), dtype=torch.float32)
     _check(load_library().rocket_transform_f16(params.handle, _dev_ptr(X, torch.float32, "X"), N, C, L,
                                                _dev_ptr(feat, torch.float32, "out"), _stream()), "rocket_transform_f16")
     return feat
@@ -280,12 +301,12 @@ def rocket_transform_f16(params, X, out=None):
 
 def rocket_transform_soft(params, X, lam, shift=3.0, out=None, argmax_out=None, want_argmax=True):
     """softPPV + max (Eq. 3-4).  Returns (features [N, 2K], argmax [N, K] int32 or None)."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X)
-    feat = out if out is not None else torch.empty((N, 2 * params.K), dtype=torch.float32, device=X.device)
+    feat = out if out is not None else X.new_empty((N, 2 * params.K), dtype=torch.float32)
     arg = argmax_out
     if arg is None and want_argmax:
-        arg = torch.empty((N, params.K), dtype=torch.int32, device=X.device)
+        arg = X.new_empty((N, params.K), dtype=torch.int32)
     _check(load_library().rocket_transform_soft(
         params.handle, _dev_ptr(X, torch.float32, "X"), N, C, L, ctypes.c_float(lam), ctypes.c_float(shift),
         _dev_ptr(feat, torch.float32, "out"),
@@ -304,10 +325,10 @@ def _stats(params, mean, inv_std):
 def rocket_transform_u8(params, X_u8, mean, inv_std, out=None):
     """Hard PPV + max of raw 8-bit intensities scaled per channel: x = (v - mean[c]) * inv_std[c].
     X_u8: CUDA uint8 [N, C, L]; mean, inv_std: host arrays of C floats."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X_u8)
     m, s = _stats(params, mean, inv_std)
-    feat = out if out is not None else torch.empty((N, 2 * params.K), dtype=torch.float32, device=X_u8.device)
+    feat = out if out is not None else X_u8.new_empty((N, 2 * params.K), dtype=torch.float32)
     _check(load_library().rocket_transform_u8(params.handle, _dev_ptr(X_u8, torch.uint8, "X_u8"), N, C, L, _np_ptr(m),
                                               _np_ptr(s), _dev_ptr(feat, torch.float32, "out"), _stream()),
            "rocket_transform_u8")
@@ -316,13 +337,13 @@ def rocket_transform_u8(params, X_u8, mean, inv_std, out=None):
 
 def rocket_transform_soft_u8(params, X_u8, mean, inv_std, lam, shift=3.0, out=None, argmax_out=None, want_argmax=True):
     """softPPV + max of raw 8-bit intensities scaled per channel.  Returns (features, argmax or None)."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X_u8)
     m, s = _stats(params, mean, inv_std)
-    feat = out if out is not None else torch.empty((N, 2 * params.K), dtype=torch.float32, device=X_u8.device)
+    feat = out if out is not None else X_u8.new_empty((N, 2 * params.K), dtype=torch.float32)
     arg = argmax_out
     if arg is None and want_argmax:
-        arg = torch.empty((N, params.K), dtype=torch.int32, device=X_u8.device)
+        arg = X_u8.new_empty((N, params.K), dtype=torch.int32)
     _check(load_library().rocket_transform_soft_u8(
         params.handle, _dev_ptr(X_u8, torch.uint8, "X_u8"), N, C, L, _np_ptr(m), _np_ptr(s), ctypes.c_float(lam),
         ctypes.c_float(shift), _dev_ptr(feat, torch.float32, "out"),
@@ -332,7 +353,7 @@ def rocket_transform_soft_u8(params, X_u8, mean, inv_std, lam, shift=3.0, out=No
 
 def rocket_transform_soft_backward(params, X, lam, shift, dfeat, argmax, dW_out=None, db_out=None):
     """Gradients of sum(dfeat * soft features) for weights (ragged like the weights) and biases."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X)
     dW = dW_out if dW_out is not None else torch.empty((params.n_weights,), dtype=torch.float32, device=X.device)
     db = db_out if db_out is not None else torch.empty((params.K,), dtype=torch.float32, device=X.device)
@@ -348,7 +369,7 @@ def rocket_transform_soft_backward_noalloc(params, X, lam, shift, dfeat, argmax,
     """Allocation-free backward: same results as rocket_transform_soft_backward, scratch in a fixed
     library-owned array (see include/rocket.h for its size limit and sharing rules).  The caller
     supplies the outputs, and the handle must already be bound to the device."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X)
     _check(load_library().rocket_transform_soft_backward_noalloc(
         params.handle, _dev_ptr(X, torch.float32, "X"), N, C, L, ctypes.c_float(lam), ctypes.c_float(shift),
@@ -361,10 +382,10 @@ def rocket_transform_soft_backward_noalloc(params, X, lam, shift, dfeat, argmax,
 def rocket_ridge_fit(feat, y, alpha):
     """Ridge regressor on pooled features (Section 3.3): feat CUDA fp32 [N, P], y CUDA fp32 [N].
     Returns (w [P], b [1]) on the device; the intercept is fitted and not penalised."""
-    import torch
+    torch = _t()
     if feat.dim() != 2 or y.dim() != 1 or y.shape[0] != feat.shape[0]:
         raise ValueError("feat must be [N, P] and y [N]")
-    N, Pn = int(feat.shape[0]), int(feat.shape[1])
+    N, Pn = feat.shape[0], feat.shape[1]
     w = torch.empty((Pn,), dtype=torch.float32, device=feat.device)
     b = torch.empty((1,), dtype=torch.float32, device=feat.device)
     _check(load_library().rocket_ridge_fit(_dev_ptr(feat, torch.float32, "feat"), N, Pn, _dev_ptr(y, torch.float32, "y"),
@@ -375,19 +396,21 @@ def rocket_ridge_fit(feat, y, alpha):
 
 def rocket_ridge_predict(feat, w, b, out=None):
     """yhat[n] = b + feat[n] . w on the device (current stream)."""
-    import torch
-    if feat.dim() != 2 or w.dim() != 1 or w.shape[0] != feat.shape[1]:
+    torch = _t()
+    shape = feat.shape
+    if len(shape) != 2 or w.dim() != 1 or w.shape[0] != shape[1]:
         raise ValueError("feat must be [N, P] and w [P]")
-    N, Pn = int(feat.shape[0]), int(feat.shape[1])
-    yhat = out if out is not None else torch.empty((N,), dtype=torch.float32, device=feat.device)
-    _check(load_library().rocket_ridge_predict(_dev_ptr(feat, torch.float32, "feat"), N, Pn, _dev_ptr(w, torch.float32, "w"),
-                                               _dev_ptr(b, torch.float32, "b"), _dev_ptr(yhat, torch.float32, "out"),
-                                               _stream()), "rocket_ridge_predict")
+    N, Pn = shape
+    f32 = torch.float32
+    yhat = out if out is not None else feat.new_empty(N, dtype=f32)
+    _check((_lib or load_library()).rocket_ridge_predict(_dev_ptr(feat, f32, "feat"), N, Pn, _dev_ptr(w, f32, "w"),
+                                                         _dev_ptr(b, f32, "b"), _dev_ptr(yhat, f32, "out"),
+                                                         _current_stream()), "rocket_ridge_predict")
     return yhat
 
 
 def _host_ptr(t, dtype, name):
-    import torch
+    torch = _torch
     if isinstance(t, np.ndarray):
         t = torch.from_numpy(t)
     if t.is_cuda or t.dtype != dtype or not t.is_contiguous():
@@ -397,7 +420,7 @@ def _host_ptr(t, dtype, name):
 
 def rocket_transform_host(params, X_host, feat_host):
     """Host-buffer form: X_host / feat_host are host tensors (pinned for asynchronous copies)."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X_host)
     _check(load_library().rocket_transform_host(params.handle, _host_ptr(X_host, torch.float32, "X_host"), N, C, L,
                                                 _host_ptr(feat_host, torch.float32, "feat_host")),
@@ -407,7 +430,7 @@ def rocket_transform_host(params, X_host, feat_host):
 
 def rocket_transform_u8_host(params, X_u8_host, mean, inv_std, feat_host):
     """Host-buffer form of rocket_transform_u8 (the bytes travel to the device inside the call)."""
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X_u8_host)
     m, s = _stats(params, mean, inv_std)
     _check(load_library().rocket_transform_u8_host(params.handle, _host_ptr(X_u8_host, torch.uint8, "X_u8_host"), N, C, L,
@@ -417,7 +440,7 @@ def rocket_transform_u8_host(params, X_u8_host, mean, inv_std, feat_host):
 
 
 def rocket_transform_soft_host(params, X_host, lam, shift, feat_host, argmax_host=None):
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X_host)
     _check(load_library().rocket_transform_soft_host(
         params.handle, _host_ptr(X_host, torch.float32, "X_host"), N, C, L, ctypes.c_float(lam),
@@ -428,7 +451,7 @@ def rocket_transform_soft_host(params, X_host, lam, shift, feat_host, argmax_hos
 
 
 def rocket_transform_soft_backward_host(params, X_host, lam, shift, dfeat_host, argmax_host, dW_host, db_host):
-    import torch
+    torch = _t()
     N, C, L = _check_x(params, X_host)
     _check(load_library().rocket_transform_soft_backward_host(
         params.handle, _host_ptr(X_host, torch.float32, "X_host"), N, C, L, ctypes.c_float(lam),
@@ -487,7 +510,7 @@ class MiniRocket:
 
     def transform(self, X, out=None):
         """PPV features [N, F] of a CUDA float32 tensor X [N, C, L]."""
-        import torch
+        torch = _t()
         _check_x(self, X)
         N = X.shape[0]
         if out is None:
