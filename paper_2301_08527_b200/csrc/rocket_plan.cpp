@@ -125,8 +125,11 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
     int d_max = 0;
     std::map<std::tuple<int, int, int>, int> map_index;
     // kernels of one length follow one another, so that the blocks running at any one time execute the same
-    // instance of the inner loops (instruction caches: backward 3.5 % faster, forward 0.1-1 %)
-    std::stable_sort(t_kernels.begin(), t_kernels.end(), [&](int a, int b) { return hp.length[a] > hp.length[b]; });
+    // instance of the inner loops (instruction caches: backward 3.5 % faster, forward 0.1-1 %); within a length by
+    // dilation, whose tile shapes decide which instance it is (backward another 2 %: 74.0 -> 72.5 ms at 32 x 20 x 50,000)
+    std::stable_sort(t_kernels.begin(), t_kernels.end(), [&](int a, int b) {
+        return hp.length[a] != hp.length[b] ? hp.length[a] > hp.length[b] : hp.dilation[a] < hp.dilation[b];
+    });
     for (int k : t_kernels) {
         const int ki = (int)out.krec.size();
         add_kernel(k);
