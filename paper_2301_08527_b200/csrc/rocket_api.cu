@@ -404,7 +404,7 @@ int rocket_transform_f16(const rocket_params_t* p, const float* X_dev, int N, in
     if (N == 0) return ROCKET_OK;
     if (!feat_dev) return ROCKET_EINVAL;
     if ((st = ensure_device(p)) != ROCKET_OK) return st;
-    if (!p->fast->host.enabled || p->fast->dev.n_generic != 0) return ROCKET_EUNSUPPORTED;
+    if (!p->fast->host.enabled || p->fast->dev.n_generic != 0 || C > fast::kF16MaxChannels) return ROCKET_EUNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(X_dev) & 3u) != 0) return ROCKET_EINVAL;
     DeviceGuard g(p->device);
     if (!g.ok) return ROCKET_ECUDA;

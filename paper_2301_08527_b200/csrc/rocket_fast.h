@@ -56,7 +56,7 @@ struct alignas(16) KRec {
     int32_t len, d, p, m;
     int32_t nout, k, lo_u, hi_u;   // k: original kernel index; lo_u = -p; hi_u = nout - p (exclusive)
     float negb;                    // 0 - bias (never -0.0)
-    int32_t ch[ROCKET_MAX_CHANNELS_PER_KERNEL];
+    int32_t ch[ROCKET_MAX_CHANNELS_PER_KERNEL];   // S regime: positions in the bucket's channel list
     int32_t tl, rl, th, rh;        // lo_u = tl * d + rl and hi_u = th * d + rh with 0 <= rl, rh < d
     int32_t woff;                  // offset of the kernel's weights in the caller's ragged weight array
     int32_t pad_[7];
@@ -71,7 +71,9 @@ static_assert(sizeof(KRec) % 16 == 0, "KRec must be copyable in 16-byte pieces")
 constexpr int kNormMaxChannels = 20;
 struct NormArgs { float mean[kNormMaxChannels], inv_std[kNormMaxChannels]; };
 
-constexpr int kSMaxChannels = 20;                                  // channels the S tile can stage
+constexpr int kSMaxPlanes = 20;                                    // (example, channel) planes the S tile can stage
+constexpr int kF16MaxChannels = 20;                                // what rocket_transform_f16 is documented to take
+constexpr int kMaxChannels = 255;                                  // channels of a series the fused kernels take (stored as bytes)
 // Output rows of a warp tile in the S regime (the band height of its rasters).  More rows per thread than in
 // the T regime: the work per (kernel, tile) grows while the per-kernel bookkeeping and the rows staged per
 // output shrink.  Measured at 60 x 20 x 50,000 (hard): 16 rows 25.7 ms, 20 rows 24.9, 22 rows 24.6, 24 to 26
@@ -87,12 +89,18 @@ static_assert(kRS >= 8 && kRS <= 32, "the row masks of the pooling hold at most 
 constexpr int kSRowsMax = kRS + ROCKET_MAX_LENGTH - 1;             // staged rows an S warp tile reads
 constexpr int kSThreads = ROCKET_S_THREADS, kSWarps = kSThreads / 32;   // one block per SM
 constexpr int kSPlaneFloats = kSRowsMax * kWarpCols;               // one channel of an S tile
+constexpr int kSManyKernels = 32, kSSomeKernels = 8;               // buckets below these share a tile among several examples
 constexpr int kSLengthOrderMin = 100;                              // buckets from this many kernels up are ordered by length
 
+// The kernels of a bucket use at most kSMaxPlanes channels between them: where the kernels of one dilation use more (series
+// of more than 20 channels), they are several buckets.  Their records hold positions in the bucket's channel list.
 struct SBucket {
     int32_t d, tmin, nbands, raster_len;  // raster_len = nbands * d
-    int32_t kbeg, kend, rows, pad_;       // kernels [kbeg, kend) of krec; rows = kRS + max len - 1
+    int32_t kbeg, kend, rows, nch;        // kernels [kbeg, kend) of krec; rows = kRS + max len - 1; channels used
+    uint8_t ch[kSMaxPlanes];              // the channels
+    int32_t pad_[3];
 };
+static_assert(sizeof(SBucket) == 64, "SBucket must be 16 words");
 // One S tile: 64 raster positions from c0 of a bucket.  interior = 1 when every (row, column) of the
 // tile is an output of every kernel of the bucket (then the kernels need no range tests).
 struct SItem { int32_t bucket, c0, interior, pad_; };
@@ -143,7 +151,7 @@ constexpr int kTStageFloats =
 constexpr int kTChunkTiles = 4;                                    // consecutive tiles a block draws at a time
 constexpr int kTWideCols = 256;                                    // columns of one half of a wide tile
 constexpr int kTWideHalves = kTConsumerWarps / 4;                  // a wide tile is one row of all consumer warps' tiles
-constexpr int kChunkExamples = 12;                                // examples per pass through the fused kernels
+constexpr int kChunkExamples = 12;                                // examples per pass through the fused kernels, at least
 constexpr int kTPadFront = 128;                                    // zero floats before every channel row
 constexpr int kTXExtra = 256;                                      // floats a box may run past a 4d run
 
@@ -175,6 +183,8 @@ struct PlanHost {
     std::vector<TMapSpec> tmaps;          // tensor maps the T tiles refer to
     std::vector<int32_t> generic_list;    // kernels the fast path does not take
     int64_t pad_pitch = 0;                // floats per channel row of the zero-margined copy
+    int s_max_nch = 0;                    // most channels of any S bucket
+    int s_class_end[3] = {0, 0, 0};       // S tiles by kernels in their bucket: at least kSManyKernels, kSSomeKernels, fewer
     double flops_s = 0.0, flops_t = 0.0;  // conv flop of one example in either regime
 };
 

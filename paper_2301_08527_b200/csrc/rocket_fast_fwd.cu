@@ -425,13 +425,15 @@ struct FwdArgs {
     long long n_weights;
     float lambda;
     long long x_row_stride;  // floats between the channel rows of X (L, or the pitch of the zero-margined copy)
+    // S kernel: tiles [s_end[i - 1], s_end[i]) are staged for s_examples[i] examples together, as s_groups[i] groups
+    int s_end[3], s_examples[3], s_groups[3];
 };
 
 // ------------------------------------------------------------------------------------------------
 // S regime
 // ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async4_zfill(uint32_t dst, const void* src, bool ok) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0) : "memory");
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, int bytes) {   // bytes: 4, or 0 for a zero
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -482,45 +484,74 @@ __device__ __forceinline__ void s_kernel_tile_h(const float* planes, const KRec*
 
 template <int MODE>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision
 __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
-    float* planes = reinterpret_cast<float*>(smem_raw);                               // [C][kRowsMax][64]
-    KRec* recs = reinterpret_cast<KRec*>(planes + a.C * kSPlaneFloats);                // [warps][2]
+    float* planes = reinterpret_cast<float*>(smem_raw);                               // [kSMaxPlanes][kSRowsMax][64]
+    KRec* recs = reinterpret_cast<KRec*>(planes + kSMaxPlanes * kSPlaneFloats);        // [warps][2]
     __shared__ unsigned s_item;
-    __shared__ int s_next;
+    __shared__ int s_next, s_n0, s_ne;
+    __shared__ SItem s_sitem;
+    __shared__ SBucket s_bucket;
+    __shared__ long long s_src[kSMaxPlanes];      // where the planes' channel rows start in X
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned n_items = (unsigned)a.plan.n_sitems;
-    const unsigned long long total = (unsigned long long)a.N * n_items;
+    // Work is handed out as (tile, group of examples), the tiles of the buckets with many kernels first.  Where a bucket has
+    // few kernels, several examples share a tile's planes, as far as they fit: the warps then find (kernel, example) pairs
+    // enough to keep busy.
+    const unsigned tiles0 = (unsigned)a.s_end[0] * (unsigned)a.s_groups[0], tiles1 = (unsigned)(a.s_end[1] - a.s_end[0]) * (unsigned)a.s_groups[1];
+    const unsigned total = tiles0 + tiles1 + (unsigned)(a.s_end[2] - a.s_end[1]) * (unsigned)a.s_groups[2];
     KRec* myrec = recs + warp * 2;
 
     for (;;) {
         __syncthreads();  // the previous tile is fully consumed
-        if (threadIdx.x == 0) s_item = atomicAdd(a.plan.counters + 0, 1u);
+        if (warp == 0) {  // draw a tile and lay its description out for the block
+            unsigned g = 0;
+            if (lane == 0) g = atomicAdd(a.plan.counters + 0, 1u);
+            g = __shfl_sync(kFull, g, 0);
+            if (lane == 0) { s_item = g; s_next = 0; }
+            if (g < total) {
+                const int cls = g < tiles0 ? 0 : g < tiles0 + tiles1 ? 1 : 2;
+                const unsigned first = cls == 0 ? 0u : (unsigned)a.s_end[cls - 1], count = (unsigned)a.s_end[cls] - first;
+                const unsigned rest = g - (cls == 0 ? 0u : cls == 1 ? tiles0 : tiles0 + tiles1);
+                const int n0 = (int)(rest / count) * a.s_examples[cls], ne = min(a.s_examples[cls], a.N - n0);
+                if (lane == 0) { s_n0 = n0; s_ne = ne; }
+                const SItem it = a.plan.sitems[first + rest % count];
+                const SBucket* __restrict__ src = a.plan.sb + it.bucket;
+                if (lane == 0) s_sitem = it;
+                if (lane < 16) reinterpret_cast<int*>(&s_bucket)[lane] = __ldg(reinterpret_cast<const int*>(src) + lane);
+                const int nch = __ldg(&src->nch), e = lane / nch;
+                if (e < ne) s_src[lane] = ((long long)(n0 + e) * a.C + __ldg(&src->ch[lane - e * nch])) * a.x_row_stride;
+            }
+        }
         __syncthreads();
-        const unsigned g = s_item;
-        if (g >= total) break;
-        const int n = (int)(g / n_items);
-        const SItem item = a.plan.sitems[g - (unsigned)n * n_items];
-        const SBucket b = a.plan.sb[item.bucket];
-        const int d = b.d;
+        if (s_item >= total) break;
+        const int n0 = s_n0, ne = s_ne;
+        const SItem item = s_sitem;
+        const SBucket& b = s_bucket;
+        const int d = b.d, kbeg = b.kbeg, n_work = (b.kend - kbeg) * ne, nch = b.nch;
         const bool tile_interior = item.interior != 0;
-        const float* __restrict__ Xn = a.X + (size_t)n * a.C * a.x_row_stride;
 
-        // stage the tile: every channel, rows 0..rows-1 of every column, zero outside the series
+        // Stage the tile: every plane, rows 0..rows-1 of every column, zero outside the series.  A thread takes one column of
+        // every eighth row; what does not depend on the plane is computed once, so that a sample costs an address and a copy.
         {
+            constexpr int kStep = kSThreads / kWarpCols, kRows = (kSRowsMax + kStep - 1) / kStep;
             const int col = threadIdx.x & (kWarpCols - 1), rg = threadIdx.x / kWarpCols;
             const int cg = item.c0 + col;
             const bool col_ok = cg < b.raster_len;
-            const int fu0 = s_column_u0(b, cg);
-            for (int s = rg; s < b.rows; s += kSThreads / kWarpCols) {
-                const int xi = fu0 + s * d;
-                const bool ok = col_ok && (unsigned)xi < (unsigned)a.L;
-                const float* __restrict__ src = Xn + (ok ? xi : 0);
-                uint32_t dst = smem_u32(planes + s * kWarpCols + col);
+            const int fu0 = s_column_u0(b, cg), n_planes = nch * ne, rows = b.rows;
+            int xi[kRows], bytes[kRows];
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                const int s = rg + i * kStep, x = fu0 + s * d;
+                const bool ok = col_ok && s < rows && (unsigned)x < (unsigned)a.L;
+                xi[i] = ok ? x : 0;
+                bytes[i] = ok ? 4 : 0;
+            }
+            uint32_t dst = smem_u32(planes + rg * kWarpCols + col);
 #pragma unroll 4
-                for (int c = 0; c < a.C; ++c) {
-                    cp_async4_zfill(dst, src, ok);
-                    src += a.x_row_stride;
-                    dst += kSPlaneFloats * 4;
-                }
+            for (int c = 0; c < n_planes; ++c) {
+                const float* __restrict__ src = a.X + s_src[c];
+#pragma unroll
+                for (int i = 0; i < kRows; ++i)
+                    if (rg + i * kStep < rows) cp_async4(dst + i * kStep * kWarpCols * 4, src + xi[i], bytes[i]);
+                dst += kSPlaneFloats * 4;
             }
             cp_async_commit();
         }
@@ -530,15 +561,16 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
         const int band0 = cg0 / d, c0 = cg0 - band0 * d;          // (first A-row, residue) of the two columns
         const int band1 = c0 + 1 < d ? band0 : band0 + 1, c1 = c0 + 1 < d ? c0 + 1 : 0;
         const int trow0 = b.tmin + band0 * kRS, trow1 = b.tmin + band1 * kRS;
-        if (threadIdx.x == 0) s_next = b.kbeg;
         cp_async_wait<0>();
         __syncthreads();
 
-        // kernels of the bucket, pulled from the shared counter; the record of the next kernel is
-        // copied into the warp's other slot while the current one computes
-        auto fetch = [&](int k, int slot) {
-            if (k < b.kend) {
-                const char* src = reinterpret_cast<const char*>(a.plan.krec + k);
+        // (kernel, example) pairs of the bucket, pulled from the shared counter, kernel by kernel; the record of the next
+        // one is copied into the warp's other slot while the current one computes
+        const unsigned inv_ne = (65536u + (unsigned)ne - 1u) / (unsigned)ne;   // several examples only with fewer than 32 kernels
+        auto kernel_of = [&](int w) { return ne == 1 ? w : (int)(((unsigned)w * inv_ne) >> 16); };
+        auto fetch = [&](int w, int slot) {
+            if (w < n_work) {
+                const char* src = reinterpret_cast<const char*>(a.plan.krec + kbeg + kernel_of(w));
                 const uint32_t dst = smem_u32(myrec + slot);
                 for (int i = lane; i < (int)(sizeof(KRec) / 16); i += 32) cp_async16(dst + 16 * i, src + 16 * i);
             }
@@ -549,13 +581,15 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
         kk = __shfl_sync(kFull, kk, 0);
         int cur = 0;
         fetch(kk, cur);
-        while (kk < b.kend) {
+        while (kk < n_work) {
             int kk_next = 0;
             if (lane == 0) kk_next = atomicAdd(&s_next, 1);
             kk_next = __shfl_sync(kFull, kk_next, 0);
             fetch(kk_next, cur ^ 1);
             cp_async_wait<1>();
             __syncwarp();
+            const int example = ne == 1 ? 0 : kk - kernel_of(kk) * ne, n = n0 + example;
+            const float* eplanes = planes + example * nch * kSPlaneFloats;   // the example's planes
             const KRec* rec = myrec + cur;
             const int len = rec->len, korig = rec->k;
             // on an interior tile (the plan's flag) every output exists for every kernel of the bucket
@@ -573,15 +607,15 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
             if constexpr (MODE == 3) {
                 h2 acch[kRS];
                 init_acc_h(acch, rec->negb);
-                if (len == 7) s_kernel_tile_h<7>(planes, rec, lane, acch);
-                else if (len == 9) s_kernel_tile_h<9>(planes, rec, lane, acch);
-                else s_kernel_tile_h<11>(planes, rec, lane, acch);
+                if (len == 7) s_kernel_tile_h<7>(eplanes, rec, lane, acch);
+                else if (len == 9) s_kernel_tile_h<9>(eplanes, rec, lane, acch);
+                else s_kernel_tile_h<11>(eplanes, rec, lane, acch);
                 widen_acc(acch, acc);
             } else {
                 if (!kFold) init_acc(acc, rec->negb, interior, lo0, hi0, lo1, hi1);
-                if (len == 7) s_kernel_tile<7, kFold>(planes, rec, lane, acc);
-                else if (len == 9) s_kernel_tile<9, kFold>(planes, rec, lane, acc);
-                else s_kernel_tile<11, kFold>(planes, rec, lane, acc);
+                if (len == 7) s_kernel_tile<7, kFold>(eplanes, rec, lane, acc);
+                else if (len == 9) s_kernel_tile<9, kFold>(eplanes, rec, lane, acc);
+                else s_kernel_tile<11, kFold>(eplanes, rec, lane, acc);
             }
             if (MODE == 2) {
                 const int64_t pair = (int64_t)n * a.K + korig;
@@ -596,9 +630,9 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
                 for (int sh = 16; sh > 0; sh >>= 1) dbs += __shfl_xor_sync(kFull, dbs, sh);
                 const double scale = __ldg(a.scale + korig);
                 if (lane == 0) add_fixed(a.accfix + a.n_weights + korig, dbs, scale);
-                if (len == 7) s_grad_tile<7>(planes, rec, lane, acc, a.accfix, scale);
-                else if (len == 9) s_grad_tile<9>(planes, rec, lane, acc, a.accfix, scale);
-                else s_grad_tile<11>(planes, rec, lane, acc, a.accfix, scale);
+                if (len == 7) s_grad_tile<7>(eplanes, rec, lane, acc, a.accfix, scale);
+                else if (len == 9) s_grad_tile<9>(eplanes, rec, lane, acc, a.accfix, scale);
+                else s_grad_tile<11>(eplanes, rec, lane, acc, a.accfix, scale);
             } else if (MODE == 1) {
                 const int p = rec->p;
                 pool_publish_soft(a.ws, (int64_t)n * a.K + korig, acc, a.c1, a.c0, interior, lo0, hi0, lo1, hi1,
@@ -1111,7 +1145,7 @@ __global__ void fast_finalize_soft_kernel(float* __restrict__ feat, int32_t* __r
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-size_t s_smem_bytes(int C) { return (size_t)C * kSPlaneFloats * 4 + (size_t)kSWarps * 2 * sizeof(KRec); }
+size_t s_smem_bytes() { return (size_t)kSMaxPlanes * kSPlaneFloats * 4 + (size_t)kSWarps * 2 * sizeof(KRec); }
 size_t t_smem_bytes() { return (size_t)kTGroups * kTGroupSmemBytes + 128; }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1139,19 +1173,19 @@ cudaError_t set_kernel_attributes(int dev) {
     bool& attr_done = attr_done_for[dev & 63];
     const size_t t_bytes = t_smem_bytes();
     if (!attr_done) {
-        e = cudaFuncSetAttribute(fast_s_forward<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(kSMaxChannels));
+        e = cudaFuncSetAttribute(fast_s_forward<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes());
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(kSMaxChannels));
+        e = cudaFuncSetAttribute(fast_s_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes());
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(fast_t_forward<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(fast_t_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(kSMaxChannels));
+        e = cudaFuncSetAttribute(fast_s_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes());
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(fast_t_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(kSMaxChannels));
+        e = cudaFuncSetAttribute(fast_s_forward<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes());
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(fast_t_forward<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
@@ -1216,6 +1250,34 @@ __global__ void fast_bwd_finalize_kernel(const long long* __restrict__ accfix, c
 }
 
 }  // namespace
+
+// Examples per pass through the fused kernels: the four staging copies of a pass stay near what 12 examples of 20 x 50,000
+// take (300 MB); passes of few short series would end in launches with nothing to do for most SMs.  Without T tiles there
+// are no copies and one pass does.
+static int chunk_examples(const FastState& fs, int C, bool copies) {
+    if (!copies) return 1 << 16;
+    return (int)std::max<int64_t>(kChunkExamples, 80000000ll / (4 * (int64_t)C * fs.host.pad_pitch));
+}
+
+// How the S kernel's tiles are shared among examples: one example where a bucket has many kernels, up to 4 and up to 16
+// where it has some or few (64 to 256 pairs per tile for its 16 warps), as far as the planes hold them and the launch keeps two
+// tiles per SM.  Returns the grid.
+static unsigned set_s_groups(FwdArgs& a, const FastState& fs, int sms) {
+    const int fit = kSMaxPlanes / std::max(1, fs.host.s_max_nch);
+    unsigned long long tiles = 0;
+    for (int shift = 0; shift < 5; ++shift) {
+        tiles = 0;
+        for (int cls = 0; cls < 3; ++cls) {
+            const int most = cls == 0 ? 1 : cls == 1 ? 4 : 16;
+            a.s_end[cls] = fs.host.s_class_end[cls];
+            a.s_examples[cls] = std::max(1, std::min({fit, most, a.N}) >> shift);
+            a.s_groups[cls] = (a.N + a.s_examples[cls] - 1) / a.s_examples[cls];
+            tiles += (unsigned long long)(a.s_end[cls] - (cls ? a.s_end[cls - 1] : 0)) * a.s_groups[cls];
+        }
+        if (tiles >= 2ull * sms || a.s_examples[2] == 1) break;
+    }
+    return (unsigned)std::min<unsigned long long>(tiles, (unsigned long long)sms);
+}
 
 // Blocks of the T kernel: as many as are resident at a time, never more than there are work units.
 static unsigned t_grid(int n_examples, int n_titems, int sms) {
@@ -1360,7 +1422,7 @@ cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N,
     if (e != cudaSuccess) return e;
     if ((e = set_kernel_attributes(dev)) != cudaSuccess) return e;
     if (fs.dev.n_titems > 0 || u8) {
-        e = ensure_pad_capacity(fs, std::min(max_N, kChunkExamples), dp.C, dp.L, u8 && fs.dev.n_titems == 0);
+        e = ensure_pad_capacity(fs, std::min(max_N, chunk_examples(fs, dp.C, true)), dp.C, dp.L, u8 && fs.dev.n_titems == 0);
         if (e != cudaSuccess) return e;
     }
     if (soft && (e = ensure_soft_ws(fs, (int64_t)max_N * dp.K)) != cudaSuccess) return e;
@@ -1380,10 +1442,11 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;
-    const size_t s_bytes = s_smem_bytes(dp.C), t_bytes = t_smem_bytes();
+    const size_t s_bytes = s_smem_bytes(), t_bytes = t_smem_bytes();
     const PlanDevice& pd = fs.dev;
+    const int chunk = chunk_examples(fs, dp.C, pd.n_titems > 0 || X_u8);
     if (pd.n_titems > 0 || X_u8) {
-        e = ensure_pad_capacity(fs, std::min(N, kChunkExamples), dp.C, dp.L, X_u8 != nullptr);
+        e = ensure_pad_capacity(fs, std::min(N, chunk), dp.C, dp.L, X_u8 != nullptr);
         if (e != cudaSuccess) return e;
     }
     const int64_t pairs = (int64_t)N * dp.K;
@@ -1400,7 +1463,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     count_launch();
     // the batch goes through in chunks of a few examples: the shifted copies of a chunk are read while
     // they are still in L2, and they stay small
-    const int n_chunks = (N + kChunkExamples - 1) / kChunkExamples;
+    const int n_chunks = (int)(((int64_t)N + chunk - 1) / chunk);
     if (fs.profile) {
         while ((int)fs.evs.size() < 3 * n_chunks) {
             cudaEvent_t ev = nullptr;
@@ -1410,7 +1473,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
         fs.ev_chunks = 0;
     }
     for (int c = 0; c < n_chunks; ++c) {
-        const int n0 = c * kChunkExamples, nc = std::min(kChunkExamples, N - n0);
+        const int n0 = c * chunk, nc = std::min(chunk, N - n0);
         if (X_u8) {   // the kernels read the normalised samples from the unshifted zero-margined copy
             a.X = fs.xpad + kTPadFront;
             a.x_row_stride = fs.host.pad_pitch;
@@ -1435,8 +1498,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
         }
         if (fs.profile) cudaEventRecord(fs.evs[3 * c], stream);
         if (pd.n_sitems > 0) {
-            const unsigned long long total = (unsigned long long)nc * pd.n_sitems;
-            const unsigned grid = (unsigned)std::min<unsigned long long>(total, (unsigned long long)sms);
+            const unsigned grid = set_s_groups(a, fs, sms);
             if (soft) fast_s_forward<1><<<grid, kSThreads, s_bytes, stream>>>(a);
             else if (half) fast_s_forward<3><<<grid, kSThreads, s_bytes, stream>>>(a);
             else fast_s_forward<0><<<grid, kSThreads, s_bytes, stream>>>(a);
@@ -1475,7 +1537,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;
-    const size_t s_bytes = s_smem_bytes(dp.C), t_bytes = t_smem_bytes();
+    const size_t s_bytes = s_smem_bytes(), t_bytes = t_smem_bytes();
     const PlanDevice& pd = fs.dev;
     // workspace: fixed-point sums [n_weights + K], scales [K], max |x| (fixed size per handle)
     const size_t acc_bytes = align256((size_t)(n_weights + dp.K) * 8), scale_bytes = align256((size_t)dp.K * 8);
@@ -1483,8 +1545,9 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     long long* accfix = static_cast<long long*>(fs.bwd_ws);
     double* scale = reinterpret_cast<double*>(static_cast<char*>(fs.bwd_ws) + acc_bytes);
     unsigned* absmax = reinterpret_cast<unsigned*>(static_cast<char*>(fs.bwd_ws) + acc_bytes + scale_bytes);
+    const int chunk = chunk_examples(fs, dp.C, pd.n_titems > 0);
     if (pd.n_titems > 0 && N > 0) {
-        e = ensure_pad_capacity(fs, std::min(N, kChunkExamples), dp.C, dp.L);
+        e = ensure_pad_capacity(fs, std::min(N, chunk), dp.C, dp.L);
         if (e != cudaSuccess) return e;
     }
     e = cudaMemsetAsync(absmax, 0, 256, stream);
@@ -1505,8 +1568,8 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     a.C = dp.C; a.L = dp.L; a.K = dp.K;
     a.accfix = accfix; a.scale = scale; a.n_weights = n_weights; a.lambda = lambda;
     a.x_row_stride = dp.L;
-    for (int n0 = 0; n0 < N; n0 += kChunkExamples) {
-        const int nc = std::min(kChunkExamples, N - n0);
+    for (int n0 = 0; n0 < N; n0 += std::min(chunk, N - n0)) {
+        const int nc = std::min(chunk, N - n0);
         a.X = X + (size_t)n0 * dp.C * dp.L;
         a.dfeat = dfeat + (size_t)n0 * 2 * dp.K;
         a.argmax = argmax + (size_t)n0 * dp.K;
@@ -1515,9 +1578,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         if (e != cudaSuccess) return e;
         if (pd.n_titems > 0) launch_pad_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
         if (pd.n_sitems > 0) {
-            const unsigned long long total = (unsigned long long)nc * pd.n_sitems;
-            const unsigned grid = (unsigned)std::min<unsigned long long>(total, (unsigned long long)sms);
-            fast_s_forward<2><<<grid, kSThreads, s_bytes, stream>>>(a);
+            fast_s_forward<2><<<set_s_groups(a, fs, sms), kSThreads, s_bytes, stream>>>(a);
             count_launch();
         }
         if (pd.n_titems > 0) {

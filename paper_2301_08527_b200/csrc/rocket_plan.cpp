@@ -1,6 +1,7 @@
 // Host-side launch plan of the fast path: buckets kernels by dilation, lays out band rasters,
 // cuts them into tiles and orders the tiles by cost (largest first).
 #include <algorithm>
+#include <climits>
 #include <map>
 #include <tuple>
 
@@ -26,12 +27,18 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
     out = PlanHost();
     out.flops_s = out.flops_t = 0.0;
     if (split < kTMinDilation) split = kTMinDilation;
-    out.split = split;
     const int K = hp.K;
-    // The fast kernels stage at most kSMaxChannels channels in an S tile.  Any series length will do: the
-    // small-dilation kernel copies single floats and the large-dilation kernel reads the zero-margined
-    // copies, whose pitch does not depend on L.
-    const bool shape_ok = hp.C <= kSMaxChannels && hp.L >= 16;
+    // Short series: where every dilation is below 128 the S kernel takes them all, which saves the staging copy and a
+    // launch for a handful of kernels (16 x 1 x 512, 1,000 kernels: 124 -> 90 us).
+    {
+        int d_top = 0;
+        for (int k = 0; k < K; ++k) d_top = std::max(d_top, hp.dilation[k]);
+        if (d_top < 2 * kTMinDilation) split = std::max(split, 2 * kTMinDilation);
+    }
+    out.split = split;
+    // Any series length will do: the small-dilation kernel copies single floats and the large-dilation kernel reads the
+    // zero-margined copies, whose pitch does not depend on L.
+    const bool shape_ok = hp.C <= kMaxChannels && hp.L >= 16;
     std::vector<int> s_kernels, t_kernels;
     for (int k = 0; k < K; ++k) {
         const int len = hp.length[k], d = hp.dilation[k];
@@ -66,7 +73,39 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
     for (int k : s_kernels) by_d[hp.dilation[k]].push_back(k);
     struct Cost { double c; int idx; };
     std::vector<Cost> s_cost;
+    // Kernels of one dilation that use more than kSMaxPlanes channels between them are split: a kernel (most channels
+    // first) joins the group whose channel set grows least, or opens a new one.
+    std::vector<std::pair<int, std::vector<int>>> groups;
     for (auto& kv : by_d) {
+        std::vector<char> used(hp.C, 0);
+        int n_used = 0;
+        for (int k : kv.second)
+            for (int q = hp.channel_offset[k]; q < hp.channel_offset[k] + hp.num_channels[k]; ++q)
+                if (!used[hp.channel_idx[q]]) { used[hp.channel_idx[q]] = 1; ++n_used; }
+        if (n_used <= kSMaxPlanes) {
+            groups.emplace_back(kv.first, std::move(kv.second));
+            continue;
+        }
+        std::stable_sort(kv.second.begin(), kv.second.end(), [&](int a, int b) { return hp.num_channels[a] > hp.num_channels[b]; });
+        struct Group { std::vector<char> has; int n; std::vector<int> ks; };
+        std::vector<Group> gs;
+        for (int k : kv.second) {
+            const int32_t* S = hp.channel_idx.data() + hp.channel_offset[k];
+            int best = -1, best_new = INT_MAX;
+            for (size_t g = 0; g < gs.size(); ++g) {
+                int fresh = 0;
+                for (int q = 0; q < hp.num_channels[k]; ++q) fresh += !gs[g].has[S[q]];
+                if (gs[g].n + fresh <= kSMaxPlanes && fresh < best_new) { best = (int)g; best_new = fresh; }
+            }
+            if (best < 0) { best = (int)gs.size(); gs.push_back({std::vector<char>(hp.C, 0), 0, {}}); }
+            Group& g = gs[best];
+            for (int q = 0; q < hp.num_channels[k]; ++q)
+                if (!g.has[S[q]]) { g.has[S[q]] = 1; ++g.n; }
+            g.ks.push_back(k);
+        }
+        for (Group& g : gs) groups.emplace_back(kv.first, std::move(g.ks));
+    }
+    for (auto& kv : groups) {
         const int d = kv.first;
         auto& ks = kv.second;
         std::stable_sort(ks.begin(), ks.end(), [&](int a, int b) {
@@ -88,6 +127,16 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
             work += (double)f.m * (f.len + 2) + 6.0;
         }
         b.kend = (int32_t)out.krec.size();
+        {   // the bucket's channel list; the records get positions in it
+            std::vector<int> at(hp.C, -1);
+            for (int f = b.kbeg; f < b.kend; ++f)
+                for (int q = 0; q < out.krec[f].m; ++q) at[out.krec[f].ch[q]] = 0;
+            for (int c = 0; c < hp.C; ++c)
+                if (at[c] == 0) { b.ch[b.nch] = (uint8_t)c; at[c] = b.nch++; }
+            for (int f = b.kbeg; f < b.kend; ++f)
+                for (int q = 0; q < out.krec[f].m; ++q) out.krec[f].ch[q] = at[out.krec[f].ch[q]];
+            out.s_max_nch = std::max(out.s_max_nch, b.nch);
+        }
         b.tmin = (int32_t)tmin;
         b.nbands = (int32_t)((tmax - tmin + 1 + kRS - 1) / kRS);
         b.raster_len = b.nbands * d;
@@ -107,7 +156,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
                 const int64_t u0 = s_column_u0(b, c);
                 interior = u0 >= lo_max && u0 + (int64_t)(kRS - 1) * d < hi_min;
             }
-            s_cost.push_back({work + 0.3 * hp.C * b.rows, (int)out.sitems.size()});
+            s_cost.push_back({work + 0.3 * b.nch * b.rows, (int)out.sitems.size()});
             out.sitems.push_back({bi, c0, interior ? 1 : 0, 0});
         }
     }
@@ -115,7 +164,14 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
         std::stable_sort(s_cost.begin(), s_cost.end(), [](const Cost& a, const Cost& b) { return a.c > b.c; });
         std::vector<SItem> sorted;
         sorted.reserve(out.sitems.size());
-        for (auto& c : s_cost) sorted.push_back(out.sitems[c.idx]);
+        for (int cls = 0; cls < 3; ++cls) {
+            for (auto& c : s_cost) {
+                const SBucket& b = out.sb[out.sitems[c.idx].bucket];
+                const int n = b.kend - b.kbeg;
+                if ((n >= kSManyKernels ? 0 : n >= kSSomeKernels ? 1 : 2) == cls) sorted.push_back(out.sitems[c.idx]);
+            }
+            out.s_class_end[cls] = (int)sorted.size();
+        }
         out.sitems.swap(sorted);
     }
 
