@@ -170,6 +170,36 @@ struct alignas(16) TItem {
     int32_t pad1_[2];
 };
 static_assert(sizeof(TItem) == 128, "TItem must be 32 words");
+// ---- stream regime (rocket_stream.cu): the large dilations, one warp per tile ------------------
+#ifndef ROCKET_W_ROWS
+#define ROCKET_W_ROWS 16
+#endif
+constexpr int kWRows = ROCKET_W_ROWS;                              // highest band
+constexpr int kWWarps = kWRows >= 24 ? 12 : 16, kWThreads = 32 * kWWarps;   // independent warps of the one block per SM
+constexpr int kWStages = 2;                                        // (tile, channel) visits in flight per warp
+constexpr int kWStageFloats = (kWRows + ROCKET_MAX_LENGTH - 1 + 3) / 4 * 4 * kWarpCols;   // input rows of a visit, whole y steps
+constexpr int kWCopies = 7;                                        // shifted copies of every channel row, next to one another
+constexpr int kWUnitVisits = 16, kWItemVisits = 32;                // visits of a unit, and of a unit for a group of examples
+constexpr int64_t kWCopyBytes = 800ll << 20;                       // what the copies of a pass may take (13 examples of 20 x 50,000)
+
+// A unit of work: consecutive tiles of one kernel (32 words).  The kernel's output rows from t0 on are cut into bands of R rows,
+// a band into ncol tiles of 64 columns; tile number band * ncol + column group.
+struct alignas(16) WUnit {
+    int32_t krec, map, t0, tile0;         // tile0: the unit's first tile
+    int32_t ntiles, shape, d, m;          // shape: R | len << 8 | row_xor << 16 (stage row of input row s: s ^ row_xor in its four)
+    int32_t k, lo_u, hi_u, p;
+    int32_t tl, rl, th, rh;
+    int32_t nout, woff, ncol, band_y;     // band_y: y steps from band to band
+    int32_t x0, y0, run, copy;            // coordinates of the first column of band 0; floats per y step; first copy
+    uint8_t ch[12];
+    int32_t bytes, pad_[4];               // bytes of a visit's copy
+};
+static_assert(sizeof(WUnit) == 128, "WUnit must be 32 words");
+// One tensor map of the stream regime: boxes of 64 columns x y_rows y steps over the copies, for dilation d.
+struct WMapSpec { int32_t d, y_rows; };
+// Rows per y step: an odd dilation takes four rows (one per alignment) as a dimension of their own, d = 2 mod 4 two.
+ROCKET_CX int w_rows_per_y(int d) { return d % 4 == 0 ? 1 : d % 4 == 2 ? 2 : 4; }
+
 // One tensor map: boxes of box_cols x box_rows floats over runs of 4 * d floats.
 struct TMapSpec { int32_t d, box_cols, box_rows; };
 
@@ -181,6 +211,10 @@ struct PlanHost {
     std::vector<SItem> sitems;
     std::vector<TItem> titems;            // kernel by kernel, in the order the blocks walk them
     std::vector<TMapSpec> tmaps;          // tensor maps the T tiles refer to
+    std::vector<WUnit> wunits;            // stream regime; empty when its copies would need too much room
+    std::vector<WMapSpec> wmaps;
+    double w_visits = 0.0;                // (tile, channel) visits of one example
+    int64_t wfront = 0, wpitch = 0;       // zeros before the first channel row; floats from copy to copy
     std::vector<int32_t> generic_list;    // kernels the fast path does not take
     int64_t pad_pitch = 0;                // floats per channel row of the zero-margined copy
     int s_max_nch = 0;                    // most channels of any S bucket
@@ -193,13 +227,16 @@ struct PlanDevice {
     const SBucket* sb = nullptr;
     const SItem* sitems = nullptr;
     const TItem* titems = nullptr;
+    const WUnit* wunits = nullptr;
+    const void* wmaps = nullptr;          // CUtensorMap[n_wmaps]
     const int32_t* generic_list = nullptr;
     unsigned* counters = nullptr;         // [0] S work counter, [1] T work counter
     int* error_flag = nullptr;            // set when a bounded wait gave up
     const void* tmaps = nullptr;          // CUtensorMap[n_tmaps], 128 bytes each
     float* xpad = nullptr;                // zero-margined copy of the batch
     int64_t pad_pitch = 0;
-    int n_krec = 0, n_sitems = 0, n_titems = 0, n_generic = 0, n_tmaps = 0;
+    int n_krec = 0, n_sitems = 0, n_titems = 0, n_generic = 0, n_tmaps = 0, n_wunits = 0;
+    double w_visits = 0.0;                // (tile, channel) visits of one example in the stream kernel
 };
 
 // Writes kernel f.k's bias and weights (negated, every weight twice) into its record.
@@ -220,6 +257,9 @@ struct FastState {
     float* xpad = nullptr;                // the four shifted zero-margined copies, capacity pad_examples
     int pad_examples = 0;
     int64_t copy_floats = 0;              // floats of one copy
+    float* wpad = nullptr;                // stream regime: the seven shifted copies, capacity wpad_examples
+    int wpad_examples = 0;
+    void* wmaps_blob = nullptr;
     void* soft_ws = nullptr;              // soft mode: 16 bytes per (example, kernel), grows with N
     size_t soft_ws_bytes = 0;
     void* bwd_ws = nullptr;               // backward: fixed-point sums [n_weights + K], scales [K], max |x|
@@ -232,6 +272,8 @@ struct FastState {
 cudaError_t upload_plan(FastState& fs);
 // Frees everything upload_plan / ensure_pad_capacity allocated.
 void release_fast_state(FastState& fs);
+// The same for the stream regime's copies.
+cudaError_t ensure_stream_capacity(FastState& fs, int N, int C, int L);
 // Makes the padded copy hold N examples and (re-)encodes the tensor maps over it.
 cudaError_t ensure_pad_capacity(FastState& fs, int N, int C, int L, bool without_maps = false);
 

@@ -2,6 +2,7 @@
 // cuts them into tiles and orders the tiles by cost (largest first).
 #include <algorithm>
 #include <climits>
+#include <functional>
 #include <map>
 #include <tuple>
 
@@ -13,6 +14,88 @@ namespace fast {
 namespace {
 
 inline int64_t floor_div(int64_t a, int64_t b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
+
+// Units of the stream kernel for the kernels whose records start at `first`.  The output rows of a kernel (their count rounded
+// up to four) become bands of 24, 16, 12 and 8 rows.  Units of one shape follow one another and within a shape in order of
+// dilation, so that the warps running at any one time share an instance of the inner loop and mostly a tensor map.
+void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost& out) {
+    if (first == out.krec.size()) return;
+    // Positions a box can reach beyond the samples: three rows before them, seven after (a y step is four rows, of which the
+    // last may start three rows further on).  Dilations of random kernels stay below L / 6; handles with larger ones keep the
+    // kernel that works on the four copies.
+    if (7ll * d_max > 2ll * hp.L + 4096) return;
+    out.wfront = (3ll * d_max + 64 + 3) / 4 * 4;
+    out.wpitch = (hp.L + std::max<int64_t>(7ll * d_max + 96, out.wfront) + 31) / 32 * 32;
+    std::vector<int> order;
+    int64_t visits = 0;
+    for (size_t f = first; f < out.krec.size(); ++f) {
+        const KRec& k = out.krec[f];
+        order.push_back((int)f);
+        visits += ((int64_t)(k.nout / ((int64_t)16 * k.d)) + 1) * ((k.d + kWarpCols - 1) / kWarpCols) * k.m;
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return out.krec[a].d < out.krec[b].d; });
+    // short units where there is little work per warp (148 x 16 of them), so that the warps end together
+    const int64_t unit_visits = std::min<int64_t>(kWUnitVisits, std::max<int64_t>(6, visits / (16 * 148 * kWWarps)));
+    // Heights for a count of rows (a multiple of four): the fewest rows, where a band costs as much as three rows on top.
+    struct Choice { int cost, R; };
+    std::vector<Choice> choice(1, {0, 0});
+    auto choose = [&](int64_t rows4) {
+        while ((int64_t)choice.size() <= rows4) {
+            const int t = (int)choice.size();
+            Choice best{INT_MAX, 0};
+            for (int R : {24, 16, 12, 8}) {
+                if (R > kWRows) continue;
+                const int rest = std::max(0, t - R / 4), cost = choice[rest].cost + R + 3;
+                if (cost < best.cost) best = {cost, R};
+            }
+            choice.push_back(best);
+        }
+        return choice[rows4].R;
+    };
+    std::map<int, std::vector<WUnit>, std::greater<int>> by_shape;   // longest kernels first, then highest bands
+    std::map<std::pair<int, int>, int> map_index;
+    for (int fi : order) {
+        const KRec& f = out.krec[fi];
+        const int64_t tmin = floor_div(f.lo_u, f.d), tmax = floor_div((int64_t)f.hi_u - 1, f.d);
+        int64_t rows = (tmax - tmin + 1 + 3) / 4 * 4;
+        const int G = w_rows_per_y(f.d), ncol = (f.d + kWarpCols - 1) / kWarpCols;
+        for (int64_t t = tmin; rows > 0;) {
+            // the bands of the highest kind that pays, all at once
+            const int R = choose(std::min<int64_t>(rows, 4096) / 4);
+            int64_t n = 1;
+            while (rows - n * R > 0 && choose(std::min<int64_t>(rows - n * R, 4096) / 4) == R) ++n;
+            out.w_visits += (double)n * ncol * f.m;
+            WUnit u{};
+            u.krec = fi; u.t0 = (int32_t)t; u.d = f.d; u.m = f.m; u.k = f.k; u.lo_u = f.lo_u; u.hi_u = f.hi_u; u.p = f.p;
+            u.tl = f.tl; u.rl = f.rl; u.th = f.th; u.rh = f.rh; u.nout = f.nout; u.woff = f.woff; u.ncol = ncol;
+            const int y_rows = (R + f.len - 1 + G - 1) / G;
+            const auto found = map_index.emplace(std::make_pair(f.d, y_rows), (int)out.wmaps.size());
+            if (found.second) out.wmaps.push_back({f.d, y_rows});
+            u.map = found.first->second;
+            u.bytes = y_rows * G * kWarpCols * 4;
+            u.run = G * f.d;
+            u.band_y = R / G;
+            // first row of a y step: the last of its four when they are taken backwards
+            const bool backwards = f.d % 4 == 3;
+            const int64_t pos = out.wfront + t * f.d + (backwards ? 3ll * f.d : 0);
+            u.copy = (int32_t)(pos & 3);
+            const int64_t start = pos - u.copy, y = floor_div(start, u.run);
+            u.x0 = (int32_t)(start - y * u.run);
+            u.y0 = (int32_t)y;
+            u.shape = R | f.len << 8 | (backwards ? 3 << 16 : 0);
+            for (int q = 0; q < f.m; ++q) u.ch[q] = (uint8_t)f.ch[q];
+            const int64_t tiles = n * ncol, per = std::max<int64_t>(1, unit_visits / f.m), units = (tiles + per - 1) / per;
+            for (int64_t i = 0; i < units; ++i) {
+                const int64_t beg = tiles * i / units, end = tiles * (i + 1) / units;
+                u.tile0 = (int32_t)beg; u.ntiles = (int32_t)(end - beg);
+                by_shape[(f.len << 8) | R].push_back(u);
+            }
+            rows -= n * R;
+            t += n * R;
+        }
+    }
+    for (auto& kv : by_shape) out.wunits.insert(out.wunits.end(), kv.second.begin(), kv.second.end());
+}
 
 }  // namespace
 
@@ -186,6 +269,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
     std::stable_sort(t_kernels.begin(), t_kernels.end(), [&](int a, int b) {
         return hp.length[a] != hp.length[b] ? hp.length[a] > hp.length[b] : hp.dilation[a] < hp.dilation[b];
     });
+    const size_t first_t = out.krec.size();
     for (int k : t_kernels) {
         const int ki = (int)out.krec.size();
         add_kernel(k);
@@ -303,6 +387,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
             }
         }
     }
+    build_stream_units(hp, first_t, d_max, out);
     // every channel row of the zero-margined copy: front zeros, L samples, zeros for the run a box may
     // read past the last sample; rounded to 128 bytes
     const int64_t pitch = (int64_t)kTPadFront + hp.L + 4ll * d_max + kTXExtra + t_box_cols(4);

@@ -1,0 +1,444 @@
+// Fused kernel of the large dilations: every warp streams its own tiles.
+//
+// With u = t d + r a dilated convolution is a dense filter down the columns of A[t][r] = x[t d + r].  A warp's tile is R rows
+// (16, 12 or 8) x 64 columns of outputs of one kernel; a thread owns two neighbouring columns, R packed accumulators.  The
+// kernel's channels come one after the other: the R + len - 1 input rows of a channel are ONE tiled bulk copy into the warp's
+// own shared memory (two stages of 7 KB per warp), issued by one of its lanes as soon as the stage has been read for the last
+// time, two (tile, channel) visits ahead, across tiles and units of work.  A warp waits on its own barriers only: no block
+// barrier, no producer warp, no other warp's pace.
+//
+// Why: kernels of large dilation share no samples worth sharing, so a block-wide tile only couples its warps.  The earlier form
+// (a producer warp, eight consumer warps behind a two-stage ring, 128 x 64 tiles; rocket_fast_fwd.cu) spent 16 of its 34 ms
+// outside the multiplications - doing them twice cost 18 ms more - because a stage is free only when the slowest warp has read
+// it, and 28 % (20 x 50,000) to 45 % (20 x 5,000) of the products lay outside a kernel's rows and columns.  Bytes: a visit
+// brings R + len - 1 rows for R rows of outputs, 0.65 B per multiply-add, 55 B/clk/SM at the rate reached; bulk copies of
+// this size deliver 75.  Heights of 16, 12 and 8 rows fit the output range to four rows.
+//
+// One copy for all rows of a tile: row s starts at position P + s d of the zero-margined row, and a bulk copy needs 16-byte
+// aligned starts.  The rows exist in seven copies, copy j moved down by j floats, one after the other per channel row, so
+// "next copy" is a stride like any other: for an odd dilation rows s = 4 y + i with i = 0..3 are a tensor dimension of stride
+// pitch + d - 1 (d = 1 mod 4) or, counted backwards, pitch - d - 1 (d = 3 mod 4), and y one of stride 4 d; for d = 2 mod 4 rows
+// come in pairs, for d = 0 mod 4 one by one.  Rows before the first and after the last y that holds samples are filled with
+// zeros by the copy engine.
+#include <algorithm>
+
+#include "rocket_fast.h"
+#include "rocket_fast_dev.cuh"
+#include "rocket_fast_geom.h"
+
+namespace rocket {
+namespace fast {
+namespace {
+
+extern __shared__ __align__(128) unsigned char smem_raw[];
+
+static_assert(kWStages == 2, "the producer runs less than a whole unit of one visit ahead");
+
+struct StreamArgs {
+    FwdArgs f;
+    const WUnit* units;
+    int n_units;
+    const void* maps;
+    int examples, groups, groups_per_set;   // examples of an item; groups of examples of the pass; groups handed out together
+};
+
+// The inner loop: one channel of a warp tile, weights handed round from lane j (conv_channel with the weight already loaded).
+template <int ELL, int R>
+__device__ __forceinline__ void stream_conv(const float* __restrict__ st, const int (&off)[4], float mine, u64 (&acc)[R]) {
+    u64 wp[ELL];
+#pragma unroll
+    for (int j = 0; j < ELL; ++j) {
+        const float w = __shfl_sync(kFull, mine, j);
+        wp[j] = pack2(w, w);
+    }
+#pragma unroll
+    for (int s = 0; s < R + ELL - 1; ++s) {
+        const u64 x = *reinterpret_cast<const u64*>(st + off[s & 3] + (s >> 2) * (4 * kWarpCols));
+#pragma unroll
+        for (int j = 0; j < ELL; ++j) {
+            const int o = s - j;
+            if (o >= 0 && o < R) fma2(acc[o], wp[j], x);
+        }
+    }
+}
+template <int ELL, int R>
+__device__ __forceinline__ void stream_conv(const float* __restrict__ st, const int (&off)[4], float mine, h2 (&acc)[R]) {
+    const h2 mh = to_h2(mine, mine);
+    h2 wp[ELL];
+#pragma unroll
+    for (int j = 0; j < ELL; ++j) wp[j] = __shfl_sync(kFull, mh, j);
+#pragma unroll
+    for (int s = 0; s < R + ELL - 1; ++s) {
+        const float2 xf = *reinterpret_cast<const float2*>(st + off[s & 3] + (s >> 2) * (4 * kWarpCols));
+        const h2 x = to_h2(xf.x, xf.y);
+#pragma unroll
+        for (int j = 0; j < ELL; ++j) {
+            const int o = s - j;
+            if (o >= 0 && o < R) hfma2(acc[o], wp[j], x);
+        }
+    }
+}
+
+// What a lane carries from tile to tile of a unit.
+struct Carry {
+    int cnt;          // hard: outputs above zero
+    float mn;         // hard, soft: min of -z
+    u64 hsum;         // soft: sum of h, fixed point
+    int idx;          // soft: lowest output index attaining the max
+    long long db;     // backward: sum of gz, fixed point
+};
+
+// Soft pooling of a tile into the lane's state (the sum as a fixed-point integer: exact and order-free from here on).
+template <int R>
+__device__ __forceinline__ void pool_soft_lane(const u64 (&acc)[R], float c1, float c0, bool interior, unsigned m0, unsigned m1, int base,
+                                               int step, Carry& st) {
+    const u64 c1p = pack2(c1, c1), c0p = pack2(c0, c0), one = pack2(1.0f, 1.0f);
+    u64 hs = pack2(0.0f, 0.0f);
+    float mt = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int o = 0; o < R; ++o) {
+        u64 t = c0p;
+        fma2(t, acc[o], c1p);
+        float ta, tb, a, b;
+        unpack2(t, ta, tb);
+        const u64 den = add2(pack2(ex2_approx(ta), ex2_approx(tb)), one);
+        unpack2(den, ta, tb);
+        float ha = rcp_approx(ta), hb = rcp_approx(tb);
+        if (!interior) {
+            if (!(m0 & (1u << o))) ha = 0.0f;
+            if (!(m1 & (1u << o))) hb = 0.0f;
+        }
+        hs = add2(hs, pack2(ha, hb));
+        unpack2(acc[o], a, b);
+        mt = min3(mt, a, b);
+    }
+    float h0, h1;
+    unpack2(hs, h0, h1);
+    st.hsum += __float2ull_rn((h0 + h1) * kSoftFixedScale);
+    if (mt <= st.mn && mt < __int_as_float(0x7f800000)) {
+        int idx = INT_MAX;
+#pragma unroll
+        for (int o = R - 1; o >= 0; --o) {
+            float a, b;
+            unpack2(acc[o], a, b);
+            if (b == mt) idx = min(idx, base + 1 + o * step);
+            if (a == mt) idx = min(idx, base + o * step);
+        }
+        if (mt < st.mn || idx < st.idx) st.idx = idx;
+        st.mn = mt;
+    }
+}
+
+__device__ __forceinline__ void publish_soft(unsigned long long* __restrict__ ws, int64_t pair, const Carry& st, int lane) {
+    u64 hsum = st.hsum;
+#pragma unroll
+    for (int sh = 16; sh > 0; sh >>= 1) hsum += __shfl_xor_sync(kFull, hsum, sh);
+    const int key = float_key(-st.mn), wkey = __reduce_max_sync(kFull, key);
+    const int idx = __reduce_min_sync(kFull, key == wkey ? st.idx : INT_MAX);
+    if (lane == 0) {
+        atomicAdd(ws + 2 * pair, hsum);
+        const unsigned long long k64 = ((unsigned long long)((unsigned)wkey ^ 0x80000000u) << 32) |
+                                       (unsigned long long)(unsigned)(INT_MAX - idx);
+        atomicMax(ws + 2 * pair + 1, k64);
+    }
+}
+
+// The rest of a wait that did not succeed at once (out of line: the fast path is one test).
+__device__ __noinline__ bool stream_wait_slow(uint32_t bar, uint32_t parity) { return mbar_wait(bar, parity); }
+
+// Announces `bytes` on the barrier and starts the copy of one box, by one lane (lead != 0), without a branch.
+__device__ __forceinline__ void stream_copy_box(int lead, uint32_t dst, const void* tmap, int x, int y, int w, uint32_t bar, uint32_t bytes) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.s32 p, %0, 0;\n\t"
+        "@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%6], %7;\n\t"
+        "@p cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%1], [%2, {%3, 0, %4, %5}], [%6];\n\t}"
+        ::"r"(lead), "r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(w), "r"(bar), "r"(bytes) : "memory");
+}
+
+template <int MODE>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision
+__global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constant__ StreamArgs a) {
+    __shared__ unsigned long long s_bar[kWWarps][kWStages];
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    const uint32_t raw = smem_u32(smem_raw);
+    float* stages = reinterpret_cast<float*>(smem_raw + (((raw + 127u) & ~127u) - raw)) + warp * kWStages * kWStageFloats;
+    const uint32_t stages0 = smem_u32(stages), bar0 = smem_u32(s_bar[warp]);
+    if (lane == 0) {
+        for (int i = 0; i < kWStages; ++i) mbar_init(bar0 + 8u * i, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+
+    // An item of work is a unit for a group of examples.  Items run over the groups of a set (whose copies stay in L2) for
+    // one unit, then over the units, then over the sets: the warps of a moment share a unit, its inner loop, weights and
+    // tensor map.  The first item of a warp goes by its place, the others by a counter.  v, vn: the unit at work and the next
+    // one, a word per lane (all zero past the last); drawn: the number of the item after that.
+    const unsigned n_units = (unsigned)a.n_units, total = (unsigned)a.groups * n_units, warps = gridDim.x * kWWarps;
+    unsigned* counter = a.f.plan.counters + 1;
+    auto item = [&](unsigned g, int& n0) {             // unit of item g, and its first example
+        const unsigned per_set = (unsigned)a.groups_per_set * n_units, set = g / per_set, rest = g - set * per_set;
+        const unsigned first = set * (unsigned)a.groups_per_set, in_set = min((unsigned)a.groups_per_set, (unsigned)a.groups - first);
+        const unsigned unit = rest / in_set;
+        n0 = (int)(first + rest - unit * in_set) * a.examples;
+        return unit;
+    };
+    auto load_unit = [&](unsigned g, int& n0) {
+        n0 = 0;
+        if (g >= total) return 0;
+        return __ldg(reinterpret_cast<const int*>(a.units + item(g, n0)) + lane);
+    };
+    unsigned g = (unsigned)warp * gridDim.x + blockIdx.x, gn = 0, drawn = 0;
+    if (g >= total) return;
+    if (lane == 0) gn = warps + atomicAdd(counter, 1u);
+    int n0, nn0;                                       // first example of v and of vn
+    int v = load_unit(g, n0);
+    if (lane == 0) drawn = warps + atomicAdd(counter, 1u);
+    gn = __shfl_sync(kFull, gn, 0);
+    int vn = load_unit(gn, nn0);
+
+    // ---- producer side: issues the copy of one visit, two visits ahead of the multiplications, into the stage just read
+    int pv = v, p_q = 0, p_visits = 0;                 // its unit's words; visit of the tile, visits per tile
+    int p_tiles = 0, p_examples = 0;                   // tiles left of the example, examples left of the item
+    int p_x = 0, p_y = 0, p_col = 0, p_rows = 0;       // box of the tile; lane q: copy row of channel q (of the q-th visit)
+    uint32_t p_bytes = 0;
+    const char* p_map = nullptr;
+    auto pfield = [&](int i) { return __shfl_sync(kFull, pv, i); };
+    auto p_tile = [&](int tile) {                      // the box of tile number `tile`
+        const int ncol = pfield(18), band = tile / ncol, run = pfield(22);
+        p_col = tile - band * ncol;
+        p_x = pfield(20) + kWarpCols * p_col;
+        p_y = pfield(21) + band * pfield(19);
+        while (p_x >= run) { p_x -= run; ++p_y; }
+    };
+    auto aim = [&](int first) {                        // the unit in pv, from example `first` on; false: there is none
+        const int m = pfield(7);
+        if (m == 0) return false;
+        p_visits = MODE == 2 ? 2 * m : m;              // the backward takes the channels twice
+        p_q = 0;
+        p_tiles = pfield(4);
+        p_examples = min(a.examples, a.f.N - first);
+        p_bytes = (uint32_t)pfield(27);
+        const int q = MODE == 2 && lane >= m ? lane - m : lane;
+        p_rows = (first * a.f.C + ((__shfl_sync(kFull, pv, 24 + ((q & 15) >> 2)) >> (8 * (q & 3))) & 0xff)) * kWCopies + pfield(23);
+        p_tile(pfield(3));
+        p_map = reinterpret_cast<const char*>(a.maps) + (size_t)pfield(1) * 128;
+        return true;
+    };
+    auto advance = [&]() {                             // to the next tile; false when no work is left
+        p_q = 0;
+        if (--p_tiles > 0) {
+            p_x += kWarpCols;
+            if (++p_col == pfield(18)) p_tile(pfield(3) + pfield(4) - p_tiles);
+            const int run = pfield(22);
+            while (p_x >= run) { p_x -= run; ++p_y; }
+            return true;
+        }
+        if (--p_examples > 0) {
+            p_tiles = pfield(4);
+            p_rows += a.f.C * kWCopies;
+            p_tile(pfield(3));
+            return true;
+        }
+        pv = vn;
+        if (aim(nn0)) return true;
+        p_visits = 0;                                  // asked again after every visit that is left
+        p_tiles = p_examples = 1;
+        return false;
+    };
+    auto issue = [&](uint32_t slot) {
+        if (p_q == p_visits && !advance()) return;
+        const int w = __shfl_sync(kFull, p_rows, p_q);
+        stream_copy_box(lane == 0, stages0 + slot * (kWStageFloats * 4), p_map, p_x, p_y, w, bar0 + 8u * slot, p_bytes);
+        ++p_q;
+    };
+    aim(n0);
+    issue(0);
+    issue(1);
+
+    uint32_t st = 0;                                   // visits consumed: stage st & 1, parity st >> 1 & 1
+    bool ok = true;
+    auto wait = [&]() {
+        const uint32_t bar = bar0 + 8u * (st & 1u), parity = (st >> 1) & 1u;
+        return mbar_try(bar, parity) || stream_wait_slow(bar, parity);
+    };
+    const int weight_lane = 2 * min(lane, ROCKET_MAX_LENGTH - 1);
+    int krec = __shfl_sync(kFull, v, 0);
+    float w_first = __ldg(&a.f.plan.krec[krec].w2[0][0] + weight_lane), negb = __ldg(&a.f.plan.krec[krec].negb);
+    while (g < total) {
+        auto field = [&](int i) { return __shfl_sync(kFull, v, i); };
+        const int t0 = field(2), tile0 = field(3), ntiles = field(4), shape = field(5), d = field(6), m = field(7), k = field(8);
+        const int ncol = field(18), R = shape & 0xff, len = (shape >> 8) & 0xff, row_xor = shape >> 16;
+        const float* __restrict__ wl = &a.f.plan.krec[krec].w2[0][0] + weight_lane;
+        const int off[4] = {(0 ^ row_xor) * kWarpCols + 2 * lane, (1 ^ row_xor) * kWarpCols + 2 * lane,
+                            (2 ^ row_xor) * kWarpCols + 2 * lane, (3 ^ row_xor) * kWarpCols + 2 * lane};
+        const int examples = min(a.examples, a.f.N - n0), band0 = tile0 / ncol, col0 = tile0 - band0 * ncol;
+        int next_krec = 0;
+        float w_first_n = 0.0f, negb_n = 0.0f;
+        Carry carry{0, __int_as_float(0x7f800000), 0ull, INT_MAX, 0ll};
+        const double scale = MODE == 2 ? __ldg(a.f.scale + k) : 0.0;
+        for (int e = 0; e < examples && ok; ++e) {
+            const int64_t pair = (int64_t)(n0 + e) * a.f.K + k;
+            float gP = 0.0f, gM = 0.0f;
+            int tA = 0, cA = 0;
+            if (MODE == 2) {
+                gP = __ldg(a.f.dfeat + 2 * pair) * a.f.lambda / (float)field(16);
+                gM = __ldg(a.f.dfeat + 2 * pair + 1);
+                const int uA = __ldg(a.f.argmax + pair) - field(11);
+                tA = uA / d;                           // floor division: uA >= -p may be negative
+                cA = uA - tA * d;
+                if (cA < 0) { cA += d; --tA; }
+            }
+            int col = col0, trow = t0 + band0 * R;
+            for (int t = 0; t < ntiles; ++t) {
+                const bool last = t + 1 == ntiles && e + 1 == examples;      // of the item
+                // the tile's channels, then its pooling; false when a wait gave up
+                auto tile = [&](auto len_tag, auto r_tag) {
+                    constexpr int ELL = decltype(len_tag)::value, RR = decltype(r_tag)::value;
+                    const int c0 = col * kWarpCols, c = c0 + 2 * lane;
+                    const bool interior = c0 + kWarpCols <= d && trow * d + c0 >= field(9) &&
+                                          (trow + RR - 1) * d + c0 + kWarpCols - 1 < field(10);
+                    int lo0 = 0, hi0 = RR, lo1 = 0, hi1 = RR;
+                    if (!interior) {
+                        const int tl = field(12), rl = field(13), th = field(14), rh = field(15);
+                        valid_rows_tc(trow, c, tl, rl, th, rh, RR, c < d, lo0, hi0);
+                        valid_rows_tc(trow, c + 1, tl, rl, th, rh, RR, c + 1 < d, lo1, hi1);
+                    }
+                    u64 acc[RR];
+                    [[maybe_unused]] h2 acch[RR];
+                    if constexpr (MODE == 3) init_acc_h(acch, negb);
+                    else init_acc(acc, negb, interior || MODE == 0, lo0, hi0, lo1, hi1);
+                    float mine = w_first;
+                    for (int q = 0; q < m; ++q) {
+                        const float mine_next = __ldg(wl + min(q + 1, m - 1) * kPairRow);
+                        if (!wait()) return false;
+                        const uint32_t slot = st & 1u;
+                        const float* stage = stages + slot * kWStageFloats;
+                        if constexpr (MODE == 3) stream_conv<ELL, RR>(stage, off, mine, acch);
+                        else stream_conv<ELL, RR>(stage, off, mine, acc);
+                        mine = mine_next;
+                        __syncwarp();                  // the stage has been read by every lane
+                        ++st;
+                        if (MODE == 2 || !last || q + 1 < m) issue(slot);
+                    }
+                    if constexpr (MODE == 3) widen_acc(acch, acc);
+                    if constexpr (MODE == 2) {
+                        const bool hit = tA >= trow && tA < trow + RR;
+                        const float dbs = make_gz(acc, a.f.c1, a.f.c0, gP, gM, interior, lo0, hi0, lo1, hi1,
+                                                  hit && c < d && c == cA ? tA - trow : -1, hit && c + 1 < d && c + 1 == cA ? tA - trow : -1);
+                        carry.db += __double2ll_rn((double)dbs * scale);
+                        for (int q = 0; q < m; ++q) {
+                            if (!wait()) return false;
+                            const uint32_t slot = st & 1u;
+                            u64 dw[ELL];
+#pragma unroll
+                            for (int j = 0; j < ELL; ++j) dw[j] = 0ull;
+                            grad_channel<ELL, 4 * kWarpCols, false, RR>(stages + slot * kWStageFloats, off, acc, dw);
+                            __syncwarp();
+                            ++st;
+                            if (!last || q + 1 < m) issue(slot);
+                            reduce_publish_dw<ELL>(dw, a.f.accfix + field(17) + q * ELL, scale, lane);
+                        }
+                    } else if constexpr (MODE == 1) {
+                        pool_soft_lane<RR>(acc, a.f.c1, a.f.c0, interior, row_mask(lo0, hi0), row_mask(lo1, hi1), trow * d + c + field(11), d,
+                                           carry);
+                    } else {
+                        if (interior) pool_hard(acc, carry.cnt, carry.mn);
+                        else pool_hard_masked(acc, row_mask(lo0, hi0), row_mask(lo1, hi1), carry.cnt, carry.mn);
+                    }
+                    return true;
+                };
+                auto by_rows = [&](auto len_tag) {
+#if ROCKET_W_ROWS >= 24
+                    if (R == 24) return tile(len_tag, std::integral_constant<int, 24>{});
+#endif
+                    if (R == 16) return tile(len_tag, std::integral_constant<int, 16>{});
+                    if (R == 12) return tile(len_tag, std::integral_constant<int, 12>{});
+                    return tile(len_tag, std::integral_constant<int, 8>{});
+                };
+                ok = len == 7 ? by_rows(std::integral_constant<int, 7>{}) : len == 9 ? by_rows(std::integral_constant<int, 9>{})
+                                                                                    : by_rows(std::integral_constant<int, 11>{});
+                if (!ok) break;
+                if (++col == ncol) { col = 0; trow += R; }
+            }
+            if (!ok) break;
+            if (e == 0) {                              // what the next unit needs first is on its way
+                next_krec = __shfl_sync(kFull, vn, 0);
+                w_first_n = __ldg(&a.f.plan.krec[next_krec].w2[0][0] + weight_lane);
+                negb_n = __ldg(&a.f.plan.krec[next_krec].negb);
+            }
+            if (e + 1 < examples && MODE != 2) {
+                if (MODE == 1) publish_soft(a.f.ws, pair, carry, lane);
+                else publish(a.f.feat_i, pair, carry.cnt, carry.mn, lane);
+                carry = Carry{0, __int_as_float(0x7f800000), 0ull, INT_MAX, 0ll};
+            }
+        }
+        if (!ok) break;
+        // the next item takes over, and the visit that this one's last still owes is issued
+        const int64_t last_pair = (int64_t)(n0 + examples - 1) * a.f.K + k;
+        v = vn;
+        g = gn;
+        n0 = nn0;
+        krec = next_krec;
+        w_first = w_first_n;
+        negb = negb_n;
+        gn = __shfl_sync(kFull, drawn, 0);
+        vn = load_unit(gn, nn0);
+        if (lane == 0) drawn = warps + atomicAdd(counter, 1u);
+        issue((st - 1u) & 1u);
+        if (MODE == 1) {
+            publish_soft(a.f.ws, last_pair, carry, lane);
+        } else if (MODE == 2) {
+            long long db = carry.db;
+#pragma unroll
+            for (int sh = 16; sh > 0; sh >>= 1) db += __shfl_xor_sync(kFull, db, sh);
+            if (lane == 0) atomicAdd(reinterpret_cast<unsigned long long*>(a.f.accfix + a.f.n_weights + k), (unsigned long long)db);
+        } else {
+            publish(a.f.feat_i, last_pair, carry.cnt, carry.mn, lane);
+        }
+    }
+    if (!ok) {
+        // a wait gave up: the results are incomplete, and nothing of this warp may be in flight when the block ends
+        if (lane == 0) atomicExch(a.f.plan.error_flag, 1);
+        for (int i = 0; i < kWStages; ++i, ++st) stream_wait_slow(bar0 + 8u * (st & 1u), (st >> 1) & 1u);
+    }
+}
+
+size_t stream_smem_bytes() { return (size_t)kWWarps * kWStages * kWStageFloats * sizeof(float) + 128; }
+
+}  // namespace
+
+cudaError_t set_stream_attributes() {
+    const int bytes = (int)stream_smem_bytes();
+    cudaError_t e = cudaFuncSetAttribute(fast_stream<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fast_stream<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fast_stream<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fast_stream<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e;
+}
+
+void launch_stream(const FwdArgs& f, int mode, int sms, cudaStream_t stream) {
+    StreamArgs a;
+    a.f = f;
+    a.units = f.plan.wunits;
+    a.n_units = f.plan.n_wunits;
+    a.maps = f.plan.wmaps;
+    // Examples of an item: as many as give it kWItemVisits visits on average, while every warp of the chip still gets a
+    // dozen items.  Examples handed out together: as many as keep their copies in a third of the L2.
+    const double per_unit = std::max(1.0, f.plan.w_visits * (mode == 2 ? 2.0 : 1.0) / std::max(1, a.n_units));
+    const long long most = (long long)f.N * a.n_units / ((long long)sms * kWWarps * 12);
+    a.examples = (int)std::max<long long>(1, std::min<long long>({(long long)(kWItemVisits / per_unit), most, (long long)f.N}));
+    a.groups = (f.N + a.examples - 1) / a.examples;
+    const long long example_bytes = (long long)f.C * kWCopies * f.L * 4;
+    a.groups_per_set = (int)std::max<long long>(1, std::min<long long>(a.groups, (40ll << 20) / (example_bytes * a.examples)));
+    const unsigned long long items = (unsigned long long)a.groups * (unsigned long long)a.n_units;
+    const unsigned grid = (unsigned)std::min<unsigned long long>((items + kWWarps - 1) / kWWarps, (unsigned long long)sms);
+    const size_t bytes = stream_smem_bytes();
+    if (mode == 1) fast_stream<1><<<grid, kWThreads, bytes, stream>>>(a);
+    else if (mode == 2) fast_stream<2><<<grid, kWThreads, bytes, stream>>>(a);
+    else if (mode == 3) fast_stream<3><<<grid, kWThreads, bytes, stream>>>(a);
+    else fast_stream<0><<<grid, kWThreads, bytes, stream>>>(a);
+    count_launch();
+}
+
+}  // namespace fast
+}  // namespace rocket
