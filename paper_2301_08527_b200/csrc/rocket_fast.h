@@ -171,11 +171,8 @@ struct alignas(16) TItem {
 };
 static_assert(sizeof(TItem) == 128, "TItem must be 32 words");
 // ---- stream regime (rocket_stream.cu): the large dilations, one warp per tile ------------------
-#ifndef ROCKET_W_ROWS
-#define ROCKET_W_ROWS 16
-#endif
-constexpr int kWRows = ROCKET_W_ROWS;                              // highest band
-constexpr int kWWarps = kWRows >= 24 ? 12 : 16, kWThreads = 32 * kWWarps;   // independent warps of the one block per SM
+constexpr int kWRows = 16;                                         // highest band
+constexpr int kWWarps = 16, kWThreads = 32 * kWWarps;              // independent warps of the one block per SM
 constexpr int kWStages = 2;                                        // (tile, channel) visits in flight per warp
 constexpr int kWStageFloats = (kWRows + ROCKET_MAX_LENGTH - 1 + 3) / 4 * 4 * kWarpCols;   // input rows of a visit, whole y steps
 constexpr int kWCopies = 7;                                        // shifted copies of every channel row, next to one another

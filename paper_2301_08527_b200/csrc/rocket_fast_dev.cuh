@@ -387,7 +387,7 @@ __device__ __forceinline__ void add_fixed(long long* dst, float v, double scale)
 // Sums dw[j] (both halves) over the warp and adds the ELL totals to dst[0..ELL).  A butterfly that
 // halves the number of live values at every step leaves total j on the lanes with (lane >> 1) == j.
 template <int ELL>
-__device__ __forceinline__ void reduce_publish_dw(const u64 (&dw)[ELL], long long* dst, double scale, int lane) {
+__device__ __forceinline__ void reduce_publish_dw(const u64 (&dw)[ELL], long long* dst, double scale, int lane, int len = ELL) {
     float v[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
@@ -412,7 +412,7 @@ __device__ __forceinline__ void reduce_publish_dw(const u64 (&dw)[ELL], long lon
     }
     const float total = v[0] + __shfl_xor_sync(kFull, v[0], 1);
     const int j = lane >> 1;
-    if ((lane & 1) == 0 && j < ELL) add_fixed(dst + j, total, scale);
+    if ((lane & 1) == 0 && j < len) add_fixed(dst + j, total, scale);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }

@@ -16,7 +16,7 @@ namespace {
 inline int64_t floor_div(int64_t a, int64_t b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
 
 // Units of the stream kernel for the kernels whose records start at `first`.  The output rows of a kernel (their count rounded
-// up to four) become bands of 24, 16, 12 and 8 rows.  Units of one shape follow one another and within a shape in order of
+// up to four) become bands of 16, 12 and 8 rows.  Units of one shape follow one another and within a shape in order of
 // dilation, so that the warps running at any one time share an instance of the inner loop and mostly a tensor map.
 void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost& out) {
     if (first == out.krec.size()) return;
@@ -43,8 +43,7 @@ void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost&
         while ((int64_t)choice.size() <= rows4) {
             const int t = (int)choice.size();
             Choice best{INT_MAX, 0};
-            for (int R : {24, 16, 12, 8}) {
-                if (R > kWRows) continue;
+            for (int R : {16, 12, 8}) {
                 const int rest = std::max(0, t - R / 4), cost = choice[rest].cost + R + 3;
                 if (cost < best.cost) best = {cost, R};
             }

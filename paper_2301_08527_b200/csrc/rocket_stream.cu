@@ -44,7 +44,7 @@ struct StreamArgs {
 
 // The inner loop: one channel of a warp tile, weights handed round from lane j (conv_channel with the weight already loaded).
 template <int ELL, int R>
-__device__ __forceinline__ void stream_conv(const float* __restrict__ st, const int (&off)[4], float mine, u64 (&acc)[R]) {
+__device__ __forceinline__ void stream_conv(const float* __restrict__ st, const int (&off)[4], float mine, u64 (&acc)[kWRows]) {
     u64 wp[ELL];
 #pragma unroll
     for (int j = 0; j < ELL; ++j) {
@@ -62,7 +62,7 @@ __device__ __forceinline__ void stream_conv(const float* __restrict__ st, const 
     }
 }
 template <int ELL, int R>
-__device__ __forceinline__ void stream_conv(const float* __restrict__ st, const int (&off)[4], float mine, h2 (&acc)[R]) {
+__device__ __forceinline__ void stream_conv(const float* __restrict__ st, const int (&off)[4], float mine, h2 (&acc)[kWRows]) {
     const h2 mh = to_h2(mine, mine);
     h2 wp[ELL];
 #pragma unroll
@@ -88,15 +88,91 @@ struct Carry {
     long long db;     // backward: sum of gz, fixed point
 };
 
+// One channel of the second half of the backward: dw[j] += gz[o] x[o + j].
+template <int ELL, int R>
+__device__ __forceinline__ void stream_grad(const float* __restrict__ st, const int (&off)[4], const u64 (&gz)[kWRows], u64 (&dw)[ROCKET_MAX_LENGTH]) {
+#pragma unroll
+    for (int s = 0; s < R + ELL - 1; ++s) {
+        const u64 x = *reinterpret_cast<const u64*>(st + off[s & 3] + (s >> 2) * (4 * kWarpCols));
+#pragma unroll
+        for (int j = 0; j < ELL; ++j) {
+            const int o = s - j;
+            if (o >= 0 && o < R) fma2(dw[j], gz[o], x);
+        }
+    }
+}
+
+// Calls f(length, rows) as compile-time constants for shape = 3 * (length index) + (rows index).
+template <typename F>
+__device__ __forceinline__ void by_shape(int shape, F&& f) {
+    using L7 = std::integral_constant<int, 7>;
+    using L9 = std::integral_constant<int, 9>;
+    using L11 = std::integral_constant<int, 11>;
+    using R16 = std::integral_constant<int, 16>;
+    using R12 = std::integral_constant<int, 12>;
+    using R8 = std::integral_constant<int, 8>;
+    switch (shape) {
+        case 0: f(L7{}, R16{}); break;
+        case 1: f(L7{}, R12{}); break;
+        case 2: f(L7{}, R8{}); break;
+        case 3: f(L9{}, R16{}); break;
+        case 4: f(L9{}, R12{}); break;
+        case 5: f(L9{}, R8{}); break;
+        case 6: f(L11{}, R16{}); break;
+        case 7: f(L11{}, R12{}); break;
+        default: f(L11{}, R8{}); break;
+    }
+}
+
+// The pooling works on the first R rows of the accumulators, four at a time from the eighth on (R is the same for the warp): one
+// instance of it serves every shape, which keeps the code that the warps of an SM run at a time small.
+template <typename F>
+__device__ __forceinline__ void for_rows(int R, F&& row) {
+#pragma unroll
+    for (int o = 0; o < 8; ++o) row(o);
+    if (R > 8) {
+#pragma unroll
+        for (int o = 8; o < 12; ++o) row(o);
+        if (R > 12) {
+#pragma unroll
+            for (int o = 12; o < 16; ++o) row(o);
+        }
+    }
+}
+
+// Hard pooling: the count of set sign bits and the minimum of -z; outputs that do not exist count as +inf.
+__device__ __forceinline__ void pool_hard_lane(const u64 (&acc)[kWRows], int R, bool interior, unsigned m0, unsigned m1, Carry& st) {
+    const float inf = __int_as_float(0x7f800000);
+    unsigned signs = 0;
+    if (interior) {
+        for_rows(R, [&](int o) {
+            float a, b;
+            unpack2(acc[o], a, b);
+            signs = __funnelshift_l(__float_as_uint(a), signs, 1);
+            signs = __funnelshift_l(__float_as_uint(b), signs, 1);
+            st.mn = min3(st.mn, a, b);
+        });
+    } else {
+        for_rows(R, [&](int o) {
+            float a, b;
+            unpack2(acc[o], a, b);
+            a = (m0 & (1u << o)) ? a : inf;
+            b = (m1 & (1u << o)) ? b : inf;
+            signs = __funnelshift_l(__float_as_uint(a), signs, 1);
+            signs = __funnelshift_l(__float_as_uint(b), signs, 1);
+            st.mn = min3(st.mn, a, b);
+        });
+    }
+    st.cnt += __popc(signs);
+}
+
 // Soft pooling of a tile into the lane's state (the sum as a fixed-point integer: exact and order-free from here on).
-template <int R>
-__device__ __forceinline__ void pool_soft_lane(const u64 (&acc)[R], float c1, float c0, bool interior, unsigned m0, unsigned m1, int base,
-                                               int step, Carry& st) {
+__device__ __forceinline__ void pool_soft_lane(const u64 (&acc)[kWRows], int R, float c1, float c0, bool interior, unsigned m0, unsigned m1,
+                                               int base, int step, Carry& st) {
     const u64 c1p = pack2(c1, c1), c0p = pack2(c0, c0), one = pack2(1.0f, 1.0f);
     u64 hs = pack2(0.0f, 0.0f);
     float mt = __int_as_float(0x7f800000);
-#pragma unroll
-    for (int o = 0; o < R; ++o) {
+    for_rows(R, [&](int o) {
         u64 t = c0p;
         fma2(t, acc[o], c1p);
         float ta, tb, a, b;
@@ -111,22 +187,54 @@ __device__ __forceinline__ void pool_soft_lane(const u64 (&acc)[R], float c1, fl
         hs = add2(hs, pack2(ha, hb));
         unpack2(acc[o], a, b);
         mt = min3(mt, a, b);
-    }
+    });
     float h0, h1;
     unpack2(hs, h0, h1);
     st.hsum += __float2ull_rn((h0 + h1) * kSoftFixedScale);
     if (mt <= st.mn && mt < __int_as_float(0x7f800000)) {
         int idx = INT_MAX;
-#pragma unroll
-        for (int o = R - 1; o >= 0; --o) {
+        for_rows(R, [&](int o) {
             float a, b;
             unpack2(acc[o], a, b);
-            if (b == mt) idx = min(idx, base + 1 + o * step);
             if (a == mt) idx = min(idx, base + o * step);
-        }
+            if (b == mt) idx = min(idx, base + 1 + o * step);
+        });
         if (mt < st.mn || idx < st.idx) st.idx = idx;
         st.mn = mt;
     }
+}
+
+// Backward: the accumulators (-z) become gz in place; returns the thread's sum of them (see make_gz).
+__device__ __forceinline__ float make_gz_lane(u64 (&acc)[kWRows], int R, float c1, float c0, float gPs, float gM, bool interior, unsigned m0,
+                                              unsigned m1, int oA0, int oA1) {
+    const u64 c1p = pack2(c1, c1), c0p = pack2(c0, c0), one = pack2(1.0f, 1.0f), neg1 = pack2(-1.0f, -1.0f), gp = pack2(gPs, gPs);
+    u64 sum = pack2(0.0f, 0.0f);
+    for_rows(R, [&](int o) {
+        u64 t = c0p;
+        fma2(t, acc[o], c1p);
+        float ta, tb;
+        unpack2(t, ta, tb);
+        const u64 den = add2(pack2(ex2_approx(ta), ex2_approx(tb)), one);
+        unpack2(den, ta, tb);
+        const u64 hh = pack2(rcp_approx(ta), rcp_approx(tb));
+        u64 omh = one;
+        fma2(omh, hh, neg1);                      // 1 - h
+        u64 g = mul2(mul2(hh, omh), gp);
+        float ga, gb;
+        unpack2(g, ga, gb);
+        if (!interior) {
+            if (!(m0 & (1u << o))) ga = 0.0f;
+            if (!(m1 & (1u << o))) gb = 0.0f;
+        }
+        if (o == oA0) ga += gM;
+        if (o == oA1) gb += gM;
+        g = pack2(ga, gb);
+        acc[o] = g;
+        sum = add2(sum, g);
+    });
+    float s0, s1;
+    unpack2(sum, s0, s1);
+    return s0 + s1;
 }
 
 __device__ __forceinline__ void publish_soft(unsigned long long* __restrict__ ws, int64_t pair, const Carry& st, int lane) {
@@ -267,7 +375,8 @@ __global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constan
     while (g < total) {
         auto field = [&](int i) { return __shfl_sync(kFull, v, i); };
         const int t0 = field(2), tile0 = field(3), ntiles = field(4), shape = field(5), d = field(6), m = field(7), k = field(8);
-        const int ncol = field(18), R = shape & 0xff, len = (shape >> 8) & 0xff, row_xor = shape >> 16;
+        const int ncol = field(18), R = shape & 0xff, len = (shape >> 8) & 0xff, row_xor = (shape >> 16) & 3;
+        const int index = 3 * ((len - 7) >> 1) + ((16 - R) >> 2);
         const float* __restrict__ wl = &a.f.plan.krec[krec].w2[0][0] + weight_lane;
         const int off[4] = {(0 ^ row_xor) * kWarpCols + 2 * lane, (1 ^ row_xor) * kWarpCols + 2 * lane,
                             (2 ^ row_xor) * kWarpCols + 2 * lane, (3 ^ row_xor) * kWarpCols + 2 * lane};
@@ -291,73 +400,75 @@ __global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constan
             int col = col0, trow = t0 + band0 * R;
             for (int t = 0; t < ntiles; ++t) {
                 const bool last = t + 1 == ntiles && e + 1 == examples;      // of the item
-                // the tile's channels, then its pooling; false when a wait gave up
-                auto tile = [&](auto len_tag, auto r_tag) {
-                    constexpr int ELL = decltype(len_tag)::value, RR = decltype(r_tag)::value;
-                    const int c0 = col * kWarpCols, c = c0 + 2 * lane;
-                    const bool interior = c0 + kWarpCols <= d && trow * d + c0 >= field(9) &&
-                                          (trow + RR - 1) * d + c0 + kWarpCols - 1 < field(10);
-                    int lo0 = 0, hi0 = RR, lo1 = 0, hi1 = RR;
-                    if (!interior) {
-                        const int tl = field(12), rl = field(13), th = field(14), rh = field(15);
-                        valid_rows_tc(trow, c, tl, rl, th, rh, RR, c < d, lo0, hi0);
-                        valid_rows_tc(trow, c + 1, tl, rl, th, rh, RR, c + 1 < d, lo1, hi1);
-                    }
-                    u64 acc[RR];
-                    [[maybe_unused]] h2 acch[RR];
-                    if constexpr (MODE == 3) init_acc_h(acch, negb);
-                    else init_acc(acc, negb, interior || MODE == 0, lo0, hi0, lo1, hi1);
-                    float mine = w_first;
-                    for (int q = 0; q < m; ++q) {
-                        const float mine_next = __ldg(wl + min(q + 1, m - 1) * kPairRow);
-                        if (!wait()) return false;
-                        const uint32_t slot = st & 1u;
-                        const float* stage = stages + slot * kWStageFloats;
-                        if constexpr (MODE == 3) stream_conv<ELL, RR>(stage, off, mine, acch);
-                        else stream_conv<ELL, RR>(stage, off, mine, acc);
-                        mine = mine_next;
-                        __syncwarp();                  // the stage has been read by every lane
-                        ++st;
-                        if (MODE == 2 || !last || q + 1 < m) issue(slot);
-                    }
-                    if constexpr (MODE == 3) widen_acc(acch, acc);
-                    if constexpr (MODE == 2) {
-                        const bool hit = tA >= trow && tA < trow + RR;
-                        const float dbs = make_gz(acc, a.f.c1, a.f.c0, gP, gM, interior, lo0, hi0, lo1, hi1,
-                                                  hit && c < d && c == cA ? tA - trow : -1, hit && c + 1 < d && c + 1 == cA ? tA - trow : -1);
-                        carry.db += __double2ll_rn((double)dbs * scale);
-                        for (int q = 0; q < m; ++q) {
-                            if (!wait()) return false;
-                            const uint32_t slot = st & 1u;
-                            u64 dw[ELL];
+                const int c0 = col * kWarpCols, c = c0 + 2 * lane;
+                const bool interior = c0 + kWarpCols <= d && trow * d + c0 >= field(9) && (trow + R - 1) * d + c0 + kWarpCols - 1 < field(10);
+                unsigned m0 = 0, m1 = 0;               // rows of the lane's two columns that are outputs
+                if (!interior) {
+                    const int tl = field(12), rl = field(13), th = field(14), rh = field(15);
+                    int lo, hi;
+                    valid_rows_tc(trow, c, tl, rl, th, rh, R, c < d, lo, hi);
+                    m0 = row_mask(lo, hi);
+                    valid_rows_tc(trow, c + 1, tl, rl, th, rh, R, c + 1 < d, lo, hi);
+                    m1 = row_mask(lo, hi);
+                }
+                u64 acc[kWRows];
+                [[maybe_unused]] h2 acch[kWRows];
+                if constexpr (MODE == 3) {
+                    init_acc_h(acch, negb);
+                } else if (MODE == 0 || interior) {
+                    const u64 start = pack2(negb, negb);
 #pragma unroll
-                            for (int j = 0; j < ELL; ++j) dw[j] = 0ull;
-                            grad_channel<ELL, 4 * kWarpCols, false, RR>(stages + slot * kWStageFloats, off, acc, dw);
-                            __syncwarp();
-                            ++st;
-                            if (!last || q + 1 < m) issue(slot);
-                            reduce_publish_dw<ELL>(dw, a.f.accfix + field(17) + q * ELL, scale, lane);
-                        }
-                    } else if constexpr (MODE == 1) {
-                        pool_soft_lane<RR>(acc, a.f.c1, a.f.c0, interior, row_mask(lo0, hi0), row_mask(lo1, hi1), trow * d + c + field(11), d,
-                                           carry);
-                    } else {
-                        if (interior) pool_hard(acc, carry.cnt, carry.mn);
-                        else pool_hard_masked(acc, row_mask(lo0, hi0), row_mask(lo1, hi1), carry.cnt, carry.mn);
-                    }
-                    return true;
-                };
-                auto by_rows = [&](auto len_tag) {
-#if ROCKET_W_ROWS >= 24
-                    if (R == 24) return tile(len_tag, std::integral_constant<int, 24>{});
-#endif
-                    if (R == 16) return tile(len_tag, std::integral_constant<int, 16>{});
-                    if (R == 12) return tile(len_tag, std::integral_constant<int, 12>{});
-                    return tile(len_tag, std::integral_constant<int, 8>{});
-                };
-                ok = len == 7 ? by_rows(std::integral_constant<int, 7>{}) : len == 9 ? by_rows(std::integral_constant<int, 9>{})
-                                                                                    : by_rows(std::integral_constant<int, 11>{});
+                    for (int o = 0; o < kWRows; ++o) acc[o] = start;
+                } else {                               // +inf where there is no output
+                    const float inf = __int_as_float(0x7f800000);
+#pragma unroll
+                    for (int o = 0; o < kWRows; ++o) acc[o] = pack2((m0 & (1u << o)) ? negb : inf, (m1 & (1u << o)) ? negb : inf);
+                }
+                float mine = w_first;
+                const float* __restrict__ wn = wl;
+                for (int q = 0; q < m; ++q) {
+                    if (q + 1 < m) wn += kPairRow;
+                    const float mine_next = __ldg(wn);
+                    if (!(ok = wait())) break;
+                    const uint32_t slot = st & 1u;
+                    const float* stage = stages + slot * kWStageFloats;
+                    by_shape(index, [&](auto len_tag, auto r_tag) {
+                        if constexpr (MODE == 3) stream_conv<decltype(len_tag)::value, decltype(r_tag)::value>(stage, off, mine, acch);
+                        else stream_conv<decltype(len_tag)::value, decltype(r_tag)::value>(stage, off, mine, acc);
+                    });
+                    mine = mine_next;
+                    __syncwarp();                      // the stage has been read by every lane
+                    ++st;
+                    if (MODE == 2 || !last || q + 1 < m) issue(slot);
+                }
                 if (!ok) break;
+                if constexpr (MODE == 3) widen_acc(acch, acc);
+                if constexpr (MODE == 2) {
+                    const bool hit = tA >= trow && tA < trow + R;
+                    const float dbs = make_gz_lane(acc, R, a.f.c1, a.f.c0, gP, gM, interior, m0, m1, hit && c < d && c == cA ? tA - trow : -1,
+                                                   hit && c + 1 < d && c + 1 == cA ? tA - trow : -1);
+                    carry.db += __double2ll_rn((double)dbs * scale);
+                    long long* dst = a.f.accfix + field(17);
+                    for (int q = 0; q < m; ++q, dst += len) {
+                        if (!(ok = wait())) break;
+                        const uint32_t slot = st & 1u;
+                        u64 dw[ROCKET_MAX_LENGTH];
+#pragma unroll
+                        for (int j = 0; j < ROCKET_MAX_LENGTH; ++j) dw[j] = 0ull;
+                        by_shape(index, [&](auto len_tag, auto r_tag) {
+                            stream_grad<decltype(len_tag)::value, decltype(r_tag)::value>(stages + slot * kWStageFloats, off, acc, dw);
+                        });
+                        __syncwarp();
+                        ++st;
+                        if (!last || q + 1 < m) issue(slot);
+                        reduce_publish_dw<ROCKET_MAX_LENGTH>(dw, dst, scale, lane, len);
+                    }
+                    if (!ok) break;
+                } else if constexpr (MODE == 1) {
+                    pool_soft_lane(acc, R, a.f.c1, a.f.c0, interior, m0, m1, trow * d + c + field(11), d, carry);
+                } else {
+                    pool_hard_lane(acc, R, interior, m0, m1, carry);
+                }
                 if (++col == ncol) { col = 0; trow += R; }
             }
             if (!ok) break;

@@ -46,7 +46,7 @@ static int check(uint64_t seed, int K, int C, int L, int rows, const HostParams*
         const WMapSpec& sp = plan.wmaps.at(u.map);
         REQUIRE(f.d == u.d && f.len == len && f.m == u.m && f.k == u.k && f.p == u.p && f.lo_u == u.lo_u && f.hi_u == u.hi_u && f.tl == u.tl &&
                 f.rl == u.rl && f.th == u.th && f.rh == u.rh && f.nout == u.nout && f.woff == u.woff && f.d >= plan.split, "unit fields");
-        REQUIRE((R == 24 || R == 16 || R == 12 || R == 8) && R <= kWRows && u.ntiles >= 1 && u.ncol == (u.d + 63) / 64 && u.run == G * u.d && u.band_y == R / G, "unit shape");
+        REQUIRE((R == 16 || R == 12 || R == 8) && u.ntiles >= 1 && u.ncol == (u.d + 63) / 64 && u.run == G * u.d && u.band_y == R / G, "unit shape");
         REQUIRE(sp.d == u.d && sp.y_rows * G >= S && u.bytes == sp.y_rows * G * kWarpCols * 4 && u.bytes <= kWStageFloats * 4, "box");
         for (int q = 0; q < u.m; ++q) REQUIRE(u.ch[q] == f.ch[q] && u.ch[q] < hp.C, "channels");
         // the tensor map, as ensure_stream_capacity encodes it
