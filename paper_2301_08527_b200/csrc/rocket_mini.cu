@@ -7,41 +7,40 @@
 //                every other (dilation, kernel) combination, a random channel subset per combination
 //   fit          rocket_mini_fit, on the host (a one-off over one training example per combination): the bias of
 //                a feature is a quantile of the combination's convolution output on that example
-//   transform    rocket_mini_transform, one fused kernel: per (example, combination) the channels are summed into
-//                a shared-memory tile of the dilated view, the nine-tap dilated convolution runs on a register
-//                window that slides down a column of the tile, and every output is compared with the
-//                combination's biases on the fly, so the convolution outputs never reach memory; feature =
-//                count / number of outputs (Eq. 1-2 against the bias)
+//   transform    rocket_mini_transform, one fused kernel: a block stages a tile of the dilated view with all the
+//                channels that the combinations of a dilation use, its warps take the combinations one by one -
+//                channels summed, nine-tap convolution, comparison with every bias of the combination, all in
+//                registers - so the convolution outputs never reach memory; a small kernel then turns counts into
+//                shares of outputs (Eq. 1-2 against the bias)
 //
 // The kernel weights take two values, so every product is one fused multiply-add with -1 or 2: on this
 // hardware an addition and a fused multiply-add take the same issue slot, and the additions-only form that
-// speeds the method up on a CPU brings nothing here.  The bound of the kernel is the traffic from L2: every
-// combination reads its channels once.
+// speeds the method up on a CPU brings nothing here.
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <new>
 #include <numeric>
 #include <thread>
-#include <type_traits>
 #include <vector>
 
+#include "rocket_fast.h"
+#include "rocket_fast_dev.cuh"
+#include "rocket_fast_geom.h"
 #include "rocket_internal.h"
 
+namespace rocket {
+namespace fast {
 namespace {
 
 constexpr int kKernels = 84, kLen = 9;
-constexpr int kMaxFeaturesPerItem = 8;      // a combination with more features becomes several items
-constexpr int kThreads = 256;
-#ifndef ROCKET_MINI_TILE
-#define ROCKET_MINI_TILE (16 * 1024)
-#endif
-constexpr int kTileSamples = ROCKET_MINI_TILE;
-#ifndef ROCKET_MINI_BLOCKS
-#define ROCKET_MINI_BLOCKS 3
-#endif   // channel-summed samples a block stages at a time (64 KB of shared memory)
+constexpr int kMRows = 12, kMInRows = kMRows + kLen - 1;      // output rows of a tile, input rows
+constexpr int kMWarps = 16, kMThreads = 32 * kMWarps;
+constexpr int kMPlanes = 20;                                  // (example, channel) planes of a tile
+constexpr int kMPlaneFloats = kMInRows * kWarpCols, kMPlaneBytes = kMPlaneFloats * 4;
 constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;
 constexpr uint64_t kStreamBase = 1ull << 32;
 constexpr double kInvGoldenRatio = 0.6180339887498949;
@@ -58,235 +57,272 @@ inline double draw_uniform(uint64_t seed, uint64_t stream, uint64_t slot) {
     return static_cast<double>(draw_u64(seed, stream, slot) >> 11) * 0x1.0p-53;
 }
 
-// One unit of device work: a combination, or a slice of at most 8 of its features, with the tiling of the
-// dilated view the kernel uses for its dilation (chosen on the host, choose_tiling).
-struct MiniItem {
-    int32_t d, padded, m, f0, nf;
-    int32_t tap[3];
-    int32_t ch[kLen];
-    int32_t width, seg_rows, segs;   // columns of a tile (= its pitch), rows a thread walks, such runs per tile
+// One combination (32 words): its outputs are u = t d + r with tl d <= u < th d + rh (A[t][r] = x[t d + r]).
+struct alignas(16) MiniRec {
+    int32_t m, f0, nf, tl, th, rh, pad_[2];
+    int32_t ch[kLen];                     // byte offsets of the channels' planes in a tile
+    float w[kLen];                        // the weights, negated
+    int32_t pad2_[6];
 };
-static_assert(sizeof(MiniItem) == 80, "MiniItem layout");
+static_assert(sizeof(MiniRec) == 128, "MiniRec must be 32 words");
+// Combinations [kbeg, kend) of one dilation that use at most kMPlanes channels between them (32 words).
+struct alignas(16) MiniBucket {
+    int32_t d, raster_len, kbeg, kend, nch, pad_[7];
+    int32_t ch[kMPlanes];
+};
+static_assert(sizeof(MiniBucket) == 128, "MiniBucket must be 32 words");
+// 64 consecutive columns of a bucket's raster: bands of kMRows rows of A, strung together band by band.
+struct MiniTile { int32_t bucket, c0; };
 
-// Sample k of a channel row through the read-only path: at a constant byte offset from the row's first sample
-// (STRIDE samples apart), or, with a run-time stride, at an address formed by one widening multiply-add.
-template <int STRIDE>
-__device__ __forceinline__ float load_at(const float* __restrict__ x0, int k, int stride) {
-    float v;
-    if constexpr (STRIDE != 0) {
-        switch (k) {   // k is a constant after unrolling; the offset must be an immediate
-            case 0: asm("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(x0)); break;
-            case 1: asm("ld.global.nc.f32 %0, [%1+%2];" : "=f"(v) : "l"(x0), "n"(4 * STRIDE)); break;
-            case 2: asm("ld.global.nc.f32 %0, [%1+%2];" : "=f"(v) : "l"(x0), "n"(8 * STRIDE)); break;
-            case 3: asm("ld.global.nc.f32 %0, [%1+%2];" : "=f"(v) : "l"(x0), "n"(12 * STRIDE)); break;
-            case 4: asm("ld.global.nc.f32 %0, [%1+%2];" : "=f"(v) : "l"(x0), "n"(16 * STRIDE)); break;
-            case 5: asm("ld.global.nc.f32 %0, [%1+%2];" : "=f"(v) : "l"(x0), "n"(20 * STRIDE)); break;
-            case 6: asm("ld.global.nc.f32 %0, [%1+%2];" : "=f"(v) : "l"(x0), "n"(24 * STRIDE)); break;
-            default: asm("ld.global.nc.f32 %0, [%1+%2];" : "=f"(v) : "l"(x0), "n"(28 * STRIDE)); break;
-        }
-    } else {
-        const float* p;
-        asm("mad.wide.s32 %0, %1, 4, %2;" : "=l"(p) : "r"(k * stride), "l"(x0));
-        asm("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    }
-    return v;
+struct MiniArgs {
+    const float* X;
+    const MiniRec* recs;
+    const MiniBucket* buckets;
+    const MiniTile* tiles;
+    const float* bias;
+    int* counts;                          // [N][F]: the features while they are counts
+    int* error_flag;
+    int N, C, L, F, n_tiles;
+    int examples, groups, parts;          // examples of a tile, groups of examples, parts a tile's combinations are dealt in
+};
+
+// A tile as a warp holds it.
+struct TileAt { int words, c0, n0, ne, kbeg, n_work; };   // words: the bucket's, one per lane
+
+__device__ __forceinline__ void mini_cp4(uint32_t dst, const void* src, int bytes) {   // bytes: 4, or 0 for a zero
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+// Arrives on the barrier when the thread's copies so far have landed.
+__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// One output of the convolution from the nine window entries (the oldest sits in slot S0; taps are taken in
-// the order 0..8 whatever the slot), compared with the first 4 NG biases of the item (Eq. 1 against the bias).
-template <int S0, int NG>
-__device__ __forceinline__ void mini_pool(const float (&win)[kLen], const float (&w)[kLen],
-                                          const float (&b)[kMaxFeaturesPerItem], int (&cnt)[kMaxFeaturesPerItem]) {
-    float z = 0.0f;
+// How many of the 2 x 12 outputs exceed a bias: the signs of bias - z (exact: the difference of two floats rounds to zero only
+// when they are equal).  acc = -z.
+__device__ __forceinline__ int mini_count(const u64 (&acc)[kMRows], float b) {
+    const u64 bp = pack2(b, b);
+    unsigned s0 = 0, s1 = 0;              // two chains
 #pragma unroll
-    for (int j = 0; j < kLen; ++j) z = fmaf(w[j], win[(S0 + j) % kLen], z);
-    // Eq. 1 against every bias: one compare and one predicated add each
-#pragma unroll
-    for (int f = 0; f < 4 * NG; ++f)
-        asm("{ .reg .pred p; setp.gt.f32 p, %1, %2; @p add.s32 %0, %0, 1; }" : "+r"(cnt[f]) : "f"(z), "f"(b[f]));
+    for (int o = 0; o < kMRows; ++o) {
+        float x, y;
+        unpack2(add2(acc[o], bp), x, y);
+        s0 = __funnelshift_l(__float_as_uint(x), s0, 1);
+        s1 = __funnelshift_l(__float_as_uint(y), s1, 1);
+    }
+    return __popc(s0 | s1 << kMRows);
 }
 
-// Steps K .. 8 of a group of nine outputs: the next row's sample enters the slot the oldest one leaves, so
-// the window never moves between registers.  GUARD: the run may end inside the group.
-template <int K, bool GUARD, int NG>
-__device__ __forceinline__ void mini_steps(const float*& p, int pitch, int left, float (&win)[kLen], const float (&w)[kLen],
-                                           const float (&b)[kMaxFeaturesPerItem], int (&cnt)[kMaxFeaturesPerItem]) {
-    if constexpr (K < kLen) {
-        if (!GUARD || K < left) {
-            win[(K + kLen - 1) % kLen] = *p;
-            p += pitch;
-            mini_pool<K, NG>(win, w, b, cnt);
+// Bound: instruction issue - per pair of outputs 9 packed multiply-adds, (m - 1) 20/12 packed adds and m 20/12 loads for the
+// channel sums (m channels, 3.9 on average) and, per bias (3.8 on average), a packed add and two shifts that collect the signs
+// of bias - z.  What the layout is for: the channels of a tile are read once for the 84 combinations of a dilation (one
+// combination per block and tile, the earlier form, read 146 GB from L2 for 60 x 20 x 50,000), the packed operations work on
+// two columns at a time, and two tiles are in shared memory so that the next one lands while this one is worked on: a warp that
+// finds no combination left goes on to the next tile without waiting for the others.
+__global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_constant__ MiniArgs a) {
+    extern __shared__ __align__(128) float planes[];              // [2][kMPlanes][kMInRows][64]
+    __shared__ unsigned long long s_full[2], s_empty[2];
+    __shared__ int s_pos;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t full0 = smem_u32(s_full), empty0 = smem_u32(s_empty);
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(full0 + 8u * i, kMThreads);
+            mbar_init(empty0 + 8u * i, kMWarps);
         }
-        mini_steps<K + 1, GUARD, NG>(p, pitch, left, win, w, b, cnt);
-    }
-}
-
-// The walks over one staged tile: thread u of cols * segs takes column u % cols over run u / cols.  Outputs of
-// column c are the rows t_min <= t < t_full + (c < c_more): t d + c < last with last = t_full d + c_more.
-template <int NG>
-__device__ __forceinline__ void mini_walk_tile(const float* s_x, int P, int cols, int rows, int seg_rows, int ta, int ca,
-                                               int t_min, int t_full, int c_more, const float (&w)[kLen],
-                                               const float (&b)[kMaxFeaturesPerItem], int (&cnt)[kMaxFeaturesPerItem]) {
-    const int segs = (rows + seg_rows - 1) / seg_rows;
-    // (run, column) of thread u, stepped without divisions: u advances by the block's threads
-    const int dq = kThreads / cols, dr = kThreads - dq * cols;
-    int seg = threadIdx.x / cols, c = threadIdx.x - seg * cols;
-    for (int u = threadIdx.x; u < cols * segs; u += kThreads) {
-        const int t_end = t_full + (ca + c < c_more ? 1 : 0);
-        const int t_lo = max(ta + seg * seg_rows, t_min);
-        const int t_hi = min(min(ta + rows, ta + (seg + 1) * seg_rows), t_end);
-        int left = t_hi - t_lo;
-        if (left > 0) {
-            // the window of output row t holds rows t - 4 .. t + 4; staged row 0 is row ta - 4
-            const float* p = s_x + (t_lo - ta) * P + c;
-            float win[kLen];
-#pragma unroll
-            for (int j = 0; j < kLen - 1; ++j) { win[j] = *p; p += P; }
-            for (; left >= kLen; left -= kLen) mini_steps<0, false, NG>(p, P, left, win, w, b, cnt);
-            if (left > 0) mini_steps<0, true, NG>(p, P, left, win, w, b, cnt);
-        }
-        seg += dq; c += dr;
-        if (c >= cols) { c -= cols; ++seg; }
-    }
-}
-
-// One block per (example, item).  The series is seen as rows of d samples (A[t][c] = x[t d + c]); a tile of it -
-// rows [ta - 4, ta + rows + 4) of `width` columns, channels already summed, zeros outside the series - is
-// staged in shared memory, then every thread walks down one column over a run of seg_rows rows with the nine
-// taps in registers: one shared-memory load, nine multiply-adds and the bias compares per output.
-__global__ void __launch_bounds__(kThreads, ROCKET_MINI_BLOCKS)
-mini_transform_kernel(const float* __restrict__ X, int C, int L, const MiniItem* __restrict__ items, int n_items,
-                      const float* __restrict__ bias, float* __restrict__ feat, int F) {
-    extern __shared__ float s_x[];
-    __shared__ int s_cnt[kMaxFeaturesPerItem];
-    __shared__ int s_choff[kLen];
-    const int n = blockIdx.x / n_items;
-    const MiniItem* __restrict__ item = items + (blockIdx.x - n * n_items);
-    const MiniItem it = *item;
-    const float* __restrict__ Xn = X + (size_t)n * C * L;
-    const int tid = threadIdx.x;
-    if (tid < kMaxFeaturesPerItem) s_cnt[tid] = 0;
-    if (tid < kLen) s_choff[tid] = __ldg(item->ch + (tid < it.m ? tid : 0)) * L;     // C L < 2^31 (checked at creation)
-    const int d = it.d, m = it.m, nf = it.nf;
-    const int first = it.padded ? 0 : 4 * d, last = it.padded ? L : L - 4 * d;
-    float w[kLen];
-#pragma unroll
-    for (int j = 0; j < kLen; ++j) w[j] = (j == it.tap[0] || j == it.tap[1] || j == it.tap[2]) ? 2.0f : -1.0f;
-    float b[kMaxFeaturesPerItem];
-#pragma unroll
-    for (int f = 0; f < kMaxFeaturesPerItem; ++f) b[f] = f < nf ? __ldg(bias + it.f0 + f) : __int_as_float(0x7f800000);
-    int cnt[kMaxFeaturesPerItem];
-#pragma unroll
-    for (int f = 0; f < kMaxFeaturesPerItem; ++f) cnt[f] = 0;
-
-    const int T = (L + d - 1) / d;                       // rows of the dilated view
-    const int P = it.width, seg_rows = it.seg_rows;      // P: columns of a tile and its pitch in shared memory
-    const int tile_rows = seg_rows * it.segs;
-    const bool whole_rows = P == d;                      // a tile spans whole rows: its samples are one contiguous run
-    const int t_min = it.padded ? 0 : 4;                 // rows below hold no output of an unpadded combination
-    const int t_full = last / d, c_more = last - t_full * d;   // column c has outputs in rows t < t_full + (c < c_more)
-    const int groups = (nf + 3) / 4;
-
-    // NK staged samples per thread at a time: position base + k * stride goes to slot + k * slot_stride.  The
-    // channels are taken two at a time, so that 2 NK loads are in flight per thread.  CHECK: a sample may lie
-    // beyond the series (then it is zero).  STRIDE = 0: the stride is a run-time value.
-    auto stage = [&](auto nk_tag, auto stride_tag, auto check_tag, int base, int stride_rt, int slot, int slot_stride) {
-        constexpr int NK = decltype(nk_tag)::value;
-        constexpr int STRIDE = decltype(stride_tag)::value;
-        constexpr bool CHECK = decltype(check_tag)::value;
-        const int stride = STRIDE ? STRIDE : stride_rt;
-        float acc[NK];
-        bool ok[NK];
-#pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            acc[k] = 0.0f;
-            ok[k] = !CHECK || (unsigned)(base + k * stride) < (unsigned)L;
-        }
-        int q = 0;
-        for (; q + 2 <= m; q += 2) {
-            const float* __restrict__ x0 = Xn + s_choff[q] + base;
-            const float* __restrict__ x1 = Xn + s_choff[q + 1] + base;
-            float v0[NK], v1[NK];
-#pragma unroll
-            for (int k = 0; k < NK; ++k) {
-                v0[k] = ok[k] ? load_at<STRIDE>(x0, k, stride) : 0.0f;
-                v1[k] = ok[k] ? load_at<STRIDE>(x1, k, stride) : 0.0f;
-            }
-#pragma unroll
-            for (int k = 0; k < NK; ++k) acc[k] = (acc[k] + v0[k]) + v1[k];
-        }
-        if (q < m) {
-            const float* __restrict__ x0 = Xn + s_choff[q] + base;
-#pragma unroll
-            for (int k = 0; k < NK; ++k)
-                if (ok[k]) acc[k] += load_at<STRIDE>(x0, k, stride);
-        }
-#pragma unroll
-        for (int k = 0; k < NK; ++k) s_x[slot + k * slot_stride] = acc[k];
-    };
-    using Strided = std::integral_constant<int, 0>;
-    using Dense = std::integral_constant<int, kThreads>;
-    using N8 = std::integral_constant<int, 8>;
-    using N4 = std::integral_constant<int, 4>;
-    using N2 = std::integral_constant<int, 2>;
-    using N1 = std::integral_constant<int, 1>;
-    using Checked = std::true_type;
-    using Inside = std::false_type;
-
-    for (int ta = 0; ta < T; ta += tile_rows) {
-        const int rows = min(tile_rows, T - ta);
-        for (int ca = 0; ca < d; ca += P) {
-            const int cols = min(P, d - ca);
-            __syncthreads();                             // the previous tile's walks are over (and s_choff is written)
-            if (whole_rows) {
-                // slots [0, count) hold positions g0 .. g0 + count: zeros before the series, the samples in
-                // rounds of 8 x 256 and of 256 without any test, one last partial round, zeros after the series
-                const int count = (rows + 8) * d, g0 = (ta - 4) * d;
-                const int z0 = min(max(-g0, 0), count), z1 = min(max(L - g0, 0), count);
-                for (int e = tid; e < z0; e += kThreads) s_x[e] = 0.0f;
-                for (int e = z1 + tid; e < count; e += kThreads) s_x[e] = 0.0f;
-                int e0 = z0;
-                for (; e0 + 8 * kThreads <= z1; e0 += 8 * kThreads) stage(N8{}, Dense{}, Inside{}, g0 + e0 + tid, 0, e0 + tid, kThreads);
-                for (; e0 + kThreads <= z1; e0 += kThreads) stage(N1{}, Dense{}, Inside{}, g0 + e0 + tid, 0, e0 + tid, kThreads);
-                if (e0 + tid < z1) stage(N1{}, Dense{}, Inside{}, g0 + e0 + tid, 0, e0 + tid, kThreads);
-            } else {
-                for (int cb = 0; cb < cols; cb += kThreads) {
-                    if (cb + tid >= cols) continue;
-                    // staged row r is row ta - 4 + r of the view: zeros above the series, rows that lie inside it
-                    // for every column of this block without any test, the rows the series ends in, zeros below
-                    const int w = min(kThreads, cols - cb), c_lo = ca + cb;
-                    const int n_rows = rows + 8;
-                    const int r_a = min(max(4 - ta, 0), n_rows);
-                    const int t_full = L >= c_lo + w ? (L - c_lo - w) / d + 1 : 0;     // rows t < t_full hold all w columns
-                    const int t_some = L > c_lo ? (L - c_lo - 1) / d + 1 : 0;          // rows t < t_some hold at least one
-                    const int r_b = min(max(t_full - (ta - 4), r_a), n_rows), r_c = min(max(t_some - (ta - 4), r_b), n_rows);
-                    const int pos0 = (ta - 4) * d + c_lo + tid, slot0 = cb + tid;
-                    for (int r = 0; r < r_a; ++r) s_x[slot0 + r * P] = 0.0f;
-                    int r = r_a;
-                    for (; r + 8 <= r_b; r += 8) stage(N8{}, Strided{}, Inside{}, pos0 + r * d, d, slot0 + r * P, P);
-                    if (r + 4 <= r_b) { stage(N4{}, Strided{}, Inside{}, pos0 + r * d, d, slot0 + r * P, P); r += 4; }
-                    if (r + 2 <= r_b) { stage(N2{}, Strided{}, Inside{}, pos0 + r * d, d, slot0 + r * P, P); r += 2; }
-                    if (r + 1 <= r_b) { stage(N1{}, Strided{}, Inside{}, pos0 + r * d, d, slot0 + r * P, P); r += 1; }
-                    for (; r < r_c; ++r) stage(N1{}, Strided{}, Checked{}, pos0 + r * d, d, slot0 + r * P, P);
-                    for (; r < n_rows; ++r) s_x[slot0 + r * P] = 0.0f;
-                }
-            }
-            __syncthreads();
-            static_assert(kMaxFeaturesPerItem == 8, "two groups of four features");
-            if (groups == 1) mini_walk_tile<1>(s_x, P, cols, rows, seg_rows, ta, ca, t_min, t_full, c_more, w, b, cnt);
-            else mini_walk_tile<2>(s_x, P, cols, rows, seg_rows, ta, ca, t_min, t_full, c_more, w, b, cnt);
-        }
-    }
-#pragma unroll
-    for (int f = 0; f < kMaxFeaturesPerItem; ++f) {
-        const int v = __reduce_add_sync(0xffffffffu, cnt[f]);
-        if ((tid & 31) == 0 && v) atomicAdd(&s_cnt[f], v);
+        s_pos = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    if (tid < nf) feat[(size_t)n * F + it.f0 + tid] = (float)s_cnt[tid] / (float)(last - first);   // Eq. 2
+
+    // The block's tiles: items blockIdx.x, blockIdx.x + gridDim.x, .. of all (tile, part, group of examples).  The (combination,
+    // example) pairs of the block's tiles form one sequence that the warps draw from.
+    const unsigned total = (unsigned)a.groups * (unsigned)a.n_tiles * (unsigned)a.parts;
+    const int K = (int)((total - blockIdx.x + gridDim.x - 1) / gridDim.x);
+    auto word = [](int v, int i) { return __shfl_sync(kFull, v, i); };
+    // Issues the thread's share of tile k's copies (every channel of the bucket, zeros outside the series).
+    auto fill = [&](int k) {
+        const unsigned g = blockIdx.x + (unsigned)k * gridDim.x, per_group = (unsigned)a.n_tiles * (unsigned)a.parts;
+        const unsigned group = g / per_group, rest = g - group * per_group, tile = rest / (unsigned)a.parts, part = rest - tile * (unsigned)a.parts;
+        TileAt t;
+        const int2 at = __ldg(reinterpret_cast<const int2*>(a.tiles + tile));
+        t.words = __ldg(reinterpret_cast<const int*>(a.buckets + at.x) + lane);
+        t.c0 = at.y;
+        t.n0 = (int)group * a.examples;
+        t.ne = min(a.examples, a.N - t.n0);
+        const int combos = word(t.words, 3) - word(t.words, 2), beg = combos * (int)part / a.parts, end = combos * ((int)part + 1) / a.parts;
+        t.kbeg = word(t.words, 2) + beg;
+        t.n_work = (end - beg) * t.ne;
+        const int d = word(t.words, 0), raster_len = word(t.words, 1), nch = word(t.words, 4);
+        constexpr int kStep = kMThreads / kWarpCols, kRows = (kMInRows + kStep - 1) / kStep;
+        static_assert((kRows - 1) * kStep < kMInRows, "only the last row of a thread may not exist");
+        const int col = tid & (kWarpCols - 1), rg = tid / kWarpCols, cg = t.c0 + col, band = cg / d;
+        const int u0 = (band * kMRows - 4 + rg) * d + (cg - band * d);
+        unsigned off[kRows];
+        int bytes[kRows];
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            const int x = u0 + i * kStep * d;
+            const bool ok = cg < raster_len && (unsigned)x < (unsigned)a.L;
+            off[i] = ok ? 4u * (unsigned)x : 0u;
+            bytes[i] = ok ? 4 : 0;
+        }
+        const bool last = rg + (kRows - 1) * kStep < kMInRows;
+        uint32_t dst = smem_u32(planes + (k & 1) * kMPlanes * kMPlaneFloats + rg * kWarpCols + col);
+        for (int e = 0; e < t.ne; ++e) {
+            const float* __restrict__ Xn = a.X + (size_t)(t.n0 + e) * a.C * a.L;
+#pragma unroll 4
+            for (int c = 0; c < nch; ++c) {
+                const char* __restrict__ src = reinterpret_cast<const char*>(Xn + (size_t)word(t.words, 12 + c) * a.L);
+#pragma unroll
+                for (int i = 0; i < kRows - 1; ++i) mini_cp4(dst + i * kStep * kWarpCols * 4, src + off[i], bytes[i]);
+                if (last) mini_cp4(dst + (kRows - 1) * kStep * kWarpCols * 4, src + off[kRows - 1], bytes[kRows - 1]);
+                dst += kMPlaneBytes;
+            }
+        }
+        cp_async_arrive(full0 + 8u * (k & 1));
+        return t;
+    };
+    auto draw = [&]() {
+        int p = 0;
+        if (lane == 0) p = atomicAdd(&s_pos, 1);
+        return __shfl_sync(kFull, p, 0);
+    };
+    auto load_rec = [&](const TileAt& t, int w) {
+        return __ldg(reinterpret_cast<const int*>(a.recs + t.kbeg + (t.ne == 1 ? w : w / t.ne)) + lane);
+    };
+
+    TileAt cur = fill(0), nxt = cur;
+    int filled = 1, k = 0, base = 0;
+    if (K > 1) { nxt = fill(1); filled = 2; }
+    int pos = draw();
+    // the lane's two columns of the tile: band of rows and column of A
+    int trow0 = 0, trow1 = 0, c0 = 0, c1 = 0;
+    bool ok0 = false, ok1 = false;
+    auto enter = [&]() {
+        const int d = word(cur.words, 0), raster_len = word(cur.words, 1), cg = cur.c0 + 2 * lane, band = (int)((unsigned)cg / (unsigned)d);
+        c0 = cg - band * d;
+        c1 = c0 + 1 < d ? c0 + 1 : 0;
+        trow0 = band * kMRows;
+        trow1 = c0 + 1 < d ? trow0 : trow0 + kMRows;
+        ok0 = cg < raster_len;
+        ok1 = cg + 1 < raster_len;
+        return mbar_wait(full0 + 8u * (k & 1), (k >> 1) & 1);
+    };
+    bool ok = enter();
+    int rec_next = pos < cur.n_work ? load_rec(cur, pos) : 0;
+    while (ok) {
+        // tile k + 1 may be copied in as soon as every warp has left tile k - 1
+        if (filled == k + 1 && filled < K && __all_sync(kFull, mbar_try(empty0 + 8u * ((k + 1) & 1), ((k - 1) >> 1) & 1))) {
+            nxt = fill(k + 1);
+            ++filled;
+        }
+        if (pos >= base + cur.n_work) {
+            if (k + 1 >= K) break;
+            if (filled == k + 1) {
+                if (!(ok = mbar_wait(empty0 + 8u * ((k + 1) & 1), ((k - 1) >> 1) & 1))) break;
+                nxt = fill(k + 1);
+                ++filled;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty0 + 8u * (k & 1));
+            base += cur.n_work;
+            cur = nxt;
+            ++k;
+            ok = enter();
+            if (pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
+            continue;
+        }
+        const int rec = rec_next, w = pos - base, e = cur.ne == 1 ? 0 : w % cur.ne;
+        const int m = word(rec, 0), f0 = word(rec, 1), nf = word(rec, 2);
+        float my_bias = lane < nf ? __ldg(a.bias + f0 + lane) : 0.0f;
+        pos = draw();
+        if (pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
+        const char* st = reinterpret_cast<const char*>(planes + (k & 1) * kMPlanes * kMPlaneFloats + 2 * lane);
+        if (e > 0) st += e * word(cur.words, 4) * kMPlaneBytes;
+
+        // the sum of the combination's channels, in the order of its list
+        u64 xs[kMInRows];
+        {
+            const u64* p = reinterpret_cast<const u64*>(st + word(rec, 8));
+#pragma unroll
+            for (int s = 0; s < kMInRows; ++s) xs[s] = p[s * (kWarpCols / 2)];
+        }
+        for (int q = 1; q < m; ++q) {
+            const u64* p = reinterpret_cast<const u64*>(st + word(rec, 8 + q));
+#pragma unroll
+            for (int s = 0; s < kMInRows; ++s) xs[s] = add2(xs[s], p[s * (kWarpCols / 2)]);
+        }
+        u64 acc[kMRows];                               // -z
+        {
+            u64 wp[kLen];
+#pragma unroll
+            for (int j = 0; j < kLen; ++j) {
+                const float v = __int_as_float(word(rec, 17 + j));
+                wp[j] = pack2(v, v);
+            }
+#pragma unroll
+            for (int s = 0; s < kMInRows; ++s)
+#pragma unroll
+                for (int j = 0; j < kLen; ++j) {
+                    const int o = s - j;
+                    if (o >= 0 && o < kMRows) {
+                        if (j == 0) acc[o] = fma2_to(wp[0], xs[s], 0ull);
+                        else fma2(acc[o], wp[j], xs[s]);
+                    }
+                }
+        }
+        // outputs that do not exist: +inf, which no bias exceeds
+        {
+            const int tl = word(rec, 3), th = word(rec, 4);
+            if (!__all_sync(kFull, ok1 && trow0 >= tl && trow1 + kMRows <= th)) {
+                const int rh = word(rec, 5);
+                int lo, hi;
+                valid_rows_tc(trow0, c0, tl, 0, th, rh, kMRows, ok0, lo, hi);
+                const unsigned m0 = row_mask(lo, hi);
+                valid_rows_tc(trow1, c1, tl, 0, th, rh, kMRows, ok1, lo, hi);
+                const unsigned m1 = row_mask(lo, hi);
+                const float inf = __int_as_float(0x7f800000);
+#pragma unroll
+                for (int o = 0; o < kMRows; ++o) {
+                    float x, y;
+                    unpack2(acc[o], x, y);
+                    acc[o] = pack2((m0 >> o) & 1 ? x : inf, (m1 >> o) & 1 ? y : inf);
+                }
+            }
+        }
+        // Eq. 1 against every bias; two of them share a reduction over the warp, lane f keeps the count of bias f
+        int* counts = a.counts + (size_t)(cur.n0 + e) * a.F + f0;
+        for (int fb = 0; fb < nf; fb += 32) {
+            if (fb > 0) my_bias = fb + lane < nf ? __ldg(a.bias + f0 + fb + lane) : 0.0f;
+            const int n = min(32, nf - fb);
+            int mine = 0;
+            for (int f = 0; f < n; f += 2) {
+                int both = mini_count(acc, __shfl_sync(kFull, my_bias, f));
+                if (f + 1 < n) both |= mini_count(acc, __shfl_sync(kFull, my_bias, f + 1)) << 16;
+                both = __reduce_add_sync(kFull, both);
+                if ((lane & ~1) == f) mine = lane & 1 ? both >> 16 : both & 0xffff;
+            }
+            if (lane < n && mine) atomicAdd(counts + fb + lane, mine);
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");   // nothing of this thread is in flight when the block ends
+    if (!ok && lane == 0) atomicExch(a.error_flag, 1);
+}
+
+// Counts to shares of outputs (Eq. 2); NaN when a wait of the tile kernel gave up.
+__global__ void __launch_bounds__(256)
+mini_finalize_kernel(float* __restrict__ feat, const int* __restrict__ nout, int F, long long total, const int* __restrict__ error_flag) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= total) return;
+    const int count = reinterpret_cast<const int*>(feat)[i];
+    feat[i] = *error_flag ? __int_as_float(0x7fc00000) : (float)count / (float)__ldg(nout + i % F);
 }
 
 }  // namespace
+}  // namespace fast
+}  // namespace rocket
+
+using namespace rocket::fast;
 
 struct rocket_mini {
     int C = 0, L = 0, F = 0, n_combos = 0;
@@ -294,92 +330,106 @@ struct rocket_mini {
     std::vector<double> example_draw, quantile;
     std::vector<float> bias;
     bool fitted = false;
-    std::vector<MiniItem> items;
+    std::vector<MiniRec> recs;
+    std::vector<MiniBucket> buckets;
+    std::vector<MiniTile> tiles;
+    std::vector<int32_t> nout;             // outputs behind every feature
+    int max_nch = 1;
     mutable std::mutex mu;
     mutable int device = -1;
-    mutable void* blob = nullptr;          // items, then biases
-    mutable const MiniItem* d_items = nullptr;
-    mutable float* d_bias = nullptr;
+    mutable void* blob = nullptr;          // records, buckets, tiles, output counts, biases, error flag
+    mutable MiniArgs dev{};
+    mutable const int* d_nout = nullptr;
     mutable bool bias_uploaded = false;
 };
 
-namespace {
-
-// Tiling of the dilated view for dilation d: the cheapest of the candidates under a simple cost model (staged
-// samples, and thread slots of the walks including the ones that idle in a partly filled round of the block).
-// Tiles either span whole rows (width = d) or 256-column multiples; runs are multiples of the window length;
-// below 32 columns only run lengths that keep the lanes of a warp on different shared-memory banks.
-void choose_tiling(int d, int L, int& width, int& seg_rows, int& segs) {
-    const int T = (L + d - 1) / d;
-    const double c_stage = 17.0, c_walk = 21.0, c_fill = 16.0;
-    double best = 1e300;
-    width = 0;
-    auto consider = [&](int w, int sr, int sg) {
-        if ((int64_t)(sg * sr + 8) * w > kTileSamples) return;
-        const int tile_rows = sr * sg;
-        double cost = 0.0;
-        for (int ta = 0; ta < T; ta += tile_rows) {
-            const int rows = std::min(tile_rows, T - ta), sgt = (rows + sr - 1) / sr;
-            for (int ca = 0; ca < d; ca += w) {
-                const int cols = std::min(w, d - ca);
-                const double rounds = std::ceil((double)cols * sgt / kThreads);
-                cost += (double)(rows + 8) * cols * c_stage + rounds * kThreads * (std::min(sr, rows) * c_walk + c_fill);
+// Groups the combinations of every dilation into buckets of at most kMPlanes channels and cuts their rasters into tiles.
+static void build_tiles(rocket_mini& p) {
+    p.recs.clear(); p.buckets.clear(); p.tiles.clear();
+    p.nout.assign(p.F, 1);
+    p.max_nch = 1;
+    std::map<int, std::vector<int>> by_d;
+    for (int c = 0; c < p.n_combos; ++c)
+        if (p.feature_offset[c + 1] > p.feature_offset[c]) by_d[p.dilation[c]].push_back(c);
+    struct Group { std::vector<char> has; int nch; std::vector<int> combos; };
+    for (auto& kv : by_d) {
+        const int d = kv.first;
+        auto& cs = kv.second;
+        // most channels first: they find room while the groups are empty, and the long ones start first in a tile
+        std::stable_sort(cs.begin(), cs.end(), [&](int a, int b) { return p.num_channels[a] > p.num_channels[b]; });
+        std::vector<Group> groups;
+        for (int c : cs) {
+            const int32_t* S = p.channel_idx.data() + p.channel_offset[c];
+            const int m = p.num_channels[c];
+            int best = -1, best_new = 1 << 30;
+            for (size_t g = 0; g < groups.size(); ++g) {
+                int fresh = 0;
+                for (int q = 0; q < m; ++q) fresh += !groups[g].has[S[q]];
+                if (groups[g].nch + fresh <= kMPlanes && fresh < best_new) { best = (int)g; best_new = fresh; }
             }
+            if (best < 0) { best = (int)groups.size(); groups.push_back({std::vector<char>(p.C, 0), 0, {}}); }
+            Group& g = groups[best];
+            for (int q = 0; q < m; ++q)
+                if (!g.has[S[q]]) { g.has[S[q]] = 1; ++g.nch; }
+            g.combos.push_back(c);
         }
-        if (cost < best) { best = cost; width = w; seg_rows = sr; segs = sg; }
-    };
-    for (int sr = kLen; sr <= 7 * kLen; sr += kLen) {
-        if (d < 32 && sr != 3 * kLen && sr != 7 * kLen) continue;
-        const int max_segs = std::max(1, (T + sr - 1) / sr);
-        for (int sg = 1; sg <= max_segs; sg = sg < 8 ? sg + 1 : sg * 2) consider(d, sr, sg);
-        consider(d, sr, max_segs);
-        if (kTileSamples / d - 8 >= sr) consider(d, sr, std::min(max_segs, (kTileSamples / d - 8) / sr));
-        for (int w = kThreads; w < d; w += kThreads)
-            for (int sg = 1; sg <= std::min(max_segs, 4); ++sg) consider(w, sr, sg);
+        const int rows = (p.L + d - 1) / d, bands = (rows + kMRows - 1) / kMRows;
+        for (Group& g : groups) {
+            MiniBucket b{};
+            b.d = d; b.raster_len = bands * d;
+            b.kbeg = (int)p.recs.size();
+            std::vector<int> at(p.C, 0);
+            for (int c = 0; c < p.C; ++c)
+                if (g.has[c]) { b.ch[b.nch] = c; at[c] = b.nch++; }
+            p.max_nch = std::max(p.max_nch, b.nch);
+            for (int c : g.combos) {
+                MiniRec r{};
+                r.m = p.num_channels[c];
+                for (int j = 0; j < kLen; ++j) r.w[j] = 1.0f;
+                for (int t = 0; t < 3; ++t) r.w[p.taps[3 * p.kernel_index[c] + t]] = -2.0f;
+                r.f0 = p.feature_offset[c]; r.nf = p.feature_offset[c + 1] - r.f0;
+                const int first = p.padded[c] ? 0 : 4 * d, last = p.padded[c] ? p.L : p.L - 4 * d;
+                r.tl = first / d; r.th = last / d; r.rh = last - r.th * d;
+                for (int q = 0; q < r.m; ++q) r.ch[q] = at[p.channel_idx[p.channel_offset[c] + q]] * kMPlaneBytes;
+                for (int f = r.f0; f < r.f0 + r.nf; ++f) p.nout[f] = last - first;
+                p.recs.push_back(r);
+            }
+            b.kend = (int)p.recs.size();
+            for (int c0 = 0; c0 < b.raster_len; c0 += kWarpCols) p.tiles.push_back({(int)p.buckets.size(), c0});
+            p.buckets.push_back(b);
+        }
     }
 }
 
-// false when a dilation has no tiling that fits the shared-memory tile (cannot happen for L >= 9; checked all the same)
-bool build_items(rocket_mini& p) {
-    p.items.clear();
-    std::map<int, std::array<int, 3>> tiling;           // by dilation
-    for (int c = 0; c < p.n_combos; ++c)
-        for (int f0 = p.feature_offset[c]; f0 < p.feature_offset[c + 1]; f0 += kMaxFeaturesPerItem) {
-            MiniItem it{};
-            it.d = p.dilation[c]; it.padded = p.padded[c]; it.m = p.num_channels[c];
-            it.f0 = f0; it.nf = std::min(kMaxFeaturesPerItem, p.feature_offset[c + 1] - f0);
-            for (int k = 0; k < 3; ++k) it.tap[k] = p.taps[3 * p.kernel_index[c] + k];
-            for (int q = 0; q < it.m; ++q) it.ch[q] = p.channel_idx[p.channel_offset[c] + q];
-            auto found = tiling.find(it.d);
-            if (found == tiling.end()) {
-                std::array<int, 3> t{};
-                choose_tiling(it.d, p.L, t[0], t[1], t[2]);
-                if (t[0] < 1 || t[1] < kLen || t[2] < 1 || (int64_t)(t[1] * t[2] + 8) * t[0] > kTileSamples) return false;
-                found = tiling.emplace(it.d, t).first;
-            }
-            it.width = found->second[0]; it.seg_rows = found->second[1]; it.segs = found->second[2];
-            p.items.push_back(it);
-        }
-    return true;
-}
+static constexpr size_t kMiniSmemBytes = (size_t)2 * kMPlanes * kMPlaneBytes;
 
-int ensure_mini_device(const rocket_mini* p) {
+static int ensure_mini_device(const rocket_mini* p) {
     std::lock_guard<std::mutex> lk(p->mu);
     if (p->device < 0) {
         int dev = -1;
         if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return ROCKET_ECUDA; }
-        const size_t ib = (p->items.size() * sizeof(MiniItem) + 255) / 256 * 256, bb = (size_t)p->F * sizeof(float);
-        cudaError_t e = rocket::device_malloc(&p->blob, ib + bb + 256);
+        struct Part { const void* src; size_t bytes, off; };
+        Part parts[6] = {{p->recs.data(), p->recs.size() * sizeof(MiniRec), 0},     {p->buckets.data(), p->buckets.size() * sizeof(MiniBucket), 0},
+                         {p->tiles.data(), p->tiles.size() * sizeof(MiniTile), 0}, {p->nout.data(), p->nout.size() * sizeof(int32_t), 0},
+                         {nullptr, (size_t)p->F * sizeof(float), 0},               {nullptr, 256, 0}};
+        size_t total = 0;
+        for (Part& pt : parts) { pt.off = total; total += (pt.bytes + 255) / 256 * 256; }
+        cudaError_t e = rocket::device_malloc(&p->blob, total);
         if (e != cudaSuccess) { cudaGetLastError(); p->blob = nullptr; return e == cudaErrorMemoryAllocation ? ROCKET_ENOMEM : ROCKET_ECUDA; }
-        if (cudaMemcpy(p->blob, p->items.data(), p->items.size() * sizeof(MiniItem), cudaMemcpyHostToDevice) != cudaSuccess) {
-            cudaGetLastError(); cudaFree(p->blob); p->blob = nullptr; return ROCKET_ECUDA;
-        }
-        if (cudaFuncSetAttribute(mini_transform_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kTileSamples * sizeof(float))) != cudaSuccess) {
-            cudaGetLastError(); cudaFree(p->blob); p->blob = nullptr; return ROCKET_ECUDA;
-        }
-        p->d_items = static_cast<const MiniItem*>(p->blob);
-        p->d_bias = reinterpret_cast<float*>(static_cast<char*>(p->blob) + ib);
+        char* base = static_cast<char*>(p->blob);
+        e = cudaMemset(base + parts[5].off, 0, 256);
+        for (const Part& pt : parts)
+            if (e == cudaSuccess && pt.src) e = cudaMemcpy(base + pt.off, pt.src, pt.bytes, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
+        if (e != cudaSuccess) { cudaGetLastError(); cudaFree(p->blob); p->blob = nullptr; return ROCKET_ECUDA; }
+        MiniArgs& a = p->dev;
+        a.recs = reinterpret_cast<const MiniRec*>(base + parts[0].off);
+        a.buckets = reinterpret_cast<const MiniBucket*>(base + parts[1].off);
+        a.tiles = reinterpret_cast<const MiniTile*>(base + parts[2].off);
+        p->d_nout = reinterpret_cast<const int*>(base + parts[3].off);
+        a.bias = reinterpret_cast<const float*>(base + parts[4].off);
+        a.error_flag = reinterpret_cast<int*>(base + parts[5].off);
+        a.C = p->C; a.L = p->L; a.F = p->F; a.n_tiles = (int)p->tiles.size();
         p->device = dev;
         p->bias_uploaded = false;
     }
@@ -387,15 +437,13 @@ int ensure_mini_device(const rocket_mini* p) {
         int prev = -1;
         cudaGetDevice(&prev);
         if (prev != p->device) cudaSetDevice(p->device);
-        const cudaError_t e = cudaMemcpy(p->d_bias, p->bias.data(), (size_t)p->F * sizeof(float), cudaMemcpyHostToDevice);
+        const cudaError_t e = cudaMemcpy(const_cast<float*>(p->dev.bias), p->bias.data(), (size_t)p->F * sizeof(float), cudaMemcpyHostToDevice);
         if (prev != p->device) cudaSetDevice(prev);
         if (e != cudaSuccess) { cudaGetLastError(); return ROCKET_ECUDA; }
         p->bias_uploaded = true;
     }
     return ROCKET_OK;
 }
-
-}  // namespace
 
 extern "C" {
 
@@ -451,10 +499,7 @@ int rocket_mini_create(uint64_t seed, int C, int L, int num_features, rocket_min
         p->quantile.resize(p->F);
         for (int f = 0; f < p->F; ++f) p->quantile[f] = std::fmod((f + 1.0) * kInvGoldenRatio, 1.0);
         p->bias.assign(p->F, 0.0f);
-        if (!build_items(*p)) {
-            delete p;
-            return ROCKET_EUNSUPPORTED;
-        }
+        build_tiles(*p);
     } catch (const std::bad_alloc&) {
         delete p;
         return ROCKET_ENOMEM;
@@ -565,16 +610,33 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     if (!p->fitted) return ROCKET_EINVAL;
     if (N == 0) return ROCKET_OK;
     if (!X_dev || !feat_dev) return ROCKET_EINVAL;
-    const long long blocks = (long long)N * (long long)p->items.size();
-    if (blocks > 0x7fffffffll) return ROCKET_EUNSUPPORTED;
+    if ((long long)N * (long long)p->tiles.size() > 0x7fffffffll / 8) return ROCKET_EUNSUPPORTED;
     const int st = ensure_mini_device(p);
     if (st != ROCKET_OK) return st;
     int prev = -1;
     if (cudaGetDevice(&prev) != cudaSuccess) { cudaGetLastError(); return ROCKET_ECUDA; }
     if (prev != p->device && cudaSetDevice(p->device) != cudaSuccess) { cudaGetLastError(); return ROCKET_ECUDA; }
-    mini_transform_kernel<<<(unsigned)blocks, kThreads, kTileSamples * sizeof(float), static_cast<cudaStream_t>(cuda_stream)>>>(
-        X_dev, C, L, p->d_items, (int)p->items.size(), p->d_bias, feat_dev, p->F);
-    rocket::count_launch();
+    int sms = 0;
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    sms = std::max(sms, 1);
+    MiniArgs args = p->dev;
+    args.X = X_dev;
+    args.counts = reinterpret_cast<int*>(feat_dev);
+    args.N = N;
+    // Examples that share a tile: as many as its planes hold, while every SM still gets four tiles; fewer tiles than SMs are
+    // dealt in parts of their combinations (84 or so) instead.
+    const long long tiles = (long long)N * args.n_tiles;
+    args.examples = (int)std::max<long long>(1, std::min<long long>({kMPlanes / p->max_nch, N, tiles / (4ll * sms)}));
+    args.groups = (N + args.examples - 1) / args.examples;
+    const long long items = (long long)args.groups * args.n_tiles;
+    args.parts = (int)std::max<long long>(1, std::min<long long>(8, 2ll * sms / items));
+    const unsigned grid = (unsigned)std::min<long long>(items * args.parts, sms);
+    cudaMemsetAsync(feat_dev, 0, (size_t)N * p->F * sizeof(float), stream);
+    mini_tile_kernel<<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
+    const long long values = (long long)N * p->F;
+    mini_finalize_kernel<<<(unsigned)((values + 255) / 256), 256, 0, stream>>>(feat_dev, p->d_nout, p->F, values, args.error_flag);
+    rocket::count_launch(2);
     const cudaError_t e = cudaGetLastError();
     if (prev != p->device) cudaSetDevice(prev);
     if (e != cudaSuccess) { cudaGetLastError(); return ROCKET_ECUDA; }
