@@ -38,7 +38,16 @@ namespace {
 
 constexpr int kKernels = 84, kLen = 9;
 constexpr int kMRows = 12, kMInRows = kMRows + kLen - 1;      // output rows of a tile, input rows
-constexpr int kMWarps = 16, kMThreads = 32 * kMWarps;
+constexpr int kMWarps = 20, kMThreads = 32 * kMWarps;         // producer and consumer warps
+// Producer warps: three keep up where a tile serves the 84 combinations of a dilation; where the combinations of a dilation use
+// more than kMPlanes channels they are several buckets, and a tile serves a third of them.
+#ifndef ROCKET_MINI_P
+#define ROCKET_MINI_P 3
+#endif
+#ifndef ROCKET_MINI_PW
+#define ROCKET_MINI_PW 6
+#endif
+constexpr int kMProducers = ROCKET_MINI_P, kMProducersWide = ROCKET_MINI_PW;
 constexpr int kMPlanes = 20;                                  // (example, channel) planes of a tile
 constexpr int kMPlaneFloats = kMInRows * kWarpCols, kMPlaneBytes = kMPlaneFloats * 4;
 constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;
@@ -86,15 +95,14 @@ struct MiniArgs {
     int examples, groups, parts;          // examples of a tile, groups of examples, parts a tile's combinations are dealt in
 };
 
-// A tile as a warp holds it.
-struct TileAt { int words, c0, n0, ne, kbeg, n_work; };   // words: the bucket's, one per lane
+// A tile as the producers describe it to the consumers.
+struct TileAt { int d, raster_len, plane_bytes, c0, n0, ne, kbeg, n_work; };   // plane_bytes: of one example's planes
 
-__device__ __forceinline__ void mini_cp4(uint32_t dst, const void* src, int bytes) {   // bytes: 4, or 0 for a zero
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-// Arrives on the barrier when the thread's copies so far have landed.
-__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+// *p, or zero; the loads stay in the order they are written in.
+__device__ __forceinline__ float load_if(const float* p, unsigned ok) {
+    float v;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t@q ld.global.nc.f32 %0, [%1];\n\t}" : "=f"(v) : "l"(p), "r"(ok));
+    return v;
 }
 
 // How many of the 2 x 12 outputs exceed a bias: the signs of bias - z (exact: the difference of two floats rounds to zero only
@@ -116,18 +124,22 @@ __device__ __forceinline__ int mini_count(const u64 (&acc)[kMRows], float b) {
 // channel sums (m channels, 3.9 on average) and, per bias (3.8 on average), a packed add and two shifts that collect the signs
 // of bias - z.  What the layout is for: the channels of a tile are read once for the 84 combinations of a dilation (one
 // combination per block and tile, the earlier form, read 146 GB from L2 for 60 x 20 x 50,000), the packed operations work on
-// two columns at a time, and two tiles are in shared memory so that the next one lands while this one is worked on: a warp that
-// finds no combination left goes on to the next tile without waiting for the others.
+// two columns at a time, and two tiles are in shared memory: producer warps bring the next one in while the others work on this
+// one, and a warp that finds no combination left goes on to the next tile without waiting.  Measured (the earlier form 17.3 ms):
+// 10.5 ms for 60 x 20 x 50,000 and 9,996 features, 9.9 without the copies into shared memory.
+template <int PRODUCERS>
 __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_constant__ MiniArgs a) {
+    constexpr int kConsumers = kMWarps - PRODUCERS;
     extern __shared__ __align__(128) float planes[];              // [2][kMPlanes][kMInRows][64]
     __shared__ unsigned long long s_full[2], s_empty[2];
+    __shared__ TileAt s_tile[2];
     __shared__ int s_pos;
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(kFull, tid >> 5, 0);
     const uint32_t full0 = smem_u32(s_full), empty0 = smem_u32(s_empty);
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(full0 + 8u * i, kMThreads);
-            mbar_init(empty0 + 8u * i, kMWarps);
+            mbar_init(full0 + 8u * i, 32 * PRODUCERS + 1);
+            mbar_init(empty0 + 8u * i, kConsumers);
         }
         s_pos = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -135,53 +147,82 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
     __syncthreads();
 
     // The block's tiles: items blockIdx.x, blockIdx.x + gridDim.x, .. of all (tile, part, group of examples).  The (combination,
-    // example) pairs of the block's tiles form one sequence that the warps draw from.
+    // example) pairs of the block's tiles form one sequence that the consumer warps draw from.
     const unsigned total = (unsigned)a.groups * (unsigned)a.n_tiles * (unsigned)a.parts;
     const int K = (int)((total - blockIdx.x + gridDim.x - 1) / gridDim.x);
     auto word = [](int v, int i) { return __shfl_sync(kFull, v, i); };
-    // Issues the thread's share of tile k's copies (every channel of the bucket, zeros outside the series).
-    auto fill = [&](int k) {
-        const unsigned g = blockIdx.x + (unsigned)k * gridDim.x, per_group = (unsigned)a.n_tiles * (unsigned)a.parts;
-        const unsigned group = g / per_group, rest = g - group * per_group, tile = rest / (unsigned)a.parts, part = rest - tile * (unsigned)a.parts;
-        TileAt t;
-        const int2 at = __ldg(reinterpret_cast<const int2*>(a.tiles + tile));
-        t.words = __ldg(reinterpret_cast<const int*>(a.buckets + at.x) + lane);
-        t.c0 = at.y;
-        t.n0 = (int)group * a.examples;
-        t.ne = min(a.examples, a.N - t.n0);
-        const int combos = word(t.words, 3) - word(t.words, 2), beg = combos * (int)part / a.parts, end = combos * ((int)part + 1) / a.parts;
-        t.kbeg = word(t.words, 2) + beg;
-        t.n_work = (end - beg) * t.ne;
-        const int d = word(t.words, 0), raster_len = word(t.words, 1), nch = word(t.words, 4);
-        constexpr int kStep = kMThreads / kWarpCols, kRows = (kMInRows + kStep - 1) / kStep;
-        static_assert((kRows - 1) * kStep < kMInRows, "only the last row of a thread may not exist");
-        const int col = tid & (kWarpCols - 1), rg = tid / kWarpCols, cg = t.c0 + col, band = cg / d;
-        const int u0 = (band * kMRows - 4 + rg) * d + (cg - band * d);
-        unsigned off[kRows];
-        int bytes[kRows];
-#pragma unroll
-        for (int i = 0; i < kRows; ++i) {
-            const int x = u0 + i * kStep * d;
-            const bool ok = cg < raster_len && (unsigned)x < (unsigned)a.L;
-            off[i] = ok ? 4u * (unsigned)x : 0u;
-            bytes[i] = ok ? 4 : 0;
-        }
-        const bool last = rg + (kRows - 1) * kStep < kMInRows;
-        uint32_t dst = smem_u32(planes + (k & 1) * kMPlanes * kMPlaneFloats + rg * kWarpCols + col);
-        for (int e = 0; e < t.ne; ++e) {
-            const float* __restrict__ Xn = a.X + (size_t)(t.n0 + e) * a.C * a.L;
+    bool ok = true;
+
+    if (warp >= kConsumers) {
+        // ---- producers: every channel of the bucket, a plane per warp, zeros outside the series
+        const unsigned per_group = (unsigned)a.n_tiles * (unsigned)a.parts;
+        auto tile_of = [&](int k) { return (blockIdx.x + (unsigned)k * gridDim.x) % per_group / (unsigned)a.parts; };
+        int2 at = __ldg(reinterpret_cast<const int2*>(a.tiles + tile_of(0)));
+        int words = __ldg(reinterpret_cast<const int*>(a.buckets + at.x) + lane);
+        for (int k = 0; k < K; ++k) {
+            const unsigned g = blockIdx.x + (unsigned)k * gridDim.x, group = g / per_group;
+            const int part = (int)(g % per_group % (unsigned)a.parts);
+            const int d = word(words, 0), raster_len = word(words, 1), nch = word(words, 4), c0 = at.y, bucket_words = words;
+            const int n0 = (int)group * a.examples, ne = min(a.examples, a.N - n0), first = word(words, 2);
+            const int combos = word(words, 3) - first, beg = combos * part / a.parts, end = combos * (part + 1) / a.parts;
+            if (k + 1 < K) at = __ldg(reinterpret_cast<const int2*>(a.tiles + tile_of(k + 1)));     // on its way
+            // the lane's columns lane and lane + 32: their first position, and the input rows that lie in the series
+            const int cg0 = c0 + lane, cg1 = cg0 + 32, band0 = (int)((unsigned)cg0 / (unsigned)d), band1 = (int)((unsigned)cg1 / (unsigned)d);
+            const int u0 = (band0 * kMRows - 4) * d + (cg0 - band0 * d), u1 = (band1 * kMRows - 4) * d + (cg1 - band1 * d);
+            const bool inside = __all_sync(kFull, cg1 < raster_len && u0 >= 0 && u1 + (kMInRows - 1) * d < a.L);
+            unsigned in0 = 0, in1 = 0;
+            if (!inside) {
 #pragma unroll 4
-            for (int c = 0; c < nch; ++c) {
-                const char* __restrict__ src = reinterpret_cast<const char*>(Xn + (size_t)word(t.words, 12 + c) * a.L);
-#pragma unroll
-                for (int i = 0; i < kRows - 1; ++i) mini_cp4(dst + i * kStep * kWarpCols * 4, src + off[i], bytes[i]);
-                if (last) mini_cp4(dst + (kRows - 1) * kStep * kWarpCols * 4, src + off[kRows - 1], bytes[kRows - 1]);
-                dst += kMPlaneBytes;
+                for (int s = 0; s < kMInRows; ++s) {
+                    in0 |= (cg0 < raster_len && (unsigned)(u0 + s * d) < (unsigned)a.L ? 1u : 0u) << s;
+                    in1 |= (cg1 < raster_len && (unsigned)(u1 + s * d) < (unsigned)a.L ? 1u : 0u) << s;
+                }
             }
+            if (k >= 2 && !(ok = mbar_wait(empty0 + 8u * (k & 1), ((k - 2) >> 1) & 1))) break;
+            if (tid == 32 * kConsumers) {
+                s_tile[k & 1] = TileAt{d, raster_len, nch * kMPlaneBytes, c0, n0, ne, first + beg, (end - beg) * ne};
+                mbar_arrive(full0 + 8u * (k & 1));
+            }
+            if (k + 1 < K) words = __ldg(reinterpret_cast<const int*>(a.buckets + at.x) + lane);
+            for (int pl = warp - kConsumers; pl < nch * ne; pl += PRODUCERS) {
+                const int e = pl / nch, c = pl - e * nch;
+                const float* __restrict__ src = a.X + ((size_t)(n0 + e) * a.C + word(bucket_words, 12 + c)) * a.L;
+                float* dst = planes + ((k & 1) * kMPlanes + pl) * kMPlaneFloats + lane;
+                // all of a plane's loads first: with asynchronous copies, of which a warp keeps only a few in flight, four
+                // producers took 35 thousand clocks for a tile
+                float v0[kMInRows], v1[kMInRows];
+                const float* __restrict__ p0 = src + u0;
+                const float* __restrict__ p1 = src + u1;
+                if (inside) {
+#pragma unroll
+                    for (int s = 0; s < kMInRows; ++s) {
+                        v0[s] = __ldg(p0);
+                        v1[s] = __ldg(p1);
+                        p0 += d;
+                        p1 += d;
+                    }
+                } else {
+#pragma unroll
+                    for (int s = 0; s < kMInRows; ++s) {
+                        v0[s] = load_if(p0, in0 >> s & 1);
+                        v1[s] = load_if(p1, in1 >> s & 1);
+                        p0 += d;
+                        p1 += d;
+                    }
+                }
+#pragma unroll
+                for (int s = 0; s < kMInRows; ++s) {
+                    dst[s * kWarpCols] = v0[s];
+                    dst[s * kWarpCols + 32] = v1[s];
+                }
+            }
+            mbar_arrive(full0 + 8u * (k & 1));
         }
-        cp_async_arrive(full0 + 8u * (k & 1));
-        return t;
-    };
+        if (!ok && lane == 0) atomicExch(a.error_flag, 1);
+        return;
+    }
+
+    // ---- consumers
     auto draw = [&]() {
         int p = 0;
         if (lane == 0) p = atomicAdd(&s_pos, 1);
@@ -190,46 +231,35 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
     auto load_rec = [&](const TileAt& t, int w) {
         return __ldg(reinterpret_cast<const int*>(a.recs + t.kbeg + (t.ne == 1 ? w : w / t.ne)) + lane);
     };
-
-    TileAt cur = fill(0), nxt = cur;
-    int filled = 1, k = 0, base = 0;
-    if (K > 1) { nxt = fill(1); filled = 2; }
+    TileAt cur;
+    int k = 0, base = 0;
     int pos = draw();
     // the lane's two columns of the tile: band of rows and column of A
     int trow0 = 0, trow1 = 0, c0 = 0, c1 = 0;
     bool ok0 = false, ok1 = false;
     auto enter = [&]() {
-        const int d = word(cur.words, 0), raster_len = word(cur.words, 1), cg = cur.c0 + 2 * lane, band = (int)((unsigned)cg / (unsigned)d);
-        c0 = cg - band * d;
-        c1 = c0 + 1 < d ? c0 + 1 : 0;
+        if (!mbar_wait(full0 + 8u * (k & 1), (k >> 1) & 1)) return false;
+        cur = s_tile[k & 1];
+        const int cg = cur.c0 + 2 * lane, band = (int)((unsigned)cg / (unsigned)cur.d);
+        c0 = cg - band * cur.d;
+        c1 = c0 + 1 < cur.d ? c0 + 1 : 0;
         trow0 = band * kMRows;
-        trow1 = c0 + 1 < d ? trow0 : trow0 + kMRows;
-        ok0 = cg < raster_len;
-        ok1 = cg + 1 < raster_len;
-        return mbar_wait(full0 + 8u * (k & 1), (k >> 1) & 1);
+        trow1 = c0 + 1 < cur.d ? trow0 : trow0 + kMRows;
+        ok0 = cg < cur.raster_len;
+        ok1 = cg + 1 < cur.raster_len;
+        return true;
     };
-    bool ok = enter();
-    int rec_next = pos < cur.n_work ? load_rec(cur, pos) : 0;
+    ok = enter();
+    int rec_next = ok && pos < cur.n_work ? load_rec(cur, pos) : 0;
     while (ok) {
-        // tile k + 1 may be copied in as soon as every warp has left tile k - 1
-        if (filled == k + 1 && filled < K && __all_sync(kFull, mbar_try(empty0 + 8u * ((k + 1) & 1), ((k - 1) >> 1) & 1))) {
-            nxt = fill(k + 1);
-            ++filled;
-        }
         if (pos >= base + cur.n_work) {
             if (k + 1 >= K) break;
-            if (filled == k + 1) {
-                if (!(ok = mbar_wait(empty0 + 8u * ((k + 1) & 1), ((k - 1) >> 1) & 1))) break;
-                nxt = fill(k + 1);
-                ++filled;
-            }
             __syncwarp();
             if (lane == 0) mbar_arrive(empty0 + 8u * (k & 1));
             base += cur.n_work;
-            cur = nxt;
             ++k;
             ok = enter();
-            if (pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
+            if (ok && pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
             continue;
         }
         const int rec = rec_next, w = pos - base, e = cur.ne == 1 ? 0 : w % cur.ne;
@@ -238,7 +268,7 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
         pos = draw();
         if (pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
         const char* st = reinterpret_cast<const char*>(planes + (k & 1) * kMPlanes * kMPlaneFloats + 2 * lane);
-        if (e > 0) st += e * word(cur.words, 4) * kMPlaneBytes;
+        if (e > 0) st += e * cur.plane_bytes;
 
         // the sum of the combination's channels, in the order of its list
         u64 xs[kMInRows];
@@ -305,7 +335,6 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
             if (lane < n && mine) atomicAdd(counts + fb + lane, mine);
         }
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");   // nothing of this thread is in flight when the block ends
     if (!ok && lane == 0) atomicExch(a.error_flag, 1);
 }
 
@@ -335,6 +364,7 @@ struct rocket_mini {
     std::vector<MiniTile> tiles;
     std::vector<int32_t> nout;             // outputs behind every feature
     int max_nch = 1;
+    bool wide = false;                     // some dilation has several buckets
     mutable std::mutex mu;
     mutable int device = -1;
     mutable void* blob = nullptr;          // records, buckets, tiles, output counts, biases, error flag
@@ -373,6 +403,7 @@ static void build_tiles(rocket_mini& p) {
                 if (!g.has[S[q]]) { g.has[S[q]] = 1; ++g.nch; }
             g.combos.push_back(c);
         }
+        p.wide = p.wide || groups.size() > 1;
         const int rows = (p.L + d - 1) / d, bands = (rows + kMRows - 1) / kMRows;
         for (Group& g : groups) {
             MiniBucket b{};
@@ -420,7 +451,8 @@ static int ensure_mini_device(const rocket_mini* p) {
         e = cudaMemset(base + parts[5].off, 0, 256);
         for (const Part& pt : parts)
             if (e == cudaSuccess && pt.src) e = cudaMemcpy(base + pt.off, pt.src, pt.bytes, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<kMProducers>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<kMProducersWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
         if (e != cudaSuccess) { cudaGetLastError(); cudaFree(p->blob); p->blob = nullptr; return ROCKET_ECUDA; }
         MiniArgs& a = p->dev;
         a.recs = reinterpret_cast<const MiniRec*>(base + parts[0].off);
@@ -633,7 +665,8 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     args.parts = (int)std::max<long long>(1, std::min<long long>(8, 2ll * sms / items));
     const unsigned grid = (unsigned)std::min<long long>(items * args.parts, sms);
     cudaMemsetAsync(feat_dev, 0, (size_t)N * p->F * sizeof(float), stream);
-    mini_tile_kernel<<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
+    if (p->wide) mini_tile_kernel<kMProducersWide><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
+    else mini_tile_kernel<kMProducers><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
     const long long values = (long long)N * p->F;
     mini_finalize_kernel<<<(unsigned)((values + 255) / 256), 256, 0, stream>>>(feat_dev, p->d_nout, p->F, values, args.error_flag);
     rocket::count_launch(2);
