@@ -38,17 +38,9 @@ namespace {
 
 constexpr int kKernels = 84, kLen = 9;
 constexpr int kMRows = 12, kMInRows = kMRows + kLen - 1;      // output rows of a tile, input rows
-constexpr int kMWarps = 20, kMThreads = 32 * kMWarps;         // producer and consumer warps
-// Producer warps: three keep up where a tile serves the 84 combinations of a dilation; where the combinations of a dilation use
-// more than kMPlanes channels they are several buckets, and a tile serves a third of them.
-#ifndef ROCKET_MINI_P
-#define ROCKET_MINI_P 3
-#endif
-#ifndef ROCKET_MINI_PW
-#define ROCKET_MINI_PW 6
-#endif
-constexpr int kMProducers = ROCKET_MINI_P, kMProducersWide = ROCKET_MINI_PW;
-constexpr int kMPlanes = 20;                                  // (example, channel) planes of a tile
+constexpr int kMWarps = 20, kMThreads = 32 * kMWarps;
+constexpr int kMProducers = 3;                                // producer warps of the double-buffered form
+constexpr int kMPlanes = 20, kMPlanesWide = 2 * kMPlanes;     // (example, channel) planes of a tile: two tiles in shared memory, or one
 constexpr int kMPlaneFloats = kMInRows * kWarpCols, kMPlaneBytes = kMPlaneFloats * 4;
 constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;
 constexpr uint64_t kStreamBase = 1ull << 32;
@@ -74,12 +66,13 @@ struct alignas(16) MiniRec {
     int32_t pad2_[6];
 };
 static_assert(sizeof(MiniRec) == 128, "MiniRec must be 32 words");
-// Combinations [kbeg, kend) of one dilation that use at most kMPlanes channels between them (32 words).
+// Combinations [kbeg, kend) of one dilation that use at most kMPlanes channels between them, kMPlanesWide in a handle whose
+// tiles have shared memory to themselves (64 words).
 struct alignas(16) MiniBucket {
     int32_t d, raster_len, kbeg, kend, nch, pad_[7];
-    int32_t ch[kMPlanes];
+    int32_t ch[kMPlanesWide], pad2_[12];
 };
-static_assert(sizeof(MiniBucket) == 128, "MiniBucket must be 32 words");
+static_assert(sizeof(MiniBucket) == 256, "MiniBucket must be 64 words");
 // 64 consecutive columns of a bucket's raster: bands of kMRows rows of A, strung together band by band.
 struct MiniTile { int32_t bucket, c0; };
 
@@ -105,6 +98,64 @@ __device__ __forceinline__ float load_if(const float* p, unsigned ok) {
     return v;
 }
 
+// The columns lane and lane + 32 of a tile: their first position, and the input rows that lie in the series.
+struct FillAt {
+    int d, u0, u1;
+    unsigned in0 = 0, in1 = 0;
+    bool inside;
+    __device__ __forceinline__ FillAt(int d_, int raster_len, int c0, int L, int lane) : d(d_) {
+        const int cg0 = c0 + lane, cg1 = cg0 + 32, band0 = (int)((unsigned)cg0 / (unsigned)d), band1 = (int)((unsigned)cg1 / (unsigned)d);
+        u0 = (band0 * kMRows - 4) * d + (cg0 - band0 * d);
+        u1 = (band1 * kMRows - 4) * d + (cg1 - band1 * d);
+        inside = __all_sync(kFull, cg1 < raster_len && u0 >= 0 && u1 + (kMInRows - 1) * d < L);
+        if (!inside) {
+#pragma unroll 4
+            for (int s = 0; s < kMInRows; ++s) {
+                in0 |= (cg0 < raster_len && (unsigned)(u0 + s * d) < (unsigned)L ? 1u : 0u) << s;
+                in1 |= (cg1 < raster_len && (unsigned)(u1 + s * d) < (unsigned)L ? 1u : 0u) << s;
+            }
+        }
+    }
+};
+
+// Planes warp, warp + warps, .. of a tile: the bucket's nch channels of ne examples, zeros outside the series.  All of a plane's
+// loads come before its stores: of 4-byte asynchronous copies a warp keeps only a few in flight, and with them four warps took
+// 35 thousand clocks for a tile.
+template <class Channel>
+__device__ __forceinline__ void fill_planes(const MiniArgs& a, const FillAt& at, float* to, Channel channel, int nch, int n0, int ne,
+                                            int warp, int warps, int lane) {
+    for (int pl = warp; pl < nch * ne; pl += warps) {
+        const int e = pl / nch, c = pl - e * nch;
+        const float* __restrict__ src = a.X + ((size_t)(n0 + e) * a.C + channel(c)) * a.L;
+        float* dst = to + pl * kMPlaneFloats + lane;
+        float v0[kMInRows], v1[kMInRows];
+        const float* __restrict__ p0 = src + at.u0;
+        const float* __restrict__ p1 = src + at.u1;
+        if (at.inside) {
+#pragma unroll
+            for (int s = 0; s < kMInRows; ++s) {
+                v0[s] = __ldg(p0);
+                v1[s] = __ldg(p1);
+                p0 += at.d;
+                p1 += at.d;
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < kMInRows; ++s) {
+                v0[s] = load_if(p0, at.in0 >> s & 1);
+                v1[s] = load_if(p1, at.in1 >> s & 1);
+                p0 += at.d;
+                p1 += at.d;
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < kMInRows; ++s) {
+            dst[s * kWarpCols] = v0[s];
+            dst[s * kWarpCols + 32] = v1[s];
+        }
+    }
+}
+
 // How many of the 2 x 12 outputs exceed a bias: the signs of bias - z (exact: the difference of two floats rounds to zero only
 // when they are equal).  acc = -z.
 __device__ __forceinline__ int mini_count(const u64 (&acc)[kMRows], float b) {
@@ -127,9 +178,9 @@ __device__ __forceinline__ int mini_count(const u64 (&acc)[kMRows], float b) {
 // two columns at a time, and two tiles are in shared memory: producer warps bring the next one in while the others work on this
 // one, and a warp that finds no combination left goes on to the next tile without waiting.  Measured (the earlier form 17.3 ms):
 // 10.5 ms for 60 x 20 x 50,000 and 9,996 features, 9.9 without the copies into shared memory.
-template <int PRODUCERS>
+template <bool WIDE>
 __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_constant__ MiniArgs a) {
-    constexpr int kConsumers = kMWarps - PRODUCERS;
+    constexpr int kConsumers = WIDE ? kMWarps : kMWarps - kMProducers;
     extern __shared__ __align__(128) float planes[];              // [2][kMPlanes][kMInRows][64]
     __shared__ unsigned long long s_full[2], s_empty[2];
     __shared__ TileAt s_tile[2];
@@ -138,7 +189,7 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
     const uint32_t full0 = smem_u32(s_full), empty0 = smem_u32(s_empty);
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(full0 + 8u * i, 32 * PRODUCERS + 1);
+            mbar_init(full0 + 8u * i, 32 * kMProducers + 1);
             mbar_init(empty0 + 8u * i, kConsumers);
         }
         s_pos = 0;
@@ -153,7 +204,7 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
     auto word = [](int v, int i) { return __shfl_sync(kFull, v, i); };
     bool ok = true;
 
-    if (warp >= kConsumers) {
+    if (!WIDE && warp >= kConsumers) {
         // ---- producers: every channel of the bucket, a plane per warp, zeros outside the series
         const unsigned per_group = (unsigned)a.n_tiles * (unsigned)a.parts;
         auto tile_of = [&](int k) { return (blockIdx.x + (unsigned)k * gridDim.x) % per_group / (unsigned)a.parts; };
@@ -166,56 +217,14 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
             const int n0 = (int)group * a.examples, ne = min(a.examples, a.N - n0), first = word(words, 2);
             const int combos = word(words, 3) - first, beg = combos * part / a.parts, end = combos * (part + 1) / a.parts;
             if (k + 1 < K) at = __ldg(reinterpret_cast<const int2*>(a.tiles + tile_of(k + 1)));     // on its way
-            // the lane's columns lane and lane + 32: their first position, and the input rows that lie in the series
-            const int cg0 = c0 + lane, cg1 = cg0 + 32, band0 = (int)((unsigned)cg0 / (unsigned)d), band1 = (int)((unsigned)cg1 / (unsigned)d);
-            const int u0 = (band0 * kMRows - 4) * d + (cg0 - band0 * d), u1 = (band1 * kMRows - 4) * d + (cg1 - band1 * d);
-            const bool inside = __all_sync(kFull, cg1 < raster_len && u0 >= 0 && u1 + (kMInRows - 1) * d < a.L);
-            unsigned in0 = 0, in1 = 0;
-            if (!inside) {
-#pragma unroll 4
-                for (int s = 0; s < kMInRows; ++s) {
-                    in0 |= (cg0 < raster_len && (unsigned)(u0 + s * d) < (unsigned)a.L ? 1u : 0u) << s;
-                    in1 |= (cg1 < raster_len && (unsigned)(u1 + s * d) < (unsigned)a.L ? 1u : 0u) << s;
-                }
-            }
+            const FillAt at_columns(d, raster_len, c0, a.L, lane);
             if (k >= 2 && !(ok = mbar_wait(empty0 + 8u * (k & 1), ((k - 2) >> 1) & 1))) break;
             if (tid == 32 * kConsumers) {
                 s_tile[k & 1] = TileAt{d, raster_len, nch * kMPlaneBytes, c0, n0, ne, first + beg, (end - beg) * ne};
                 mbar_arrive(full0 + 8u * (k & 1));
             }
             if (k + 1 < K) words = __ldg(reinterpret_cast<const int*>(a.buckets + at.x) + lane);
-            for (int pl = warp - kConsumers; pl < nch * ne; pl += PRODUCERS) {
-                const int e = pl / nch, c = pl - e * nch;
-                const float* __restrict__ src = a.X + ((size_t)(n0 + e) * a.C + word(bucket_words, 12 + c)) * a.L;
-                float* dst = planes + ((k & 1) * kMPlanes + pl) * kMPlaneFloats + lane;
-                // all of a plane's loads first: with asynchronous copies, of which a warp keeps only a few in flight, four
-                // producers took 35 thousand clocks for a tile
-                float v0[kMInRows], v1[kMInRows];
-                const float* __restrict__ p0 = src + u0;
-                const float* __restrict__ p1 = src + u1;
-                if (inside) {
-#pragma unroll
-                    for (int s = 0; s < kMInRows; ++s) {
-                        v0[s] = __ldg(p0);
-                        v1[s] = __ldg(p1);
-                        p0 += d;
-                        p1 += d;
-                    }
-                } else {
-#pragma unroll
-                    for (int s = 0; s < kMInRows; ++s) {
-                        v0[s] = load_if(p0, in0 >> s & 1);
-                        v1[s] = load_if(p1, in1 >> s & 1);
-                        p0 += d;
-                        p1 += d;
-                    }
-                }
-#pragma unroll
-                for (int s = 0; s < kMInRows; ++s) {
-                    dst[s * kWarpCols] = v0[s];
-                    dst[s * kWarpCols + 32] = v1[s];
-                }
-            }
+            fill_planes(a, at_columns, planes + (k & 1) * kMPlanes * kMPlaneFloats, [&](int c) { return word(bucket_words, 12 + c); }, nch, n0, ne, warp - kConsumers, kMProducers, lane);
             mbar_arrive(full0 + 8u * (k & 1));
         }
         if (!ok && lane == 0) atomicExch(a.error_flag, 1);
@@ -238,8 +247,22 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
     int trow0 = 0, trow1 = 0, c0 = 0, c1 = 0;
     bool ok0 = false, ok1 = false;
     auto enter = [&]() {
-        if (!mbar_wait(full0 + 8u * (k & 1), (k >> 1) & 1)) return false;
-        cur = s_tile[k & 1];
+        if constexpr (WIDE) {
+            const unsigned g = blockIdx.x + (unsigned)k * gridDim.x, per_group = (unsigned)a.n_tiles * (unsigned)a.parts;
+            const unsigned group = g / per_group, in_group = g - group * per_group, tile = in_group / (unsigned)a.parts;
+            const int part = (int)(in_group - tile * (unsigned)a.parts);
+            const int2 at = __ldg(reinterpret_cast<const int2*>(a.tiles + tile));
+            const MiniBucket* b = a.buckets + at.x;
+            const int words = __ldg(reinterpret_cast<const int*>(b) + lane), first = word(words, 2), combos = word(words, 3) - first;
+            const int nch = word(words, 4), n0 = (int)group * a.examples, ne = min(a.examples, a.N - n0), beg = combos * part / a.parts;
+            cur = TileAt{word(words, 0), word(words, 1), nch * kMPlaneBytes, at.y, n0, ne, first + beg, (combos * (part + 1) / a.parts - beg) * ne};
+            const FillAt columns(cur.d, cur.raster_len, cur.c0, a.L, lane);
+            fill_planes(a, columns, planes, [&](int c) { return __ldg(b->ch + c); }, nch, n0, ne, warp, kMWarps, lane);
+            __syncthreads();
+        } else {
+            if (!mbar_wait(full0 + 8u * (k & 1), (k >> 1) & 1)) return false;
+            cur = s_tile[k & 1];
+        }
         const int cg = cur.c0 + 2 * lane, band = (int)((unsigned)cg / (unsigned)cur.d);
         c0 = cg - band * cur.d;
         c1 = c0 + 1 < cur.d ? c0 + 1 : 0;
@@ -254,8 +277,12 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
     while (ok) {
         if (pos >= base + cur.n_work) {
             if (k + 1 >= K) break;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(empty0 + 8u * (k & 1));
+            if constexpr (WIDE) {
+                __syncthreads();
+            } else {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty0 + 8u * (k & 1));
+            }
             base += cur.n_work;
             ++k;
             ok = enter();
@@ -267,7 +294,7 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
         float my_bias = lane < nf ? __ldg(a.bias + f0 + lane) : 0.0f;
         pos = draw();
         if (pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
-        const char* st = reinterpret_cast<const char*>(planes + (k & 1) * kMPlanes * kMPlaneFloats + 2 * lane);
+        const char* st = reinterpret_cast<const char*>(planes + (WIDE ? 0 : (k & 1) * kMPlanes * kMPlaneFloats) + 2 * lane);
         if (e > 0) st += e * cur.plane_bytes;
 
         // the sum of the combination's channels, in the order of its list
@@ -364,7 +391,7 @@ struct rocket_mini {
     std::vector<MiniTile> tiles;
     std::vector<int32_t> nout;             // outputs behind every feature
     int max_nch = 1;
-    bool wide = false;                     // some dilation has several buckets
+    bool wide = false;                     // the combinations of some dilation use more than kMPlanes channels
     mutable std::mutex mu;
     mutable int device = -1;
     mutable void* blob = nullptr;          // records, buckets, tiles, output counts, biases, error flag
@@ -381,6 +408,16 @@ static void build_tiles(rocket_mini& p) {
     std::map<int, std::vector<int>> by_d;
     for (int c = 0; c < p.n_combos; ++c)
         if (p.feature_offset[c + 1] > p.feature_offset[c]) by_d[p.dilation[c]].push_back(c);
+    // A handle whose dilations all fit has two tiles in shared memory.  With more channels one large tile is better than several
+    // small buckets for each dilation, which repeat channels and leave a tile only a dozen combinations.
+    p.wide = false;
+    for (const auto& kv : by_d) {
+        std::vector<char> has(p.C, 0);
+        for (int c : kv.second)
+            for (int q = p.channel_offset[c]; q < p.channel_offset[c + 1]; ++q) has[p.channel_idx[q]] = 1;
+        p.wide = p.wide || std::count(has.begin(), has.end(), 1) > kMPlanes;
+    }
+    const int planes = p.wide ? kMPlanesWide : kMPlanes;
     struct Group { std::vector<char> has; int nch; std::vector<int> combos; };
     for (auto& kv : by_d) {
         const int d = kv.first;
@@ -395,7 +432,7 @@ static void build_tiles(rocket_mini& p) {
             for (size_t g = 0; g < groups.size(); ++g) {
                 int fresh = 0;
                 for (int q = 0; q < m; ++q) fresh += !groups[g].has[S[q]];
-                if (groups[g].nch + fresh <= kMPlanes && fresh < best_new) { best = (int)g; best_new = fresh; }
+                if (groups[g].nch + fresh <= planes && fresh < best_new) { best = (int)g; best_new = fresh; }
             }
             if (best < 0) { best = (int)groups.size(); groups.push_back({std::vector<char>(p.C, 0), 0, {}}); }
             Group& g = groups[best];
@@ -403,7 +440,6 @@ static void build_tiles(rocket_mini& p) {
                 if (!g.has[S[q]]) { g.has[S[q]] = 1; ++g.nch; }
             g.combos.push_back(c);
         }
-        p.wide = p.wide || groups.size() > 1;
         const int rows = (p.L + d - 1) / d, bands = (rows + kMRows - 1) / kMRows;
         for (Group& g : groups) {
             MiniBucket b{};
@@ -451,8 +487,8 @@ static int ensure_mini_device(const rocket_mini* p) {
         e = cudaMemset(base + parts[5].off, 0, 256);
         for (const Part& pt : parts)
             if (e == cudaSuccess && pt.src) e = cudaMemcpy(base + pt.off, pt.src, pt.bytes, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<kMProducers>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<kMProducersWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
         if (e != cudaSuccess) { cudaGetLastError(); cudaFree(p->blob); p->blob = nullptr; return ROCKET_ECUDA; }
         MiniArgs& a = p->dev;
         a.recs = reinterpret_cast<const MiniRec*>(base + parts[0].off);
@@ -659,14 +695,14 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     // Examples that share a tile: as many as its planes hold, while every SM still gets four tiles; fewer tiles than SMs are
     // dealt in parts of their combinations (84 or so) instead.
     const long long tiles = (long long)N * args.n_tiles;
-    args.examples = (int)std::max<long long>(1, std::min<long long>({kMPlanes / p->max_nch, N, tiles / (4ll * sms)}));
+    args.examples = (int)std::max<long long>(1, std::min<long long>({(p->wide ? kMPlanesWide : kMPlanes) / p->max_nch, N, tiles / (4ll * sms)}));
     args.groups = (N + args.examples - 1) / args.examples;
     const long long items = (long long)args.groups * args.n_tiles;
     args.parts = (int)std::max<long long>(1, std::min<long long>(8, 2ll * sms / items));
     const unsigned grid = (unsigned)std::min<long long>(items * args.parts, sms);
     cudaMemsetAsync(feat_dev, 0, (size_t)N * p->F * sizeof(float), stream);
-    if (p->wide) mini_tile_kernel<kMProducersWide><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
-    else mini_tile_kernel<kMProducers><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
+    if (p->wide) mini_tile_kernel<true><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
+    else mini_tile_kernel<false><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
     const long long values = (long long)N * p->F;
     mini_finalize_kernel<<<(unsigned)((values + 255) / 256), 256, 0, stream>>>(feat_dev, p->d_nout, p->F, values, args.error_flag);
     rocket::count_launch(2);
