@@ -49,7 +49,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int ELL>
 __device__ __forceinline__ void s_grad_tile(const float* planes, const KRec* rec, int lane, const u64 (&gz)[kRS],
                                             long long* accfix, double scale) {
-    const int m = rec->m;
+    const int m = __shfl_sync(kFull, rec->m, 0);
     const int off[4] = {2 * lane, kWarpCols + 2 * lane, 2 * kWarpCols + 2 * lane, 3 * kWarpCols + 2 * lane};
     for (int q = 0; q < m; ++q) {
         u64 dw[ELL];
@@ -64,7 +64,7 @@ __device__ __forceinline__ void s_grad_tile(const float* planes, const KRec* rec
 // kernel's 0 - bias inside the first channel's pass (every output of the warp tile exists).
 template <int ELL, bool FOLD>
 __device__ __forceinline__ void s_kernel_tile(const float* planes, const KRec* rec, int lane, u64 (&acc)[kRS]) {
-    const int m = rec->m;
+    const int m = __shfl_sync(kFull, rec->m, 0);
     const int off[4] = {2 * lane, kWarpCols + 2 * lane, 2 * kWarpCols + 2 * lane, 3 * kWarpCols + 2 * lane};
     int q = 0;
     if constexpr (FOLD) {
@@ -79,7 +79,7 @@ __device__ __forceinline__ void s_kernel_tile(const float* planes, const KRec* r
 // The same in half precision (mode 3).
 template <int ELL>
 __device__ __forceinline__ void s_kernel_tile_h(const float* planes, const KRec* rec, int lane, h2 (&acc)[kRS]) {
-    const int m = rec->m;
+    const int m = __shfl_sync(kFull, rec->m, 0);
     const int off[4] = {2 * lane, kWarpCols + 2 * lane, 2 * kWarpCols + 2 * lane, 3 * kWarpCols + 2 * lane};
     for (int q = 0; q < m; ++q)
         conv_channel_h<ELL, 4 * kWarpCols, false, kRS>(planes + rec->ch[q] * kSPlaneFloats, off, rec->w2[q], acc);
@@ -194,7 +194,8 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
             const int example = ne == 1 ? 0 : kk - kernel_of(kk) * ne, n = n0 + example;
             const float* eplanes = planes + example * nch * kSPlaneFloats;   // the example's planes
             const KRec* rec = myrec + cur;
-            const int len = rec->len, korig = rec->k;
+            // the same for the warp: as a shuffle's result the compiler takes it for uniform and keeps the branches on it cheap
+            const int len = __shfl_sync(kFull, rec->len, 0), korig = rec->k;
             // on an interior tile (the plan's flag) every output exists for every kernel of the bucket
             int lo0 = 0, hi0 = kRS, lo1 = 0, hi1 = kRS;
             bool interior = tile_interior;
