@@ -241,8 +241,9 @@ void fill_record_weights(const HostParams& hp, KRec& f);
 // Copies the records of the host plan to the device again (after their weights changed).
 cudaError_t upload_records(FastState& fs);
 
-// Builds the launch plan for the kernels in hp (host side, once per handle).
-void build_plan(const HostParams& hp, int split, PlanHost& out);
+// Builds the launch plan for the kernels in hp (host side, once per handle).  all_tiles: also the T tiles of kernels that have
+// stream units, which no launch uses.
+void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles = true);
 
 // Device-side state of the fast path owned by a handle.
 struct FastState {

@@ -83,16 +83,20 @@ void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost&
             u.y0 = (int32_t)y;
             u.shape = R | f.len << 8 | (backwards ? 3 << 16 : 0);
             for (int q = 0; q < f.m; ++q) u.ch[q] = (uint8_t)f.ch[q];
+            std::vector<WUnit>& shape_units = by_shape[(f.len << 8) | R];
             const int64_t tiles = n * ncol, per = std::max<int64_t>(1, unit_visits / f.m), units = (tiles + per - 1) / per;
             for (int64_t i = 0; i < units; ++i) {
                 const int64_t beg = tiles * i / units, end = tiles * (i + 1) / units;
                 u.tile0 = (int32_t)beg; u.ntiles = (int32_t)(end - beg);
-                by_shape[(f.len << 8) | R].push_back(u);
+                shape_units.push_back(u);
             }
             rows -= n * R;
             t += n * R;
         }
     }
+    size_t total = 0;
+    for (auto& kv : by_shape) total += kv.second.size();
+    out.wunits.reserve(total);
     for (auto& kv : by_shape) out.wunits.insert(out.wunits.end(), kv.second.begin(), kv.second.end());
 }
 
@@ -105,7 +109,7 @@ void fill_record_weights(const HostParams& hp, KRec& f) {
         for (int j = 0; j < f.len; ++j) f.w2[q][2 * j] = f.w2[q][2 * j + 1] = 0.0f - W[q * f.len + j];
 }
 
-void build_plan(const HostParams& hp, int split, PlanHost& out) {
+void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) {
     out = PlanHost();
     out.flops_s = out.flops_t = 0.0;
     if (split < kTMinDilation) split = kTMinDilation;
@@ -132,8 +136,10 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
     out.enabled = !(s_kernels.empty() && t_kernels.empty());
     if (!out.enabled) return;
 
+    out.krec.reserve(s_kernels.size() + t_kernels.size());
     auto add_kernel = [&](int k) {
-        KRec f{};
+        out.krec.emplace_back();
+        KRec& f = out.krec.back();
         f.len = hp.length[k]; f.d = hp.dilation[k]; f.p = hp.padding[k]; f.m = hp.num_channels[k];
         f.nout = (int32_t)((int64_t)hp.L + 2 * (int64_t)f.p - (int64_t)(f.len - 1) * f.d);
         f.k = k; f.lo_u = -f.p; f.hi_u = f.nout - f.p;
@@ -143,7 +149,6 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
         const int32_t* S = hp.channel_idx.data() + hp.channel_offset[k];
         for (int q = 0; q < f.m; ++q) f.ch[q] = S[q];
         fill_record_weights(hp, f);
-        out.krec.push_back(f);
     };
 
     // ---- S regime: one bucket per dilation, kernels inside ordered by cost (largest first: the warps of a
@@ -270,11 +275,16 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
     });
     const size_t first_t = out.krec.size();
     for (int k : t_kernels) {
-        const int ki = (int)out.krec.size();
         add_kernel(k);
-        const KRec f = out.krec.back();
+        const KRec& f = out.krec.back();
         out.flops_t += 2.0 * f.len * f.m * (double)f.nout;
         d_max = std::max(d_max, f.d);
+    }
+    build_stream_units(hp, first_t, d_max, out);
+    // the tiles are for handles without stream units (a third of the time to make a handle of 10,000 kernels)
+    const size_t end_t = all_tiles || out.wunits.empty() ? out.krec.size() : first_t;
+    for (size_t ki = first_t; ki < end_t; ++ki) {
+        const KRec& f = out.krec[ki];
         const int64_t tmin = floor_div(f.lo_u, f.d);
         const int64_t tmax = floor_div((int64_t)f.hi_u - 1, f.d);
         const int R16 = (int)((tmax - tmin + 1 + kR - 1) / kR), C64 = (f.d + kWarpCols - 1) / kWarpCols;
@@ -354,7 +364,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
                     it.g_hi = it.wide ? win.g_hi : t_box_rows(it.rg, f.len);
                     it.box_rows = it.g_hi - it.g_lo;
                     for (int q = 0; q < f.m; ++q) it.ch[q] = (uint8_t)f.ch[q];
-                    it.krec = ki;
+                    it.krec = (int)ki;
                     const auto key = std::make_tuple(f.d, t_box_cols(it.cg), it.box_rows);
                     auto found = map_index.find(key);
                     if (found == map_index.end()) {
@@ -386,7 +396,6 @@ void build_plan(const HostParams& hp, int split, PlanHost& out) {
             }
         }
     }
-    build_stream_units(hp, first_t, d_max, out);
     // every channel row of the zero-margined copy: front zeros, L samples, zeros for the run a box may
     // read past the last sample; rounded to 128 bytes
     const int64_t pitch = (int64_t)kTPadFront + hp.L + 4ll * d_max + kTXExtra + t_box_cols(4);
