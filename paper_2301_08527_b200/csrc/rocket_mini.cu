@@ -37,7 +37,7 @@ namespace fast {
 namespace {
 
 constexpr int kKernels = 84, kLen = 9;
-constexpr int kMRows = 12, kMInRows = kMRows + kLen - 1;      // output rows of a tile, input rows
+constexpr int kMRows = 14, kMInRows = kMRows + kLen - 1;      // output rows of a tile, input rows
 constexpr int kMWarps = 20, kMThreads = 32 * kMWarps;
 constexpr int kMProducers = 3;                                // producer warps of the double-buffered form
 constexpr int kMPlanes = 20, kMPlanesWide = 2 * kMPlanes;     // (example, channel) planes of a tile: two tiles in shared memory, or one
@@ -156,7 +156,7 @@ __device__ __forceinline__ void fill_planes(const MiniArgs& a, const FillAt& at,
     }
 }
 
-// How many of the 2 x 12 outputs exceed a bias: the signs of bias - z (exact: the difference of two floats rounds to zero only
+// How many of the 2 x 14 outputs exceed a bias: the signs of bias - z (exact: the difference of two floats rounds to zero only
 // when they are equal).  acc = -z.
 __device__ __forceinline__ int mini_count(const u64 (&acc)[kMRows], float b) {
     const u64 bp = pack2(b, b);
@@ -171,13 +171,14 @@ __device__ __forceinline__ int mini_count(const u64 (&acc)[kMRows], float b) {
     return __popc(s0 | s1 << kMRows);
 }
 
-// Bound: instruction issue - per pair of outputs 9 packed multiply-adds, (m - 1) 20/12 packed adds and m 20/12 loads for the
+// Bound: instruction issue - per pair of outputs 9 packed multiply-adds, (m - 1) 22/14 packed adds and m 22/14 loads for the
 // channel sums (m channels, 3.9 on average) and, per bias (3.8 on average), a packed add and two shifts that collect the signs
 // of bias - z.  What the layout is for: the channels of a tile are read once for the 84 combinations of a dilation (one
 // combination per block and tile, the earlier form, read 146 GB from L2 for 60 x 20 x 50,000), the packed operations work on
 // two columns at a time, and two tiles are in shared memory: producer warps bring the next one in while the others work on this
 // one, and a warp that finds no combination left goes on to the next tile without waiting.  Measured (the earlier form 17.3 ms):
-// 10.5 ms for 60 x 20 x 50,000 and 9,996 features, 9.9 without the copies into shared memory.
+// 10.4 ms for 60 x 20 x 50,000 and 9,996 features (12 rows: 10.75, of which 9.9 remain without the copies into shared memory;
+// the shared memory's bandwidth counts, so the tile is as high as two of them fit: 22 input rows for 14 rows of outputs).
 template <bool WIDE>
 __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_constant__ MiniArgs a) {
     constexpr int kConsumers = WIDE ? kMWarps : kMWarps - kMProducers;
