@@ -89,18 +89,25 @@ static_assert(kRS >= 8 && kRS <= 32, "the row masks of the pooling hold at most 
 constexpr int kSRowsMax = kRS + ROCKET_MAX_LENGTH - 1;             // staged rows an S warp tile reads
 constexpr int kSThreads = ROCKET_S_THREADS, kSWarps = kSThreads / 32;   // one block per SM
 constexpr int kSPlaneFloats = kSRowsMax * kWarpCols;               // one channel of an S tile
+// Wide handles: the kernels of some dilation use more than kSMaxPlanes channels, none more than kSWidePlanes.  Their tiles are staged in two halves of kRS / 2
+// rows, of which kSWidePlanes planes fit, so that a dilation stays one bucket.  With buckets of 20 channels the
+// 200 kernels of a dilation over 32 channels were 15 buckets of a dozen kernels each, and a tile's copies took longer than the
+// work on it (24 x 32 x 1,751, 2,000 kernels).
+constexpr int kSHalfRows = kRS / 2, kSWidePlanes = 34;
+ROCKET_CX int s_plane_floats(int rows) { return (rows + ROCKET_MAX_LENGTH - 1) * kWarpCols; }
 constexpr int kSManyKernels = 32, kSSomeKernels = 8;               // buckets below these share a tile among several examples
 constexpr int kSLengthOrderMin = 100;                              // buckets from this many kernels up are ordered by length
 
-// The kernels of a bucket use at most kSMaxPlanes channels between them: where the kernels of one dilation use more (series
-// of more than 20 channels), they are several buckets.  Their records hold positions in the bucket's channel list.
+// The kernels of a bucket use at most kSMaxPlanes channels between them (kSWidePlanes in a wide handle): where the kernels of one
+// dilation use more, they are several buckets.  Their records hold positions in the bucket's channel list.
 struct SBucket {
     int32_t d, tmin, nbands, raster_len;  // raster_len = nbands * d
     int32_t kbeg, kend, rows, nch;        // kernels [kbeg, kend) of krec; rows = kRS + max len - 1; channels used
-    uint8_t ch[kSMaxPlanes];              // the channels
-    int32_t pad_[3];
+    uint8_t ch[40];                       // the channels (at most kSWidePlanes)
+    int32_t pad_[2];
 };
-static_assert(sizeof(SBucket) == 64, "SBucket must be 16 words");
+constexpr int kSBucketWords = 20;
+static_assert(sizeof(SBucket) == 4 * kSBucketWords && kSWidePlanes <= 40, "SBucket layout");
 // One S tile: 64 raster positions from c0 of a bucket.  interior = 1 when every (row, column) of the
 // tile is an output of every kernel of the bucket (then the kernels need no range tests).
 struct SItem { int32_t bucket, c0, interior, pad_; };
@@ -215,6 +222,7 @@ struct PlanHost {
     std::vector<int32_t> generic_list;    // kernels the fast path does not take
     int64_t pad_pitch = 0;                // floats per channel row of the zero-margined copy
     int s_max_nch = 0;                    // most channels of any S bucket
+    bool s_wide = false;                  // the S tiles are staged in halves of up to kSWidePlanes planes
     int s_class_end[3] = {0, 0, 0};       // S tiles by kernels in their bucket: at least kSManyKernels, kSSomeKernels, fewer
     double flops_s = 0.0, flops_t = 0.0;  // conv flop of one example in either regime
 };

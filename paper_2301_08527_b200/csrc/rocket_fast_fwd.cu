@@ -46,8 +46,8 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Backward second half for one kernel on an S tile: per channel, dW sums of the warp tile.
-template <int ELL>
-__device__ __forceinline__ void s_grad_tile(const float* planes, const KRec* rec, int lane, const u64 (&gz)[kRS],
+template <int ELL, int R>
+__device__ __forceinline__ void s_grad_tile(const float* planes, const KRec* rec, int lane, const u64 (&gz)[R],
                                             long long* accfix, double scale) {
     const int m = __shfl_sync(kFull, rec->m, 0);
     const int off[4] = {2 * lane, kWarpCols + 2 * lane, 2 * kWarpCols + 2 * lane, 3 * kWarpCols + 2 * lane};
@@ -55,51 +55,52 @@ __device__ __forceinline__ void s_grad_tile(const float* planes, const KRec* rec
         u64 dw[ELL];
 #pragma unroll
         for (int j = 0; j < ELL; ++j) dw[j] = 0ull;
-        grad_channel<ELL, 4 * kWarpCols, false, kRS>(planes + rec->ch[q] * kSPlaneFloats, off, gz, dw);
+        grad_channel<ELL, 4 * kWarpCols, false, R>(planes + rec->ch[q] * s_plane_floats(R), off, gz, dw);
         reduce_publish_dw<ELL>(dw, accfix + rec->woff + q * ELL, scale, lane);
     }
 }
 
 // The channels of one kernel on an S tile.  fold: the accumulators come in undefined and start at the
 // kernel's 0 - bias inside the first channel's pass (every output of the warp tile exists).
-template <int ELL, bool FOLD>
-__device__ __forceinline__ void s_kernel_tile(const float* planes, const KRec* rec, int lane, u64 (&acc)[kRS]) {
+template <int ELL, bool FOLD, int R>
+__device__ __forceinline__ void s_kernel_tile(const float* planes, const KRec* rec, int lane, u64 (&acc)[R]) {
     const int m = __shfl_sync(kFull, rec->m, 0);
     const int off[4] = {2 * lane, kWarpCols + 2 * lane, 2 * kWarpCols + 2 * lane, 3 * kWarpCols + 2 * lane};
     int q = 0;
     if constexpr (FOLD) {
         const float nb = rec->negb;
-        conv_channel<ELL, 4 * kWarpCols, false, true, kRS>(planes + rec->ch[0] * kSPlaneFloats, off, rec->w2[0], acc, 0, 0, pack2(nb, nb));
+        conv_channel<ELL, 4 * kWarpCols, false, true, R>(planes + rec->ch[0] * s_plane_floats(R), off, rec->w2[0], acc, 0, 0, pack2(nb, nb));
         q = 1;
     }
     for (; q < m; ++q)
-        conv_channel<ELL, 4 * kWarpCols, false, false, kRS>(planes + rec->ch[q] * kSPlaneFloats, off, rec->w2[q], acc);
+        conv_channel<ELL, 4 * kWarpCols, false, false, R>(planes + rec->ch[q] * s_plane_floats(R), off, rec->w2[q], acc);
 }
 
 // The same in half precision (mode 3).
-template <int ELL>
-__device__ __forceinline__ void s_kernel_tile_h(const float* planes, const KRec* rec, int lane, h2 (&acc)[kRS]) {
+template <int ELL, int R>
+__device__ __forceinline__ void s_kernel_tile_h(const float* planes, const KRec* rec, int lane, h2 (&acc)[R]) {
     const int m = __shfl_sync(kFull, rec->m, 0);
     const int off[4] = {2 * lane, kWarpCols + 2 * lane, 2 * kWarpCols + 2 * lane, 3 * kWarpCols + 2 * lane};
     for (int q = 0; q < m; ++q)
-        conv_channel_h<ELL, 4 * kWarpCols, false, kRS>(planes + rec->ch[q] * kSPlaneFloats, off, rec->w2[q], acc);
+        conv_channel_h<ELL, 4 * kWarpCols, false, R>(planes + rec->ch[q] * s_plane_floats(R), off, rec->w2[q], acc);
 }
 
-template <int MODE>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision
+template <int MODE, bool HALF = false>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision; HALF: a wide handle
 __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
-    float* planes = reinterpret_cast<float*>(smem_raw);                               // [kSMaxPlanes][kSRowsMax][64]
-    KRec* recs = reinterpret_cast<KRec*>(planes + kSMaxPlanes * kSPlaneFloats);        // [warps][2]
+    constexpr int R = HALF ? kSHalfRows : kRS, kPlanes = HALF ? kSWidePlanes : kSMaxPlanes, kPlaneFloats = s_plane_floats(R);
+    float* planes = reinterpret_cast<float*>(smem_raw);                               // [kPlanes][rows][64]
+    KRec* recs = reinterpret_cast<KRec*>(planes + kPlanes * kPlaneFloats);             // [warps][2]
     __shared__ unsigned s_item;
-    __shared__ int s_next, s_n0, s_ne;
+    __shared__ int s_next, s_n0, s_ne, s_half;
     __shared__ SItem s_sitem;
     __shared__ SBucket s_bucket;
-    __shared__ long long s_src[kSMaxPlanes];      // where the planes' channel rows start in X
+    __shared__ long long s_src[kPlanes];      // where the planes' channel rows start in X
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // Work is handed out as (tile, group of examples), the tiles of the buckets with many kernels first.  Where a bucket has
     // few kernels, several examples share a tile's planes, as far as they fit: the warps then find (kernel, example) pairs
     // enough to keep busy.
     const unsigned tiles0 = (unsigned)a.s_end[0] * (unsigned)a.s_groups[0], tiles1 = (unsigned)(a.s_end[1] - a.s_end[0]) * (unsigned)a.s_groups[1];
-    const unsigned total = tiles0 + tiles1 + (unsigned)(a.s_end[2] - a.s_end[1]) * (unsigned)a.s_groups[2];
+    const unsigned total = (tiles0 + tiles1 + (unsigned)(a.s_end[2] - a.s_end[1]) * (unsigned)a.s_groups[2]) * (HALF ? 2u : 1u);
     KRec* myrec = recs + warp * 2;
 
     for (;;) {
@@ -110,6 +111,10 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
             g = __shfl_sync(kFull, g, 0);
             if (lane == 0) { s_item = g; s_next = 0; }
             if (g < total) {
+                if (HALF) {
+                    if (lane == 0) s_half = (int)(g & 1u);
+                    g >>= 1;
+                }
                 const int cls = g < tiles0 ? 0 : g < tiles0 + tiles1 ? 1 : 2;
                 const unsigned first = cls == 0 ? 0u : (unsigned)a.s_end[cls - 1], count = (unsigned)a.s_end[cls] - first;
                 const unsigned rest = g - (cls == 0 ? 0u : cls == 1 ? tiles0 : tiles0 + tiles1);
@@ -118,9 +123,14 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
                 const SItem it = a.plan.sitems[first + rest % count];
                 const SBucket* __restrict__ src = a.plan.sb + it.bucket;
                 if (lane == 0) s_sitem = it;
-                if (lane < 16) reinterpret_cast<int*>(&s_bucket)[lane] = __ldg(reinterpret_cast<const int*>(src) + lane);
-                const int nch = __ldg(&src->nch), e = lane / nch;
-                if (e < ne) s_src[lane] = ((long long)(n0 + e) * a.C + __ldg(&src->ch[lane - e * nch])) * a.x_row_stride;
+                if (lane < kSBucketWords) reinterpret_cast<int*>(&s_bucket)[lane] = __ldg(reinterpret_cast<const int*>(src) + lane);
+                const int nch = __ldg(&src->nch);
+                auto plane_src = [&](int pl) {
+                    const int e = pl / nch;
+                    if (e < ne) s_src[pl] = ((long long)(n0 + e) * a.C + __ldg(&src->ch[pl - e * nch])) * a.x_row_stride;
+                };
+                plane_src(lane);
+                if (HALF) plane_src(lane + 32);
             }
         }
         __syncthreads();
@@ -130,15 +140,16 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
         const SBucket& b = s_bucket;
         const int d = b.d, kbeg = b.kbeg, n_work = (b.kend - kbeg) * ne, nch = b.nch;
         const bool tile_interior = item.interior != 0;
+        const int half_row = HALF ? s_half * R : 0;              // the first row of the half
 
         // Stage the tile: every plane, rows 0..rows-1 of every column, zero outside the series.  A thread takes one column of
         // every eighth row; what does not depend on the plane is computed once, so that a sample costs an address and a copy.
         {
-            constexpr int kStep = kSThreads / kWarpCols, kRows = (kSRowsMax + kStep - 1) / kStep;
+            constexpr int kStep = kSThreads / kWarpCols, kRows = (R + ROCKET_MAX_LENGTH - 1 + kStep - 1) / kStep;
             const int col = threadIdx.x & (kWarpCols - 1), rg = threadIdx.x / kWarpCols;
             const int cg = item.c0 + col;
             const bool col_ok = cg < b.raster_len;
-            const int fu0 = s_column_u0(b, cg), n_planes = nch * ne, rows = b.rows;
+            const int fu0 = s_column_u0(b, cg) + half_row * d, n_planes = nch * ne, rows = b.rows - (kRS - R);
             int xi[kRows], bytes[kRows];
 #pragma unroll
             for (int i = 0; i < kRows; ++i) {
@@ -154,7 +165,7 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
 #pragma unroll
                 for (int i = 0; i < kRows; ++i)
                     if (rg + i * kStep < rows) cp_async4(dst + i * kStep * kWarpCols * 4, src + xi[i], bytes[i]);
-                dst += kSPlaneFloats * 4;
+                dst += kPlaneFloats * 4;
             }
             cp_async_commit();
         }
@@ -163,7 +174,7 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
         const bool ok0 = cg0 < b.raster_len, ok1 = cg0 + 1 < b.raster_len;
         const int band0 = cg0 / d, c0 = cg0 - band0 * d;          // (first A-row, residue) of the two columns
         const int band1 = c0 + 1 < d ? band0 : band0 + 1, c1 = c0 + 1 < d ? c0 + 1 : 0;
-        const int trow0 = b.tmin + band0 * kRS, trow1 = b.tmin + band1 * kRS;
+        const int trow0 = b.tmin + band0 * kRS + half_row, trow1 = b.tmin + band1 * kRS + half_row;
         cp_async_wait<0>();
         __syncthreads();
 
@@ -192,24 +203,24 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
             cp_async_wait<1>();
             __syncwarp();
             const int example = ne == 1 ? 0 : kk - kernel_of(kk) * ne, n = n0 + example;
-            const float* eplanes = planes + example * nch * kSPlaneFloats;   // the example's planes
+            const float* eplanes = planes + example * nch * kPlaneFloats;   // the example's planes
             const KRec* rec = myrec + cur;
             // the same for the warp: as a shuffle's result the compiler takes it for uniform and keeps the branches on it cheap
             const int len = __shfl_sync(kFull, rec->len, 0), korig = rec->k;
             // on an interior tile (the plan's flag) every output exists for every kernel of the bucket
-            int lo0 = 0, hi0 = kRS, lo1 = 0, hi1 = kRS;
+            int lo0 = 0, hi0 = R, lo1 = 0, hi1 = R;
             bool interior = tile_interior;
             if (!tile_interior) {
-                valid_rows_tc(trow0, c0, rec->tl, rec->rl, rec->th, rec->rh, kRS, ok0, lo0, hi0);
-                valid_rows_tc(trow1, c1, rec->tl, rec->rl, rec->th, rec->rh, kRS, ok1, lo1, hi1);
-                interior = __all_sync(kFull, lo0 == 0 && lo1 == 0 && hi0 == kRS && hi1 == kRS);
+                valid_rows_tc(trow0, c0, rec->tl, rec->rl, rec->th, rec->rh, R, ok0, lo0, hi0);
+                valid_rows_tc(trow1, c1, rec->tl, rec->rl, rec->th, rec->rh, R, ok1, lo1, hi1);
+                interior = __all_sync(kFull, lo0 == 0 && lo1 == 0 && hi0 == R && hi1 == R);
             }
-            u64 acc[kRS];
+            u64 acc[R];
             // hard mode: the pooling masks the outputs that do not exist, so the accumulators always start inside
             // the first channel's pass; the other modes start them at 0 - bias, or +inf where there is no output
             constexpr bool kFold = MODE == 0;
             if constexpr (MODE == 3) {
-                h2 acch[kRS];
+                h2 acch[R];
                 init_acc_h(acch, rec->negb);
                 if (len == 7) s_kernel_tile_h<7>(eplanes, rec, lane, acch);
                 else if (len == 9) s_kernel_tile_h<9>(eplanes, rec, lane, acch);
@@ -227,8 +238,8 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
                 const int uA = __ldg(a.argmax + pair) - rec->p;
                 int tA = uA / d, cA = uA - tA * d;                        // floor division: uA >= -p may be negative
                 if (cA < 0) { cA += d; --tA; }
-                const int oA0 = (ok0 && c0 == cA && tA >= trow0 && tA < trow0 + kRS) ? tA - trow0 : -1;
-                const int oA1 = (ok1 && c1 == cA && tA >= trow1 && tA < trow1 + kRS) ? tA - trow1 : -1;
+                const int oA0 = (ok0 && c0 == cA && tA >= trow0 && tA < trow0 + R) ? tA - trow0 : -1;
+                const int oA1 = (ok1 && c1 == cA && tA >= trow1 && tA < trow1 + R) ? tA - trow1 : -1;
                 float dbs = make_gz(acc, a.c1, a.c0, gP * a.lambda / (float)rec->nout, gM, interior, lo0, hi0, lo1, hi1, oA0, oA1);
 #pragma unroll
                 for (int sh = 16; sh > 0; sh >>= 1) dbs += __shfl_xor_sync(kFull, dbs, sh);
@@ -765,7 +776,9 @@ __global__ void fast_finalize_soft_kernel(float* __restrict__ feat, int32_t* __r
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-size_t s_smem_bytes() { return (size_t)kSMaxPlanes * kSPlaneFloats * 4 + (size_t)kSWarps * 2 * sizeof(KRec); }
+size_t s_smem_bytes(bool wide) {
+    return (size_t)(wide ? kSWidePlanes * s_plane_floats(kSHalfRows) : kSMaxPlanes * kSPlaneFloats) * 4 + (size_t)kSWarps * 2 * sizeof(KRec);
+}
 size_t t_smem_bytes() { return (size_t)kTGroups * kTGroupSmemBytes + 128; }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -793,19 +806,25 @@ cudaError_t set_kernel_attributes(int dev) {
     bool& attr_done = attr_done_for[dev & 63];
     const size_t t_bytes = t_smem_bytes();
     if (!attr_done) {
-        e = cudaFuncSetAttribute(fast_s_forward<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes());
+        e = cudaFuncSetAttribute(fast_s_forward<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes());
+        e = cudaFuncSetAttribute(fast_s_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(fast_t_forward<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(fast_t_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes());
+        e = cudaFuncSetAttribute(fast_s_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(fast_t_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes());
+        e = cudaFuncSetAttribute(fast_s_forward<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(fast_s_forward<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(true));
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(fast_s_forward<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(true));
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(fast_s_forward<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(true));
         if (e != cudaSuccess) return e;
         e = set_stream_attributes();
         if (e != cudaSuccess) return e;
@@ -886,7 +905,7 @@ static int chunk_examples(const FastState& fs, int C, bool stream, bool copies) 
 // where it has some or few (64 to 256 pairs per tile for its 16 warps), as far as the planes hold them and the launch keeps two
 // tiles per SM.  Returns the grid.
 static unsigned set_s_groups(FwdArgs& a, const FastState& fs, int sms) {
-    const int fit = kSMaxPlanes / std::max(1, fs.host.s_max_nch);
+    const int fit = (fs.host.s_wide ? kSWidePlanes : kSMaxPlanes) / std::max(1, fs.host.s_max_nch);
     unsigned long long tiles = 0;
     for (int shift = 0; shift < 5; ++shift) {
         tiles = 0;
@@ -895,11 +914,26 @@ static unsigned set_s_groups(FwdArgs& a, const FastState& fs, int sms) {
             a.s_end[cls] = fs.host.s_class_end[cls];
             a.s_examples[cls] = std::max(1, std::min({fit, most, a.N}) >> shift);
             a.s_groups[cls] = (a.N + a.s_examples[cls] - 1) / a.s_examples[cls];
-            tiles += (unsigned long long)(a.s_end[cls] - (cls ? a.s_end[cls - 1] : 0)) * a.s_groups[cls];
+            tiles += (unsigned long long)(a.s_end[cls] - (cls ? a.s_end[cls - 1] : 0)) * a.s_groups[cls] * (fs.host.s_wide ? 2 : 1);
         }
         if (tiles >= 2ull * sms || a.s_examples[2] == 1) break;
     }
     return (unsigned)std::min<unsigned long long>(tiles, (unsigned long long)sms);
+}
+
+// The S tiles of a pass (mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half precision, whose series are never wide).
+static void launch_s(FwdArgs& a, const FastState& fs, int mode, int sms, cudaStream_t stream) {
+    const unsigned grid = set_s_groups(a, fs, sms);
+    const bool wide = fs.host.s_wide;
+    const size_t bytes = s_smem_bytes(wide);
+    if (mode == 3) fast_s_forward<3><<<grid, kSThreads, bytes, stream>>>(a);
+    else if (mode == 0 && wide) fast_s_forward<0, true><<<grid, kSThreads, bytes, stream>>>(a);
+    else if (mode == 0) fast_s_forward<0><<<grid, kSThreads, bytes, stream>>>(a);
+    else if (mode == 1 && wide) fast_s_forward<1, true><<<grid, kSThreads, bytes, stream>>>(a);
+    else if (mode == 1) fast_s_forward<1><<<grid, kSThreads, bytes, stream>>>(a);
+    else if (wide) fast_s_forward<2, true><<<grid, kSThreads, bytes, stream>>>(a);
+    else fast_s_forward<2><<<grid, kSThreads, bytes, stream>>>(a);
+    count_launch();
 }
 
 // Blocks of the T kernel: as many as are resident at a time, never more than there are work units.
@@ -1122,7 +1156,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;
-    const size_t s_bytes = s_smem_bytes(), t_bytes = t_smem_bytes();
+    const size_t t_bytes = t_smem_bytes();
     const PlanDevice& pd = fs.dev;
     // the stream kernel takes the dilations the S kernel leaves; the T kernel where the stream kernel's copies have no room
     const bool streamed = pd.n_wunits > 0, copied = pd.n_titems > 0 || X_u8;
@@ -1184,13 +1218,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
             launch_pad_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
         }
         if (fs.profile) cudaEventRecord(fs.evs[3 * c], stream);
-        if (pd.n_sitems > 0) {
-            const unsigned grid = set_s_groups(a, fs, sms);
-            if (soft) fast_s_forward<1><<<grid, kSThreads, s_bytes, stream>>>(a);
-            else if (half) fast_s_forward<3><<<grid, kSThreads, s_bytes, stream>>>(a);
-            else fast_s_forward<0><<<grid, kSThreads, s_bytes, stream>>>(a);
-            count_launch();
-        }
+        if (pd.n_sitems > 0) launch_s(a, fs, soft ? 1 : half ? 3 : 0, sms, stream);
         if (fs.profile) cudaEventRecord(fs.evs[3 * c + 1], stream);
         if (streamed) {
             launch_stream(a, soft ? 1 : half ? 3 : 0, sms, stream);
@@ -1226,7 +1254,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;
-    const size_t s_bytes = s_smem_bytes(), t_bytes = t_smem_bytes();
+    const size_t t_bytes = t_smem_bytes();
     const PlanDevice& pd = fs.dev;
     // workspace: fixed-point sums [n_weights + K], scales [K], max |x| (fixed size per handle)
     const size_t acc_bytes = align256((size_t)(n_weights + dp.K) * 8), scale_bytes = align256((size_t)dp.K * 8);
@@ -1269,10 +1297,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         if (e != cudaSuccess) return e;
         if (streamed) launch_stream_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
         else if (copied) launch_pad_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
-        if (pd.n_sitems > 0) {
-            fast_s_forward<2><<<set_s_groups(a, fs, sms), kSThreads, s_bytes, stream>>>(a);
-            count_launch();
-        }
+        if (pd.n_sitems > 0) launch_s(a, fs, 2, sms, stream);
         if (streamed) {
             launch_stream(a, 2, sms, stream);
         } else if (pd.n_titems > 0) {

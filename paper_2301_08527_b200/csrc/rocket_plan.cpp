@@ -160,16 +160,25 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
     for (int k : s_kernels) by_d[hp.dilation[k]].push_back(k);
     struct Cost { double c; int idx; };
     std::vector<Cost> s_cost;
-    // Kernels of one dilation that use more than kSMaxPlanes channels between them are split: a kernel (most channels
+    // Kernels of one dilation that use more channels than a tile has planes are split: a kernel (most channels
     // first) joins the group whose channel set grows least, or opens a new one.
     std::vector<std::pair<int, std::vector<int>>> groups;
-    for (auto& kv : by_d) {
+    std::map<int, int> channels_of;
+    for (const auto& kv : by_d) {
         std::vector<char> used(hp.C, 0);
-        int n_used = 0;
+        int& n_used = channels_of[kv.first];
         for (int k : kv.second)
             for (int q = hp.channel_offset[k]; q < hp.channel_offset[k] + hp.num_channels[k]; ++q)
                 if (!used[hp.channel_idx[q]]) { used[hp.channel_idx[q]] = 1; ++n_used; }
-        if (n_used <= kSMaxPlanes) {
+    }
+    {   // halves where that lets every dilation be one bucket; two of 34 channels are no better than several of 20 (64 channels)
+        int most = 0;
+        for (const auto& c : channels_of) most = std::max(most, c.second);
+        out.s_wide = most > kSMaxPlanes && most <= kSWidePlanes;
+    }
+    const int max_planes = out.s_wide ? kSWidePlanes : kSMaxPlanes;
+    for (auto& kv : by_d) {
+        if (channels_of[kv.first] <= max_planes) {
             groups.emplace_back(kv.first, std::move(kv.second));
             continue;
         }
@@ -182,7 +191,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
             for (size_t g = 0; g < gs.size(); ++g) {
                 int fresh = 0;
                 for (int q = 0; q < hp.num_channels[k]; ++q) fresh += !gs[g].has[S[q]];
-                if (gs[g].n + fresh <= kSMaxPlanes && fresh < best_new) { best = (int)g; best_new = fresh; }
+                if (gs[g].n + fresh <= max_planes && fresh < best_new) { best = (int)g; best_new = fresh; }
             }
             if (best < 0) { best = (int)gs.size(); gs.push_back({std::vector<char>(hp.C, 0), 0, {}}); }
             Group& g = gs[best];
