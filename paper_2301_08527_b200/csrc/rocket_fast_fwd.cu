@@ -836,14 +836,22 @@ cudaError_t set_kernel_attributes(int dev) {
 }
 
 // ---- backward helpers ----------------------------------------------------------------------------
-// Largest |x| of the batch, as the bit pattern of a non-negative float (integer order = float order).
+// Largest |x| of the batch, as the bit pattern of a non-negative float (integer order = float order).  One atomic per block of 256
+// threads: one per warp, all to the same word, took 8 us of a minibatch.
+__device__ __forceinline__ void block_max(float m, unsigned* __restrict__ out) {
+    __shared__ unsigned s_max;
+    if (threadIdx.x == 0) s_max = 0u;
+    __syncthreads();
+    const unsigned b = __reduce_max_sync(kFull, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_max, b);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(out, s_max);
+}
 __global__ void fast_absmax_scalar_kernel(const float* __restrict__ X, int64_t n, unsigned* __restrict__ out) {
     float m = 0.0f;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
         m = fmaxf(m, fabsf(__ldg(X + e)));
-    unsigned b = __float_as_uint(m);
-    b = __reduce_max_sync(kFull, b);
-    if ((threadIdx.x & 31) == 0) atomicMax(out, b);
+    block_max(m, out);
 }
 
 __global__ void fast_absmax_kernel(const float4* __restrict__ X, int64_t n4, unsigned* __restrict__ out) {
@@ -852,42 +860,46 @@ __global__ void fast_absmax_kernel(const float4* __restrict__ X, int64_t n4, uns
         const float4 v = __ldg(X + e);
         m = fmaxf(fmaxf(m, fabsf(v.x)), fmaxf(fabsf(v.y), fmaxf(fabsf(v.z), fabsf(v.w))));
     }
-    unsigned b = __float_as_uint(m);
-    b = __reduce_max_sync(kFull, b);
-    if ((threadIdx.x & 31) == 0) atomicMax(out, b);
+    block_max(m, out);
 }
 
 // Per kernel: a bound on sum |gz| |x| over the batch gives the fixed-point scale of its sums
-// (|sum_i gz_i| <= |gP| lambda / 4 + |gM| per example since h (1 - h) <= 1/4), and its sums are cleared.
+// (|sum_i gz_i| <= |gP| lambda / 4 + |gM| per example since h (1 - h) <= 1/4), and its sums are cleared.  A warp per kernel here
+// and in the finalise kernel: a thread per kernel went through up to 121 weights one by one (8 and 13 us of a minibatch).
 __global__ void fast_bwd_prepare_kernel(const float* __restrict__ dfeat, const KRec* __restrict__ krec, int n_krec, int N,
                                         int K, float lambda, const unsigned* __restrict__ absmax_bits,
-                                        double* __restrict__ scale, long long* __restrict__ accfix, long long n_weights) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
+                                        double* __restrict__ scale, long long* __restrict__ accfix, long long n_weights,
+                                        unsigned* __restrict__ counters) {
+    const int f = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (f >= n_krec) return;
-    const int k = krec[f].k;
+    const KRec& r = krec[f];
+    const int k = r.k, taps = r.m * r.len;
     double bound = 0.0;
-    for (int n = 0; n < N; ++n) {
-        const float gP = dfeat[((int64_t)n * K + k) * 2], gM = dfeat[((int64_t)n * K + k) * 2 + 1];
+    for (int n = lane; n < N; n += 32) {
+        const float gP = __ldg(dfeat + ((int64_t)n * K + k) * 2), gM = __ldg(dfeat + ((int64_t)n * K + k) * 2 + 1);
         bound += (double)fabsf(gP) * (double)fabsf(lambda) * 0.25 + (double)fabsf(gM);
     }
+#pragma unroll
+    for (int sh = 16; sh > 0; sh >>= 1) bound += __shfl_xor_sync(kFull, bound, sh);
+    for (int t = lane; t < taps; t += 32) accfix[r.woff + t] = 0;
+    if (lane > 0) return;
     const double xmax = fmax((double)__uint_as_float(*absmax_bits), 1.0);
     bound *= xmax * 1.01;
     scale[k] = (bound > 0.0 && bound < 1e300) ? 1152921504606846976.0 / bound : 0.0;  // 2^60 / bound
-    const int taps = krec[f].m * krec[f].len;
-    for (int t = 0; t < taps; ++t) accfix[krec[f].woff + t] = 0;
     accfix[n_weights + k] = 0;
+    if (f == 0) { counters[0] = 0u; counters[1] = 0u; }
 }
 
 __global__ void fast_bwd_finalize_kernel(const long long* __restrict__ accfix, const double* __restrict__ scale,
                                          const KRec* __restrict__ krec, int n_krec, long long n_weights,
                                          float* __restrict__ dW, float* __restrict__ db) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
+    const int f = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (f >= n_krec) return;
-    const int k = krec[f].k;
+    const KRec& r = krec[f];
+    const int k = r.k, taps = r.m * r.len;
     const double sc = scale[k], inv = sc > 0.0 ? 1.0 / sc : 0.0;
-    const int taps = krec[f].m * krec[f].len;
-    for (int t = 0; t < taps; ++t) dW[krec[f].woff + t] = (float)((double)accfix[krec[f].woff + t] * inv);
-    db[k] = (float)((double)accfix[n_weights + k] * inv);
+    for (int t = lane; t < taps; t += 32) dW[r.woff + t] = (float)((double)accfix[r.woff + t] * inv);
+    if (lane == 0) db[k] = (float)((double)accfix[n_weights + k] * inv);
 }
 
 }  // namespace
@@ -1273,13 +1285,14 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     if (e != cudaSuccess) return e;
     const int64_t n_x = (int64_t)N * dp.C * dp.L;
     if (n_x > 0) {
+        auto blocks = [&](int64_t loads) { return (unsigned)std::min<int64_t>(sms * 8, (loads + 1023) / 1024); };   // four loads per thread
         if (dp.L % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0)
-            fast_absmax_kernel<<<sms * 8, 256, 0, stream>>>(reinterpret_cast<const float4*>(X), n_x / 4, absmax);
-        else fast_absmax_scalar_kernel<<<sms * 8, 256, 0, stream>>>(X, n_x, absmax);
+            fast_absmax_kernel<<<blocks(n_x / 4), 256, 0, stream>>>(reinterpret_cast<const float4*>(X), n_x / 4, absmax);
+        else fast_absmax_scalar_kernel<<<blocks(n_x), 256, 0, stream>>>(X, n_x, absmax);
         count_launch();
     }
-    fast_bwd_prepare_kernel<<<(pd.n_krec + 127) / 128, 128, 0, stream>>>(dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale,
-                                                                         accfix, n_weights);
+    fast_bwd_prepare_kernel<<<(pd.n_krec + 7) / 8, 256, 0, stream>>>(dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale, accfix,
+                                                                     n_weights, pd.counters);
     count_launch();
     FwdArgs a;
     a.plan = fs.dev; a.feat_i = nullptr; a.ws = nullptr;
@@ -1293,8 +1306,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         a.dfeat = dfeat + (size_t)n0 * 2 * dp.K;
         a.argmax = argmax + (size_t)n0 * dp.K;
         a.N = nc;
-        e = cudaMemsetAsync(pd.counters, 0, 8, stream);
-        if (e != cudaSuccess) return e;
+        if (n0 > 0 && (e = cudaMemsetAsync(pd.counters, 0, 8, stream)) != cudaSuccess) return e;
         if (streamed) launch_stream_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
         else if (copied) launch_pad_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
         if (pd.n_sitems > 0) launch_s(a, fs, 2, sms, stream);
@@ -1305,7 +1317,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
             count_launch();
         }
     }
-    fast_bwd_finalize_kernel<<<(pd.n_krec + 127) / 128, 128, 0, stream>>>(accfix, scale, pd.krec, pd.n_krec, n_weights, dW, db);
+    fast_bwd_finalize_kernel<<<(pd.n_krec + 7) / 8, 256, 0, stream>>>(accfix, scale, pd.krec, pd.n_krec, n_weights, dW, db);
     count_launch();
     return cudaGetLastError();
 }
