@@ -10,13 +10,16 @@
 // (fma.rn.f32x2), so every input is loaded once and used len times.  Lanes of a warp own
 // adjacent column pairs: a warp tile is 16 rows x 64 columns.
 //
-// Two regimes share the arithmetic core:
+// Three kernels share the arithmetic core:
 //   S (d < split): kernels of one dilation form a bucket.  Columns of successive bands of kRS rows
 //     are strung together into one "raster" (band-major, r-minor) and a tile is 64 consecutive
 //     raster positions, so lanes stay busy even when d < 64.  A block stages one tile of ALL
 //     channels in shared memory, then its warps pull kernels of the bucket from a shared
 //     counter, so one staged tile serves dozens to hundreds of kernels.
-//   T (d >= split): few kernels share a dilation, so a block of eight consumer warps takes one
+//   stream (d >= split; rocket_stream.cu): few kernels share a dilation, so every warp takes tiles of
+//     one kernel of its own and streams the kernel's channels through its own shared memory.
+//   T (d >= split, handles with dilations near L / 3.5 and above, for which the stream kernel's copies
+//     would be mostly margins): a block of eight consumer warps takes one
 //     kernel and one tile of up to eight warp tiles (128 x 64, 64 x 128, 32 x 256, or 16 x 512 for
 //     kernels whose outputs span at most 16 rows of A) and streams the kernel's channels through a
 //     ring of shared-memory stages.  A producer warp fills the
@@ -47,7 +50,9 @@ constexpr int kRowsMax = kR + ROCKET_MAX_LENGTH - 1;               // staged row
 #ifndef ROCKET_SPLIT
 #define ROCKET_SPLIT 64
 #endif
-constexpr int kSplitDefault = ROCKET_SPLIT;                        // S below, T at or above
+// S below, stream (or T) at or above.  The stream kernel's tiles are 64 columns of one band, so it cannot start lower; with 96 to
+// 256 the S kernel's buckets hold too few kernels for the 16 warps of a block (the hard transform loses 0.5 to 4 %).
+constexpr int kSplitDefault = ROCKET_SPLIT;
 constexpr int kTMinDilation = 64;                                  // a T tile needs 64 residues in one band
 
 // ---- kernel record: one fast kernel as the device reads it (header + duplicated weights) ----

@@ -82,6 +82,9 @@ __device__ __forceinline__ void conv_channel(const float* __restrict__ st, const
                                              const float* __restrict__ w2, u64 (&acc)[R], int gl = 0, int gh = 0,
                                              u64 init = 0ull) {
     static_assert(!(WIN && FIRST), "a windowed pass may skip an accumulator's first product");
+    // A warp loads its weights once, lane j weight j, and hands them round: loads of every weight by every lane are ELL more trips
+    // through shared memory per channel.  The loop alone went from 94 to 104 multiply-adds/clk/SM at length 9 and 16 rows, from 98
+    // to 108 at 24 rows; the hard transform of 60 x 20 x 50,000 from 60.1 to 56.9 ms.
     u64 wp[ELL];
     {
         const int lane = threadIdx.x & 31;

@@ -85,6 +85,13 @@ __device__ __forceinline__ void s_kernel_tile_h(const float* planes, const KRec*
         conv_channel_h<ELL, 4 * kWarpCols, false, R>(planes + rec->ch[q] * s_plane_floats(R), off, rec->w2[q], acc);
 }
 
+// Bound: the packed multiply-adds of the inner loops (78 % of a tile's time at dilations below 8), and for the larger dilations, where
+// a bucket has few kernels, what a tile costs besides: 2,600 clocks to draw it, 7,400 (dilations 32 to 63) to 20,000 (dilation 1,
+// whose columns are 24 samples apart) to copy it in - the lines an SM can have in flight, about 24 B/clk, whether the copies are
+// asynchronous, plain loads in batches or 16 bytes wide - and 800 to 5,400 that the warps wait for the last kernel; of 27,000 clocks
+// at dilations 32 to 63, 11,400 are work.  Measured at 60 x 20 x 50,000, hard: 24.1 ms with weights read by every lane, 22.6 now.
+// Tried and not kept: two half tiles in flight behind producer warps (22.9 ms; 22 input rows for 12 rows of outputs make the
+// shared memory the limit), drawing the next tile during the copies (22.5 to 22.6, and late draws matter for small batches).
 template <int MODE, bool HALF = false>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision; HALF: a wide handle
 __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
     constexpr int R = HALF ? kSHalfRows : kRS, kPlanes = HALF ? kSWidePlanes : kSMaxPlanes, kPlaneFloats = s_plane_floats(R);

@@ -8,9 +8,9 @@
 // to fp32 before w and b are stored.  Every sum is taken in an order that depends on the sizes alone, so two fits
 // of the same data are bitwise identical.
 //
-// Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights took
-// 55 / 2,607 / 20,270 / 174 us as one thread per column, 2 x 2 outputs per thread, one block and one thread per
-// column.
+// Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights take
+// 18 / 496 / 381 / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
+// 55 / 2,607 / 20,270 / 174.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -391,7 +391,7 @@ ridge_weights_kernel(const float* __restrict__ F, int N, int P, const double* __
 // yhat[n] = b + sum_p F[n][p] w[p], products summed in double.  A row is shared by the blocks of a cluster (as many as
 // it takes to put a block on every SM, at most eight): each sums its contiguous part, the first adds the parts in rank
 // order through distributed shared memory.  Bound: the latency of one trip to memory; a block per row and one float
-// per load took 14.7 us for 60 rows of 20,000.
+// per load took 14.7 us for 60 rows of 20,000, this takes 7.6.
 constexpr int kPThreads = 512;
 template <bool VEC>
 __global__ void __launch_bounds__(kPThreads)
