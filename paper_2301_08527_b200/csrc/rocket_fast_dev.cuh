@@ -362,9 +362,9 @@ __device__ __forceinline__ float make_gz(u64 (&acc)[R], float c1, float c0, floa
 
 // Backward, second half, one channel of one warp tile: dw[j] += gz[o] * x[o + j] for the thread's
 // column pair (same traversal as conv_channel with the roles of weights and accumulators swapped).
-template <int ELL, int STEP, bool WIN, int R = kR>
+template <int ELL, int STEP, bool WIN, int R = kR, int A = ELL>
 __device__ __forceinline__ void grad_channel(const float* __restrict__ st, const int (&off)[4], const u64 (&gz)[R],
-                                             u64 (&dw)[ELL], int gl = 0, int gh = 0) {
+                                             u64 (&dw)[A], int gl = 0, int gh = 0) {
 #pragma unroll
     for (int g = 0; g < (R + ELL - 1 + 3) / 4; ++g) {
         if (!WIN || (g >= gl && g < gh)) {

@@ -45,18 +45,22 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Backward second half for one kernel on an S tile: per channel, dW sums of the warp tile.
-template <int ELL, int R>
-__device__ __forceinline__ void s_grad_tile(const float* planes, const KRec* rec, int lane, const u64 (&gz)[R],
-                                            long long* accfix, double scale) {
+// Backward second half for one kernel on an S tile: per channel, dW sums of the warp tile.  One instance of the reduction for all
+// lengths: the code that the warps of an SM run at a time decides how long the backward waits for instructions.
+template <int R>
+__device__ __forceinline__ void s_grad_tile(const float* planes, const KRec* rec, int len, int lane, const u64 (&gz)[R], long long* accfix,
+                                            double scale) {
     const int m = __shfl_sync(kFull, rec->m, 0);
     const int off[4] = {2 * lane, kWarpCols + 2 * lane, 2 * kWarpCols + 2 * lane, 3 * kWarpCols + 2 * lane};
     for (int q = 0; q < m; ++q) {
-        u64 dw[ELL];
+        u64 dw[ROCKET_MAX_LENGTH];
 #pragma unroll
-        for (int j = 0; j < ELL; ++j) dw[j] = 0ull;
-        grad_channel<ELL, 4 * kWarpCols, false, R>(planes + rec->ch[q] * s_plane_floats(R), off, gz, dw);
-        reduce_publish_dw<ELL>(dw, accfix + rec->woff + q * ELL, scale, lane);
+        for (int j = 0; j < ROCKET_MAX_LENGTH; ++j) dw[j] = 0ull;
+        const float* st = planes + rec->ch[q] * s_plane_floats(R);
+        if (len == 7) grad_channel<7, 4 * kWarpCols, false, R>(st, off, gz, dw);
+        else if (len == 9) grad_channel<9, 4 * kWarpCols, false, R>(st, off, gz, dw);
+        else grad_channel<11, 4 * kWarpCols, false, R>(st, off, gz, dw);
+        reduce_publish_dw<ROCKET_MAX_LENGTH>(dw, accfix + rec->woff + q * len, scale, lane, len);
     }
 }
 
@@ -252,9 +256,7 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
                 for (int sh = 16; sh > 0; sh >>= 1) dbs += __shfl_xor_sync(kFull, dbs, sh);
                 const double scale = __ldg(a.scale + korig);
                 if (lane == 0) add_fixed(a.accfix + a.n_weights + korig, dbs, scale);
-                if (len == 7) s_grad_tile<7>(eplanes, rec, lane, acc, a.accfix, scale);
-                else if (len == 9) s_grad_tile<9>(eplanes, rec, lane, acc, a.accfix, scale);
-                else s_grad_tile<11>(eplanes, rec, lane, acc, a.accfix, scale);
+                s_grad_tile(eplanes, rec, len, lane, acc, a.accfix, scale);
             } else if (MODE == 1) {
                 const int p = rec->p;
                 pool_publish_soft(a.ws, (int64_t)n * a.K + korig, acc, a.c1, a.c0, interior, lo0, hi0, lo1, hi1,

@@ -34,6 +34,12 @@ extern __shared__ __align__(128) unsigned char smem_raw[];
 
 static_assert(kWStages == 2, "the producer runs less than a whole unit of one visit ahead");
 
+// The channel loop either chooses the inner loop of the tile's shape for every channel, or exists once per shape as a whole (WHOLE).
+// As a whole a channel costs less (soft transform of 32 x 20 x 50,000 33.1 -> 32.1 ms, backward 67.1 -> 65.6), but there is more
+// code to fetch, which launches of a few dozen visits per warp do not make up for (10 x 6 x 1,251: 89 -> 97 us; even at 160
+// visits per warp).  The hard modes, whose other code is small, lose by it at every size.
+constexpr int kWWholeVisits = 300;
+
 struct StreamArgs {
     FwdArgs f;
     const WUnit* units;
@@ -264,7 +270,7 @@ __device__ __forceinline__ void stream_copy_box(int lead, uint32_t dst, const vo
         ::"r"(lead), "r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(w), "r"(bar), "r"(bytes) : "memory");
 }
 
-template <int MODE>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision
+template <int MODE, bool WHOLE = false>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision; WHOLE: see kWWholeVisits
 __global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constant__ StreamArgs a) {
     __shared__ unsigned long long s_bar[kWWarps][kWStages];
     const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
@@ -426,20 +432,32 @@ __global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constan
                 }
                 float mine = w_first;
                 const float* __restrict__ wn = wl;
-                for (int q = 0; q < m; ++q) {
+                auto channel = [&](int q, auto&& conv) {
                     if (q + 1 < m) wn += kPairRow;
                     const float mine_next = __ldg(wn);
-                    if (!(ok = wait())) break;
+                    if (!(ok = wait())) return false;
                     const uint32_t slot = st & 1u;
-                    const float* stage = stages + slot * kWStageFloats;
-                    by_shape(index, [&](auto len_tag, auto r_tag) {
-                        if constexpr (MODE == 3) stream_conv<decltype(len_tag)::value, decltype(r_tag)::value>(stage, off, mine, acch);
-                        else stream_conv<decltype(len_tag)::value, decltype(r_tag)::value>(stage, off, mine, acc);
-                    });
+                    conv(stages + slot * kWStageFloats);
                     mine = mine_next;
                     __syncwarp();                      // the stage has been read by every lane
                     ++st;
                     if (MODE == 2 || !last || q + 1 < m) issue(slot);
+                    return true;
+                };
+                if constexpr (WHOLE) {
+                    by_shape(index, [&](auto len_tag, auto r_tag) {
+                        for (int q = 0; q < m; ++q)
+                            if (!channel(q, [&](const float* stage) { stream_conv<decltype(len_tag)::value, decltype(r_tag)::value>(stage, off, mine, acc); })) break;
+                    });
+                } else {
+                    for (int q = 0; q < m; ++q) {
+                        if (!channel(q, [&](const float* stage) {
+                                by_shape(index, [&](auto len_tag, auto r_tag) {
+                                    if constexpr (MODE == 3) stream_conv<decltype(len_tag)::value, decltype(r_tag)::value>(stage, off, mine, acch);
+                                    else stream_conv<decltype(len_tag)::value, decltype(r_tag)::value>(stage, off, mine, acc);
+                                });
+                            })) break;
+                    }
                 }
                 if (!ok) break;
                 if constexpr (MODE == 3) widen_acc(acch, acc);
@@ -523,6 +541,8 @@ cudaError_t set_stream_attributes() {
     cudaError_t e = cudaFuncSetAttribute(fast_stream<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fast_stream<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fast_stream<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fast_stream<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fast_stream<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fast_stream<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     return e;
 }
@@ -544,7 +564,10 @@ void launch_stream(const FwdArgs& f, int mode, int sms, cudaStream_t stream) {
     const unsigned long long items = (unsigned long long)a.groups * (unsigned long long)a.n_units;
     const unsigned grid = (unsigned)std::min<unsigned long long>((items + kWWarps - 1) / kWWarps, (unsigned long long)sms);
     const size_t bytes = stream_smem_bytes();
-    if (mode == 1) fast_stream<1><<<grid, kWThreads, bytes, stream>>>(a);
+    const bool whole = f.plan.w_visits * f.N >= (double)kWWholeVisits * sms * kWWarps;
+    if (mode == 1 && whole) fast_stream<1, true><<<grid, kWThreads, bytes, stream>>>(a);
+    else if (mode == 1) fast_stream<1><<<grid, kWThreads, bytes, stream>>>(a);
+    else if (mode == 2 && whole) fast_stream<2, true><<<grid, kWThreads, bytes, stream>>>(a);
     else if (mode == 2) fast_stream<2><<<grid, kWThreads, bytes, stream>>>(a);
     else if (mode == 3) fast_stream<3><<<grid, kWThreads, bytes, stream>>>(a);
     else fast_stream<0><<<grid, kWThreads, bytes, stream>>>(a);
