@@ -33,10 +33,32 @@ struct FwdArgs {
 
 // The stream kernel over a pass of f.N examples (rocket_stream.cu); mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half
 // precision.
-void launch_stream(const FwdArgs& f, int mode, int sms, cudaStream_t stream);
+void launch_stream(const FwdArgs& f, int mode, int sms, bool after_s, cudaStream_t stream);   // after_s: directly behind the S kernel
 cudaError_t set_stream_attributes();   // opts the kernel into its shared-memory size
 
+// A launch that may begin while its predecessor in the stream ends (programmatic dependent launch): the kernel itself waits for the
+// predecessor with dependency_wait() before it touches anything, or states why it need not.
+template <typename... P, typename... A>
+inline void launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 namespace {
+
+// Waits until the kernels before this one in the stream are complete and their results visible.
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the stream begin once every block has come here.
+__device__ __forceinline__ void dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 typedef unsigned long long u64;
 constexpr unsigned kFull = 0xffffffffu;

@@ -98,6 +98,10 @@ __device__ __forceinline__ void s_kernel_tile_h(const float* planes, const KRec*
 // shared memory the limit), drawing the next tile during the copies (22.5 to 22.6, and late draws matter for small batches).
 template <int MODE, bool HALF = false>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision; HALF: a wide handle
 __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
+    dependency_wait();
+    // The stream kernel needs what came before this one, not this one: it may begin on the SMs that run out of tiles (8 x 20 x 10,001:
+    // 1.52 -> 1.45 ms; 10 x 6 x 1,251, 1,000 kernels: soft transform 88 -> 72 us).
+    dependency_release();
     constexpr int R = HALF ? kSHalfRows : kRS, kPlanes = HALF ? kSWidePlanes : kSMaxPlanes, kPlaneFloats = s_plane_floats(R);
     float* planes = reinterpret_cast<float*>(smem_raw);                               // [kPlanes][rows][64]
     KRec* recs = reinterpret_cast<KRec*>(planes + kPlanes * kPlaneFloats);             // [warps][2]
@@ -703,6 +707,7 @@ __device__ __forceinline__ void write_stream_copies(float* __restrict__ row0, in
 }
 template <bool VEC>   // VEC: rows start at 16-byte boundaries
 __global__ void stream_copy_kernel(const float* __restrict__ X, float* __restrict__ wpad, int64_t rows, int L, int64_t pitch, int front) {
+    dependency_wait();
     const int per = (L + 3) / 4 + 2;
     const int64_t total = rows * per;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -753,6 +758,7 @@ __global__ void fast_init_kernel(int* __restrict__ feat_i, int64_t pairs, unsign
 
 __global__ void fast_finalize_kernel(float* __restrict__ feat, const KRec* __restrict__ krec, int n_krec, int N,
                                      int K) {
+    dependency_wait();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)N * n_krec) return;
     const int n = (int)(e / n_krec), f = (int)(e - (int64_t)n * n_krec);
@@ -772,6 +778,7 @@ __global__ void fast_init_soft_kernel(unsigned long long* __restrict__ ws, int64
 __global__ void fast_finalize_soft_kernel(float* __restrict__ feat, int32_t* __restrict__ argmax,
                                           const unsigned long long* __restrict__ ws, const KRec* __restrict__ krec,
                                           int n_krec, int N, int K) {
+    dependency_wait();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)N * n_krec) return;
     const int n = (int)(e / n_krec), f = (int)(e - (int64_t)n * n_krec);
@@ -879,6 +886,7 @@ __global__ void fast_bwd_prepare_kernel(const float* __restrict__ dfeat, const K
                                         int K, float lambda, const unsigned* __restrict__ absmax_bits,
                                         double* __restrict__ scale, long long* __restrict__ accfix, long long n_weights,
                                         unsigned* __restrict__ counters) {
+    dependency_wait();
     const int f = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (f >= n_krec) return;
     const KRec& r = krec[f];
@@ -902,6 +910,7 @@ __global__ void fast_bwd_prepare_kernel(const float* __restrict__ dfeat, const K
 __global__ void fast_bwd_finalize_kernel(const long long* __restrict__ accfix, const double* __restrict__ scale,
                                          const KRec* __restrict__ krec, int n_krec, long long n_weights,
                                          float* __restrict__ dW, float* __restrict__ db) {
+    dependency_wait();
     const int f = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (f >= n_krec) return;
     const KRec& r = krec[f];
@@ -947,13 +956,13 @@ static void launch_s(FwdArgs& a, const FastState& fs, int mode, int sms, cudaStr
     const unsigned grid = set_s_groups(a, fs, sms);
     const bool wide = fs.host.s_wide;
     const size_t bytes = s_smem_bytes(wide);
-    if (mode == 3) fast_s_forward<3><<<grid, kSThreads, bytes, stream>>>(a);
-    else if (mode == 0 && wide) fast_s_forward<0, true><<<grid, kSThreads, bytes, stream>>>(a);
-    else if (mode == 0) fast_s_forward<0><<<grid, kSThreads, bytes, stream>>>(a);
-    else if (mode == 1 && wide) fast_s_forward<1, true><<<grid, kSThreads, bytes, stream>>>(a);
-    else if (mode == 1) fast_s_forward<1><<<grid, kSThreads, bytes, stream>>>(a);
-    else if (wide) fast_s_forward<2, true><<<grid, kSThreads, bytes, stream>>>(a);
-    else fast_s_forward<2><<<grid, kSThreads, bytes, stream>>>(a);
+    if (mode == 3) launch_dependent(fast_s_forward<3>, grid, kSThreads, bytes, stream, a);
+    else if (mode == 0 && wide) launch_dependent(fast_s_forward<0, true>, grid, kSThreads, bytes, stream, a);
+    else if (mode == 0) launch_dependent(fast_s_forward<0>, grid, kSThreads, bytes, stream, a);
+    else if (mode == 1 && wide) launch_dependent(fast_s_forward<1, true>, grid, kSThreads, bytes, stream, a);
+    else if (mode == 1) launch_dependent(fast_s_forward<1>, grid, kSThreads, bytes, stream, a);
+    else if (wide) launch_dependent(fast_s_forward<2, true>, grid, kSThreads, bytes, stream, a);
+    else launch_dependent(fast_s_forward<2>, grid, kSThreads, bytes, stream, a);
     count_launch();
 }
 
@@ -1067,10 +1076,11 @@ cudaError_t ensure_stream_capacity(FastState& fs, int N, int C, int L) {
 }
 
 // Writes `rows` channel rows of X into the stream kernel's copies.
-static void launch_stream_copy(FastState& fs, const float* X, int64_t rows, int L, int sms, cudaStream_t stream) {
+static void launch_stream_copy(FastState& fs, const float* X, int64_t rows, int L, int sms, bool dependent, cudaStream_t stream) {
     const bool vec = L % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
     auto kernel = vec ? stream_copy_kernel<true> : stream_copy_kernel<false>;
-    kernel<<<sms * 8, 256, 0, stream>>>(X, fs.wpad, rows, L, fs.host.wpitch, (int)fs.host.wfront);
+    if (dependent) launch_dependent(kernel, sms * 8, 256, 0, stream, X, fs.wpad, rows, L, fs.host.wpitch, (int)fs.host.wfront);
+    else kernel<<<sms * 8, 256, 0, stream>>>(X, fs.wpad, rows, L, fs.host.wpitch, (int)fs.host.wfront);
     count_launch();
 }
 
@@ -1229,7 +1239,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
                                                                fs.host.wpitch, (int)fs.host.wfront, *norm);
             count_launch();
         } else if (streamed) {
-            launch_stream_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
+            launch_stream_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, c == 0, stream);
         } else if (X_u8) {
             fast_pad_copy_u8_kernel<<<sms * 8, 256, 0, stream>>>(
                 reinterpret_cast<const uchar4*>(X_u8 + (size_t)n0 * dp.C * dp.L), fs.xpad, (int64_t)nc * dp.C, dp.L / 4, dp.C,
@@ -1242,7 +1252,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
         if (pd.n_sitems > 0) launch_s(a, fs, soft ? 1 : half ? 3 : 0, sms, stream);
         if (fs.profile) cudaEventRecord(fs.evs[3 * c + 1], stream);
         if (streamed) {
-            launch_stream(a, soft ? 1 : half ? 3 : 0, sms, stream);
+            launch_stream(a, soft ? 1 : half ? 3 : 0, sms, pd.n_sitems > 0, stream);
         } else if (pd.n_titems > 0) {
             const unsigned grid = t_grid(nc, pd.n_titems, sms);
             if (soft) fast_t_forward<1><<<grid, kTBlockThreads, t_bytes, stream>>>(a);
@@ -1257,8 +1267,8 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     }
     const int64_t fin = (int64_t)N * pd.n_krec;
     if (fin > 0) {
-        if (soft) fast_finalize_soft_kernel<<<(unsigned)((fin + 255) / 256), 256, 0, stream>>>(feat, argmax, ws, pd.krec, pd.n_krec, N, dp.K);
-        else fast_finalize_kernel<<<(unsigned)((fin + 255) / 256), 256, 0, stream>>>(feat, pd.krec, pd.n_krec, N, dp.K);
+        if (soft) launch_dependent(fast_finalize_soft_kernel, (unsigned)((fin + 255) / 256), 256, 0, stream, feat, argmax, ws, pd.krec, pd.n_krec, N, dp.K);
+        else launch_dependent(fast_finalize_kernel, (unsigned)((fin + 255) / 256), 256, 0, stream, feat, pd.krec, pd.n_krec, N, dp.K);
         count_launch();
     }
     return cudaGetLastError();
@@ -1300,7 +1310,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         else fast_absmax_scalar_kernel<<<blocks(n_x), 256, 0, stream>>>(X, n_x, absmax);
         count_launch();
     }
-    fast_bwd_prepare_kernel<<<(pd.n_krec + 7) / 8, 256, 0, stream>>>(dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale, accfix,
+    launch_dependent(fast_bwd_prepare_kernel, (pd.n_krec + 7) / 8, 256, 0, stream, dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale, accfix,
                                                                      n_weights, pd.counters);
     count_launch();
     FwdArgs a;
@@ -1316,17 +1326,17 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         a.argmax = argmax + (size_t)n0 * dp.K;
         a.N = nc;
         if (n0 > 0 && (e = cudaMemsetAsync(pd.counters, 0, 8, stream)) != cudaSuccess) return e;
-        if (streamed) launch_stream_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
+        if (streamed) launch_stream_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, n0 == 0, stream);
         else if (copied) launch_pad_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
         if (pd.n_sitems > 0) launch_s(a, fs, 2, sms, stream);
         if (streamed) {
-            launch_stream(a, 2, sms, stream);
+            launch_stream(a, 2, sms, pd.n_sitems > 0, stream);
         } else if (pd.n_titems > 0) {
             fast_t_forward<2><<<t_grid(nc, pd.n_titems, sms), kTBlockThreads, t_bytes, stream>>>(a);
             count_launch();
         }
     }
-    fast_bwd_finalize_kernel<<<(pd.n_krec + 7) / 8, 256, 0, stream>>>(accfix, scale, pd.krec, pd.n_krec, n_weights, dW, db);
+    launch_dependent(fast_bwd_finalize_kernel, (pd.n_krec + 7) / 8, 256, 0, stream, accfix, scale, pd.krec, pd.n_krec, n_weights, dW, db);
     count_launch();
     return cudaGetLastError();
 }

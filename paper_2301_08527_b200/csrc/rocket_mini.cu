@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
 // Counts to shares of outputs (Eq. 2); NaN when a wait of the tile kernel gave up.
 __global__ void __launch_bounds__(256)
 mini_finalize_kernel(float* __restrict__ feat, const int* __restrict__ nout, int F, long long total, const int* __restrict__ error_flag) {
+    dependency_wait();
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
     if (i >= total) return;
     const int count = reinterpret_cast<const int*>(feat)[i];
@@ -705,7 +706,7 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     if (p->wide) mini_tile_kernel<true><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
     else mini_tile_kernel<false><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
     const long long values = (long long)N * p->F;
-    mini_finalize_kernel<<<(unsigned)((values + 255) / 256), 256, 0, stream>>>(feat_dev, p->d_nout, p->F, values, args.error_flag);
+    launch_dependent(mini_finalize_kernel, (unsigned)((values + 255) / 256), 256, 0, stream, feat_dev, p->d_nout, p->F, values, args.error_flag);
     rocket::count_launch(2);
     const cudaError_t e = cudaGetLastError();
     if (prev != p->device) cudaSetDevice(prev);

@@ -530,6 +530,7 @@ __global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constan
         if (lane == 0) atomicExch(a.f.plan.error_flag, 1);
         for (int i = 0; i < kWStages; ++i, ++st) stream_wait_slow(bar0 + 8u * (st & 1u), (st >> 1) & 1u);
     }
+    dependency_wait();                                 // this grid ends after the one before it: whoever waits for this one waits for both
 }
 
 size_t stream_smem_bytes() { return (size_t)kWWarps * kWStages * kWStageFloats * sizeof(float) + 128; }
@@ -547,7 +548,7 @@ cudaError_t set_stream_attributes() {
     return e;
 }
 
-void launch_stream(const FwdArgs& f, int mode, int sms, cudaStream_t stream) {
+void launch_stream(const FwdArgs& f, int mode, int sms, bool after_s, cudaStream_t stream) {
     StreamArgs a;
     a.f = f;
     a.units = f.plan.wunits;
@@ -565,12 +566,18 @@ void launch_stream(const FwdArgs& f, int mode, int sms, cudaStream_t stream) {
     const unsigned grid = (unsigned)std::min<unsigned long long>((items + kWWarps - 1) / kWWarps, (unsigned long long)sms);
     const size_t bytes = stream_smem_bytes();
     const bool whole = f.plan.w_visits * f.N >= (double)kWWholeVisits * sms * kWWarps;
-    if (mode == 1 && whole) fast_stream<1, true><<<grid, kWThreads, bytes, stream>>>(a);
-    else if (mode == 1) fast_stream<1><<<grid, kWThreads, bytes, stream>>>(a);
-    else if (mode == 2 && whole) fast_stream<2, true><<<grid, kWThreads, bytes, stream>>>(a);
-    else if (mode == 2) fast_stream<2><<<grid, kWThreads, bytes, stream>>>(a);
-    else if (mode == 3) fast_stream<3><<<grid, kWThreads, bytes, stream>>>(a);
-    else fast_stream<0><<<grid, kWThreads, bytes, stream>>>(a);
+    // Behind the S kernel this one may begin as SMs run out of S tiles: every block of the S kernel has by then seen the kernels before
+    // it complete, and those wrote all that this one reads.
+    auto launch = [&](auto kernel) {
+        if (after_s) launch_dependent(kernel, grid, kWThreads, bytes, stream, a);
+        else kernel<<<grid, kWThreads, bytes, stream>>>(a);
+    };
+    if (mode == 1 && whole) launch(fast_stream<1, true>);
+    else if (mode == 1) launch(fast_stream<1>);
+    else if (mode == 2 && whole) launch(fast_stream<2, true>);
+    else if (mode == 2) launch(fast_stream<2>);
+    else if (mode == 3) launch(fast_stream<3>);
+    else launch(fast_stream<0>);
     count_launch();
 }
 
