@@ -758,7 +758,6 @@ __global__ void fast_init_kernel(int* __restrict__ feat_i, int64_t pairs, unsign
 
 __global__ void fast_finalize_kernel(float* __restrict__ feat, const KRec* __restrict__ krec, int n_krec, int N,
                                      int K) {
-    dependency_wait();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)N * n_krec) return;
     const int n = (int)(e / n_krec), f = (int)(e - (int64_t)n * n_krec);
@@ -778,7 +777,6 @@ __global__ void fast_init_soft_kernel(unsigned long long* __restrict__ ws, int64
 __global__ void fast_finalize_soft_kernel(float* __restrict__ feat, int32_t* __restrict__ argmax,
                                           const unsigned long long* __restrict__ ws, const KRec* __restrict__ krec,
                                           int n_krec, int N, int K) {
-    dependency_wait();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)N * n_krec) return;
     const int n = (int)(e / n_krec), f = (int)(e - (int64_t)n * n_krec);
@@ -910,7 +908,6 @@ __global__ void fast_bwd_prepare_kernel(const float* __restrict__ dfeat, const K
 __global__ void fast_bwd_finalize_kernel(const long long* __restrict__ accfix, const double* __restrict__ scale,
                                          const KRec* __restrict__ krec, int n_krec, long long n_weights,
                                          float* __restrict__ dW, float* __restrict__ db) {
-    dependency_wait();
     const int f = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (f >= n_krec) return;
     const KRec& r = krec[f];
@@ -1267,8 +1264,9 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     }
     const int64_t fin = (int64_t)N * pd.n_krec;
     if (fin > 0) {
-        if (soft) launch_dependent(fast_finalize_soft_kernel, (unsigned)((fin + 255) / 256), 256, 0, stream, feat, argmax, ws, pd.krec, pd.n_krec, N, dp.K);
-        else launch_dependent(fast_finalize_kernel, (unsigned)((fin + 255) / 256), 256, 0, stream, feat, pd.krec, pd.n_krec, N, dp.K);
+        // in stream order: behind the stream kernel alone it would not wait for the small-dilation kernel
+        if (soft) fast_finalize_soft_kernel<<<(unsigned)((fin + 255) / 256), 256, 0, stream>>>(feat, argmax, ws, pd.krec, pd.n_krec, N, dp.K);
+        else fast_finalize_kernel<<<(unsigned)((fin + 255) / 256), 256, 0, stream>>>(feat, pd.krec, pd.n_krec, N, dp.K);
         count_launch();
     }
     return cudaGetLastError();
@@ -1336,7 +1334,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
             count_launch();
         }
     }
-    launch_dependent(fast_bwd_finalize_kernel, (pd.n_krec + 7) / 8, 256, 0, stream, accfix, scale, pd.krec, pd.n_krec, n_weights, dW, db);
+    fast_bwd_finalize_kernel<<<(pd.n_krec + 7) / 8, 256, 0, stream>>>(accfix, scale, pd.krec, pd.n_krec, n_weights, dW, db);
     count_launch();
     return cudaGetLastError();
 }

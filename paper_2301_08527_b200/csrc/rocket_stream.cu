@@ -530,7 +530,6 @@ __global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constan
         if (lane == 0) atomicExch(a.f.plan.error_flag, 1);
         for (int i = 0; i < kWStages; ++i, ++st) stream_wait_slow(bar0 + 8u * (st & 1u), (st >> 1) & 1u);
     }
-    dependency_wait();                                 // this grid ends after the one before it: whoever waits for this one waits for both
 }
 
 size_t stream_smem_bytes() { return (size_t)kWWarps * kWStages * kWStageFloats * sizeof(float) + 128; }
