@@ -37,9 +37,9 @@ MINI_FEATURES = 9996          # MINIROCKET's default 10,000 rounded down to a mu
 # DRAM bytes (read + write) of one launch of either fused kernel, from the committed ncu capture (profiles/),
 # per launch = one chunk of 12 examples.  The figures belong to one state of the kernel sources: they are
 # reported only while the digest of those sources still equals NCU_SOURCES_DIGEST, and as null otherwise.
-NCU_DRAM_BYTES_PER_LAUNCH = {"fast_s_forward": 55.9e6, "fast_t_forward": 311.5e6}
-NCU_SOURCES_DIGEST = "7353b8ccfa8d2918"
-KERNEL_SOURCES = ("rocket_fast_fwd.cu", "rocket_fast.h", "rocket_fast_geom.h", "rocket_plan.cpp")
+NCU_DRAM_BYTES_PER_LAUNCH = {"fast_s_forward": 55.9e6, "fast_stream": 2071.1e6}
+NCU_SOURCES_DIGEST = "6878b2100711e21e"
+KERNEL_SOURCES = ("rocket_fast_fwd.cu", "rocket_stream.cu", "rocket_fast_dev.cuh", "rocket_fast.h", "rocket_fast_geom.h", "rocket_plan.cpp")
 
 
 def kernel_sources_digest():
@@ -415,7 +415,7 @@ def main():
     ms_s = float(np.mean([k["ms_small_dilations"] for k in kernel_ms]))
     ms_t = float(np.mean([k["ms_large_dilations"] for k in kernel_ms]))
     fl_s, fl_t = kernel_ms[-1]["flops_small_dilations"], kernel_ms[-1]["flops_large_dilations"]
-    dom = "fast_t_forward (dilations >= 64)" if ms_t >= ms_s else "fast_s_forward (dilations < 64)"
+    dom = "fast_stream (dilations >= 64)" if ms_t >= ms_s else "fast_s_forward (dilations < 64)"
     dom_ms, dom_fl = (ms_t, fl_t) if ms_t >= ms_s else (ms_s, fl_s)
     achieved = dom_fl * w["N"] / (dom_ms * 1e-3) / 1e12 if dom_ms > 0 else 0.0
     step_tflops = flops_ex * w["N"] / float(np.mean(per_step)) / 1e12
@@ -435,7 +435,7 @@ def main():
                 "flop_count": "2*len*channels*L_out per kernel per example; whole path %.4g flop/example, "
                               "this kernel %.4g" % (flops_ex, dom_fl),
                 "kernels": {"fast_s_forward": {"ms": ms_s, "tflops": fl_s * w["N"] / (ms_s * 1e-3) / 1e12 if ms_s else None},
-                            "fast_t_forward": {"ms": ms_t, "tflops": fl_t * w["N"] / (ms_t * 1e-3) / 1e12 if ms_t else None}},
+                            "fast_stream": {"ms": ms_t, "tflops": fl_t * w["N"] / (ms_t * 1e-3) / 1e12 if ms_t else None}},
                 "whole_step_tflops": step_tflops, "whole_step_frac": step_tflops / peak,
                 "pooling_ops_per_example": 2.0 * outputs_ex}
     # the three denominators: lanes x maximum clock (peak / frac above), lanes x the clock observed during the timed
