@@ -118,12 +118,15 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
     const unsigned total = (tiles0 + tiles1 + (unsigned)(a.s_end[2] - a.s_end[1]) * (unsigned)a.s_groups[2]) * (HALF ? 2u : 1u);
     KRec* myrec = recs + warp * 2;
 
+    bool first = true;
     for (;;) {
         __syncthreads();  // the previous tile is fully consumed
         if (warp == 0) {  // draw a tile and lay its description out for the block
             unsigned g = 0;
-            if (lane == 0) g = atomicAdd(a.plan.counters + 0, 1u);
+            if (first) g = blockIdx.x;            // a block's first tile goes by its place, which spares a trip to the counter
+            else if (lane == 0) g = gridDim.x + atomicAdd(a.plan.counters + 0, 1u);
             g = __shfl_sync(kFull, g, 0);
+            first = false;
             if (lane == 0) { s_item = g; s_next = 0; }
             if (g < total) {
                 if (HALF) {
