@@ -241,12 +241,16 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
     auto load_rec = [&](const TileAt& t, int w) {
         return __ldg(reinterpret_cast<const int*>(a.recs + t.kbeg + (t.ne == 1 ? w : w / t.ne)) + lane);
     };
-    TileAt cur;
+    TileAt cur{};
     int k = 0, base = 0;
     int pos = draw();
     // the lane's two columns of the tile: band of rows and column of A
     int trow0 = 0, trow1 = 0, c0 = 0, c1 = 0;
     bool ok0 = false, ok1 = false;
+    int rec_next = 0;                                  // the record of the pair at pos, on its way
+    auto fetch_rec = [&]() {
+        if (pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
+    };
     auto enter = [&]() {
         if constexpr (WIDE) {
             const unsigned g = blockIdx.x + (unsigned)k * gridDim.x, per_group = (unsigned)a.n_tiles * (unsigned)a.parts;
@@ -257,12 +261,14 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
             const int words = __ldg(reinterpret_cast<const int*>(b) + lane), more_words = __ldg(reinterpret_cast<const int*>(b) + 32 + lane), first = word(words, 2), combos = word(words, 3) - first;
             const int nch = word(words, 4), n0 = (int)group * a.examples, ne = min(a.examples, a.N - n0), beg = combos * part / a.parts;
             cur = TileAt{word(words, 0), word(words, 1), nch * kMPlaneBytes, at.y, n0, ne, first + beg, (combos * (part + 1) / a.parts - beg) * ne};
+            fetch_rec();
             const FillAt columns(cur.d, cur.raster_len, cur.c0, a.L, lane);
             fill_planes(a, columns, planes, [&](int c) { return c < 20 ? word(words, 12 + c) : word(more_words, c - 20); }, nch, n0, ne, warp, kMWarps, lane);
             __syncthreads();
         } else {
             if (!mbar_wait(full0 + 8u * (k & 1), (k >> 1) & 1)) return false;
             cur = s_tile[k & 1];
+            fetch_rec();
         }
         const int cg = cur.c0 + 2 * lane, band = (int)((unsigned)cg / (unsigned)cur.d);
         c0 = cg - band * cur.d;
@@ -274,7 +280,6 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
         return true;
     };
     ok = enter();
-    int rec_next = ok && pos < cur.n_work ? load_rec(cur, pos) : 0;
     while (ok) {
         if (pos >= base + cur.n_work) {
             if (k + 1 >= K) break;
@@ -287,14 +292,13 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
             base += cur.n_work;
             ++k;
             ok = enter();
-            if (ok && pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
             continue;
         }
         const int rec = rec_next, w = pos - base, e = cur.ne == 1 ? 0 : w % cur.ne;
         const int m = word(rec, 0), f0 = word(rec, 1), nf = word(rec, 2);
         float my_bias = lane < nf ? __ldg(a.bias + f0 + lane) : 0.0f;
         pos = draw();
-        if (pos < base + cur.n_work) rec_next = load_rec(cur, pos - base);
+        fetch_rec();
         const char* st = reinterpret_cast<const char*>(planes + (WIDE ? 0 : (k & 1) * kMPlanes * kMPlaneFloats) + 2 * lane);
         if (e > 0) st += e * cur.plane_bytes;
 
