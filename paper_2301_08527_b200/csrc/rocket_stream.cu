@@ -530,6 +530,9 @@ __global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constan
         if (lane == 0) atomicExch(a.f.plan.error_flag, 1);
         for (int i = 0; i < kWStages; ++i, ++st) stream_wait_slow(bar0 + 8u * (st & 1u), (st >> 1) & 1u);
     }
+    // Begun early, this kernel may end before the S kernel does.  Every block has a warp with work, which waits for the S kernel
+    // here: what follows in the stream, or behind this kernel's node of a captured graph, then follows the S kernel too.
+    dependency_wait();
 }
 
 size_t stream_smem_bytes() { return (size_t)kWWarps * kWStages * kWStageFloats * sizeof(float) + 128; }
