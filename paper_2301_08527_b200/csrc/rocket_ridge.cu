@@ -401,6 +401,9 @@ ridge_predict_kernel(const float* __restrict__ F, int P, const float* __restrict
     __shared__ double s_part[8];
     cg::cluster_group cluster = cg::this_cluster();
     const int parts = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // No block may write to the first one's shared memory before that block runs: every block says here that it does, and waits for
+    // the others behind its loop.
+    if (parts > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     const float* __restrict__ f = F + (size_t)blockIdx.y * P;
     double s = 0.0;
     if (VEC) {
@@ -421,13 +424,17 @@ ridge_predict_kernel(const float* __restrict__ F, int P, const float* __restrict
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) red[warp] = s;
     __syncthreads();
+    if (parts > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (warp == 0) {
         s = lane < kPThreads / 32 ? red[lane] : 0.0;
 #pragma unroll
         for (int o = kPThreads / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) *cluster.map_shared_rank(&s_part[rank], 0) = s;
+        if (lane == 0) {
+            if (parts > 1) *cluster.map_shared_rank(&s_part[rank], 0) = s;
+            else s_part[0] = s;
+        }
     }
-    cluster.sync();
+    if (parts > 1) cluster.sync();
     if (rank == 0 && threadIdx.x == 0) {
         s = s_part[0];
         for (int r = 1; r < parts; ++r) s += s_part[r];

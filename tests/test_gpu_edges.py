@@ -78,3 +78,16 @@ def test_ridge_predict(N, P_, offset):
     got = rk.rocket_ridge_predict(raw[offset:].view(N, P_), _dev(w), _dev(np.array([1.2], np.float32))).cpu().numpy()
     want = F.astype(np.float64) @ w.astype(np.float64) + np.float32(1.2)
     assert np.abs(got - want).max() <= 2e-6 * max(1.0, float(np.abs(want).max()), float((np.abs(F) @ np.abs(w)).max()))
+
+
+@pytest.mark.parametrize("N,P_", [(70, 4100), (3, 8196), (37, 16388), (1, 20000), (148, 4096), (149, 4100)])
+def test_ridge_predict_rows_shared_by_a_cluster(N, P_):
+    # rows of whole 16-byte loads shared by 2, 4 and 8 blocks, in parts that are not of one size; 148 rows are the most that
+    # two blocks share
+    F, y = _problem(N + P_, N, P_)
+    w = np.random.default_rng(P_).normal(0, 1.0 / np.sqrt(P_), P_).astype(np.float32)
+    got = [rk.rocket_ridge_predict(_dev(F), _dev(w), _dev(np.array([1.2], np.float32))).cpu().numpy() for _ in range(20)]
+    want = F.astype(np.float64) @ w.astype(np.float64) + np.float32(1.2)
+    # summed in double and rounded once: half a unit of the result, and the double sum's own error far below that
+    assert np.abs(got[0] - want).max() <= 1.2e-7 * max(1.0, float(np.abs(want).max()))
+    assert all(np.array_equal(g, got[0]) for g in got)
