@@ -388,11 +388,48 @@ ridge_weights_kernel(const float* __restrict__ F, int N, int P, const double* __
     }
 }
 
-// yhat[n] = b + sum_p F[n][p] w[p], products summed in double.  A row is shared by the blocks of a cluster (as many as
-// it takes to put a block on every SM, at most eight): each sums its contiguous part, the first adds the parts in rank
-// order through distributed shared memory.  Bound: the latency of one trip to memory; a block per row and one float
-// per load took 14.7 us for 60 rows of 20,000, this takes 7.6.
+// yhat[n] = b + sum_p F[n][p] w[p], products summed in double: a row per block of 256 threads (W = 8 warps), half a
+// block or a warp.  (Eight loads of a lane gathered in registers before the first product: 68 us for 4,000 rows of 20,000 against 64.)
+template <bool VEC, int W>
+__global__ void __launch_bounds__(kRThreads)
+ridge_predict_rows_kernel(const float* __restrict__ F, int N, int P, const float* __restrict__ w, const float* __restrict__ b,
+                          float* __restrict__ yhat) {
+    __shared__ double red[kRWarps];
+    const int warp = threadIdx.x >> 5, at = threadIdx.x % (32 * W);
+    const long long n = (long long)blockIdx.x * (kRWarps / W) + warp / W;
+    double s = 0.0;
+    if (n < N) {
+        const float* __restrict__ f = F + (size_t)n * P;
+        if (VEC) {
+            const float4* __restrict__ f4 = reinterpret_cast<const float4*>(f);
+            const float4* __restrict__ w4 = reinterpret_cast<const float4*>(w);
+            const int n4 = P / 4;
+#pragma unroll 4
+            for (int i = at; i < n4; i += 32 * W) {
+                const float4 x = __ldg(f4 + i), v = __ldg(w4 + i);
+                s += (double)x.x * (double)v.x + (double)x.y * (double)v.y + ((double)x.z * (double)v.z + (double)x.w * (double)v.w);
+            }
+        } else {
+#pragma unroll 4
+            for (int i = at; i < P; i += 32 * W) s += (double)__ldg(f + i) * (double)__ldg(w + i);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (W > 1) {
+        if ((threadIdx.x & 31) == 0) red[warp] = s;
+        __syncthreads();
+        if (at == 0)
+            for (int v = 1; v < W; ++v) s += red[warp + v];
+    }
+    if (n < N && at == 0) yhat[n] = (float)(s + (double)*b);
+}
+
+// The same for few, long rows: the blocks of a cluster (as many as it takes to put two blocks on every SM, at most eight) share a
+// row, each sums its contiguous part, the first adds the parts in rank order through distributed shared memory.  Bound: the
+// latency of a few trips to memory: 60 rows of 20,000 take 3.7 us on the device, 5.8 with a block per row.
 constexpr int kPThreads = 512;
+constexpr int kPPairs = 148;                            // rows that two blocks each share: two blocks per SM of this GPU
 template <bool VEC>
 __global__ void __launch_bounds__(kPThreads)
 ridge_predict_kernel(const float* __restrict__ F, int P, const float* __restrict__ w, const float* __restrict__ b,
@@ -403,7 +440,7 @@ ridge_predict_kernel(const float* __restrict__ F, int P, const float* __restrict
     const int parts = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // No block may write to the first one's shared memory before that block runs: every block says here that it does, and waits for
     // the others behind its loop.
-    if (parts > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     const float* __restrict__ f = F + (size_t)blockIdx.y * P;
     double s = 0.0;
     if (VEC) {
@@ -424,17 +461,14 @@ ridge_predict_kernel(const float* __restrict__ F, int P, const float* __restrict
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) red[warp] = s;
     __syncthreads();
-    if (parts > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (warp == 0) {
         s = lane < kPThreads / 32 ? red[lane] : 0.0;
 #pragma unroll
         for (int o = kPThreads / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            if (parts > 1) *cluster.map_shared_rank(&s_part[rank], 0) = s;
-            else s_part[0] = s;
-        }
+        if (lane == 0) *cluster.map_shared_rank(&s_part[rank], 0) = s;
     }
-    if (parts > 1) cluster.sync();
+    cluster.sync();
     if (rank == 0 && threadIdx.x == 0) {
         s = s_part[0];
         for (int r = 1; r < parts; ++r) s += s_part[r];
@@ -575,16 +609,16 @@ extern "C" int rocket_ridge_predict(const float* feat_dev, int N, int P, const f
     if (N == 0) return ROCKET_OK;
     if (!feat_dev || !w_dev || !b_dev || !yhat_dev) return ROCKET_EINVAL;
     const bool vec = P % 4 == 0 && ((reinterpret_cast<uintptr_t>(feat_dev) | reinterpret_cast<uintptr_t>(w_dev)) & 15u) == 0;
-    // grid.y is limited to 65,535 rows
-    for (int n0 = 0; n0 < N; n0 += 65535) {
-        const int n = std::min(N - n0, 65535);
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    // A cluster per row where two blocks per row leave no SM with more than two, and a part is at least three loads per thread: 10 rows
+    // of 20,000 take 3.1 us so and 5.6 with a block per row, 60 of 8,000 3.3 and 3.7; rows of 4,096 2.8 and 2.3.
+    if (N <= kPPairs && P >= 6144) {
+        unsigned parts = 2;
+        while (parts < 8 && (int)parts * N <= kPPairs && (int)parts * 2 * kPThreads * 4 <= P) parts *= 2;
         cudaLaunchConfig_t cfg = {};
-        // blocks per row: up to two per SM of this GPU's 148, and no fewer than one step of a block's threads each
-        unsigned parts = 1;
-        while (parts < 8 && (long long)n * parts * 2 <= 296 && (int)parts * 2 * kPThreads * 4 <= P) parts *= 2;
-        cfg.gridDim = dim3(parts, (unsigned)n);
+        cfg.gridDim = dim3(parts, (unsigned)N);
         cfg.blockDim = dim3(kPThreads);
-        cfg.stream = static_cast<cudaStream_t>(cuda_stream);
+        cfg.stream = stream;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = parts;
@@ -592,12 +626,21 @@ extern "C" int rocket_ridge_predict(const float* feat_dev, int N, int P, const f
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const float* f = feat_dev + (size_t)n0 * P;
-        float* out = yhat_dev + n0;
-        const cudaError_t e = vec ? cudaLaunchKernelEx(&cfg, ridge_predict_kernel<true>, f, P, w_dev, b_dev, out)
-                                  : cudaLaunchKernelEx(&cfg, ridge_predict_kernel<false>, f, P, w_dev, b_dev, out);
+        const cudaError_t e = vec ? cudaLaunchKernelEx(&cfg, ridge_predict_kernel<true>, feat_dev, P, w_dev, b_dev, yhat_dev)
+                                  : cudaLaunchKernelEx(&cfg, ridge_predict_kernel<false>, feat_dev, P, w_dev, b_dev, yhat_dev);
         count_launch();
-        if (e != cudaSuccess) return status_of(e);
+        return status_of(e);
     }
-    return ROCKET_OK;
+    // A warp per row where a lane's loads are one, or few for the number of rows (30,000 rows of 200: 6.7 us, of 2,000: 55; a block
+    // per row takes 28 and 65, a cluster of one block 128 and 167; 700 rows of 600: 2.8 us so, 2.2 with a block per row).  Half a
+    // block for the longer of many rows (4,000 rows of 20,000: 60 us against 64, of 4,096 the same).
+    const long long loads = ((long long)P / (vec ? 4 : 1) + 31) / 32;
+    auto launch = [&](auto kernel, int rows) {
+        kernel<<<(unsigned)(((long long)N + rows - 1) / rows), kRThreads, 0, stream>>>(feat_dev, N, P, w_dev, b_dev, yhat_dev);
+    };
+    if (loads <= 1 || N >= 300 * loads) vec ? launch(ridge_predict_rows_kernel<true, 1>, 8) : launch(ridge_predict_rows_kernel<false, 1>, 8);
+    else if (N >= 2000) vec ? launch(ridge_predict_rows_kernel<true, 4>, 2) : launch(ridge_predict_rows_kernel<false, 4>, 2);
+    else vec ? launch(ridge_predict_rows_kernel<true, 8>, 1) : launch(ridge_predict_rows_kernel<false, 8>, 1);
+    count_launch();
+    return status_of(cudaGetLastError());
 }

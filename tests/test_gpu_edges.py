@@ -91,3 +91,19 @@ def test_ridge_predict_rows_shared_by_a_cluster(N, P_):
     # summed in double and rounded once: half a unit of the result, and the double sum's own error far below that
     assert np.abs(got[0] - want).max() <= 1.2e-7 * max(1.0, float(np.abs(want).max()))
     assert all(np.array_equal(g, got[0]) for g in got)
+
+
+@pytest.mark.parametrize("N,P_,offset", [(299, 127, 0), (300, 128, 0), (600, 256, 0), (599, 256, 0), (1201, 512, 0), (301, 31, 1), (600, 33, 3),
+                                         (70001, 5, 0), (66000, 64, 0), (149, 6144, 0), (148, 6145, 1), (7, 1023, 0), (9, 4100, 0),
+                                         (2000, 897, 0), (2001, 4092, 0), (2001, 2049, 2)])
+def test_ridge_predict_of_many_rows(N, P_, offset):
+    # a warp (one load per lane, or many rows), half a block and a block per row, at the edges between them and in both widths of load
+    rng = np.random.default_rng(N + P_)
+    F = rng.normal(0.5, 1.0, (N, P_)).astype(np.float32)
+    w = rng.normal(0, 1.0 / np.sqrt(P_), P_).astype(np.float32)
+    import torch
+    raw = torch.zeros(N * P_ + offset, device="cuda")
+    raw[offset:] = _dev(F).reshape(-1)
+    got = rk.rocket_ridge_predict(raw[offset:].view(N, P_), _dev(w), _dev(np.array([1.2], np.float32))).cpu().numpy()
+    want = F.astype(np.float64) @ w.astype(np.float64) + np.float32(1.2)
+    assert np.abs(got - want).max() <= 1.2e-7 * max(1.0, float(np.abs(want).max()))   # summed in double, rounded once
