@@ -189,6 +189,7 @@ constexpr int kWStages = 2;                                        // (tile, cha
 constexpr int kWStageFloats = (kWRows + ROCKET_MAX_LENGTH - 1 + 3) / 4 * 4 * kWarpCols;   // input rows of a visit, whole y steps
 constexpr int kWCopies = 7;                                        // shifted copies of every channel row, next to one another
 constexpr int kWUnitVisits = 16, kWItemVisits = 32;                // visits of a unit, and of a unit for a group of examples
+constexpr int kWSoftSetItems = 24;                                 // items per warp of a set, soft and backward
 constexpr int64_t kWCopyBytes = 800ll << 20;                       // what the copies of a pass may take (13 examples of 20 x 50,000)
 
 // A unit of work: consecutive tiles of one kernel (32 words).  The kernel's output rows from t0 on are cut into bands of R rows,
@@ -204,6 +205,10 @@ struct alignas(16) WUnit {
     int32_t bytes, pad_[4];               // bytes of a visit's copy
 };
 static_assert(sizeof(WUnit) == 128, "WUnit must be 32 words");
+// How a pass of N examples is handed out to the warps of the stream kernel (mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half
+// precision): an item is a unit for `examples` examples, the items of `groups_per_set` such groups go through all units together.
+struct StreamItems { int examples, groups, groups_per_set; };
+StreamItems stream_items(int N, int C, int L, int n_units, double visits, int mode, int sms, int64_t l2_bytes);
 // One tensor map of the stream regime: boxes of 64 columns x y_rows y steps over the copies, for dilation d.
 struct WMapSpec { int32_t d, y_rows; };
 // Rows per y step: an odd dilation takes four rows (one per alignment) as a dimension of their own, d = 2 mod 4 two.

@@ -33,7 +33,7 @@ struct FwdArgs {
 
 // The stream kernel over a pass of f.N examples (rocket_stream.cu); mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half
 // precision.
-void launch_stream(const FwdArgs& f, int mode, int sms, bool after_s, cudaStream_t stream);   // after_s: directly behind the S kernel
+void launch_stream(const FwdArgs& f, int mode, int sms, int64_t l2_bytes, bool after_s, cudaStream_t stream);   // after_s: directly behind the S kernel
 cudaError_t set_stream_attributes();   // opts the kernel into its shared-memory size
 
 // A launch that may begin while its predecessor in the stream ends (programmatic dependent launch): the kernel itself waits for the

@@ -1180,10 +1180,11 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
                                 const uint8_t* X_u8, const NormArgs* norm, bool half) {
     if (half && soft) return cudaErrorInvalidValue;
     std::lock_guard<std::mutex> lk(fs.mu);
-    int dev = 0, sms = 0;
+    int dev = 0, sms = 0, l2 = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;
@@ -1252,7 +1253,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
         if (pd.n_sitems > 0) launch_s(a, fs, soft ? 1 : half ? 3 : 0, sms, stream);
         if (fs.profile) cudaEventRecord(fs.evs[3 * c + 1], stream);
         if (streamed) {
-            launch_stream(a, soft ? 1 : half ? 3 : 0, sms, pd.n_sitems > 0, stream);
+            launch_stream(a, soft ? 1 : half ? 3 : 0, sms, l2, pd.n_sitems > 0, stream);
         } else if (pd.n_titems > 0) {
             const unsigned grid = t_grid(nc, pd.n_titems, sms);
             if (soft) fast_t_forward<1><<<grid, kTBlockThreads, t_bytes, stream>>>(a);
@@ -1279,10 +1280,11 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
                                  float lambda, float shift, const float* dfeat, const int32_t* argmax, float* dW,
                                  float* db, cudaStream_t stream) {
     std::lock_guard<std::mutex> lk(fs.mu);
-    int dev = 0, sms = 0;
+    int dev = 0, sms = 0, l2 = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;
@@ -1331,7 +1333,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         else if (copied) launch_pad_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
         if (pd.n_sitems > 0) launch_s(a, fs, 2, sms, stream);
         if (streamed) {
-            launch_stream(a, 2, sms, pd.n_sitems > 0, stream);
+            launch_stream(a, 2, sms, l2, pd.n_sitems > 0, stream);
         } else if (pd.n_titems > 0) {
             fast_t_forward<2><<<t_grid(nc, pd.n_titems, sms), kTBlockThreads, t_bytes, stream>>>(a);
             count_launch();

@@ -102,6 +102,27 @@ void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost&
 
 }  // namespace
 
+// Examples of an item: as many as give it kWItemVisits visits on average, while every warp of the chip still gets a dozen items and
+// their copies take no more than half of the L2: two examples of 20 x 200,000 do not, and 60 of them took 245 ms two at a time, 218
+// one at a time (10,000 kernels; 20 x 100,000: 106 and 103 ms; 20 x 50,000, where two fit: 50.7 and 51.6).
+// Groups of a set: as many as keep their copies in a third of the L2.  The soft transform and the backward take more of them where a
+// handle has few units: in the course of a set the warps pass through all nine shapes of the inner loop, and with fewer than
+// kWSoftSetItems items per warp they wait for instructions (24 x 12 x 50,000, 340 kernels, both passes: 8.68 ms by bytes alone,
+// 7.44, 6.46, 6.40 and 6.40 with 4, 8, 16 and 24 items; 24 x 20 x 14,002, 1,200 kernels: 6.32 and 4.56).  The hard modes, whose code
+// is smaller, lose by it (24 x 12 x 50,000, 340 kernels: 1.91 and 2.06).
+StreamItems stream_items(int N, int C, int L, int n_units, double visits, int mode, int sms, int64_t l2_bytes) {
+    StreamItems s;
+    const int64_t warps = (int64_t)sms * kWWarps, example_bytes = (int64_t)C * kWCopies * L * 4;
+    const double per_unit = std::max(1.0, visits * (mode == 2 ? 2.0 : 1.0) / std::max(1, n_units));
+    s.examples = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)(kWItemVisits / per_unit), (int64_t)N * n_units / (warps * 12), (int64_t)N,
+                                                              l2_bytes / 2 / example_bytes}));
+    s.groups = (N + s.examples - 1) / s.examples;
+    int64_t per_set = l2_bytes / 3 / (example_bytes * s.examples);
+    if (mode == 1 || mode == 2) per_set = std::max(per_set, (kWSoftSetItems * warps + n_units - 1) / std::max(1, n_units));
+    s.groups_per_set = (int)std::max<int64_t>(1, std::min<int64_t>(s.groups, per_set));
+    return s;
+}
+
 void fill_record_weights(const HostParams& hp, KRec& f) {
     const float* W = hp.weights.data() + hp.weight_offset[f.k];
     f.negb = 0.0f - hp.bias[f.k];

@@ -552,20 +552,16 @@ cudaError_t set_stream_attributes() {
     return e;
 }
 
-void launch_stream(const FwdArgs& f, int mode, int sms, bool after_s, cudaStream_t stream) {
+void launch_stream(const FwdArgs& f, int mode, int sms, int64_t l2_bytes, bool after_s, cudaStream_t stream) {
     StreamArgs a;
     a.f = f;
     a.units = f.plan.wunits;
     a.n_units = f.plan.n_wunits;
     a.maps = f.plan.wmaps;
-    // Examples of an item: as many as give it kWItemVisits visits on average, while every warp of the chip still gets a
-    // dozen items.  Examples handed out together: as many as keep their copies in a third of the L2.
-    const double per_unit = std::max(1.0, f.plan.w_visits * (mode == 2 ? 2.0 : 1.0) / std::max(1, a.n_units));
-    const long long most = (long long)f.N * a.n_units / ((long long)sms * kWWarps * 12);
-    a.examples = (int)std::max<long long>(1, std::min<long long>({(long long)(kWItemVisits / per_unit), most, (long long)f.N}));
-    a.groups = (f.N + a.examples - 1) / a.examples;
-    const long long example_bytes = (long long)f.C * kWCopies * f.L * 4;
-    a.groups_per_set = (int)std::max<long long>(1, std::min<long long>(a.groups, (40ll << 20) / (example_bytes * a.examples)));
+    const StreamItems it = stream_items(f.N, f.C, f.L, a.n_units, f.plan.w_visits, mode, sms, l2_bytes);
+    a.examples = it.examples;
+    a.groups = it.groups;
+    a.groups_per_set = it.groups_per_set;
     const unsigned long long items = (unsigned long long)a.groups * (unsigned long long)a.n_units;
     const unsigned grid = (unsigned)std::min<unsigned long long>((items + kWWarps - 1) / kWWarps, (unsigned long long)sms);
     const size_t bytes = stream_smem_bytes();
