@@ -360,7 +360,8 @@ int rocket_transform_soft_backward_noalloc(const rocket_params_t* p, const float
  * rocket_mini_transform   X_dev [N][C][L] fp32 and feat_dev [N][n_features] fp32 on the device; one fused kernel
  *                      (and a small one that divides the counts) on the caller's stream (convolution outputs never
  *                      reach memory; any L, any 4-byte aligned X_dev); the first call binds the handle to the current
- *                      device, uploads its parameters (one allocation) and opts the kernel into 200 KB of shared memory.  ROCKET_EINVAL before
+ *                      device, uploads its parameters (one allocation) and opts the kernel into 220 KB of shared memory.  Every wait inside the
+ *                      kernel is bounded; should one give up, all features of that call (and of no other) are NaN.  ROCKET_EINVAL before
  *                      a fit or set_biases; ROCKET_ESHAPE when C or L differ from the handle's.
  * rocket_mini_host_view   read-only views of the host arrays (taps [84][3], per combination: dilation,
  *                      kernel_index, padded, num_channels, ragged channel_idx, feature_offset [n + 1],

@@ -18,6 +18,7 @@
 // speeds the method up on a CPU brings nothing here.
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -83,7 +84,7 @@ struct MiniArgs {
     const MiniTile* tiles;
     const float* bias;
     int* counts;                          // [N][F]: the features while they are counts
-    int* error_flag;
+    int* failed;                          // the call's flag
     int N, C, L, F, n_tiles;
     int examples, groups, parts;          // examples of a tile, groups of examples, parts a tile's combinations are dealt in
 };
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
             fill_planes(a, at_columns, planes + (k & 1) * kMPlanes * kMPlaneFloats, [&](int c) { return word(bucket_words, 12 + c); }, nch, n0, ne, warp - kConsumers, kMProducers, lane);
             mbar_arrive(full0 + 8u * (k & 1));
         }
-        if (!ok && lane == 0) atomicExch(a.error_flag, 1);
+        if (!ok && lane == 0) atomicExch(a.failed, 1);
         return;
     }
 
@@ -367,17 +368,33 @@ __global__ void __launch_bounds__(kMThreads, 1) mini_tile_kernel(const __grid_co
             if (lane < n && mine) atomicAdd(counts + fb + lane, mine);
         }
     }
-    if (!ok && lane == 0) atomicExch(a.error_flag, 1);
+    if (!ok && lane == 0) atomicExch(a.failed, 1);
 }
 
-// Counts to shares of outputs (Eq. 2); NaN when a wait of the tile kernel gave up.
+// A call's flag, set when one of its waits gave up, and the blocks of its finalising kernel that have read it then.
+struct MiniFlag { int failed; unsigned readers; };
+constexpr int kMFlags = 64;               // calls take them in turn
+
+// Counts to shares of outputs (Eq. 2); NaN when a wait of the tile kernel gave up, in which case the last block clears the flag, so
+// that the failure stays the call's own (also where a graph repeats the call).
 __global__ void __launch_bounds__(256)
-mini_finalize_kernel(float* __restrict__ feat, const int* __restrict__ nout, int F, long long total, const int* __restrict__ error_flag) {
+mini_finalize_kernel(float* __restrict__ feat, const int* __restrict__ nout, int F, long long total, MiniFlag* flag) {
     dependency_wait();
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-    if (i >= total) return;
-    const int count = reinterpret_cast<const int*>(feat)[i];
-    feat[i] = *error_flag ? __int_as_float(0x7fc00000) : (float)count / (float)__ldg(nout + i % F);
+    const bool failed = *(volatile int*)&flag->failed != 0;
+    if (i < total) {
+        const int count = reinterpret_cast<const int*>(feat)[i];
+        feat[i] = failed ? __int_as_float(0x7fc00000) : (float)count / (float)__ldg(nout + i % F);
+    }
+    if (!failed) return;
+    __syncthreads();                      // every thread of the block has read the flag
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&flag->readers, 1u) == gridDim.x - 1) {
+            flag->readers = 0u;
+            flag->failed = 0;
+        }
+    }
 }
 
 }  // namespace
@@ -400,9 +417,11 @@ struct rocket_mini {
     bool wide = false;                     // the combinations of some dilation use more than kMPlanes channels
     mutable std::mutex mu;
     mutable int device = -1;
-    mutable void* blob = nullptr;          // records, buckets, tiles, output counts, biases, error flag
+    mutable void* blob = nullptr;          // records, buckets, tiles, output counts, biases, the calls' flags
     mutable MiniArgs dev{};
     mutable const int* d_nout = nullptr;
+    mutable MiniFlag* flags = nullptr;
+    mutable std::atomic<unsigned> calls{0};
     mutable bool bias_uploaded = false;
 };
 
@@ -484,13 +503,13 @@ static int ensure_mini_device(const rocket_mini* p) {
         struct Part { const void* src; size_t bytes, off; };
         Part parts[6] = {{p->recs.data(), p->recs.size() * sizeof(MiniRec), 0},     {p->buckets.data(), p->buckets.size() * sizeof(MiniBucket), 0},
                          {p->tiles.data(), p->tiles.size() * sizeof(MiniTile), 0}, {p->nout.data(), p->nout.size() * sizeof(int32_t), 0},
-                         {nullptr, (size_t)p->F * sizeof(float), 0},               {nullptr, 256, 0}};
+                         {nullptr, (size_t)p->F * sizeof(float), 0},               {nullptr, kMFlags * sizeof(MiniFlag), 0}};
         size_t total = 0;
         for (Part& pt : parts) { pt.off = total; total += (pt.bytes + 255) / 256 * 256; }
         cudaError_t e = rocket::device_malloc(&p->blob, total);
         if (e != cudaSuccess) { cudaGetLastError(); p->blob = nullptr; return e == cudaErrorMemoryAllocation ? ROCKET_ENOMEM : ROCKET_ECUDA; }
         char* base = static_cast<char*>(p->blob);
-        e = cudaMemset(base + parts[5].off, 0, 256);
+        e = cudaMemset(base + parts[5].off, 0, parts[5].bytes);
         for (const Part& pt : parts)
             if (e == cudaSuccess && pt.src) e = cudaMemcpy(base + pt.off, pt.src, pt.bytes, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
@@ -502,7 +521,7 @@ static int ensure_mini_device(const rocket_mini* p) {
         a.tiles = reinterpret_cast<const MiniTile*>(base + parts[2].off);
         p->d_nout = reinterpret_cast<const int*>(base + parts[3].off);
         a.bias = reinterpret_cast<const float*>(base + parts[4].off);
-        a.error_flag = reinterpret_cast<int*>(base + parts[5].off);
+        p->flags = reinterpret_cast<MiniFlag*>(base + parts[5].off);
         a.C = p->C; a.L = p->L; a.F = p->F; a.n_tiles = (int)p->tiles.size();
         p->device = dev;
         p->bias_uploaded = false;
@@ -698,6 +717,8 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     args.X = X_dev;
     args.counts = reinterpret_cast<int*>(feat_dev);
     args.N = N;
+    MiniFlag* flag = p->flags + p->calls.fetch_add(1, std::memory_order_relaxed) % kMFlags;
+    args.failed = &flag->failed;
     // Examples that share a tile: as many as its planes hold, while every SM still gets four tiles; fewer tiles than SMs are
     // dealt in parts of their combinations (84 or so) instead.
     const long long tiles = (long long)N * args.n_tiles;
@@ -714,7 +735,7 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     const bool all_copy = p->wide || items * args.parts <= grid;
     if (all_copy) mini_tile_kernel<true><<<grid, kMThreads, (size_t)args.examples * p->max_nch * kMPlaneBytes, stream>>>(args);
     else mini_tile_kernel<false><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
-    launch_dependent(mini_finalize_kernel, value_blocks, 256, 0, stream, feat_dev, p->d_nout, p->F, values, args.error_flag);
+    launch_dependent(mini_finalize_kernel, value_blocks, 256, 0, stream, feat_dev, p->d_nout, p->F, values, flag);
     rocket::count_launch(2);
     const cudaError_t e = cudaGetLastError();
     if (prev != p->device) cudaSetDevice(prev);
