@@ -413,6 +413,7 @@ struct rocket_mini {
     std::vector<MiniBucket> buckets;
     std::vector<MiniTile> tiles;
     std::vector<int32_t> nout;             // outputs behind every feature
+    int64_t slices = 0;                    // slices of at most eight features of one combination
     int max_nch = 1;
     bool wide = false;                     // the combinations of some dilation use more than kMPlanes channels
     mutable std::mutex mu;
@@ -429,6 +430,8 @@ struct rocket_mini {
 static void build_tiles(rocket_mini& p) {
     p.recs.clear(); p.buckets.clear(); p.tiles.clear();
     p.nout.assign(p.F, 1);
+    p.slices = 0;
+    for (int c = 0; c < p.n_combos; ++c) p.slices += (p.feature_offset[c + 1] - p.feature_offset[c] + 7) / 8;
     p.max_nch = 1;
     std::map<int, std::vector<int>> by_d;
     for (int c = 0; c < p.n_combos; ++c)
@@ -492,6 +495,12 @@ static void build_tiles(rocket_mini& p) {
         }
     }
 }
+
+// Examples of one launch of the tile kernel: (tile, example) pairs, eight parts of each, are counted in 32 bits.
+#ifndef ROCKET_MINI_LAUNCH_TILES
+#define ROCKET_MINI_LAUNCH_TILES (0x7fffffffll / 8)
+#endif
+static int mini_launch_examples(long long n_tiles) { return (int)std::max<long long>(1, std::min<long long>(0x7fffffff, ROCKET_MINI_LAUNCH_TILES / n_tiles)); }
 
 static constexpr size_t kMiniSmemBytes = (size_t)2 * kMPlanes * kMPlaneBytes;
 
@@ -703,7 +712,7 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     if (!p->fitted) return ROCKET_EINVAL;
     if (N == 0) return ROCKET_OK;
     if (!X_dev || !feat_dev) return ROCKET_EINVAL;
-    if ((long long)N * (long long)p->tiles.size() > 0x7fffffffll / 8) return ROCKET_EUNSUPPORTED;
+    if (N * p->slices > 0x7fffffffll) return ROCKET_EUNSUPPORTED;
     const int st = ensure_mini_device(p);
     if (st != ROCKET_OK) return st;
     int prev = -1;
@@ -713,30 +722,34 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
     sms = std::max(sms, 1);
-    MiniArgs args = p->dev;
-    args.X = X_dev;
-    args.counts = reinterpret_cast<int*>(feat_dev);
-    args.N = N;
     MiniFlag* flag = p->flags + p->calls.fetch_add(1, std::memory_order_relaxed) % kMFlags;
-    args.failed = &flag->failed;
-    // Examples that share a tile: as many as its planes hold, while every SM still gets four tiles; fewer tiles than SMs are
-    // dealt in parts of their combinations (84 or so) instead.
-    const long long tiles = (long long)N * args.n_tiles;
-    args.examples = (int)std::max<long long>(1, std::min<long long>({(p->wide ? kMPlanesWide : kMPlanes) / p->max_nch, N, tiles / (4ll * sms)}));
-    args.groups = (N + args.examples - 1) / args.examples;
-    const long long items = (long long)args.groups * args.n_tiles;
-    args.parts = (int)std::max<long long>(1, std::min<long long>(8, 2ll * sms / items));
-    const unsigned grid = (unsigned)std::min<long long>(items * args.parts, sms);
     const long long values = (long long)N * p->F;
     const unsigned value_blocks = (unsigned)((values + 255) / 256);
     cudaMemsetAsync(feat_dev, 0, (size_t)values * sizeof(float), stream);
-    // A block that has one tile only has nothing to overlap its copies with: all warps make them (1 x 20 x 300, 840 features:
-    // 16.4 us with three warps, 14.4 so), into no more shared memory than the tile takes (1 x 12 x 900: 16.4 -> 14.4 us).
-    const bool all_copy = p->wide || items * args.parts <= grid;
-    if (all_copy) mini_tile_kernel<true><<<grid, kMThreads, (size_t)args.examples * p->max_nch * kMPlaneBytes, stream>>>(args);
-    else mini_tile_kernel<false><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
+    const int most = mini_launch_examples(p->dev.n_tiles);
+    for (int n0 = 0; n0 < N; n0 += std::min(most, N - n0)) {
+        MiniArgs args = p->dev;
+        args.X = X_dev + (size_t)n0 * C * L;
+        args.counts = reinterpret_cast<int*>(feat_dev) + (size_t)n0 * p->F;
+        args.N = std::min(most, N - n0);
+        args.failed = &flag->failed;
+        // Examples that share a tile: as many as its planes hold, while every SM still gets four tiles; fewer tiles than SMs are
+        // dealt in parts of their combinations (84 or so) instead.
+        const long long tiles = (long long)args.N * args.n_tiles;
+        args.examples = (int)std::max<long long>(1, std::min<long long>({(p->wide ? kMPlanesWide : kMPlanes) / p->max_nch, args.N, tiles / (4ll * sms)}));
+        args.groups = (args.N + args.examples - 1) / args.examples;
+        const long long items = (long long)args.groups * args.n_tiles;
+        args.parts = (int)std::max<long long>(1, std::min<long long>(8, 2ll * sms / items));
+        const unsigned grid = (unsigned)std::min<long long>(items * args.parts, sms);
+        // A block that has one tile only has nothing to overlap its copies with: all warps make them (1 x 20 x 300, 840 features:
+        // 16.4 us with three warps, 14.4 so), into no more shared memory than the tile takes (1 x 12 x 900: 16.4 -> 14.4 us).
+        const bool all_copy = p->wide || items * args.parts <= grid;
+        if (all_copy) mini_tile_kernel<true><<<grid, kMThreads, (size_t)args.examples * p->max_nch * kMPlaneBytes, stream>>>(args);
+        else mini_tile_kernel<false><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
+        rocket::count_launch();
+    }
     launch_dependent(mini_finalize_kernel, value_blocks, 256, 0, stream, feat_dev, p->d_nout, p->F, values, flag);
-    rocket::count_launch(2);
+    rocket::count_launch();
     const cudaError_t e = cudaGetLastError();
     if (prev != p->device) cudaSetDevice(prev);
     if (e != cudaSuccess) { cudaGetLastError(); return ROCKET_ECUDA; }

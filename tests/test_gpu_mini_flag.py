@@ -22,3 +22,10 @@ def _run(tmp_path, name, *defines):
 
 def test_a_failed_wait_marks_its_own_call_only(tmp_path):
     _run(tmp_path, "whole")
+
+
+def test_a_batch_in_several_launches_gives_the_same_bits(tmp_path):
+    # 50 examples, 7 and 1 per launch
+    whole = _run(tmp_path, "whole")
+    assert _run(tmp_path, "seven", "-DROCKET_MINI_LAUNCH_TILES=(7 * n_tiles)") == whole
+    assert _run(tmp_path, "one", "-DROCKET_MINI_LAUNCH_TILES=1") == whole
