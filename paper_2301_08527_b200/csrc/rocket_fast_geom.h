@@ -34,6 +34,15 @@ ROCKET_HD void valid_rows_tc(int t_row0, int c, int tl, int rl, int th, int rh, 
     if (!col_ok) o_hi = 0;
 }
 
+// Rows t0 .. t0 + rows - 1 of column r of A that hold samples of a series of th * d + rh (the first of them at or above -rows):
+// [lo, hi), counted from t0.  No step leaves 32 bits, however long the series.
+ROCKET_HD void rows_in_series(int t0, int r, int th, int rh, int rows, int& lo, int& hi) {
+    const int end = th + (r < rh ? 1 : 0);
+    lo = t0 >= 0 ? 0 : imin(-t0, rows);
+    const unsigned left = end > t0 ? (unsigned)end - (unsigned)t0 : 0u;
+    hi = left < (unsigned)rows ? (int)left : rows;
+}
+
 // S regime: the u of the first output row of raster column cg of a bucket.
 ROCKET_HD int s_column_u0(const SBucket& b, int cg) {
     const int band = cg / b.d, r = cg - band * b.d;

@@ -99,23 +99,26 @@ __device__ __forceinline__ float load_if(const float* p, unsigned ok) {
     return v;
 }
 
-// The columns lane and lane + 32 of a tile: their first position, and the input rows that lie in the series.
+// The columns lane and lane + 32 of a tile: their first position (64 bits: columns that do not exist lie anywhere), and the input
+// rows that lie in the series.
 struct FillAt {
-    int d, u0, u1;
-    unsigned in0 = 0, in1 = 0;
+    int d;
+    long long u0, u1;
+    unsigned in0, in1;
     bool inside;
     __device__ __forceinline__ FillAt(int d_, int raster_len, int c0, int L, int lane) : d(d_) {
         const int cg0 = c0 + lane, cg1 = cg0 + 32, band0 = (int)((unsigned)cg0 / (unsigned)d), band1 = (int)((unsigned)cg1 / (unsigned)d);
-        u0 = (band0 * kMRows - 4) * d + (cg0 - band0 * d);
-        u1 = (band1 * kMRows - 4) * d + (cg1 - band1 * d);
-        inside = __all_sync(kFull, cg1 < raster_len && u0 >= 0 && u1 + (kMInRows - 1) * d < L);
-        if (!inside) {
-#pragma unroll 4
-            for (int s = 0; s < kMInRows; ++s) {
-                in0 |= (cg0 < raster_len && (unsigned)(u0 + s * d) < (unsigned)L ? 1u : 0u) << s;
-                in1 |= (cg1 < raster_len && (unsigned)(u1 + s * d) < (unsigned)L ? 1u : 0u) << s;
-            }
-        }
+        const int t0 = band0 * kMRows - 4, t1 = band1 * kMRows - 4, r0 = cg0 - band0 * d, r1 = cg1 - band1 * d;
+        const int th = (int)((unsigned)L / (unsigned)d), rh = L - th * d;
+        u0 = (long long)t0 * d + r0;
+        u1 = (long long)t1 * d + r1;
+        int lo, hi;
+        rows_in_series(t0, r0, th, rh, kMInRows, lo, hi);
+        in0 = cg0 < raster_len ? row_mask(lo, hi) : 0u;
+        rows_in_series(t1, r1, th, rh, kMInRows, lo, hi);
+        in1 = cg1 < raster_len ? row_mask(lo, hi) : 0u;
+        constexpr unsigned kAll = (1u << kMInRows) - 1u;
+        inside = __all_sync(kFull, (in0 & in1) == kAll);
     }
 };
 
@@ -468,7 +471,7 @@ static void build_tiles(rocket_mini& p) {
                 if (!g.has[S[q]]) { g.has[S[q]] = 1; ++g.nch; }
             g.combos.push_back(c);
         }
-        const int rows = (p.L + d - 1) / d, bands = (rows + kMRows - 1) / kMRows;
+        const int rows = (int)(((int64_t)p.L + d - 1) / d), bands = (rows + kMRows - 1) / kMRows;
         for (Group& g : groups) {
             MiniBucket b{};
             b.d = d; b.raster_len = bands * d;

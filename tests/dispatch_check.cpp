@@ -44,7 +44,28 @@ static void check_stream_items() {
                     }
 }
 
+// The rows of a column that lie in a series, for the longest series there are: positions beyond 2^31 must not wrap.
+static void check_rows_in_series() {
+    const int kRows = 22;
+    for (long long L : {9ll, 64ll, 50001ll, 700000000ll, 900000000ll, 1300000001ll, 2147483647ll})
+        for (long long d : {1ll, 2ll, 7ll, (L - 1) / 8, (L - 1) / 9, (L - 1) / 13}) {
+            if (d < 1) continue;
+            const long long rows = (L + d - 1) / d;
+            for (long long t0 : {-4ll, -3ll, 0ll, 10ll, rows - 30, rows - 22, rows - 21, rows - 9, rows - 1, rows + 5})
+                for (long long r : {0ll, 1ll, d / 2, d - 1}) {
+                    if (r >= d || t0 < -kRows || t0 > 0x7fffffffll) continue;
+                    int lo, hi;
+                    rows_in_series((int)t0, (int)r, (int)(L / d), (int)(L % d), kRows, lo, hi);
+                    for (int s = 0; s < kRows; ++s) {
+                        const long long u = (t0 + s) * d + r;
+                        REQUIRE((s >= lo && s < hi) == (u >= 0 && u < L), "L %lld d %lld row %lld + %d column %lld", L, d, t0, s, r);
+                    }
+                }
+        }
+}
+
 int main() {
+    check_rows_in_series();
     check_stream_items();
     if (failures == 0) std::printf("ok\n");
     return failures ? 1 : 0;
