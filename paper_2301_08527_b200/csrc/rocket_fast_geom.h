@@ -49,6 +49,12 @@ ROCKET_HD int s_column_u0(const SBucket& b, int cg) {
     return (b.tmin + band * kRS) * b.d + r;
 }
 
+// Stream regime: every one of the R rows x 64 columns from (row trow, column c0) is an output of a kernel of dilation d.  The last
+// row of a band may lie 16 d beyond the series, which takes more than 32 bits from 380 million samples on.
+ROCKET_HD bool tile_interior(int trow, int c0, int R, int d, int lo_u, int hi_u) {
+    return c0 + kWarpCols <= d && (long long)trow * d + c0 >= lo_u && (long long)(trow + R - 1) * d + c0 + kWarpCols - 1 < hi_u;
+}
+
 // T regime.  A tile starts at A-row t0 and residue r0 (a multiple of 64).  Row s of the tile
 // (A-row t0 + s) arrives with the box of phase s & 3, as that box's row s >> 2.  In the
 // zero-margined copy the element (A-row t, residue r) of a channel row sits at float

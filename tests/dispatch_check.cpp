@@ -64,7 +64,31 @@ static void check_rows_in_series() {
         }
 }
 
+// A tile of the stream kernel is interior exactly when the masks of its columns say so, at every length.
+static void check_tile_interior() {
+    for (long long nout : {1000ll, 100000ll, 400000000ll, 700000001ll, 1073741824ll})
+        for (long long d : {64ll, 65ll, 1000ll, nout / 7, nout / 6 + 1})
+            for (long long p : {0ll, 4 * d, 5 * d - 3})
+                for (int R : {8, 12, 16}) {
+                    if (d < 64) continue;
+                    const long long lo = -p, hi = nout - p, tl = lo >= 0 ? lo / d : -((-lo + d - 1) / d), th = hi / d;
+                    if (hi < 0) continue;
+                    for (long long t : {tl, tl + 1, 0ll, th - R - 1, th - R, th - R + 1, th - 1, th})
+                        for (long long c0 : {0ll, 64ll, (d - 1) / 64 * 64}) {
+                            bool all = true;
+                            for (int l = 0; l < 64; ++l) {
+                                int a, b;
+                                valid_rows_tc((int)t, (int)(c0 + l), (int)tl, (int)(lo - tl * d), (int)th, (int)(hi - th * d), R, c0 + l < d, a, b);
+                                all = all && a == 0 && b == R;
+                            }
+                            REQUIRE(tile_interior((int)t, (int)c0, R, (int)d, (int)lo, (int)hi) == all, "nout %lld d %lld p %lld R %d row %lld column %lld",
+                                    nout, d, p, R, t, c0);
+                        }
+                }
+}
+
 int main() {
+    check_tile_interior();
     check_rows_in_series();
     check_stream_items();
     if (failures == 0) std::printf("ok\n");
