@@ -35,6 +35,10 @@
  *     covers a call - after rocket_params_reserve for its size and passes, or after an earlier
  *     call at least as large - the device calls only enqueue kernels and return without
  *     allocating or synchronising.  rocket_device_alloc_count lets a caller verify that.
+ *     The staging copies take up to 800 MB, or four examples' (up to 4 GB; one example's beyond), and less where the
+ *     device has less: the batch then goes through in smaller parts, and where not even one example's copies fit,
+ *     the generic kernels, which need none, serve the call (rocket_transform_f16, which they do not serve, returns
+ *     ROCKET_ENOMEM).  rocket_params_reserve asks for the full size again.
  *   - Every function returns a rocket_status_t (0 = success).  Argument errors are detected
  *     on the host before anything is launched and leave the outputs untouched.  Nothing
  *     aborts and nothing throws across this boundary.  There is no CPU fallback: without a

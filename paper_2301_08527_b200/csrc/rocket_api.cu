@@ -138,6 +138,13 @@ int cuda_status(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? ROCKET_ENOMEM : ROCKET_ECUDA;
 }
 
+// Whether the fused kernels launched nothing for want of room for their copies: the generic kernels, which need none, serve the call.
+bool no_room(cudaError_t e) {
+    if (e != cudaErrorMemoryAllocation) return false;
+    cudaGetLastError();
+    return true;
+}
+
 // Makes the handle's device current for the duration of a call.
 struct DeviceGuard {
     int prev = -1;
@@ -356,13 +363,15 @@ int rocket_params_reserve(rocket_params_t* p, int max_N, int passes) {
     const bool soft = (passes & ROCKET_PASS_SOFT) != 0, backward = (passes & ROCKET_PASS_BACKWARD) != 0;
     const bool u8 = (passes & ROCKET_PASS_U8_INPUT) != 0;
     const int64_t nW = n_weights_of(p);
-    if (p->fast->host.enabled) {
+    bool fused = p->fast->host.enabled;
+    if (fused) {
         cudaError_t e = fast::reserve_fast_state(*p->fast, p->dp, max_N, soft, backward, u8, nW);
-        if (e != cudaSuccess) return cuda_status(e);
+        if (no_room(e)) fused = false;
+        else if (e != cudaSuccess) return cuda_status(e);
     }
     std::lock_guard<std::mutex> lk(p->mu);
     // kernels outside the fused path: the backward's per-example partial sums; 8-bit input: its fp32 copy
-    const bool some_generic = !p->fast->host.enabled || !p->fast->host.generic_list.empty() || p->path == 1;
+    const bool some_generic = !fused || !p->fast->host.generic_list.empty() || p->path == 1;
     if (backward && some_generic) {
         cudaError_t e = p->scratch.reserve(generic_backward_scratch_floats(max_N, nW, p->host.K) * sizeof(float));
         if (e != cudaSuccess) return cuda_status(e);
@@ -388,10 +397,11 @@ int rocket_transform(const rocket_params_t* p, const float* X_dev, int N, int C,
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
     if (p->path == 0 && p->fast->host.enabled && aligned) {
         cudaError_t e = fast::launch_fast_forward(*p->fast, p->dp, X_dev, N, feat_dev, stream);
-        if (e != cudaSuccess) return cuda_status(e);
-        if (p->fast->dev.n_generic == 0) return ROCKET_OK;
-        return cuda_status(launch_generic_forward(p->dp, X_dev, N, false, 0.0f, 0.0f, feat_dev, nullptr, stream,
-                                                  p->fast->dev.generic_list, p->fast->dev.n_generic));
+        if (e != cudaSuccess && !no_room(e)) return cuda_status(e);
+        if (e == cudaSuccess && p->fast->dev.n_generic == 0) return ROCKET_OK;
+        if (e == cudaSuccess)
+            return cuda_status(launch_generic_forward(p->dp, X_dev, N, false, 0.0f, 0.0f, feat_dev, nullptr, stream,
+                                                      p->fast->dev.generic_list, p->fast->dev.n_generic));
     }
     return cuda_status(launch_generic_forward(p->dp, X_dev, N, false, 0.0f, 0.0f, feat_dev, nullptr, stream));
 }
@@ -426,10 +436,11 @@ int rocket_transform_soft(const rocket_params_t* p, const float* X_dev, int N, i
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
     if (p->path == 0 && p->fast->host.enabled && aligned) {
         cudaError_t e = fast::launch_fast_forward(*p->fast, p->dp, X_dev, N, feat_dev, stream, true, lambda, shift, argmax_dev);
-        if (e != cudaSuccess) return cuda_status(e);
-        if (p->fast->dev.n_generic == 0) return ROCKET_OK;
-        return cuda_status(launch_generic_forward(p->dp, X_dev, N, true, lambda, shift, feat_dev, argmax_dev, stream,
-                                                  p->fast->dev.generic_list, p->fast->dev.n_generic));
+        if (e != cudaSuccess && !no_room(e)) return cuda_status(e);
+        if (e == cudaSuccess && p->fast->dev.n_generic == 0) return ROCKET_OK;
+        if (e == cudaSuccess)
+            return cuda_status(launch_generic_forward(p->dp, X_dev, N, true, lambda, shift, feat_dev, argmax_dev, stream,
+                                                      p->fast->dev.generic_list, p->fast->dev.n_generic));
     }
     return cuda_status(launch_generic_forward(p->dp, X_dev, N, true, lambda, shift, feat_dev, argmax_dev, stream));
 }
@@ -458,8 +469,9 @@ static int transform_u8(const rocket_params_t* p, const uint8_t* X_u8_dev, int N
             norm.mean[c] = c < C ? mean[c] : 0.0f;
             norm.inv_std[c] = c < C ? inv_std[c] : 0.0f;
         }
-        return cuda_status(fast::launch_fast_forward(*p->fast, p->dp, nullptr, N, feat_dev, stream, soft, lambda, shift,
-                                                     argmax_dev, X_u8_dev, &norm));
+        const cudaError_t e = fast::launch_fast_forward(*p->fast, p->dp, nullptr, N, feat_dev, stream, soft, lambda, shift,
+                                                        argmax_dev, X_u8_dev, &norm);
+        if (!no_room(e)) return cuda_status(e);
     }
     // otherwise: a scaled fp32 copy of the batch in a buffer of the handle, then the fp32 route
     const float* Xf = nullptr;
@@ -507,14 +519,15 @@ int rocket_transform_soft_backward(const rocket_params_t* p, const float* X_dev,
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const int64_t nW = n_weights_of(p);
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
-    const bool use_fast = p->path == 0 && p->fast->host.enabled && (aligned || N == 0);
-    const int n_generic = use_fast ? (int)p->fast->host.generic_list.size() : p->host.K;
+    bool use_fast = p->path == 0 && p->fast->host.enabled && (aligned || N == 0);
     if (use_fast) {   // the fused kernels assign dW / db of the kernels they serve
         cudaError_t e = fast::launch_fast_backward(*p->fast, p->dp, nW, X_dev, N, lambda, shift, dfeat_dev, argmax_dev,
                                                    dW_dev, db_dev, stream);
-        if (e != cudaSuccess) return cuda_status(e);
-        if (n_generic == 0) return ROCKET_OK;
+        if (no_room(e)) use_fast = false;
+        else if (e != cudaSuccess) return cuda_status(e);
     }
+    const int n_generic = use_fast ? (int)p->fast->host.generic_list.size() : p->host.K;
+    if (use_fast && n_generic == 0) return ROCKET_OK;
     float* scratch = nullptr;
     if (N > 0) {
         std::lock_guard<std::mutex> lk(p->mu);

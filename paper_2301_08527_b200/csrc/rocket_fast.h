@@ -190,7 +190,9 @@ constexpr int kWStageFloats = (kWRows + ROCKET_MAX_LENGTH - 1 + 3) / 4 * 4 * kWa
 constexpr int kWCopies = 7;                                        // shifted copies of every channel row, next to one another
 constexpr int kWUnitVisits = 16, kWItemVisits = 32;                // visits of a unit, and of a unit for a group of examples
 constexpr int kWSoftSetItems = 24;                                 // items per warp of a set, soft and backward
-constexpr int64_t kWCopyBytes = 800ll << 20;                       // what the copies of a pass may take (13 examples of 20 x 50,000)
+// What the copies of a pass take: 800 MB (13 examples of 20 x 50,000), or four examples where those take no more than 4 GB.
+constexpr int64_t kWCopyBytes = 800ll << 20, kWMostCopyBytes = 4ll << 30;
+constexpr int kWFewExamples = 4;
 
 // A unit of work: consecutive tiles of one kernel (32 words).  The kernel's output rows from t0 on are cut into bands of R rows,
 // a band into ncol tiles of 64 columns; tile number band * ncol + column group.
@@ -205,6 +207,15 @@ struct alignas(16) WUnit {
     int32_t bytes, pad_[4];               // bytes of a visit's copy
 };
 static_assert(sizeof(WUnit) == 128, "WUnit must be 32 words");
+// Examples of a pass of the stream regime for rows of `pitch` floats.
+int stream_chunk(int C, int64_t pitch);
+// Capacity for `want` examples, or as many as there is room for: alloc(n) makes room for n examples.  0 when there is none for one.
+template <class Alloc>
+int fit_examples(int want, Alloc&& alloc) {
+    for (int n = want; n >= 1; n /= 2)
+        if (alloc(n)) return n;
+    return 0;
+}
 // How a pass of N examples is handed out to the warps of the stream kernel (mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half
 // precision): an item is a unit for `examples` examples, the items of `groups_per_set` such groups go through all units together.
 struct StreamItems { int examples, groups, groups_per_set; };
@@ -272,6 +283,7 @@ struct FastState {
     void* maps_blob = nullptr;            // tensor maps
     float* xpad = nullptr;                // the four shifted zero-margined copies, capacity pad_examples
     int pad_examples = 0;
+    int most_examples = 1 << 30;          // of either kind of copies: fewer than wanted once there was no room for more (until the next reserve)
     int64_t copy_floats = 0;              // floats of one copy
     float* wpad = nullptr;                // stream regime: the seven shifted copies, capacity wpad_examples
     int wpad_examples = 0;
@@ -290,7 +302,8 @@ cudaError_t upload_plan(FastState& fs);
 void release_fast_state(FastState& fs);
 // The same for the stream regime's copies.
 cudaError_t ensure_stream_capacity(FastState& fs, int N, int C, int L);
-// Makes the padded copy hold N examples and (re-)encodes the tensor maps over it.
+// Makes the padded copy hold N examples, or as many as there is room for (at least one, or cudaErrorMemoryAllocation), and
+// (re-)encodes the tensor maps over it.
 cudaError_t ensure_pad_capacity(FastState& fs, int N, int C, int L, bool without_maps = false);
 
 // Allocates, once, everything the fused kernels need for calls of up to max_N examples (the zero-margined
@@ -305,6 +318,8 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
                                  float lambda, float shift, const float* dfeat, const int32_t* argmax, float* dW,
                                  float* db, cudaStream_t stream);
 
+// The launches below return cudaErrorMemoryAllocation, having launched nothing, when there is no room for the copies of one example.
+//
 // Forward through the fast path: init, pad copy, S kernel, T kernel, finalise.  soft = false:
 // PPV + max; soft = true: softPPV + max (+ argmax when argmax != nullptr).
 // With X_u8 (raw 8-bit intensities [N][C][L], 4-byte aligned) the samples are normalised per channel

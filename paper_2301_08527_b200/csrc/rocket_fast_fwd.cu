@@ -926,7 +926,7 @@ __global__ void fast_bwd_finalize_kernel(const long long* __restrict__ accfix, c
 // or near what 12 examples of that size take in the four-copy form; passes of few short series would end in launches with
 // nothing to do for most SMs.  Without copies one pass does.
 static int chunk_examples(const FastState& fs, int C, bool stream, bool copies) {
-    if (stream) return (int)std::min<int64_t>(1 << 16, std::max<int64_t>(4, kWCopyBytes / (4 * kWCopies * (int64_t)C * fs.host.wpitch)));
+    if (stream) return stream_chunk(C, fs.host.wpitch);
     if (!copies) return 1 << 16;
     return (int)std::max<int64_t>(kChunkExamples, 80000000ll / (4 * (int64_t)C * fs.host.pad_pitch));
 }
@@ -1033,19 +1033,38 @@ void release_fast_state(FastState& fs) {
     fs.pad_examples = fs.wpad_examples = 0;
 }
 
+// Room for the copies of N examples in place of what *buf holds; N comes back smaller when there is room for fewer, which later
+// calls then ask for (a failed allocation of this size takes milliseconds).
+template <class Bytes>
+static cudaError_t allocate_copies(FastState& fs, float** buf, int& held, int& N, Bytes&& bytes_of) {
+    if (*buf) cudaFree(*buf);  // waits for work that still reads it
+    *buf = nullptr;
+    held = 0;
+    cudaError_t e = cudaSuccess;
+    const int got = fit_examples(N, [&](int n) {
+        e = device_malloc(reinterpret_cast<void**>(buf), bytes_of(n));
+        if (e != cudaSuccess) *buf = nullptr;
+        return e != cudaErrorMemoryAllocation;
+    });
+    if (got < N) fs.most_examples = got;
+    if (got > 0 && e == cudaSuccess && got < N) cudaGetLastError();   // of the larger sizes
+    N = got;
+    return e;
+}
+
 cudaError_t ensure_stream_capacity(FastState& fs, int N, int C, int L) {
+    N = std::min(N, fs.most_examples);
+    if (N == 0) return cudaErrorMemoryAllocation;
     if (N <= fs.wpad_examples) return cudaSuccess;
     EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return cudaErrorNotSupported;
-    const int64_t pitch = fs.host.wpitch, front = fs.host.wfront, copies = (int64_t)N * C * kWCopies;
-    const size_t bytes = (size_t)(copies * pitch + front + pitch) * sizeof(float);   // a box may run past the last copy
-    if (fs.wpad) cudaFree(fs.wpad);  // waits for work that still reads it
-    fs.wpad = nullptr;
-    fs.wpad_examples = 0;
-    cudaError_t e = device_malloc(reinterpret_cast<void**>(&fs.wpad), bytes);
-    if (e != cudaSuccess) { fs.wpad = nullptr; return e; }
-    e = cudaMemset(fs.wpad, 0, bytes);  // the margins stay zero from here on
+    const int64_t pitch = fs.host.wpitch, front = fs.host.wfront;
+    auto bytes_of = [&](int n) { return (size_t)((int64_t)n * C * kWCopies * pitch + front + pitch) * sizeof(float); };   // a box may run past the last copy
+    cudaError_t e = allocate_copies(fs, &fs.wpad, fs.wpad_examples, N, bytes_of);
     if (e != cudaSuccess) return e;
+    e = cudaMemset(fs.wpad, 0, bytes_of(N));  // the margins stay zero from here on
+    if (e != cudaSuccess) return e;
+    const int64_t copies = (int64_t)N * C * kWCopies;
     const size_t n_maps = fs.host.wmaps.size();
     std::vector<CUtensorMap> maps(n_maps);
     for (size_t i = 0; i < n_maps; ++i) {
@@ -1085,18 +1104,18 @@ static void launch_stream_copy(FastState& fs, const float* X, int64_t rows, int 
 }
 
 cudaError_t ensure_pad_capacity(FastState& fs, int N, int C, int L, bool without_maps) {
-    if ((fs.host.tmaps.empty() && !without_maps) || N <= fs.pad_examples) return cudaSuccess;
+    if (fs.host.tmaps.empty() && !without_maps) return cudaSuccess;
+    N = std::min(N, fs.most_examples);
+    if (N == 0) return cudaErrorMemoryAllocation;
+    if (N <= fs.pad_examples) return cudaSuccess;
     EncodeTiledFn encode = fs.host.tmaps.empty() ? nullptr : encode_tiled_fn();
     if (!encode && !fs.host.tmaps.empty()) return cudaErrorNotSupported;
-    const int64_t pitch = fs.host.pad_pitch, rows = (int64_t)N * C;
-    const int64_t copy_floats = (rows + 1) * pitch;   // pitch is a multiple of 32 floats
-    const size_t bytes = (size_t)copy_floats * 4 * 4;
-    if (fs.xpad) cudaFree(fs.xpad);  // waits for work that still reads it
-    fs.xpad = nullptr;
-    fs.pad_examples = 0;
-    cudaError_t e = device_malloc(reinterpret_cast<void**>(&fs.xpad), bytes);
-    if (e != cudaSuccess) { fs.xpad = nullptr; return e; }
-    e = cudaMemset(fs.xpad, 0, bytes);  // the margins stay zero from here on: the pad copy writes samples only
+    const int64_t pitch = fs.host.pad_pitch;          // a multiple of 32 floats
+    auto bytes_of = [&](int n) { return (size_t)((int64_t)n * C + 1) * pitch * 4 * 4; };
+    cudaError_t e = allocate_copies(fs, &fs.xpad, fs.pad_examples, N, bytes_of);
+    if (e != cudaSuccess) return e;
+    const int64_t rows = (int64_t)N * C, copy_floats = (rows + 1) * pitch;
+    e = cudaMemset(fs.xpad, 0, bytes_of(N));  // the margins stay zero from here on: the pad copy writes samples only
     if (e != cudaSuccess) return e;
     const size_t n_maps = fs.host.tmaps.size();
     std::vector<CUtensorMap> maps(n_maps);
@@ -1166,6 +1185,7 @@ cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N,
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = set_kernel_attributes(dev)) != cudaSuccess) return e;
+    fs.most_examples = 1 << 30;           // asked again
     const bool stream = fs.dev.n_wunits > 0, copies = fs.dev.n_titems > 0 || u8;
     const int chunk = std::min(max_N, chunk_examples(fs, dp.C, stream, copies));
     if (stream && (e = ensure_stream_capacity(fs, chunk, dp.C, dp.L)) != cudaSuccess) return e;
@@ -1192,10 +1212,11 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     const PlanDevice& pd = fs.dev;
     // the stream kernel takes the dilations the S kernel leaves; the T kernel where the stream kernel's copies have no room
     const bool streamed = pd.n_wunits > 0, copied = pd.n_titems > 0 || X_u8;
-    const int chunk = chunk_examples(fs, dp.C, streamed, copied);
+    int chunk = chunk_examples(fs, dp.C, streamed, copied);
     if (streamed) e = ensure_stream_capacity(fs, std::min(N, chunk), dp.C, dp.L);
     else if (copied) e = ensure_pad_capacity(fs, std::min(N, chunk), dp.C, dp.L, X_u8 != nullptr);
     if (e != cudaSuccess) return e;
+    if (streamed || copied) chunk = std::min(chunk, fs.most_examples);
     const int64_t pairs = (int64_t)N * dp.K;
     if (soft && (e = ensure_soft_ws(fs, pairs)) != cudaSuccess) return e;
     FwdArgs a;
@@ -1297,11 +1318,12 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     double* scale = reinterpret_cast<double*>(static_cast<char*>(fs.bwd_ws) + acc_bytes);
     unsigned* absmax = reinterpret_cast<unsigned*>(static_cast<char*>(fs.bwd_ws) + acc_bytes + scale_bytes);
     const bool streamed = pd.n_wunits > 0, copied = pd.n_titems > 0;
-    const int chunk = chunk_examples(fs, dp.C, streamed, copied);
+    int chunk = chunk_examples(fs, dp.C, streamed, copied);
     if (N > 0) {
         if (streamed) e = ensure_stream_capacity(fs, std::min(N, chunk), dp.C, dp.L);
         else if (copied) e = ensure_pad_capacity(fs, std::min(N, chunk), dp.C, dp.L);
         if (e != cudaSuccess) return e;
+        if (streamed || copied) chunk = std::min(chunk, fs.most_examples);
     }
     e = cudaMemsetAsync(absmax, 0, 256, stream);
     if (e != cudaSuccess) return e;

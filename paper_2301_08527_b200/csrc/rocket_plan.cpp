@@ -102,6 +102,12 @@ void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost&
 
 }  // namespace
 
+int stream_chunk(int C, int64_t pitch) {
+    const int64_t example = 4 * kWCopies * (int64_t)C * pitch;
+    const int64_t few = std::max<int64_t>(1, std::min<int64_t>(kWFewExamples, kWMostCopyBytes / example));
+    return (int)std::min<int64_t>(1 << 16, std::max<int64_t>(few, kWCopyBytes / example));
+}
+
 // Examples of an item: as many as give it kWItemVisits visits on average, while every warp of the chip still gets a dozen items and
 // their copies take no more than half of the L2: two examples of 20 x 200,000 do not, and 60 of them took 245 ms two at a time, 218
 // one at a time (10,000 kernels; 20 x 100,000: 106 and 103 ms; 20 x 50,000, where two fit: 50.7 and 51.6).

@@ -1,4 +1,5 @@
 // Host-side checks of the rules by which a call is handed out to the kernels (no GPU needed).
+#include <algorithm>
 #include <cstdio>
 
 #include "rocket_fast.h"
@@ -87,7 +88,25 @@ static void check_tile_interior() {
                 }
 }
 
+// The copies of a pass stay within their budget, whatever the channels and the length, and shrink to what there is room for.
+static void check_copies() {
+    for (int C : {1, 3, 20, 32, 255})
+        for (int64_t pitch : {1000ll, 110000ll, 440000ll, 2200000ll, 220000000ll}) {
+            const int n = stream_chunk(C, pitch);
+            const int64_t example = 4 * kWCopies * (int64_t)C * pitch;
+            REQUIRE(n >= 1 && (n == 1 || n * example <= std::max<int64_t>(kWCopyBytes, kWMostCopyBytes)), "%d examples of %lld", n, (long long)example);
+            REQUIRE(n <= kWFewExamples || n * example <= kWCopyBytes, "%d examples of %lld", n, (long long)example);
+        }
+    REQUIRE(stream_chunk(20, 108416) == 13 && stream_chunk(20, 433440) == 4, "the benchmark's lengths");
+    for (int room : {0, 1, 2, 5, 12, 13, 40}) {
+        int tries = 0;
+        const int got = fit_examples(13, [&](int n) { ++tries; return n <= room; });
+        REQUIRE(got <= room && (got > 0) == (room > 0) && (room < 13 || got == 13) && tries <= 4 && (room < 1 || got > room / 4), "%d of %d", got, room);
+    }
+}
+
 int main() {
+    check_copies();
     check_tile_interior();
     check_rows_in_series();
     check_stream_items();
