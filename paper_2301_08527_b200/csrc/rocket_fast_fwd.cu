@@ -952,17 +952,22 @@ static unsigned set_s_groups(FwdArgs& a, const FastState& fs, int sms) {
 }
 
 // The S tiles of a pass (mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half precision, whose series are never wide).
-static void launch_s(FwdArgs& a, const FastState& fs, int mode, int sms, cudaStream_t stream) {
+// after_kernel: what comes before it in the stream is a kernel of this call (a programmatic launch depends on nothing else).
+static void launch_s(FwdArgs& a, const FastState& fs, int mode, int sms, bool after_kernel, cudaStream_t stream) {
     const unsigned grid = set_s_groups(a, fs, sms);
     const bool wide = fs.host.s_wide;
     const size_t bytes = s_smem_bytes(wide);
-    if (mode == 3) launch_dependent(fast_s_forward<3>, grid, kSThreads, bytes, stream, a);
-    else if (mode == 0 && wide) launch_dependent(fast_s_forward<0, true>, grid, kSThreads, bytes, stream, a);
-    else if (mode == 0) launch_dependent(fast_s_forward<0>, grid, kSThreads, bytes, stream, a);
-    else if (mode == 1 && wide) launch_dependent(fast_s_forward<1, true>, grid, kSThreads, bytes, stream, a);
-    else if (mode == 1) launch_dependent(fast_s_forward<1>, grid, kSThreads, bytes, stream, a);
-    else if (wide) launch_dependent(fast_s_forward<2, true>, grid, kSThreads, bytes, stream, a);
-    else launch_dependent(fast_s_forward<2>, grid, kSThreads, bytes, stream, a);
+    auto launch = [&](auto kernel) {
+        if (after_kernel) launch_dependent(kernel, grid, kSThreads, bytes, stream, a);
+        else kernel<<<grid, kSThreads, bytes, stream>>>(a);
+    };
+    if (mode == 3) launch(fast_s_forward<3>);
+    else if (mode == 0 && wide) launch(fast_s_forward<0, true>);
+    else if (mode == 0) launch(fast_s_forward<0>);
+    else if (mode == 1 && wide) launch(fast_s_forward<1, true>);
+    else if (mode == 1) launch(fast_s_forward<1>);
+    else if (wide) launch(fast_s_forward<2, true>);
+    else launch(fast_s_forward<2>);
     count_launch();
 }
 
@@ -1271,7 +1276,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
             launch_pad_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
         }
         if (fs.profile) cudaEventRecord(fs.evs[3 * c], stream);
-        if (pd.n_sitems > 0) launch_s(a, fs, soft ? 1 : half ? 3 : 0, sms, stream);
+        if (pd.n_sitems > 0) launch_s(a, fs, soft ? 1 : half ? 3 : 0, sms, c == 0 || streamed || copied, stream);
         if (fs.profile) cudaEventRecord(fs.evs[3 * c + 1], stream);
         if (streamed) {
             launch_stream(a, soft ? 1 : half ? 3 : 0, sms, l2, pd.n_sitems > 0, stream);
@@ -1335,8 +1340,12 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         else fast_absmax_scalar_kernel<<<blocks(n_x), 256, 0, stream>>>(X, n_x, absmax);
         count_launch();
     }
-    launch_dependent(fast_bwd_prepare_kernel, (pd.n_krec + 7) / 8, 256, 0, stream, dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale, accfix,
-                                                                     n_weights, pd.counters);
+    if (n_x > 0)
+        launch_dependent(fast_bwd_prepare_kernel, (pd.n_krec + 7) / 8, 256, 0, stream, dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale,
+                         accfix, n_weights, pd.counters);
+    else
+        fast_bwd_prepare_kernel<<<(pd.n_krec + 7) / 8, 256, 0, stream>>>(dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale, accfix,
+                                                                         n_weights, pd.counters);
     count_launch();
     FwdArgs a;
     a.plan = fs.dev; a.feat_i = nullptr; a.ws = nullptr;
@@ -1353,7 +1362,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         if (n0 > 0 && (e = cudaMemsetAsync(pd.counters, 0, 8, stream)) != cudaSuccess) return e;
         if (streamed) launch_stream_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, n0 == 0, stream);
         else if (copied) launch_pad_copy(fs, a.X, (int64_t)nc * dp.C, dp.L, sms, stream);
-        if (pd.n_sitems > 0) launch_s(a, fs, 2, sms, stream);
+        if (pd.n_sitems > 0) launch_s(a, fs, 2, sms, n0 == 0 || streamed || copied, stream);
         if (streamed) {
             launch_stream(a, 2, sms, l2, pd.n_sitems > 0, stream);
         } else if (pd.n_titems > 0) {

@@ -19,7 +19,7 @@ def _handle(C, L, small, large):
     for i in range(small + large):
         ln = (7, 9, 11)[i % 3]
         d = 1 if i < small else 130 + i
-        m = 4 if i < small else 1
+        m = min(C, 4) if i < small else 1
         ks.append(dict(dilation=d, padding=(ln - 1) * d // 2 if i % 2 else 0, channels=sorted(rng.choice(C, m, replace=False).tolist()),
                        weights=rng.normal(size=(m, ln)), bias=float(rng.uniform(-1, 1))))
     return rk.RocketParams.from_kernel_params(kernels_from_lists(C, L, ks))
@@ -60,4 +60,26 @@ def test_captured_calls_give_the_bits_of_plain_calls(small, large):
         for name, t in want.items():
             assert torch.equal(t, got[name]), name
     assert p.device_status() == 0
+    p.close()
+
+
+def test_captured_backward_of_an_empty_batch():
+    # no kernel of the call before the one that clears the sums
+    import torch
+    p = _handle(2, 501, 6, 2)
+    p.reserve(1, rk.PASS_SOFT | rk.PASS_BACKWARD)
+    X, g = torch.empty((0, 2, 501), device="cuda"), torch.empty((0, 16), device="cuda")
+    arg = torch.empty((0, 8), dtype=torch.int32, device="cuda")
+    dW, db = torch.full((p.n_weights,), -7.0, device="cuda"), torch.full((8,), -7.0, device="cuda")
+    rk.rocket_transform_soft_backward(p, X, 10.0, 3.0, g, arg, dW, db)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        rk.rocket_transform_soft_backward(p, X, 10.0, 3.0, g, arg, dW, db)
+    for _ in range(2):
+        dW.fill_(-7)
+        db.fill_(-7)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert not dW.any() and not db.any()
     p.close()
