@@ -248,6 +248,11 @@ struct PlanHost {
     double flops_s = 0.0, flops_t = 0.0;  // conv flop of one example in either regime
 };
 
+// How the S kernel's tiles are shared among the examples of a pass: tiles [end[i - 1], end[i]) for examples[i] examples together, as
+// groups[i] groups; grid: its blocks.
+struct SGroups { int end[3], examples[3], groups[3]; unsigned grid; };
+SGroups s_groups(const PlanHost& plan, int N, int sms);
+
 struct PlanDevice {
     const KRec* krec = nullptr;
     const SBucket* sb = nullptr;

@@ -931,30 +931,16 @@ static int chunk_examples(const FastState& fs, int C, bool stream, bool copies) 
     return (int)std::max<int64_t>(kChunkExamples, 80000000ll / (4 * (int64_t)C * fs.host.pad_pitch));
 }
 
-// How the S kernel's tiles are shared among examples: one example where a bucket has many kernels, up to 4 and up to 16
-// where it has some or few (64 to 256 pairs per tile for its 16 warps), as far as the planes hold them and the launch keeps two
-// tiles per SM.  Returns the grid.
-static unsigned set_s_groups(FwdArgs& a, const FastState& fs, int sms) {
-    const int fit = (fs.host.s_wide ? kSWidePlanes : kSMaxPlanes) / std::max(1, fs.host.s_max_nch);
-    unsigned long long tiles = 0;
-    for (int shift = 0; shift < 5; ++shift) {
-        tiles = 0;
-        for (int cls = 0; cls < 3; ++cls) {
-            const int most = cls == 0 ? 1 : cls == 1 ? 4 : 16;
-            a.s_end[cls] = fs.host.s_class_end[cls];
-            a.s_examples[cls] = std::max(1, std::min({fit, most, a.N}) >> shift);
-            a.s_groups[cls] = (a.N + a.s_examples[cls] - 1) / a.s_examples[cls];
-            tiles += (unsigned long long)(a.s_end[cls] - (cls ? a.s_end[cls - 1] : 0)) * a.s_groups[cls] * (fs.host.s_wide ? 2 : 1);
-        }
-        if (tiles >= 2ull * sms || a.s_examples[2] == 1) break;
-    }
-    return (unsigned)std::min<unsigned long long>(tiles, (unsigned long long)sms);
-}
-
 // The S tiles of a pass (mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half precision, whose series are never wide).
 // after_kernel: what comes before it in the stream is a kernel of this call (a programmatic launch depends on nothing else).
 static void launch_s(FwdArgs& a, const FastState& fs, int mode, int sms, bool after_kernel, cudaStream_t stream) {
-    const unsigned grid = set_s_groups(a, fs, sms);
+    const SGroups share = s_groups(fs.host, a.N, sms);
+    for (int cls = 0; cls < 3; ++cls) {
+        a.s_end[cls] = share.end[cls];
+        a.s_examples[cls] = share.examples[cls];
+        a.s_groups[cls] = share.groups[cls];
+    }
+    const unsigned grid = share.grid;
     const bool wide = fs.host.s_wide;
     const size_t bytes = s_smem_bytes(wide);
     auto launch = [&](auto kernel) {

@@ -102,6 +102,27 @@ void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost&
 
 }  // namespace
 
+// One example where a bucket has many kernels, up to 4 and up to 16 where it has some or few (64 to 256 pairs per tile for its 16
+// warps), as far as the planes hold them and the launch keeps two tiles per SM.
+SGroups s_groups(const PlanHost& plan, int N, int sms) {
+    const int fit = (plan.s_wide ? kSWidePlanes : kSMaxPlanes) / std::max(1, plan.s_max_nch);
+    SGroups a{};
+    unsigned long long tiles = 0;
+    for (int shift = 0; shift < 5; ++shift) {
+        tiles = 0;
+        for (int cls = 0; cls < 3; ++cls) {
+            const int most = cls == 0 ? 1 : cls == 1 ? 4 : 16;
+            a.end[cls] = plan.s_class_end[cls];
+            a.examples[cls] = std::max(1, std::min({fit, most, N}) >> shift);
+            a.groups[cls] = (N + a.examples[cls] - 1) / a.examples[cls];
+            tiles += (unsigned long long)(a.end[cls] - (cls ? a.end[cls - 1] : 0)) * a.groups[cls] * (plan.s_wide ? 2 : 1);
+        }
+        if (tiles >= 2ull * sms || a.examples[2] == 1) break;
+    }
+    a.grid = (unsigned)std::min<unsigned long long>(tiles, (unsigned long long)sms);
+    return a;
+}
+
 int stream_chunk(int C, int64_t pitch) {
     const int64_t example = 4 * kWCopies * (int64_t)C * pitch;
     const int64_t few = std::max<int64_t>(1, std::min<int64_t>(kWFewExamples, kWMostCopyBytes / example));

@@ -1,6 +1,7 @@
 // Host-side checks of the rules by which a call is handed out to the kernels (no GPU needed).
 #include <algorithm>
 #include <cstdio>
+#include <cstdlib>
 
 #include "rocket_fast.h"
 #include "rocket_fast_geom.h"
@@ -105,7 +106,33 @@ static void check_copies() {
     }
 }
 
-int main() {
+// Kernels from standard input (C, L, K, then per kernel length, dilation, padding and its channels): prints, for N examples, how many
+// examples the tiles of each class share and how many tiles there are of each.
+static int print_sharing(int N) {
+    HostParams hp;
+    if (std::scanf("%d %d %d", &hp.C, &hp.L, &hp.K) != 3) return 2;
+    hp.channel_offset.assign(1, 0);
+    hp.weight_offset.assign(1, 0);
+    for (int k = 0; k < hp.K; ++k) {
+        int len, d, p, m, c;
+        if (std::scanf("%d %d %d %d", &len, &d, &p, &m) != 4) return 2;
+        hp.length.push_back(len); hp.dilation.push_back(d); hp.padding.push_back(p); hp.num_channels.push_back(m);
+        for (int q = 0; q < m && std::scanf("%d", &c) == 1; ++q) hp.channel_idx.push_back(c);
+        hp.channel_offset.push_back((int)hp.channel_idx.size());
+        hp.weight_offset.push_back(hp.weight_offset.back() + m * len);
+        hp.bias.push_back(0.5f);
+    }
+    hp.weights.assign(hp.weight_offset.back(), 1.0f);
+    PlanHost plan;
+    build_plan(hp, kSplitDefault, plan, false);
+    const SGroups s = s_groups(plan, N, kSms);
+    for (int i = 0; i < 3; ++i) std::printf("%d %d ", s.examples[i], s.end[i] - (i ? s.end[i - 1] : 0));
+    std::printf("\n");
+    return 0;
+}
+
+int main(int argc, char** argv) {
+    if (argc > 1) return print_sharing(std::atoi(argv[1]));
     check_copies();
     check_tile_interior();
     check_rows_in_series();

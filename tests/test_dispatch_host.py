@@ -2,14 +2,37 @@
 import os
 import subprocess
 
+import pytest
+
+from test_gpu_sharing import CASES, kernels
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-def test_dispatch_rules(tmp_path):
+@pytest.fixture(scope="module")
+def check(tmp_path_factory):
     csrc = os.path.join(ROOT, "paper_2301_08527_b200", "csrc")
-    exe = str(tmp_path / "dispatch_check")
+    exe = str(tmp_path_factory.mktemp("dispatch") / "dispatch_check")
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-I", csrc, "-I", os.path.join(ROOT, "include"), "-I", "/usr/local/cuda/include",
                            os.path.join(ROOT, "tests", "dispatch_check.cpp"), os.path.join(csrc, "rocket_plan.cpp"),
                            os.path.join(csrc, "rocket_generate.cpp"), "-o", exe])
-    out = subprocess.run([exe], capture_output=True, text=True)
+    return exe
+
+
+def test_dispatch_rules(check):
+    out = subprocess.run([check], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_the_sharing_cases_share_tiles(check, case):
+    C, L, N, K, dilations, classes = case
+    kp = kernels(C, L, K, dilations)
+    text = "%d %d %d\n" % (C, L, K)
+    for k in range(K):
+        ch = kp.channel_idx[kp.channel_offset[k]:kp.channel_offset[k + 1]]
+        text += " ".join(map(str, [kp.length[k], kp.dilation[k], kp.padding[k], len(ch), *ch])) + "\n"
+    out = subprocess.run([check, str(N)], input=text, capture_output=True, text=True, check=True).stdout.split()
+    examples, tiles = list(map(int, out[0::2])), list(map(int, out[1::2]))
+    for cls in classes:
+        assert tiles[cls] > 0 and examples[cls] > 1 and N % examples[cls] != 0, (examples, tiles)

@@ -66,9 +66,9 @@ def test_captured_calls_give_the_bits_of_plain_calls(small, large):
 def test_captured_backward_of_an_empty_batch():
     # no kernel of the call before the one that clears the sums
     import torch
-    p = _handle(2, 501, 6, 2)
+    p = _handle(2, 6001, 6, 2)
     p.reserve(1, rk.PASS_SOFT | rk.PASS_BACKWARD)
-    X, g = torch.empty((0, 2, 501), device="cuda"), torch.empty((0, 16), device="cuda")
+    X, g = torch.empty((0, 2, 6001), device="cuda"), torch.empty((0, 16), device="cuda")
     arg = torch.empty((0, 8), dtype=torch.int32, device="cuda")
     dW, db = torch.full((p.n_weights,), -7.0, device="cuda"), torch.full((8,), -7.0, device="cuda")
     rk.rocket_transform_soft_backward(p, X, 10.0, 3.0, g, arg, dW, db)

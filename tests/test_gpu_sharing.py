@@ -1,0 +1,51 @@
+"""Small-dilation tiles shared among examples, with a last group that is not full, against the oracles (every mode).
+
+Which tiles are shared, and by how many examples, test_dispatch_host.py checks on the host for the cases below (buckets of 8 to 31
+kernels are class 1, of fewer class 2; 148 SMs).
+"""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2301_08527_b200 as rk
+from rocket_inputs import ar1_spike_series, normal_array
+
+import parity as P
+from test_gpu_edges import _kernels
+from test_gpu_f16 import _check_bitwise
+
+# channels, steps, examples, kernels, dilations; classes whose tiles are shared
+CASES = [(1, 65, 401, 60, (1, 2, 9), (1,)), (3, 207, 233, 40, (1, 2, 3, 5, 6, 7, 11, 13), (2,)),
+         (2, 120, 401, 52, (1, 1, 1, 1, 1, 1, 1, 2, 3, 4, 5, 6, 7), (1, 2)), (4, 99, 403, 30, (1, 2, 3, 4, 5), (2,))]
+
+
+def kernels(C, L, K, dilations):
+    return _kernels(np.random.default_rng(1000 * C + L), C, L, K, dilations, 9)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", CASES)
+def test_shared_tiles(case):
+    import torch
+    C, L, N, K, dilations, _ = case
+    kp = kernels(C, L, K, dilations)
+    X = ar1_spike_series(C + L, N, C, L)
+    lam, shift = 10.0, 3.0
+    p = rk.RocketParams.from_kernel_params(kp)
+    Xd = torch.from_numpy(X).cuda()
+    ref = oracle.forward(kp, X, lam=lam, shift=shift)
+    ppv, mx = P.split_features(rk.rocket_transform(p, Xd).cpu().numpy())
+    P.check_hard_ppv(ppv, ref)
+    P.check_max(mx, ref)
+    _check_bitwise(kp, X, rk.rocket_transform_f16(p, Xd).cpu().numpy())
+    feat, arg = rk.rocket_transform_soft(p, Xd, lam, shift)
+    soft, mx = P.split_features(feat.cpu().numpy())
+    P.check_soft_ppv(soft, ref)
+    P.check_max(mx, ref)
+    P.check_argmax(arg.cpu().numpy(), ref)
+    g = normal_array(L, (N, 2 * kp.K))
+    dW, db = rk.rocket_transform_soft_backward(p, Xd, lam, shift, torch.from_numpy(g).cuda(), arg)
+    rW, rb = oracle.backward(kp, X, g, arg.cpu().numpy(), lam=lam, shift=shift)
+    P.check_grads(dW.cpu().numpy(), db.cpu().numpy(), rW, rb)
+    assert p.device_status() == 0
+    p.close()
