@@ -175,7 +175,7 @@ __device__ __forceinline__ int mini_count(const u64 (&acc)[kMRows], float b) {
     return __popc(s0 | s1 << kMRows);
 }
 
-// Bound: instruction issue - per pair of outputs 9 packed multiply-adds, (m - 1) 22/14 packed adds and m 22/14 loads for the
+// Bound: shared memory (67 % of its wavefronts at 60 x 20 x 50,000) and instruction issue (59 %) together - per pair of outputs 9 packed multiply-adds, (m - 1) 22/14 packed adds and m 22/14 loads for the
 // channel sums (m channels, 3.9 on average) and, per bias (3.8 on average), a packed add and two shifts that collect the signs
 // of bias - z.  What the layout is for: the channels of a tile are read once for the 84 combinations of a dilation (one
 // combination per block and tile, the earlier form, read 146 GB from L2 for 60 x 20 x 50,000), the packed operations work on

@@ -565,7 +565,7 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     if (e != cudaSuccess) return status_of(e);
     const int col_blocks = (P + 31) / 32;
     // Slices of the feature axis: about two waves of the four blocks an SM holds, at least 128 columns each, and no more
-    // than 40 MB of partial tiles.
+    // than 40 MB of partial tiles (or one slice, 65 MB at the most examples).
     const int nt = (N + kGT - 1) / kGT, tiles = nt * (nt + 1) / 2;
     const size_t tile_bytes = (size_t)kGT * kGT * sizeof(double);
     int slices = std::max(1, std::min({8 * sms / tiles, P / 128, (int)(((size_t)40 << 20) / (tile_bytes * tiles))}));
