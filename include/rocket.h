@@ -90,7 +90,8 @@ int rocket_params_generate(uint64_t seed, int K, int C, int L, rocket_params_t**
  * L_out,k >= 1; 1 <= num_channels[k] <= min(C, 11); channel indices of one kernel distinct and
  * in [0, C).  Any such kernel is accepted, up to L_out,k <= 2^30 (ROCKET_EUNSUPPORTED beyond);
  * kernels of length 7, 9 or 11 are served by the fused kernels (for C <= 255 channels and L >= 16),
- * every other kernel of the same handle by the generic ones, in every pass.
+ * every other kernel of the same handle by the generic ones, in every pass.  With more than 20 channels
+ * a call too small for the fused kernels to pay goes to the generic ones as a whole.
  */
 int rocket_params_from_arrays(int K, int C, int L, const int32_t* length, const int32_t* dilation,
                               const int32_t* padding, const int32_t* num_channels,

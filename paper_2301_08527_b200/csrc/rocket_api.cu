@@ -145,6 +145,15 @@ bool no_room(cudaError_t e) {
     return true;
 }
 
+// Whether the fused kernels serve a call of N examples (with the handle's kernels that they take).
+bool fused_call(const rocket_params* p, bool aligned, int N) {
+    if (p->path != 0 || !p->fast->host.enabled || !aligned) return false;
+    if (p->host.C <= fast::kSMaxPlanes || N == 0) return true;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    return !fast::generic_pays(p->fast->host, N, std::max(1, sms));
+}
+
 // Makes the handle's device current for the duration of a call.
 struct DeviceGuard {
     int prev = -1;
@@ -372,8 +381,14 @@ int rocket_params_reserve(rocket_params_t* p, int max_N, int passes) {
     std::lock_guard<std::mutex> lk(p->mu);
     // kernels outside the fused path: the backward's per-example partial sums; 8-bit input: its fp32 copy
     const bool some_generic = !fused || !p->fast->host.generic_list.empty() || p->path == 1;
-    if (backward && some_generic) {
-        cudaError_t e = p->scratch.reserve(generic_backward_scratch_floats(max_N, nW, p->host.K) * sizeof(float));
+    int generic_N = some_generic ? max_N : 0;
+    if (!some_generic && p->host.C > fast::kSMaxPlanes) {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+        generic_N = fast::generic_pays_up_to(p->fast->host, max_N, std::max(1, sms));
+    }
+    if (backward && generic_N > 0) {
+        cudaError_t e = p->scratch.reserve(generic_backward_scratch_floats(generic_N, nW, p->host.K) * sizeof(float));
         if (e != cudaSuccess) return cuda_status(e);
     }
     if (u8 && (some_generic || p->host.C > fast::kNormMaxChannels)) {
@@ -395,7 +410,7 @@ int rocket_transform(const rocket_params_t* p, const float* X_dev, int N, int C,
     if (!g.ok) return ROCKET_ECUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
-    if (p->path == 0 && p->fast->host.enabled && aligned) {
+    if (fused_call(p, aligned, N)) {
         cudaError_t e = fast::launch_fast_forward(*p->fast, p->dp, X_dev, N, feat_dev, stream);
         if (e != cudaSuccess && !no_room(e)) return cuda_status(e);
         if (e == cudaSuccess && p->fast->dev.n_generic == 0) return ROCKET_OK;
@@ -434,7 +449,7 @@ int rocket_transform_soft(const rocket_params_t* p, const float* X_dev, int N, i
     if (!g.ok) return ROCKET_ECUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
-    if (p->path == 0 && p->fast->host.enabled && aligned) {
+    if (fused_call(p, aligned, N)) {
         cudaError_t e = fast::launch_fast_forward(*p->fast, p->dp, X_dev, N, feat_dev, stream, true, lambda, shift, argmax_dev);
         if (e != cudaSuccess && !no_room(e)) return cuda_status(e);
         if (e == cudaSuccess && p->fast->dev.n_generic == 0) return ROCKET_OK;
@@ -519,7 +534,7 @@ int rocket_transform_soft_backward(const rocket_params_t* p, const float* X_dev,
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const int64_t nW = n_weights_of(p);
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
-    bool use_fast = p->path == 0 && p->fast->host.enabled && (aligned || N == 0);
+    bool use_fast = fused_call(p, aligned || N == 0, N);
     if (use_fast) {   // the fused kernels assign dW / db of the kernels they serve
         cudaError_t e = fast::launch_fast_backward(*p->fast, p->dp, nW, X_dev, N, lambda, shift, dfeat_dev, argmax_dev,
                                                    dW_dev, db_dev, stream);

@@ -246,7 +246,15 @@ struct PlanHost {
     bool s_wide = false;                  // the S tiles are staged in halves of up to kSWidePlanes planes
     int s_class_end[3] = {0, 0, 0};       // S tiles by kernels in their bucket: at least kSManyKernels, kSSomeKernels, fewer
     double flops_s = 0.0, flops_t = 0.0;  // conv flop of one example in either regime
+    // What generic_pays compares, in us: work of one example for one SM (small dilations) and for the GPU (large dilations and their
+    // copies, generic kernels), and what one tile or one kernel takes at least.
+    double us_s = 0.0, us_s_tile = 0.0, us_t = 0.0, us_g = 0.0, us_g_kernel = 0.0;
 };
+
+// Whether the generic kernels serve a call of N examples in less time than the fused ones (asked where C > kSMaxPlanes).
+bool generic_pays(const PlanHost& plan, int N, int sms);
+// The most examples up to max_N of a call that the generic kernels serve for that reason.
+int generic_pays_up_to(const PlanHost& plan, int max_N, int sms);
 
 // How the S kernel's tiles are shared among the examples of a pass: tiles [end[i - 1], end[i]) for examples[i] examples together, as
 // groups[i] groups; grid: its blocks.

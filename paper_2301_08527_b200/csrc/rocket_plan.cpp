@@ -2,6 +2,7 @@
 // cuts them into tiles and orders the tiles by cost (largest first).
 #include <algorithm>
 #include <climits>
+#include <cmath>
 #include <functional>
 #include <map>
 #include <tuple>
@@ -148,6 +149,63 @@ StreamItems stream_items(int N, int C, int L, int n_units, double visits, int mo
     if (mode == 1 || mode == 2) per_set = std::max(per_set, (kWSoftSetItems * warps + n_units - 1) / std::max(1, n_units));
     s.groups_per_set = (int)std::max<int64_t>(1, std::min<int64_t>(s.groups, per_set));
     return s;
+}
+
+namespace {
+
+// Costs for generic_pays, fitted to the device times of 220 calls of 21 to 255 channels, 24 to 20,000 steps, 30 to 5,000 kernels and
+// 1 to 128 examples (hard transform; 8 % rms for the fused kernels, 14 % for the generic ones; the training passes take three times
+// as long on either side).
+constexpr double kUsFused = 6.4, kUsTile = 3.7, kUsPlane = 0.125, kUsTap = 0.0105, kUsVisit = 6.3e-4, kUsCopiedByte = 1.66e-7;
+constexpr double kUsGeneric = 2.3, kUsPair = 1.4e-3, kUsWarpTap = 6.1e-6, kUsBlockTap = 1.2e-4, kUsTapLatency = 0.076;
+
+void estimate_costs(const HostParams& hp, PlanHost& p) {
+    const double halves = p.s_wide ? 2.0 : 1.0, plane = kUsPlane * (p.s_wide ? 23.0 / 34.0 : 1.0);
+    std::vector<double> taps(p.sb.size(), 0.0);
+    for (size_t b = 0; b < p.sb.size(); ++b)
+        for (int f = p.sb[b].kbeg; f < p.sb[b].kend; ++f) taps[b] += (double)p.krec[f].m * p.krec[f].len;
+    double most = -1.0;
+    for (const SItem& it : p.sitems) {
+        const double tile = kUsTile + p.sb[it.bucket].nch * plane, work = taps[it.bucket] * kUsTap;
+        p.us_s += halves * tile + work;
+        if (work > most) {                                     // the longest tile, not the widest
+            most = work;
+            p.us_s_tile = tile + work / halves;
+        }
+    }
+    double visits = p.w_visits;
+    int64_t row_bytes = p.wunits.empty() ? 0 : 4 * kWCopies * p.wpitch;
+    for (const TItem& it : p.titems) visits += (double)it.m * kTConsumerWarps;
+    if (p.wunits.empty() && !p.titems.empty()) row_bytes = 4 * 4 * p.pad_pitch;
+    p.us_t = visits * kUsVisit + (double)hp.C * row_bytes * kUsCopiedByte;
+    for (int k = 0; k < hp.K; ++k) {
+        const int64_t nout = (int64_t)hp.L + 2 * (int64_t)hp.padding[k] - (int64_t)(hp.length[k] - 1) * hp.dilation[k];
+        const double t = (double)hp.length[k] * hp.num_channels[k], rounds = t * (double)((nout + 255) / 256);
+        p.us_g += kUsPair + kUsWarpTap * t * (double)((nout + 31) / 32) + kUsBlockTap * rounds;
+        p.us_g_kernel = std::max(p.us_g_kernel, kUsTapLatency * rounds);
+    }
+}
+
+// A launch whose blocks share `total` and whose longest block takes `longest`.
+double launch_time(double total, double longest) { return std::sqrt(std::sqrt(total * total * total * total + longest * longest * longest * longest)); }
+
+}  // namespace
+
+// A series of more channels than a tile has planes for needs buckets and copies that few or short kernels do not pay for: the generic
+// kernels, which read what a kernel uses and no more, take 14 us for 1 x 32 x 32 and 1,500 kernels where the fused ones take 140,
+// 71 us for 32 x 255 x 1,002 and 60 kernels against 113; from some 500 steps on the fused ones are ahead (24 x 32 x 1,751, 2,000
+// kernels: 1,445 us against 477).  Within the error of the estimates the generic kernels have it.
+bool generic_pays(const PlanHost& plan, int N, int sms) {
+    const double fused = kUsFused + launch_time(N * plan.us_s / sms, plan.us_s_tile) + N * plan.us_t;
+    const double generic = kUsGeneric + launch_time(N * plan.us_g, plan.us_g_kernel);
+    return 0.93 * generic < fused;
+}
+
+int generic_pays_up_to(const PlanHost& plan, int max_N, int sms) {
+    if (max_N > 65536) return max_N;
+    int n = max_N;
+    while (n > 0 && !generic_pays(plan, n, sms)) --n;
+    return n;
 }
 
 void fill_record_weights(const HostParams& hp, KRec& f) {
@@ -457,6 +515,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
     // read past the last sample; rounded to 128 bytes
     const int64_t pitch = (int64_t)kTPadFront + hp.L + 4ll * d_max + kTXExtra + t_box_cols(4);
     out.pad_pitch = (pitch + 31) / 32 * 32;
+    estimate_costs(hp, out);
 }
 
 }  // namespace fast

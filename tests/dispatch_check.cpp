@@ -106,8 +106,30 @@ static void check_copies() {
     }
 }
 
+// Many channels: the generic kernels where they were measured to be faster, the fused ones where those were.
+static void check_generic() {
+    struct Case { int N, C, L, K, generic; };
+    for (const Case& c : {Case{1, 32, 32, 1500, 1}, Case{1, 21, 100, 300, 1}, Case{32, 255, 102, 1500, 1}, Case{32, 255, 1002, 60, 1}, Case{1, 64, 31, 300, 1},
+                          Case{6, 32, 102, 1500, 1}, Case{24, 32, 1751, 2000, 0}, Case{1, 32, 4000, 300, 0}, Case{32, 255, 4002, 1500, 0}, Case{6, 64, 4000, 60, 0},
+                          Case{32, 21, 300, 1500, 0}, Case{1, 30, 100000, 100, 0}, Case{4, 100, 20000, 500, 0}}) {
+        HostParams hp;
+        generate_host_params(8527, c.K, c.C, c.L, hp);
+        hp.channel_offset.assign(hp.K + 1, 0);
+        hp.weight_offset.assign(hp.K + 1, 0);
+        for (int k = 0; k < hp.K; ++k) {
+            hp.channel_offset[k + 1] = hp.channel_offset[k] + hp.num_channels[k];
+            hp.weight_offset[k + 1] = hp.weight_offset[k] + hp.num_channels[k] * hp.length[k];
+        }
+        PlanHost plan;
+        build_plan(hp, kSplitDefault, plan, false);
+        REQUIRE(generic_pays(plan, c.N, kSms) == (c.generic != 0), "%d x %d x %d, %d kernels", c.N, c.C, c.L, c.K);
+        const int up_to = generic_pays_up_to(plan, 300, kSms);
+        for (int n = 1; n <= 300; ++n) REQUIRE(n <= up_to || !generic_pays(plan, n, kSms), "%d of at most %d examples", n, up_to);
+    }
+}
+
 // Kernels from standard input (C, L, K, then per kernel length, dilation, padding and its channels): prints, for N examples, how many
-// examples the tiles of each class share and how many tiles there are of each.
+// examples the tiles of each class share and how many tiles there are of each, and whether the generic kernels serve the call.
 static int print_sharing(int N) {
     HostParams hp;
     if (std::scanf("%d %d %d", &hp.C, &hp.L, &hp.K) != 3) return 2;
@@ -127,7 +149,7 @@ static int print_sharing(int N) {
     build_plan(hp, kSplitDefault, plan, false);
     const SGroups s = s_groups(plan, N, kSms);
     for (int i = 0; i < 3; ++i) std::printf("%d %d ", s.examples[i], s.end[i] - (i ? s.end[i - 1] : 0));
-    std::printf("\n");
+    std::printf("%d\n", hp.C > kSMaxPlanes && generic_pays(plan, N, kSms) ? 1 : 0);
     return 0;
 }
 
@@ -137,6 +159,7 @@ int main(int argc, char** argv) {
     check_tile_interior();
     check_rows_in_series();
     check_stream_items();
+    check_generic();
     if (failures == 0) std::printf("ok\n");
     return failures ? 1 : 0;
 }

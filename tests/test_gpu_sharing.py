@@ -1,7 +1,8 @@
-"""Small-dilation tiles shared among examples, with a last group that is not full, against the oracles (every mode).
+"""Small-dilation tiles shared among examples, with a last group that is not full, and series of more than 20 channels on either side of
+the line between the fused and the generic kernels, against the oracles (every mode).
 
-Which tiles are shared, and by how many examples, test_dispatch_host.py checks on the host for the cases below (buckets of 8 to 31
-kernels are class 1, of fewer class 2; 148 SMs).
+Which tiles are shared, and by how many examples, and which kernels serve the wide series, test_dispatch_host.py checks on the host
+for the cases below (buckets of 8 to 31 kernels are class 1, of fewer class 2; 148 SMs).
 """
 import numpy as np
 import pytest
@@ -17,6 +18,9 @@ from test_gpu_f16 import _check_bitwise
 # channels, steps, examples, kernels, dilations; classes whose tiles are shared
 CASES = [(1, 65, 401, 60, (1, 2, 9), (1,)), (3, 207, 233, 40, (1, 2, 3, 5, 6, 7, 11, 13), (2,)),
          (2, 120, 401, 52, (1, 1, 1, 1, 1, 1, 1, 2, 3, 4, 5, 6, 7), (1, 2)), (4, 99, 403, 30, (1, 2, 3, 4, 5), (2,))]
+# channels, steps, examples, kernels, dilations; served by the generic kernels
+WIDE_CASES = [(21, 1501, 9, 120, (1, 5, 40), False), (34, 1701, 8, 160, (1, 3, 63, 90), False), (35, 1500, 8, 160, (2, 9, 130), False),
+              (48, 2003, 6, 90, (1, 2, 7, 66, 160), False), (25, 86, 3, 60, (1, 2, 5), True), (255, 130, 5, 40, (1, 4, 9), True)]
 
 
 def kernels(C, L, K, dilations):
@@ -24,8 +28,8 @@ def kernels(C, L, K, dilations):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("case", CASES)
-def test_shared_tiles(case):
+@pytest.mark.parametrize("case", CASES + WIDE_CASES)
+def test_every_mode(case):
     import torch
     C, L, N, K, dilations, _ = case
     kp = kernels(C, L, K, dilations)
@@ -37,7 +41,8 @@ def test_shared_tiles(case):
     ppv, mx = P.split_features(rk.rocket_transform(p, Xd).cpu().numpy())
     P.check_hard_ppv(ppv, ref)
     P.check_max(mx, ref)
-    _check_bitwise(kp, X, rk.rocket_transform_f16(p, Xd).cpu().numpy())
+    if C <= 20:
+        _check_bitwise(kp, X, rk.rocket_transform_f16(p, Xd).cpu().numpy())
     feat, arg = rk.rocket_transform_soft(p, Xd, lam, shift)
     soft, mx = P.split_features(feat.cpu().numpy())
     P.check_soft_ppv(soft, ref)
