@@ -204,7 +204,7 @@ struct alignas(16) WUnit {
     int32_t nout, woff, ncol, band_y;     // band_y: y steps from band to band
     int32_t x0, y0, run, copy;            // coordinates of the first column of band 0; floats per y step; first copy
     uint8_t ch[12];
-    int32_t bytes, pad_[4];               // bytes of a visit's copy
+    int32_t bytes, span, pad_[3];         // bytes of a visit's copy; positions from a band's first row to its last (w_span)
 };
 static_assert(sizeof(WUnit) == 128, "WUnit must be 32 words");
 // Examples of a pass of the stream regime for rows of `pitch` floats.

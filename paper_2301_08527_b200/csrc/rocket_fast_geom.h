@@ -49,10 +49,16 @@ ROCKET_HD int s_column_u0(const SBucket& b, int cg) {
     return (b.tmin + band * kRS) * b.d + r;
 }
 
-// Stream regime: every one of the R rows x 64 columns from (row trow, column c0) is an output of a kernel of dilation d.  The last
-// row of a band may lie 16 d beyond the series, which takes more than 32 bits from 380 million samples on.
-ROCKET_HD bool tile_interior(int trow, int c0, int R, int d, int lo_u, int hi_u) {
-    return c0 + kWarpCols <= d && (long long)trow * d + c0 >= lo_u && (long long)(trow + R - 1) * d + c0 + kWarpCols - 1 < hi_u;
+// Stream regime: every one of the rows x 64 columns from (row trow, column c0) is an output of a kernel of dilation d.  span is
+// (rows - 1) * d: the end of a tile may lie 16 d beyond the series, which takes more than 32 bits from 380 million samples on, while the
+// distance from its first output to the last one of the kernel never does.
+ROCKET_HD int w_span(int rows, int d) {
+    const long long span = (long long)(rows - 1) * d;
+    return span < 0x7fffffff ? (int)span : 0x7fffffff;
+}
+ROCKET_HD bool tile_interior(int trow, int c0, int span, int d, int lo_u, int hi_u) {
+    const int u = trow * d + c0;
+    return c0 + kWarpCols <= d && u >= lo_u && hi_u - kWarpCols - u >= span;
 }
 
 // T regime.  A tile starts at A-row t0 and residue r0 (a multiple of 64).  Row s of the tile

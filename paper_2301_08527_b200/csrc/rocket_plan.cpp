@@ -75,6 +75,7 @@ void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost&
             u.bytes = y_rows * G * kWarpCols * 4;
             u.run = G * f.d;
             u.band_y = R / G;
+            u.span = w_span(R, f.d);
             // first row of a y step: the last of its four when they are taken backwards
             const bool backwards = f.d % 4 == 3;
             const int64_t pos = out.wfront + t * f.d + (backwards ? 3ll * f.d : 0);

@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kWThreads, 1) fast_stream(const __grid_constan
             for (int t = 0; t < ntiles; ++t) {
                 const bool last = t + 1 == ntiles && e + 1 == examples;      // of the item
                 const int c0 = col * kWarpCols, c = c0 + 2 * lane;
-                const bool interior = tile_interior(trow, c0, R, d, field(9), field(10));
+                const bool interior = tile_interior(trow, c0, field(28), d, field(9), field(10));
                 unsigned m0 = 0, m1 = 0;               // rows of the lane's two columns that are outputs
                 if (!interior) {
                     const int tl = field(12), rl = field(13), th = field(14), rh = field(15);
