@@ -364,7 +364,7 @@ int rocket_transform_soft_backward_noalloc(const rocket_params_t* p, const float
  *                      combination, on the host's cores); returns when done.
  * rocket_mini_set_biases  installs biases computed elsewhere ([n_features] floats, host).
  * rocket_mini_transform   X_dev [N][C][L] fp32 and feat_dev [N][n_features] fp32 on the device; one fused kernel
- *                      (and a small one that divides the counts) on the caller's stream (convolution outputs never
+ *                      (and, in one of its two forms, a small one that divides the counts) on the caller's stream (convolution outputs never
  *                      reach memory; any L, any 4-byte aligned X_dev); the first call binds the handle to the current
  *                      device, uploads its parameters (one allocation) and opts the kernel into 220 KB of shared memory.  Every wait inside the
  *                      kernel is bounded; should one give up, all features of that call (and of no other) are NaN.  ROCKET_EINVAL before

@@ -7,7 +7,7 @@
 //                every other (dilation, kernel) combination, a random channel subset per combination
 //   fit          rocket_mini_fit, on the host (a one-off over one training example per combination): the bias of
 //                a feature is a quantile of the combination's convolution output on that example
-//   transform    rocket_mini_transform, one fused kernel: a block stages a tile of the dilated view with all the
+//   transform    rocket_mini_transform, one fused kernel of two (the other: rocket_mini_walk.cuh): a block stages a tile of the dilated view with all the
 //                channels that the combinations of a dilation use, its warps take the combinations one by one -
 //                channels summed, nine-tap convolution, comparison with every bias of the combination, all in
 //                registers - so the convolution outputs never reach memory; a small kernel then turns counts into
@@ -32,6 +32,7 @@
 #include "rocket_fast_dev.cuh"
 #include "rocket_fast_geom.h"
 #include "rocket_internal.h"
+#include "rocket_mini_walk.cuh"
 
 namespace rocket {
 namespace fast {
@@ -415,6 +416,9 @@ struct rocket_mini {
     std::vector<MiniRec> recs;
     std::vector<MiniBucket> buckets;
     std::vector<MiniTile> tiles;
+    std::vector<WalkItem> walk_items;
+    // what mini_walks compares, in us: copies and work of all tiles of one example; all walks of one example and the longest walk
+    double us_copies = 0.0, us_work = 0.0, us_walks = 0.0, us_walk = 0.0;
     std::vector<int32_t> nout;             // outputs behind every feature
     int64_t slices = 0;                    // slices of at most eight features of one combination
     int max_nch = 1;
@@ -424,6 +428,7 @@ struct rocket_mini {
     mutable void* blob = nullptr;          // records, buckets, tiles, output counts, biases, the calls' flags
     mutable MiniArgs dev{};
     mutable const int* d_nout = nullptr;
+    mutable const WalkItem* d_walk = nullptr;
     mutable MiniFlag* flags = nullptr;
     mutable std::atomic<unsigned> calls{0};
     mutable bool bias_uploaded = false;
@@ -499,6 +504,91 @@ static void build_tiles(rocket_mini& p) {
     }
 }
 
+// Costs for mini_walks, fitted to the device times of 260 calls of 1 to 250 channels, 24 to 60,000 steps, 84 to 9,996 features and 1 to
+// 128 examples (12 % rms for the walks, 21 % for the tiles).
+constexpr double kUsTiles = 7.1, kUsTile = 2.8, kUsPlane = 0.19, kUsPair = 0.067, kUsChannel = 0.0174, kUsBias = 0.0119;
+constexpr double kUsWalks = 2.8, kUsItem = 1.03, kUsLoad = 3.55e-5, kUsStaged = 1.69e-4, kUsSlot = 8.9e-6, kUsLongest = 2.52e-4;
+
+// The items of the kernel that takes one combination at a time, and the costs of either kernel.
+static void build_walk_items(rocket_mini& p) {
+    p.us_copies = p.us_work = p.us_walks = p.us_walk = 0.0;
+    std::vector<double> work(p.buckets.size(), 0.0);
+    for (size_t b = 0; b < p.buckets.size(); ++b)
+        for (int r = p.buckets[b].kbeg; r < p.buckets[b].kend; ++r) work[b] += kUsPair + p.recs[r].m * kUsChannel + p.recs[r].nf * kUsBias;
+    for (const MiniTile& t : p.tiles) {
+        p.us_copies += kUsPlane * p.buckets[t.bucket].nch;
+        p.us_work += work[t.bucket];
+    }
+    p.walk_items.clear();
+    if (p.L > kWalkMostSamples) return;
+    struct Tiling { int width, seg_rows, segs; double staged, slots; };
+    std::map<int, Tiling> tiling;                        // by dilation
+    for (int c = 0; c < p.n_combos; ++c)
+        for (int f0 = p.feature_offset[c]; f0 < p.feature_offset[c + 1]; f0 += kWalkFeatures) {
+            WalkItem it{};
+            it.d = p.dilation[c]; it.padded = p.padded[c]; it.m = p.num_channels[c];
+            it.f0 = f0; it.nf = std::min(kWalkFeatures, p.feature_offset[c + 1] - f0);
+            for (int k = 0; k < 3; ++k) it.tap[k] = p.taps[3 * p.kernel_index[c] + k];
+            for (int q = 0; q < it.m; ++q) it.ch[q] = p.channel_idx[p.channel_offset[c] + q];
+            auto found = tiling.find(it.d);
+            if (found == tiling.end()) {
+                Tiling t{};
+                choose_walk(it.d, p.L, t.width, t.seg_rows, t.segs);
+                if (t.width < 1 || t.seg_rows < kLen || t.segs < 1 || (int64_t)(t.seg_rows * t.segs + 8) * t.width > kWalkSamples) {
+                    p.walk_items.clear();                // no tiling fits (does not happen from L = 9 on)
+                    return;
+                }
+                const int T = (p.L + it.d - 1) / it.d, tile_rows = t.seg_rows * t.segs;
+                for (int ta = 0; ta < T; ta += tile_rows) {
+                    const int rows = std::min(tile_rows, T - ta), segs = (rows + t.seg_rows - 1) / t.seg_rows;
+                    for (int ca = 0; ca < it.d; ca += t.width) {
+                        const int cols = std::min(t.width, it.d - ca);
+                        t.staged += (rows + 8.0) * cols;
+                        t.slots += (double)(((int64_t)cols * segs + kWalkThreads - 1) / kWalkThreads * kWalkThreads) * (std::min(t.seg_rows, rows) + 1);
+                    }
+                }
+                found = tiling.emplace(it.d, t).first;
+            }
+            const Tiling& t = found->second;
+            it.width = t.width; it.seg_rows = t.seg_rows; it.segs = t.segs;
+            p.walk_items.push_back(it);
+            p.us_walks += kUsItem + t.staged * it.m * kUsLoad + t.staged * kUsStaged + t.slots * (it.nf > 4 ? 1.6 : 1.0) * kUsSlot;
+            p.us_walk = std::max(p.us_walk, kUsLongest * (0.3 * t.staged * it.m + t.slots));
+        }
+}
+
+// How the tile kernel goes over N examples.
+struct MiniLaunch { int examples, groups, parts; unsigned grid; bool all_copy; };
+static MiniLaunch mini_launch(const rocket_mini& p, int N, int sms) {
+    MiniLaunch a;
+    // Examples that share a tile: as many as its planes hold, while every SM still gets four tiles; fewer tiles than SMs are
+    // dealt in parts of their combinations (84 or so) instead.
+    const long long n_tiles = (long long)p.tiles.size(), tiles = N * n_tiles;
+    a.examples = (int)std::max<long long>(1, std::min<long long>({(p.wide ? kMPlanesWide : kMPlanes) / p.max_nch, N, tiles / (4ll * sms)}));
+    a.groups = (N + a.examples - 1) / a.examples;
+    const long long items = (long long)a.groups * n_tiles;
+    a.parts = (int)std::max<long long>(1, std::min<long long>(8, 2ll * sms / items));
+    a.grid = (unsigned)std::min<long long>(items * a.parts, sms);
+    // A block that has one tile only has nothing to overlap its copies with: all warps make them (1 x 20 x 300, 840 features:
+    // 16.4 us with three warps, 14.4 so), into no more shared memory than the tile takes (1 x 12 x 900: 16.4 -> 14.4 us).
+    a.all_copy = p.wide || items * a.parts <= a.grid;
+    return a;
+}
+
+// Whether the kernel that takes one combination at a time serves a call of N examples in less time.  It does where a tile's channels are
+// many and each is used by few combinations (24 x 250 x 10,000, 9,996 features: 1.65 ms against 4.5; 24 x 100 x 10,000, 840: 0.56
+// against 1.35), and where there are few tiles (5 x 20 x 10,000, 84 features: 18.6 us against 26.7; 1 x 20 x 1,500, 840: 16 against
+// 25).  The tiles have it from a few examples on where they share (24 x 20 x 10,000, 9,996 features: 0.88 ms against 1.6).
+static bool mini_walks(const rocket_mini& p, int N, int sms) {
+    if (p.walk_items.empty()) return false;
+    const MiniLaunch a = mini_launch(p, N, sms);
+    const double n_tiles = (double)p.tiles.size(), items = (double)a.groups * n_tiles * a.parts;
+    auto both = [](double x, double y) { return std::sqrt(std::sqrt(x * x * x * x + y * y * y * y)); };   // near the larger
+    const double copies = kUsTile + p.us_copies / n_tiles * a.examples, work = p.us_work / n_tiles * a.examples / a.parts;
+    const double tiles = kUsTiles + std::ceil(items / a.grid) * (a.all_copy ? copies + work : both(copies, work));
+    return kUsWalks + both(N * p.us_walks / sms, p.us_walk) < tiles;
+}
+
 // Examples of one launch of the tile kernel: (tile, example) pairs, eight parts of each, are counted in 32 bits.
 #ifndef ROCKET_MINI_LAUNCH_TILES
 #define ROCKET_MINI_LAUNCH_TILES (0x7fffffffll / 8)
@@ -513,9 +603,10 @@ static int ensure_mini_device(const rocket_mini* p) {
         int dev = -1;
         if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return ROCKET_ECUDA; }
         struct Part { const void* src; size_t bytes, off; };
-        Part parts[6] = {{p->recs.data(), p->recs.size() * sizeof(MiniRec), 0},     {p->buckets.data(), p->buckets.size() * sizeof(MiniBucket), 0},
+        Part parts[7] = {{p->recs.data(), p->recs.size() * sizeof(MiniRec), 0},     {p->buckets.data(), p->buckets.size() * sizeof(MiniBucket), 0},
                          {p->tiles.data(), p->tiles.size() * sizeof(MiniTile), 0}, {p->nout.data(), p->nout.size() * sizeof(int32_t), 0},
-                         {nullptr, (size_t)p->F * sizeof(float), 0},               {nullptr, kMFlags * sizeof(MiniFlag), 0}};
+                         {nullptr, (size_t)p->F * sizeof(float), 0},               {nullptr, kMFlags * sizeof(MiniFlag), 0},
+                         {p->walk_items.data(), p->walk_items.size() * sizeof(WalkItem), 0}};
         size_t total = 0;
         for (Part& pt : parts) { pt.off = total; total += (pt.bytes + 255) / 256 * 256; }
         cudaError_t e = rocket::device_malloc(&p->blob, total);
@@ -523,9 +614,10 @@ static int ensure_mini_device(const rocket_mini* p) {
         char* base = static_cast<char*>(p->blob);
         e = cudaMemset(base + parts[5].off, 0, parts[5].bytes);
         for (const Part& pt : parts)
-            if (e == cudaSuccess && pt.src) e = cudaMemcpy(base + pt.off, pt.src, pt.bytes, cudaMemcpyHostToDevice);
+            if (e == cudaSuccess && pt.src && pt.bytes) e = cudaMemcpy(base + pt.off, pt.src, pt.bytes, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_tile_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMiniSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(mini_walk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kWalkSamples * sizeof(float)));
         if (e != cudaSuccess) { cudaGetLastError(); cudaFree(p->blob); p->blob = nullptr; return ROCKET_ECUDA; }
         MiniArgs& a = p->dev;
         a.recs = reinterpret_cast<const MiniRec*>(base + parts[0].off);
@@ -533,6 +625,7 @@ static int ensure_mini_device(const rocket_mini* p) {
         a.tiles = reinterpret_cast<const MiniTile*>(base + parts[2].off);
         p->d_nout = reinterpret_cast<const int*>(base + parts[3].off);
         a.bias = reinterpret_cast<const float*>(base + parts[4].off);
+        p->d_walk = reinterpret_cast<const WalkItem*>(base + parts[6].off);
         p->flags = reinterpret_cast<MiniFlag*>(base + parts[5].off);
         a.C = p->C; a.L = p->L; a.F = p->F; a.n_tiles = (int)p->tiles.size();
         p->device = dev;
@@ -605,6 +698,7 @@ int rocket_mini_create(uint64_t seed, int C, int L, int num_features, rocket_min
         for (int f = 0; f < p->F; ++f) p->quantile[f] = std::fmod((f + 1.0) * kInvGoldenRatio, 1.0);
         p->bias.assign(p->F, 0.0f);
         build_tiles(*p);
+        build_walk_items(*p);
     } catch (const std::bad_alloc&) {
         delete p;
         return ROCKET_ENOMEM;
@@ -725,6 +819,15 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
     sms = std::max(sms, 1);
+    if (mini_walks(*p, N, sms)) {
+        mini_walk_kernel<<<(unsigned)(N * (long long)p->walk_items.size()), kWalkThreads, kWalkSamples * sizeof(float), stream>>>(
+            X_dev, C, L, p->d_walk, (int)p->walk_items.size(), p->dev.bias, feat_dev, p->F);
+        rocket::count_launch();
+        const cudaError_t e = cudaGetLastError();
+        if (prev != p->device) cudaSetDevice(prev);
+        if (e != cudaSuccess) { cudaGetLastError(); return ROCKET_ECUDA; }
+        return ROCKET_OK;
+    }
     MiniFlag* flag = p->flags + p->calls.fetch_add(1, std::memory_order_relaxed) % kMFlags;
     const long long values = (long long)N * p->F;
     const unsigned value_blocks = (unsigned)((values + 255) / 256);
@@ -736,19 +839,12 @@ int rocket_mini_transform(const rocket_mini_t* p, const float* X_dev, int N, int
         args.counts = reinterpret_cast<int*>(feat_dev) + (size_t)n0 * p->F;
         args.N = std::min(most, N - n0);
         args.failed = &flag->failed;
-        // Examples that share a tile: as many as its planes hold, while every SM still gets four tiles; fewer tiles than SMs are
-        // dealt in parts of their combinations (84 or so) instead.
-        const long long tiles = (long long)args.N * args.n_tiles;
-        args.examples = (int)std::max<long long>(1, std::min<long long>({(p->wide ? kMPlanesWide : kMPlanes) / p->max_nch, args.N, tiles / (4ll * sms)}));
-        args.groups = (args.N + args.examples - 1) / args.examples;
-        const long long items = (long long)args.groups * args.n_tiles;
-        args.parts = (int)std::max<long long>(1, std::min<long long>(8, 2ll * sms / items));
-        const unsigned grid = (unsigned)std::min<long long>(items * args.parts, sms);
-        // A block that has one tile only has nothing to overlap its copies with: all warps make them (1 x 20 x 300, 840 features:
-        // 16.4 us with three warps, 14.4 so), into no more shared memory than the tile takes (1 x 12 x 900: 16.4 -> 14.4 us).
-        const bool all_copy = p->wide || items * args.parts <= grid;
-        if (all_copy) mini_tile_kernel<true><<<grid, kMThreads, (size_t)args.examples * p->max_nch * kMPlaneBytes, stream>>>(args);
-        else mini_tile_kernel<false><<<grid, kMThreads, kMiniSmemBytes, stream>>>(args);
+        const MiniLaunch at = mini_launch(*p, args.N, sms);
+        args.examples = at.examples;
+        args.groups = at.groups;
+        args.parts = at.parts;
+        if (at.all_copy) mini_tile_kernel<true><<<at.grid, kMThreads, (size_t)args.examples * p->max_nch * kMPlaneBytes, stream>>>(args);
+        else mini_tile_kernel<false><<<at.grid, kMThreads, kMiniSmemBytes, stream>>>(args);
         rocket::count_launch();
     }
     launch_dependent(mini_finalize_kernel, value_blocks, 256, 0, stream, feat_dev, p->d_nout, p->F, values, flag);
