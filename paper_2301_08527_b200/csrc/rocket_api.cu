@@ -145,13 +145,32 @@ bool no_room(cudaError_t e) {
     return true;
 }
 
+int sms_of(const rocket_params* p) {
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    return std::max(1, sms);
+}
+
 // Whether the fused kernels serve a call of N examples (with the handle's kernels that they take).
 bool fused_call(const rocket_params* p, bool aligned, int N) {
     if (p->path != 0 || !p->fast->host.enabled || !aligned) return false;
     if (p->host.C <= fast::kSMaxPlanes || N == 0) return true;
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-    return !fast::generic_pays(p->fast->host, N, std::max(1, sms));
+    return !fast::generic_pays(p->fast->host, N, sms_of(p));
+}
+
+// A call covers every smaller one of its kind, also those that take the other kernels: their workspace is made with it.  Without room
+// for it they find that out themselves.
+void cover_smaller_calls(const rocket_params* p, int N, bool soft, bool backward, bool fused) {
+    if (p->path != 0 || !p->fast->host.enabled || p->host.C <= fast::kSMaxPlanes || N < 2) return;
+    const int n = fast::pays_up_to(p->fast->host, N - 1, sms_of(p), fused);
+    if (n == 0) return;
+    const int64_t nW = n_weights_of(p);
+    if (!fused) {
+        no_room(fast::reserve_fast_state(*p->fast, p->dp, n, soft, backward, false, nW, false));
+    } else if (backward) {
+        std::lock_guard<std::mutex> lk(p->mu);
+        no_room(p->scratch.reserve(generic_backward_scratch_floats(n, nW, p->host.K) * sizeof(float)));
+    }
 }
 
 // Makes the handle's device current for the duration of a call.
@@ -382,11 +401,7 @@ int rocket_params_reserve(rocket_params_t* p, int max_N, int passes) {
     // kernels outside the fused path: the backward's per-example partial sums; 8-bit input: its fp32 copy
     const bool some_generic = !fused || !p->fast->host.generic_list.empty() || p->path == 1;
     int generic_N = some_generic ? max_N : 0;
-    if (!some_generic && p->host.C > fast::kSMaxPlanes) {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-        generic_N = fast::generic_pays_up_to(p->fast->host, max_N, std::max(1, sms));
-    }
+    if (!some_generic && p->host.C > fast::kSMaxPlanes) generic_N = fast::pays_up_to(p->fast->host, max_N, sms_of(p), true);
     if (backward && generic_N > 0) {
         cudaError_t e = p->scratch.reserve(generic_backward_scratch_floats(generic_N, nW, p->host.K) * sizeof(float));
         if (e != cudaSuccess) return cuda_status(e);
@@ -410,7 +425,9 @@ int rocket_transform(const rocket_params_t* p, const float* X_dev, int N, int C,
     if (!g.ok) return ROCKET_ECUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
-    if (fused_call(p, aligned, N)) {
+    const bool use_fast = fused_call(p, aligned, N);
+    cover_smaller_calls(p, N, false, false, use_fast);
+    if (use_fast) {
         cudaError_t e = fast::launch_fast_forward(*p->fast, p->dp, X_dev, N, feat_dev, stream);
         if (e != cudaSuccess && !no_room(e)) return cuda_status(e);
         if (e == cudaSuccess && p->fast->dev.n_generic == 0) return ROCKET_OK;
@@ -449,7 +466,9 @@ int rocket_transform_soft(const rocket_params_t* p, const float* X_dev, int N, i
     if (!g.ok) return ROCKET_ECUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
-    if (fused_call(p, aligned, N)) {
+    const bool use_fast = fused_call(p, aligned, N);
+    cover_smaller_calls(p, N, true, false, use_fast);
+    if (use_fast) {
         cudaError_t e = fast::launch_fast_forward(*p->fast, p->dp, X_dev, N, feat_dev, stream, true, lambda, shift, argmax_dev);
         if (e != cudaSuccess && !no_room(e)) return cuda_status(e);
         if (e == cudaSuccess && p->fast->dev.n_generic == 0) return ROCKET_OK;
@@ -535,6 +554,7 @@ int rocket_transform_soft_backward(const rocket_params_t* p, const float* X_dev,
     const int64_t nW = n_weights_of(p);
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
     bool use_fast = fused_call(p, aligned || N == 0, N);
+    cover_smaller_calls(p, N, false, true, use_fast);
     if (use_fast) {   // the fused kernels assign dW / db of the kernels they serve
         cudaError_t e = fast::launch_fast_backward(*p->fast, p->dp, nW, X_dev, N, lambda, shift, dfeat_dev, argmax_dev,
                                                    dW_dev, db_dev, stream);

@@ -253,8 +253,9 @@ struct PlanHost {
 
 // Whether the generic kernels serve a call of N examples in less time than the fused ones (asked where C > kSMaxPlanes).
 bool generic_pays(const PlanHost& plan, int N, int sms);
-// The most examples up to max_N of a call that the generic kernels serve for that reason.
-int generic_pays_up_to(const PlanHost& plan, int max_N, int sms);
+// A bound on the examples of the calls of up to max_N that the generic kernels serve for that reason (pays), or that the fused ones do:
+// what either needs a workspace for.
+int pays_up_to(const PlanHost& plan, int max_N, int sms, bool generic);
 
 // How the S kernel's tiles are shared among the examples of a pass: tiles [end[i - 1], end[i]) for examples[i] examples together, as
 // groups[i] groups; grid: its blocks.
@@ -322,8 +323,9 @@ cudaError_t ensure_pad_capacity(FastState& fs, int N, int C, int L, bool without
 // Allocates, once, everything the fused kernels need for calls of up to max_N examples (the zero-margined
 // copies and their tensor maps, the soft transform's and the backward's workspaces) and opts the kernels
 // into their shared-memory sizes; later calls within that size allocate nothing.
+// again: the full size, where there was no room for it before.
 cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N, bool soft, bool backward, bool u8,
-                               int64_t n_weights);
+                               int64_t n_weights, bool again = true);
 
 // Backward of the soft transform through the fast path (every kernel must be a fast-path kernel):
 // dW (ragged like the weights, n_weights floats) and db [K] are assigned.

@@ -1170,13 +1170,13 @@ static cudaError_t ensure_bwd_ws(FastState& fs, const DeviceParams& dp, int64_t 
 }
 
 cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N, bool soft, bool backward, bool u8,
-                               int64_t n_weights) {
+                               int64_t n_weights, bool again) {
     std::lock_guard<std::mutex> lk(fs.mu);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = set_kernel_attributes(dev)) != cudaSuccess) return e;
-    fs.most_examples = 1 << 30;           // asked again
+    if (again) fs.most_examples = 1 << 30;
     const bool stream = fs.dev.n_wunits > 0, copies = fs.dev.n_titems > 0 || u8;
     const int chunk = std::min(max_N, chunk_examples(fs, dp.C, stream, copies));
     if (stream && (e = ensure_stream_capacity(fs, chunk, dp.C, dp.L)) != cudaSuccess) return e;

@@ -202,11 +202,11 @@ bool generic_pays(const PlanHost& plan, int N, int sms) {
     return 0.93 * generic < fused;
 }
 
-int generic_pays_up_to(const PlanHost& plan, int max_N, int sms) {
-    if (max_N > 65536) return max_N;
-    int n = max_N;
-    while (n > 0 && !generic_pays(plan, n, sms)) --n;
-    return n;
+int pays_up_to(const PlanHost& plan, int max_N, int sms, bool generic) {
+    if (generic_pays(plan, max_N, sms) == generic) return max_N;
+    for (int n = 1 << 16; n >= 1; n /= 2)
+        if (n < max_N && generic_pays(plan, n, sms) == generic) return std::min(max_N, 2 * n - 1);
+    return 0;
 }
 
 void fill_record_weights(const HostParams& hp, KRec& f) {

@@ -123,8 +123,12 @@ static void check_generic() {
         PlanHost plan;
         build_plan(hp, kSplitDefault, plan, false);
         REQUIRE(generic_pays(plan, c.N, kSms) == (c.generic != 0), "%d x %d x %d, %d kernels", c.N, c.C, c.L, c.K);
-        const int up_to = generic_pays_up_to(plan, 300, kSms);
-        for (int n = 1; n <= 300; ++n) REQUIRE(n <= up_to || !generic_pays(plan, n, kSms), "%d of at most %d examples", n, up_to);
+        for (int generic = 0; generic < 2; ++generic)
+            for (int most : {1, 7, 32, 300}) {
+                const int up_to = pays_up_to(plan, most, kSms, generic != 0);
+                for (int n = 1; n <= most; ++n)
+                    REQUIRE(n <= up_to || generic_pays(plan, n, kSms) != (generic != 0), "%d of at most %d examples", n, up_to);
+            }
     }
 }
 

@@ -54,3 +54,26 @@ def test_every_mode(case):
     P.check_grads(dW.cpu().numpy(), db.cpu().numpy(), rW, rb)
     assert p.device_status() == 0
     p.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("C,L,K,N", [(255, 4000, 60, 32), (32, 301, 1500, 40), (21, 33, 1500, 64)])
+def test_a_call_covers_the_smaller_ones_of_its_kind(C, L, K, N):
+    # whichever kernels serve them: no call allocates after a larger one
+    import torch
+    p = rk.RocketParams.generate(8527, K, C, L)
+    X = torch.from_numpy(ar1_spike_series(C + L, N, C, L)).cuda()
+    g = torch.from_numpy(normal_array(L, (N, 2 * K))).cuda()
+
+    def calls(n):
+        rk.rocket_transform(p, X[:n])
+        _, arg = rk.rocket_transform_soft(p, X[:n], 10.0, 3.0)
+        return rk.rocket_transform_soft_backward(p, X[:n], 10.0, 3.0, g[:n].contiguous(), arg)
+
+    calls(N)
+    before = rk.device_alloc_count()
+    for n in [*range(1, N, 3), N]:
+        calls(n)
+    torch.cuda.synchronize()
+    assert rk.device_alloc_count() == before
+    p.close()
