@@ -145,24 +145,18 @@ bool no_room(cudaError_t e) {
     return true;
 }
 
-int sms_of(const rocket_params* p) {
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-    return std::max(1, sms);
-}
-
 // Whether the fused kernels serve a call of N examples (with the handle's kernels that they take).
 bool fused_call(const rocket_params* p, bool aligned, int N) {
     if (p->path != 0 || !p->fast->host.enabled || !aligned) return false;
     if (p->host.C <= fast::kSMaxPlanes || N == 0) return true;
-    return !fast::generic_pays(p->fast->host, N, sms_of(p));
+    return !fast::generic_pays(p->fast->host, N, p->fast->sms);
 }
 
 // A call covers every smaller one of its kind, also those that take the other kernels: their workspace is made with it.  Without room
 // for it they find that out themselves.
 void cover_smaller_calls(const rocket_params* p, int N, bool soft, bool backward, bool fused) {
     if (p->path != 0 || !p->fast->host.enabled || p->host.C <= fast::kSMaxPlanes || N < 2) return;
-    const int n = fast::pays_up_to(p->fast->host, N - 1, sms_of(p), fused);
+    const int n = fast::pays_up_to(p->fast->host, N - 1, p->fast->sms, fused);
     if (n == 0) return;
     const int64_t nW = n_weights_of(p);
     if (!fused) {
@@ -401,7 +395,7 @@ int rocket_params_reserve(rocket_params_t* p, int max_N, int passes) {
     // kernels outside the fused path: the backward's per-example partial sums; 8-bit input: its fp32 copy
     const bool some_generic = !fused || !p->fast->host.generic_list.empty() || p->path == 1;
     int generic_N = some_generic ? max_N : 0;
-    if (!some_generic && p->host.C > fast::kSMaxPlanes) generic_N = fast::pays_up_to(p->fast->host, max_N, sms_of(p), true);
+    if (!some_generic && p->host.C > fast::kSMaxPlanes) generic_N = fast::pays_up_to(p->fast->host, max_N, p->fast->sms, true);
     if (backward && generic_N > 0) {
         cudaError_t e = p->scratch.reserve(generic_backward_scratch_floats(generic_N, nW, p->host.K) * sizeof(float));
         if (e != cudaSuccess) return cuda_status(e);

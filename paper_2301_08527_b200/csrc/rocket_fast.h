@@ -291,6 +291,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles =
 // Device-side state of the fast path owned by a handle.
 struct FastState {
     std::mutex mu;                        // guards the grow-only buffers below and the launch sequence of a call
+    int sms = 0, l2_bytes = 0;            // of the handle's device
     PlanHost host;
     PlanDevice dev;
     void* plan_blob = nullptr;            // records, buckets, items, counters, error flag

@@ -967,6 +967,11 @@ cudaError_t upload_plan(FastState& fs) {
     const PlanHost& h = fs.host;
     PlanDevice& d = fs.dev;
     d = PlanDevice();
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&fs.sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&fs.l2_bytes, cudaDevAttrL2CacheSize, dev);
+    if (e != cudaSuccess) return e;
     struct Part { const void* src; size_t bytes; size_t off; };
     Part parts[8] = {
         {h.krec.data(), h.krec.size() * sizeof(KRec), 0},   {h.sb.data(), h.sb.size() * sizeof(SBucket), 0},
@@ -975,7 +980,7 @@ cudaError_t upload_plan(FastState& fs) {
         {h.wunits.data(), h.wunits.size() * sizeof(WUnit), 0}};
     size_t total = 0;
     for (auto& pt : parts) { pt.off = total; total += align256(pt.bytes); }
-    cudaError_t e = device_malloc(&fs.plan_blob, std::max<size_t>(total, 256));
+    e = device_malloc(&fs.plan_blob, std::max<size_t>(total, 256));
     if (e != cudaSuccess) { fs.plan_blob = nullptr; return e; }
     char* base = static_cast<char*>(fs.plan_blob);
     e = cudaMemset(base, 0, std::max<size_t>(total, 256));
@@ -1191,11 +1196,9 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
                                 const uint8_t* X_u8, const NormArgs* norm, bool half) {
     if (half && soft) return cudaErrorInvalidValue;
     std::lock_guard<std::mutex> lk(fs.mu);
-    int dev = 0, sms = 0, l2 = 0;
+    const int sms = fs.sms, l2 = fs.l2_bytes;
+    int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;
@@ -1292,11 +1295,9 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
                                  float lambda, float shift, const float* dfeat, const int32_t* argmax, float* dW,
                                  float* db, cudaStream_t stream) {
     std::lock_guard<std::mutex> lk(fs.mu);
-    int dev = 0, sms = 0, l2 = 0;
+    const int sms = fs.sms, l2 = fs.l2_bytes;
+    int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;

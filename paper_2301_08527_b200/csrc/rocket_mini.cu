@@ -504,10 +504,10 @@ static void build_tiles(rocket_mini& p) {
     }
 }
 
-// Costs for mini_walks, fitted to the device times of 260 calls of 1 to 250 channels, 24 to 60,000 steps, 84 to 9,996 features and 1 to
-// 128 examples (12 % rms for the walks, 21 % for the tiles).
-constexpr double kUsTiles = 7.1, kUsTile = 2.8, kUsPlane = 0.19, kUsPair = 0.067, kUsChannel = 0.0174, kUsBias = 0.0119;
-constexpr double kUsWalks = 2.8, kUsItem = 1.03, kUsLoad = 3.55e-5, kUsStaged = 1.69e-4, kUsSlot = 8.9e-6, kUsLongest = 2.52e-4;
+// Costs for mini_walks, fitted to the device times of 400 calls of 1 to 250 channels, 24 to 60,000 steps, 84 to 9,996 features and 1 to
+// 128 examples (13 % rms for the walks, 23 % for the tiles).
+constexpr double kUsTiles = 6.75, kUsTile = 4.68, kUsPlane = 0.092, kUsPair = 0.0673, kUsChannel = 0.0176, kUsBias = 0.0131;
+constexpr double kUsWalks = 2.86, kUsItem = 1.17, kUsLoad = 5.1e-5, kUsStaged = 1.13e-4, kUsLongest = 2.69e-4;
 
 // The items of the kernel that takes one combination at a time, and the costs of either kernel.
 static void build_walk_items(rocket_mini& p) {
@@ -552,7 +552,7 @@ static void build_walk_items(rocket_mini& p) {
             const Tiling& t = found->second;
             it.width = t.width; it.seg_rows = t.seg_rows; it.segs = t.segs;
             p.walk_items.push_back(it);
-            p.us_walks += kUsItem + t.staged * it.m * kUsLoad + t.staged * kUsStaged + t.slots * (it.nf > 4 ? 1.6 : 1.0) * kUsSlot;
+            p.us_walks += kUsItem + t.staged * it.m * kUsLoad + t.staged * kUsStaged;
             p.us_walk = std::max(p.us_walk, kUsLongest * (0.3 * t.staged * it.m + t.slots));
         }
 }
@@ -585,8 +585,8 @@ static bool mini_walks(const rocket_mini& p, int N, int sms) {
     const double n_tiles = (double)p.tiles.size(), items = (double)a.groups * n_tiles * a.parts;
     auto both = [](double x, double y) { return std::sqrt(std::sqrt(x * x * x * x + y * y * y * y)); };   // near the larger
     const double copies = kUsTile + p.us_copies / n_tiles * a.examples, work = p.us_work / n_tiles * a.examples / a.parts;
-    const double tiles = kUsTiles + std::ceil(items / a.grid) * (a.all_copy ? copies + work : both(copies, work));
-    return kUsWalks + both(N * p.us_walks / sms, p.us_walk) < tiles;
+    const double rounds = items / a.grid, tiles = kUsTiles + (rounds < 4.0 ? std::ceil(rounds) : rounds + 0.5) * (a.all_copy ? copies + work : both(copies, work));
+    return 1.1 * (kUsWalks + both(N * p.us_walks / sms, p.us_walk)) < tiles;     // the tiles have it within the error of the estimates
 }
 
 // Examples of one launch of the tile kernel: (tile, example) pairs, eight parts of each, are counted in 32 bits.

@@ -154,11 +154,11 @@ StreamItems stream_items(int N, int C, int L, int n_units, double visits, int mo
 
 namespace {
 
-// Costs for generic_pays, fitted to the device times of 220 calls of 21 to 255 channels, 24 to 20,000 steps, 30 to 5,000 kernels and
-// 1 to 128 examples (hard transform; 8 % rms for the fused kernels, 14 % for the generic ones; the training passes take three times
+// Costs for generic_pays, fitted to the device times of 340 calls of 21 to 255 channels, 24 to 20,000 steps, 30 to 5,000 kernels and
+// 1 to 128 examples (hard transform; 7 % rms for the fused kernels, 14 % for the generic ones; the training passes take three times
 // as long on either side).
-constexpr double kUsFused = 6.4, kUsTile = 3.7, kUsPlane = 0.125, kUsTap = 0.0105, kUsVisit = 6.3e-4, kUsCopiedByte = 1.66e-7;
-constexpr double kUsGeneric = 2.3, kUsPair = 1.4e-3, kUsWarpTap = 6.1e-6, kUsBlockTap = 1.2e-4, kUsTapLatency = 0.076;
+constexpr double kUsFused = 5.5, kUsStream = 6.7, kUsTile = 3.37, kUsPlane = 0.166, kUsTap = 0.0105, kUsVisit = 5.5e-4, kUsCopiedByte = 1.4e-7;
+constexpr double kUsGeneric = 3.6, kUsPair = 1.41e-3, kUsWarpTap = 6.5e-6, kUsBlockTap = 1.11e-4, kUsTapLatency = 0.0758;
 
 void estimate_costs(const HostParams& hp, PlanHost& p) {
     const double halves = p.s_wide ? 2.0 : 1.0, plane = kUsPlane * (p.s_wide ? 23.0 / 34.0 : 1.0);
@@ -195,11 +195,11 @@ double launch_time(double total, double longest) { return std::sqrt(std::sqrt(to
 // A series of more channels than a tile has planes for needs buckets and copies that few or short kernels do not pay for: the generic
 // kernels, which read what a kernel uses and no more, take 14 us for 1 x 32 x 32 and 1,500 kernels where the fused ones take 140,
 // 71 us for 32 x 255 x 1,002 and 60 kernels against 113; from some 500 steps on the fused ones are ahead (24 x 32 x 1,751, 2,000
-// kernels: 1,445 us against 477).  Within the error of the estimates the generic kernels have it.
+// kernels: 1,445 us against 477).  Within the error of the estimates the fused kernels have it.
 bool generic_pays(const PlanHost& plan, int N, int sms) {
-    const double fused = kUsFused + launch_time(N * plan.us_s / sms, plan.us_s_tile) + N * plan.us_t;
+    const double fused = kUsFused + launch_time(N * plan.us_s / sms, plan.us_s_tile) + (plan.us_t > 0.0 ? kUsStream : 0.0) + N * plan.us_t;
     const double generic = kUsGeneric + launch_time(N * plan.us_g, plan.us_g_kernel);
-    return 0.93 * generic < fused;
+    return 1.05 * generic < fused;
 }
 
 int pays_up_to(const PlanHost& plan, int max_N, int sms, bool generic) {
