@@ -251,11 +251,12 @@ struct PlanHost {
     double us_s = 0.0, us_s_tile = 0.0, us_t = 0.0, us_g = 0.0, us_g_kernel = 0.0;
 };
 
-// Whether the generic kernels serve a call of N examples in less time than the fused ones (asked where C > kSMaxPlanes).
-bool generic_pays(const PlanHost& plan, int N, int sms);
+// Whether the generic kernels serve a call of N examples in less time than the fused ones (asked where C > kSMaxPlanes); soft: the
+// soft transform or its backward.
+bool generic_pays(const PlanHost& plan, int N, int sms, bool soft);
 // A bound on the examples of the calls of up to max_N that the generic kernels serve for that reason (pays), or that the fused ones do:
 // what either needs a workspace for.
-int pays_up_to(const PlanHost& plan, int max_N, int sms, bool generic);
+int pays_up_to(const PlanHost& plan, int max_N, int sms, bool soft, bool generic);
 
 // How the S kernel's tiles are shared among the examples of a pass: tiles [end[i - 1], end[i]) for examples[i] examples together, as
 // groups[i] groups; grid: its blocks.

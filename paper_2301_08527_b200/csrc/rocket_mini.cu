@@ -504,19 +504,22 @@ static void build_tiles(rocket_mini& p) {
     }
 }
 
-// Costs for mini_walks, fitted to the device times of 400 calls of 1 to 250 channels, 24 to 60,000 steps, 84 to 9,996 features and 1 to
-// 128 examples (13 % rms for the walks, 23 % for the tiles).
-constexpr double kUsTiles = 6.75, kUsTile = 4.68, kUsPlane = 0.092, kUsPair = 0.0673, kUsChannel = 0.0176, kUsBias = 0.0131;
+// Costs for mini_walks, fitted to the device times of 600 calls of 1 to 250 channels, 24 to 60,000 steps, 84 to 9,996 features and 1 to
+// 128 examples (13 % rms for the walks, 25 % for the tiles, which have costs of their own where a dilation is several buckets).
+struct TileCosts { double call, tile, plane, pair, channel, bias; };
+constexpr TileCosts kUsOneBucket{6.75, 4.68, 0.092, 0.0673, 0.0176, 0.0131}, kUsBuckets{6.81, 7.81, 0.0, 0.179, 0.0, 0.0023};
 constexpr double kUsWalks = 2.86, kUsItem = 1.17, kUsLoad = 5.1e-5, kUsStaged = 1.13e-4, kUsLongest = 2.69e-4;
+static const TileCosts& tile_costs(const rocket_mini& p) { return p.C > kMPlanesWide ? kUsBuckets : kUsOneBucket; }
 
 // The items of the kernel that takes one combination at a time, and the costs of either kernel.
 static void build_walk_items(rocket_mini& p) {
     p.us_copies = p.us_work = p.us_walks = p.us_walk = 0.0;
+    const TileCosts& us = tile_costs(p);
     std::vector<double> work(p.buckets.size(), 0.0);
     for (size_t b = 0; b < p.buckets.size(); ++b)
-        for (int r = p.buckets[b].kbeg; r < p.buckets[b].kend; ++r) work[b] += kUsPair + p.recs[r].m * kUsChannel + p.recs[r].nf * kUsBias;
+        for (int r = p.buckets[b].kbeg; r < p.buckets[b].kend; ++r) work[b] += us.pair + p.recs[r].m * us.channel + p.recs[r].nf * us.bias;
     for (const MiniTile& t : p.tiles) {
-        p.us_copies += kUsPlane * p.buckets[t.bucket].nch;
+        p.us_copies += us.plane * p.buckets[t.bucket].nch;
         p.us_work += work[t.bucket];
     }
     p.walk_items.clear();
@@ -584,8 +587,9 @@ static bool mini_walks(const rocket_mini& p, int N, int sms) {
     const MiniLaunch a = mini_launch(p, N, sms);
     const double n_tiles = (double)p.tiles.size(), items = (double)a.groups * n_tiles * a.parts;
     auto both = [](double x, double y) { return std::sqrt(std::sqrt(x * x * x * x + y * y * y * y)); };   // near the larger
-    const double copies = kUsTile + p.us_copies / n_tiles * a.examples, work = p.us_work / n_tiles * a.examples / a.parts;
-    const double rounds = items / a.grid, tiles = kUsTiles + (rounds < 4.0 ? std::ceil(rounds) : rounds + 0.5) * (a.all_copy ? copies + work : both(copies, work));
+    const TileCosts& us = tile_costs(p);
+    const double copies = us.tile + p.us_copies / n_tiles * a.examples, work = p.us_work / n_tiles * a.examples / a.parts;
+    const double rounds = items / a.grid, tiles = us.call + (rounds < 4.0 ? std::ceil(rounds) : rounds + 0.5) * (a.all_copy ? copies + work : both(copies, work));
     return 1.1 * (kUsWalks + both(N * p.us_walks / sms, p.us_walk)) < tiles;     // the tiles have it within the error of the estimates
 }
 

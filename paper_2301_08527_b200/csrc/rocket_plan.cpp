@@ -154,11 +154,12 @@ StreamItems stream_items(int N, int C, int L, int n_units, double visits, int mo
 
 namespace {
 
-// Costs for generic_pays, fitted to the device times of 340 calls of 21 to 255 channels, 24 to 20,000 steps, 30 to 5,000 kernels and
-// 1 to 128 examples (hard transform; 7 % rms for the fused kernels, 14 % for the generic ones; the training passes take three times
-// as long on either side).
-constexpr double kUsFused = 5.5, kUsStream = 6.7, kUsTile = 3.37, kUsPlane = 0.166, kUsTap = 0.0105, kUsVisit = 5.5e-4, kUsCopiedByte = 1.4e-7;
-constexpr double kUsGeneric = 3.6, kUsPair = 1.41e-3, kUsWarpTap = 6.5e-6, kUsBlockTap = 1.11e-4, kUsTapLatency = 0.0758;
+// Costs for generic_pays, fitted to the device times of 570 calls of 21 to 255 channels, 24 to 20,000 steps, 30 to 5,000 kernels and
+// 1 to 128 examples (9 % rms on either side).  The costs are the hard transform's; training takes 3.1 times as long through the fused
+// kernels and 3.4 times through the generic ones.
+constexpr double kUsFused = 6.2, kUsStream = 6.0, kUsTile = 3.25, kUsPlane = 0.159, kUsTap = 0.0112, kUsVisit = 5.9e-4, kUsCopiedByte = 1.28e-7;
+constexpr double kUsGeneric = 1.9, kUsPair = 2.2e-3, kUsWarpTap = 8.35e-6, kUsBlockTap = 8.2e-5, kUsTapLatency = 0.0696;
+constexpr double kSoftGeneric = 3.4 / 3.1, kNearTie = 1.03;    // within the error of the estimates the fused kernels have it
 
 void estimate_costs(const HostParams& hp, PlanHost& p) {
     const double halves = p.s_wide ? 2.0 : 1.0, plane = kUsPlane * (p.s_wide ? 23.0 / 34.0 : 1.0);
@@ -187,25 +188,25 @@ void estimate_costs(const HostParams& hp, PlanHost& p) {
     }
 }
 
-// A launch whose blocks share `total` and whose longest block takes `longest`.
-double launch_time(double total, double longest) { return std::sqrt(std::sqrt(total * total * total * total + longest * longest * longest * longest)); }
-
 }  // namespace
 
 // A series of more channels than a tile has planes for needs buckets and copies that few or short kernels do not pay for: the generic
 // kernels, which read what a kernel uses and no more, take 14 us for 1 x 32 x 32 and 1,500 kernels where the fused ones take 140,
 // 71 us for 32 x 255 x 1,002 and 60 kernels against 113; from some 500 steps on the fused ones are ahead (24 x 32 x 1,751, 2,000
-// kernels: 1,445 us against 477).  Within the error of the estimates the fused kernels have it.
-bool generic_pays(const PlanHost& plan, int N, int sms) {
-    const double fused = kUsFused + launch_time(N * plan.us_s / sms, plan.us_s_tile) + (plan.us_t > 0.0 ? kUsStream : 0.0) + N * plan.us_t;
-    const double generic = kUsGeneric + launch_time(N * plan.us_g, plan.us_g_kernel);
-    return 1.05 * generic < fused;
+// kernels: 1,445 us against 477).
+bool generic_pays(const PlanHost& plan, int N, int sms, bool soft) {
+    // a launch lasts as long as its work for the SMs or its longest block, whichever is more, and near a tie somewhat longer than both;
+    // the generic kernels' blocks, as long as their kernels' outputs, pack worse
+    auto both = [](double work, double longest, double q) { return std::pow(std::pow(work, q) + std::pow(longest, q), 1.0 / q); };
+    const double fused = kUsFused + both(N * plan.us_s / sms, plan.us_s_tile, 4.0) + (plan.us_t > 0.0 ? kUsStream : 0.0) + N * plan.us_t;
+    const double generic = kUsGeneric + both(N * plan.us_g, plan.us_g_kernel, 1.5);
+    return kNearTie * (soft ? kSoftGeneric : 1.0) * generic < fused;
 }
 
-int pays_up_to(const PlanHost& plan, int max_N, int sms, bool generic) {
-    if (generic_pays(plan, max_N, sms) == generic) return max_N;
+int pays_up_to(const PlanHost& plan, int max_N, int sms, bool soft, bool generic) {
+    if (generic_pays(plan, max_N, sms, soft) == generic) return max_N;
     for (int n = 1 << 16; n >= 1; n /= 2)
-        if (n < max_N && generic_pays(plan, n, sms) == generic) return std::min(max_N, 2 * n - 1);
+        if (n < max_N && generic_pays(plan, n, sms, soft) == generic) return std::min(max_N, 2 * n - 1);
     return 0;
 }
 
@@ -516,7 +517,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
     // read past the last sample; rounded to 128 bytes
     const int64_t pitch = (int64_t)kTPadFront + hp.L + 4ll * d_max + kTXExtra + t_box_cols(4);
     out.pad_pitch = (pitch + 31) / 32 * 32;
-    estimate_costs(hp, out);
+    if (hp.C > kSMaxPlanes) estimate_costs(hp, out);
 }
 
 }  // namespace fast

@@ -111,7 +111,7 @@ static void check_generic() {
     struct Case { int N, C, L, K, generic; };
     for (const Case& c : {Case{1, 32, 32, 1500, 1}, Case{1, 21, 100, 300, 1}, Case{32, 255, 102, 1500, 1}, Case{32, 255, 1002, 60, 1}, Case{1, 64, 31, 300, 1},
                           Case{6, 32, 102, 1500, 1}, Case{24, 32, 1751, 2000, 0}, Case{1, 32, 4000, 300, 0}, Case{32, 255, 4002, 1500, 0}, Case{6, 64, 4000, 60, 0},
-                          Case{32, 21, 300, 1500, 0}, Case{1, 30, 100000, 100, 0}, Case{4, 100, 20000, 500, 0}}) {
+                          Case{32, 21, 300, 1500, 0}, Case{1, 30, 100000, 100, 0}, Case{4, 100, 20000, 500, 0}, Case{32, 64, 4003, 60, 0}, Case{32, 32, 4000, 60, 0}}) {
         HostParams hp;
         generate_host_params(8527, c.K, c.C, c.L, hp);
         hp.channel_offset.assign(hp.K + 1, 0);
@@ -122,12 +122,13 @@ static void check_generic() {
         }
         PlanHost plan;
         build_plan(hp, kSplitDefault, plan, false);
-        REQUIRE(generic_pays(plan, c.N, kSms) == (c.generic != 0), "%d x %d x %d, %d kernels", c.N, c.C, c.L, c.K);
-        for (int generic = 0; generic < 2; ++generic)
+        REQUIRE(generic_pays(plan, c.N, kSms, false) == (c.generic != 0), "%d x %d x %d, %d kernels", c.N, c.C, c.L, c.K);
+        for (int way = 0; way < 4; ++way)
             for (int most : {1, 7, 32, 300}) {
-                const int up_to = pays_up_to(plan, most, kSms, generic != 0);
+                const bool generic = (way & 1) != 0, soft = (way & 2) != 0;
+                const int up_to = pays_up_to(plan, most, kSms, soft, generic);
                 for (int n = 1; n <= most; ++n)
-                    REQUIRE(n <= up_to || generic_pays(plan, n, kSms) != (generic != 0), "%d of at most %d examples", n, up_to);
+                    REQUIRE(n <= up_to || generic_pays(plan, n, kSms, soft) != generic, "%d of at most %d examples", n, up_to);
             }
     }
 }
@@ -153,7 +154,7 @@ static int print_sharing(int N) {
     build_plan(hp, kSplitDefault, plan, false);
     const SGroups s = s_groups(plan, N, kSms);
     for (int i = 0; i < 3; ++i) std::printf("%d %d ", s.examples[i], s.end[i] - (i ? s.end[i - 1] : 0));
-    std::printf("%d\n", hp.C > kSMaxPlanes && generic_pays(plan, N, kSms) ? 1 : 0);
+    std::printf("%d\n", hp.C > kSMaxPlanes && generic_pays(plan, N, kSms, false) && generic_pays(plan, N, kSms, true) ? 1 : 0);
     return 0;
 }
 

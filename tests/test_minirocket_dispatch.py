@@ -11,7 +11,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 # channels, steps, features, examples; walks
 MEASURED = [(250, 10000, 9996, 24, 1), (100, 10000, 840, 24, 1), (20, 10000, 84, 5, 1), (20, 1500, 840, 1, 1), (64, 1500, 840, 1, 1),
-            (20, 50000, 9996, 60, 0), (20, 10000, 9996, 24, 0), (1, 512, 9996, 16, 0), (9, 1500, 4200, 24, 0), (100, 300, 9996, 24, 0)]
+            (20, 50000, 9996, 60, 0), (20, 10000, 9996, 24, 0), (1, 512, 9996, 16, 0), (41, 10000, 84, 24, 1), (41, 10000, 4200, 5, 1), (250, 1500, 84, 24, 1), (9, 1500, 4200, 24, 0), (100, 300, 9996, 24, 0)]
 
 
 def test_dispatch(tmp_path):
