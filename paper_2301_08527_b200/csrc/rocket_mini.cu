@@ -506,8 +506,8 @@ static void build_tiles(rocket_mini& p) {
 
 // Costs for mini_walks, fitted to the device times of 600 calls of 1 to 250 channels, 24 to 60,000 steps, 84 to 9,996 features and 1 to
 // 128 examples (13 % rms for the walks, 25 % for the tiles, which have costs of their own where a dilation is several buckets).
-struct TileCosts { double call, tile, plane, pair, channel, bias; };
-constexpr TileCosts kUsOneBucket{6.75, 4.68, 0.092, 0.0673, 0.0176, 0.0131}, kUsBuckets{6.81, 7.81, 0.0, 0.179, 0.0, 0.0023};
+struct TileCosts { double call, tile, plane, pair, channel, bias, tie; };      // tie: the tiles have it within this
+constexpr TileCosts kUsOneBucket{6.75, 4.68, 0.092, 0.0673, 0.0176, 0.0131, 1.1}, kUsBuckets{6.81, 7.81, 0.0, 0.179, 0.0, 0.0023, 1.02};
 constexpr double kUsWalks = 2.86, kUsItem = 1.17, kUsLoad = 5.1e-5, kUsStaged = 1.13e-4, kUsLongest = 2.69e-4;
 static const TileCosts& tile_costs(const rocket_mini& p) { return p.C > kMPlanesWide ? kUsBuckets : kUsOneBucket; }
 
@@ -590,7 +590,7 @@ static bool mini_walks(const rocket_mini& p, int N, int sms) {
     const TileCosts& us = tile_costs(p);
     const double copies = us.tile + p.us_copies / n_tiles * a.examples, work = p.us_work / n_tiles * a.examples / a.parts;
     const double rounds = items / a.grid, tiles = us.call + (rounds < 4.0 ? std::ceil(rounds) : rounds + 0.5) * (a.all_copy ? copies + work : both(copies, work));
-    return 1.1 * (kUsWalks + both(N * p.us_walks / sms, p.us_walk)) < tiles;     // the tiles have it within the error of the estimates
+    return us.tie * (kUsWalks + both(N * p.us_walks / sms, p.us_walk)) < tiles;
 }
 
 // Examples of one launch of the tile kernel: (tile, example) pairs, eight parts of each, are counted in 32 bits.
