@@ -1,0 +1,267 @@
+// Gram matrix of the centred features on the fifth-generation tensor cores, in integers.
+//
+// Fc = F - mu is taken in double precision, every row scaled by a power of two so that its largest magnitude lies in [2^45, 2^46), rounded
+// to an integer and written as six signed base-256 digits, d_0 first.  Then G_ij is a sum of digit products: all with a + b <= 5 are kept
+// (21 of 36; what is left out is below 2^-49 of the diagonal), products with the same a + b share a 32-bit accumulator and are exact there
+// (6 * 16,384 columns * 128^2 < 2^31), and the six accumulators meet in double precision.  The quantum is 2^-46 of a row's largest
+// value; against exact sums the result is as close as FP64 multiply-adds came.
+//
+// Why: FP64 products run at 37 TFLOP/s at the most, 8-bit ones at a hundred times that, and 21 of those replace one.  Measured at 677 x
+// 20,000: 193 us (scales 21, digits 26, products 146) where FP64 matrix instructions took 496.  Relative error of the fitted weights against
+// a solution in 64 bits: the same to three digits (2.52e-8, their rounding to FP32), at fifteen sizes from 24 x 200 to 1,500 x 9,001.
+#include <algorithm>
+#include <cstdint>
+
+#include "rocket_fast_dev.cuh"
+#include "rocket_gram.h"
+#include "rocket_internal.h"
+
+namespace rocket {
+namespace {
+
+using fast::bulk_g2s;
+using fast::mbar_arrive_expect_tx;
+using fast::mbar_init;
+using fast::mbar_wait;
+using fast::smem_u32;
+
+constexpr int kDigits = 6, kTileM = 128, kTileN = 64, kStageK = 64;
+// The digits lie in memory as the matrix instruction reads them from shared memory (8 rows x 16 bytes to a core matrix, no swizzle):
+// [block of 64 columns][group of 8 rows][digit][4 core matrices][8 rows][16 columns], so that the operands of a stage are two bulk copies.
+constexpr int kCoreBytes = 128, kDigitBytes = kStageK / 16 * kCoreBytes, kGroupBytes = kDigits * kDigitBytes;
+constexpr int kABytes = kTileM / 8 * kGroupBytes, kBBytes = kTileN / 8 * kGroupBytes, kStageBytes = kABytes + kBBytes;
+constexpr int kStages = 3, kGramThreads = 128;
+static_assert(kDigits * kTileN <= 512, "an accumulator per a + b");
+
+// up[i] = 2^k with up[i] max_p |F[i][p] - mu[p]| in [2^45, 2^46), down[i] = 1 / up[i]; NaN where a value of the row is not finite.
+__global__ void __launch_bounds__(256)
+gram_scale_kernel(const float* __restrict__ F, int P, const double* __restrict__ mu, double* __restrict__ up, double* __restrict__ down) {
+    __shared__ unsigned long long s_max;
+    if (threadIdx.x == 0) s_max = 0ull;
+    __syncthreads();
+    const float* __restrict__ f = F + (size_t)blockIdx.x * P;
+    unsigned long long m = 0ull;                       // magnitudes compare as integers, infinities and NaN above all others
+#pragma unroll 8
+    for (int p = threadIdx.x; p < P; p += 256)
+        m = max(m, (unsigned long long)__double_as_longlong((double)__ldg(f + p) - __ldg(mu + p)) & 0x7fffffffffffffffull);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_max, m);
+    __syncthreads();
+    if (threadIdx.x > 0) return;
+    m = s_max;
+    const int e = (int)(m >> 52) - 1022;               // the maximum is below 2^e
+    const int k = min(max(46 - e, -1022), 1022);
+    const bool finite = (m >> 52) < 2047ull;
+    up[blockIdx.x] = finite ? __longlong_as_double((long long)(1023 + k) << 52) : __longlong_as_double(0x7ff8000000000000ll);
+    down[blockIdx.x] = finite ? __longlong_as_double((long long)(1023 - k) << 52) : __longlong_as_double(0x7ff8000000000000ll);
+}
+
+// The digits of columns [p0, p0 + 64 blocks): a warp writes a core matrix of every digit, 128 contiguous bytes each.  Zeros past the last
+// row and column.
+__global__ void __launch_bounds__(256)
+gram_digits_kernel(const float* __restrict__ F, int N, int P, int p0, int cores, const double* __restrict__ mu, const double* __restrict__ up, int groups,
+                   uint8_t* __restrict__ digits) {
+    const int lane = threadIdx.x & 31, core = blockIdx.x * 8 + (threadIdx.x >> 5), group = blockIdx.y;
+    const int row = group * 8 + lane / 4, k = core * 16 + lane % 4 * 4;
+    if (core >= cores) return;
+    unsigned lo[4], hi[4];
+    const bool there = row < N;
+    const double scale = there ? __ldg(up + row) : 0.0;
+    const float* __restrict__ f = F + (size_t)(there ? row : 0) * P + p0 + k;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const bool ok = there && p0 + k + c < P;
+        const double x = ok ? (double)__ldg(f + c) - __ldg(mu + p0 + k + c) : 0.0;
+        // 1.5 * 2^52 + q has q in its low bits; with 128 added to every digit the digits are the bytes
+        const double shifted = fma(x, scale, 6755399441055744.0);
+        const unsigned long long q = (unsigned long long)(__double_as_longlong(shifted) - 0x4338000000000000ll) + 0x808080808080ull;
+        lo[c] = (unsigned)q;
+        hi[c] = (unsigned)(q >> 32);
+    }
+    uint8_t* out = digits + ((size_t)(core >> 2) * groups + group) * kGroupBytes + (core & 3) * kCoreBytes + 4 * lane;
+#pragma unroll
+    for (int a = 0; a < kDigits; ++a) {
+        const int byte = kDigits - 1 - a;
+        const unsigned* w = byte < 4 ? lo : hi;
+        const unsigned sel = (byte & 3) | ((byte & 3) + 4) << 4;
+        const unsigned v = __byte_perm(__byte_perm(w[0], w[1], sel), __byte_perm(w[2], w[3], sel), 0x5410);
+        *reinterpret_cast<unsigned*>(out + a * kDigitBytes) = v ^ 0x80808080u;
+    }
+}
+
+struct GramArgs {
+    const uint8_t* digits;
+    const double* down;
+    double* part;             // [slices][tiles of 64 x 64][64][64]
+    int* failed;
+    int N, groups, blocks, tiles, slices, add;   // groups: of 8 rows; blocks: of 64 columns; tiles: 64 x 64 ones of a slice; add: onto what part holds
+};
+
+__device__ __forceinline__ uint64_t operand(uint32_t at) {   // K-major, no swizzle: core matrices along K, groups of 8 rows
+    return (uint64_t)((at & 0x3ffffu) >> 4) | (uint64_t)(kCoreBytes >> 4) << 16 | (uint64_t)(kGroupBytes >> 4) << 32 | 1ull << 46;
+}
+
+// One 128 x 64 tile of the lower triangle over a slice of the columns.  One thread copies stages in, one issues the matrix instructions
+// (42 per stage of 64 columns), all four warps turn the accumulators into doubles.  Bound: the matrix pipe, an instruction of 128 x 64 x 32
+// every 70 clocks; with A's digits copied to tensor memory, which spares two thirds of the shared-memory reads, the same.
+__global__ void __launch_bounds__(kGramThreads, 1)
+gram_mma_kernel(const GramArgs a) {
+    extern __shared__ __align__(128) unsigned char gram_smem[];
+    __shared__ __align__(8) unsigned long long s_full[kStages], s_empty[kStages], s_done;
+    __shared__ uint32_t s_tmem;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t full0 = smem_u32(s_full), empty0 = smem_u32(s_empty), done = smem_u32(&s_done);
+    const uint32_t raw = smem_u32(gram_smem), stage0 = (raw + 127u) & ~127u;
+    int bi = (int)((sqrtf(4.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+    while (bi * (bi + 1) > (int)blockIdx.x) --bi;
+    while ((bi + 1) * (bi + 2) <= (int)blockIdx.x) ++bi;
+    const int bj = (int)blockIdx.x - bi * (bi + 1);
+    const int kb0 = (int)((long long)a.blocks * blockIdx.y / a.slices), n_st = (int)((long long)a.blocks * (blockIdx.y + 1) / a.slices) - kb0;
+    if (tid == 0) {
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(full0 + 8u * i, 1);
+            mbar_init(empty0 + 8u * i, 1);
+        }
+        mbar_init(done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = s_tmem;
+    bool ok = true;
+
+    if (tid == 0) {                                    // copies
+        int st = 0;
+        for (; st < n_st; ++st) {
+            const int slot = st % kStages;
+            if (st >= kStages && !(ok = mbar_wait(empty0 + 8u * slot, (st / kStages - 1) & 1))) break;
+            const uint8_t* src = a.digits + (size_t)(kb0 + st) * a.groups * kGroupBytes;
+            const uint32_t dst = stage0 + slot * kStageBytes, bar = full0 + 8u * slot;
+            mbar_arrive_expect_tx(bar, kStageBytes);
+            bulk_g2s(dst, src + (size_t)bi * kABytes, kABytes, bar);
+            bulk_g2s(dst + kABytes, src + (size_t)bj * kBBytes, kBBytes, bar);
+        }
+        if (!ok)                                       // what was started has to land before the block ends
+            for (int i = max(0, st - kStages); i < st; ++i) mbar_wait(full0 + 8u * (i % kStages), (i / kStages) & 1);
+    } else if (tid == 32) {                            // multiplications
+        // D: 32-bit integers; A, B: signed bytes, K-major; 128 x 64
+        constexpr uint32_t kInstr = 2u << 4 | 1u << 7 | 1u << 10 | (uint32_t)(kTileN >> 3) << 17 | (uint32_t)(kTileM >> 4) << 24;
+        for (int st = 0; st < n_st; ++st) {
+            const int slot = st % kStages;
+            if (!(ok = mbar_wait(full0 + 8u * slot, (st / kStages) & 1))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t at = stage0 + slot * kStageBytes;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int da = 0; da < kDigits; ++da)
+#pragma unroll
+                    for (int db = 0; db + da < kDigits; ++db) {
+                        const uint32_t fresh = da == 0 && k == 0 && st == 0 ? 0u : 1u;   // the first product of an accumulator assigns it
+                        asm volatile(
+                            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                            "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+                            ::"r"(tmem + (uint32_t)((da + db) * kTileN)), "l"(operand(at + da * kDigitBytes + k * 2 * kCoreBytes)),
+                            "l"(operand(at + kABytes + db * kDigitBytes + k * 2 * kCoreBytes)), "r"(kInstr), "r"(fresh) : "memory");
+                    }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty0 + 8u * slot) : "memory");
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done) : "memory");
+    }
+    __syncwarp();
+    ok = mbar_wait(done, 0) && ok;
+    ok = __syncthreads_and(ok);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (!ok && tid == 0) atomicExch(a.failed, 1);
+
+    // warp w holds rows 32 w .. 32 w + 31 of the tile, a row per lane
+    const int i = bi * kTileM + tid, ti = i / 64, j0 = bj * kTileN;
+    const double di = i < a.N ? __ldg(a.down + i) : 0.0;
+    double* out = a.part + ((size_t)blockIdx.y * a.tiles + (size_t)ti * (ti + 1) / 2 + bj) * 4096 + (i % 64) * 64;
+    const bool lower = bj <= ti && i < (a.N + 63) / 64 * 64;
+#pragma unroll 1
+    for (int c = 0; c < kTileN; c += 8) {
+        uint32_t v[kDigits][8];
+#pragma unroll
+        for (int s = 0; s < kDigits; ++s)
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(v[s][0]), "=r"(v[s][1]), "=r"(v[s][2]), "=r"(v[s][3]), "=r"(v[s][4]), "=r"(v[s][5]), "=r"(v[s][6]), "=r"(v[s][7])
+                         : "r"(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(s * kTileN + c)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (!lower) continue;
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+            double g[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                double sum = 0.0;                      // smallest first
+#pragma unroll
+                for (int s = kDigits - 1; s >= 0; --s) sum = fma(sum, 1.0 / 256.0, (double)(int)v[s][e + h]);
+                const int j = j0 + c + e + h;
+                // 256^5 per factor between the leading digit and the integer
+                g[h] = sum * (1099511627776.0 * di) * (1099511627776.0 * (j < a.N ? __ldg(a.down + j) : 0.0));
+            }
+            double2* to = reinterpret_cast<double2*>(out + c + e);
+            if (a.add) {
+                const double2 old = *to;
+                *to = make_double2(old.x + g[0], old.y + g[1]);
+            } else {
+                *to = make_double2(g[0], g[1]);
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+}
+
+constexpr size_t kGramSmem = (size_t)kStages * kStageBytes + 128;
+
+}  // namespace
+
+GramPlan gram_plan(int N, int P, int sms) {
+    GramPlan g{};
+    g.groups = (N + kTileM - 1) / kTileM * (kTileM / 8);
+    const int nt = (N + 63) / 64, last = (N + kTileM - 1) / kTileM - 1;
+    g.blocks_mn = last * (last + 1) + std::min(2 * last + 2, nt);
+    const size_t block_bytes = (size_t)g.groups * kGroupBytes;
+    const int blocks = (P + kStageK - 1) / kStageK;
+    g.chunk = (int)std::max<size_t>(1, std::min<size_t>(blocks, kGramDigitBytes / block_bytes));
+    g.chunk = (blocks + (blocks + g.chunk - 1) / g.chunk - 1) / ((blocks + g.chunk - 1) / g.chunk);   // evenly
+    // Slices of a chunk: the fewest clocks, where a stage takes 2,050 and a block's beginning and end 9,000; no more than 16,384 columns each
+    // (32-bit sums), and 24 MB of partial tiles (or one slice).
+    const size_t slice_bytes = (size_t)nt * (nt + 1) / 2 * 4096 * sizeof(double);
+    const int least = (g.chunk * kStageK + 16383) / 16384, most = std::max<int>(least, std::min<int>(16, (int)(((size_t)24 << 20) / slice_bytes)));
+    double best = 1e300;
+    for (int s = least; s <= most && s <= g.chunk; ++s) {
+        const double t = (double)(((long long)g.blocks_mn * s + sms - 1) / sms) * ((g.chunk + s - 1) / s * 2050.0 + 9000.0);
+        if (t < best) { best = t; g.slices = s; }
+    }
+    g.digit_bytes = (size_t)g.chunk * block_bytes;
+    return g;
+}
+
+cudaError_t launch_gram(const GramPlan& g, const float* F, int N, int P, const double* mu, double* up, double* down, uint8_t* digits, double* part,
+                        int* failed, cudaStream_t stream) {
+    cudaError_t e = cudaFuncSetAttribute(gram_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmem);
+    if (e != cudaSuccess) return e;
+    gram_scale_kernel<<<N, 256, 0, stream>>>(F, P, mu, up, down);
+    count_launch();
+    const int nt = (N + 63) / 64, blocks = (P + kStageK - 1) / kStageK;
+    for (int b0 = 0; b0 < blocks; b0 += g.chunk) {
+        const int nb = std::min(g.chunk, blocks - b0);
+        gram_digits_kernel<<<dim3((nb * 4 + 7) / 8, g.groups), 256, 0, stream>>>(F, N, P, b0 * kStageK, nb * 4, mu, up, g.groups, digits);
+        const GramArgs a{digits, down, part, failed, N, g.groups, nb, nt * (nt + 1) / 2, g.slices, b0 > 0 ? 1 : 0};
+        gram_mma_kernel<<<dim3(g.blocks_mn, g.slices), kGramThreads, kGramSmem, stream>>>(a);
+        count_launch(2);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace rocket

@@ -3,13 +3,13 @@
 //
 // Fit, with an intercept that is not penalised: centre the columns of F [N][P] and y, solve the dual
 // system (Fc Fc^T + alpha I) a = yc (N x N, N examples << P features), w = Fc^T a,
-// b = mean(y) - mean(F) . w.  The Gram matrix, its Cholesky factor and the two triangular solves are
+// b = mean(y) - mean(F) . w.  The Gram matrix (of larger problems by rocket_gram.cu), its Cholesky factor and the two triangular solves are
 // kept in double precision: the features are fp32 data, everything derived from them is not rounded
 // to fp32 before w and b are stored.  Every sum is taken in an order that depends on the sizes alone, so two fits
 // of the same data are bitwise identical.
 //
 // Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights take
-// 18 / 496 / 381 / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
+// 18 / 193 (in FP64 496) / 381 / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
 // 55 / 2,607 / 20,270 / 174.
 #include <cooperative_groups.h>
 
@@ -17,6 +17,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "rocket_gram.h"
 #include "rocket_internal.h"
 
 namespace rocket {
@@ -31,10 +32,10 @@ constexpr int kRWarps = kRThreads / 32;
 // eight warps share the rows; the warps' sums are added in warp order.
 //
 // mu[p] = mean over the N rows of F[.][p]; the block past the last column takes ybar = mean(y) and clears the ticket
-// the weights kernel counts its blocks with.
+// the weights kernel counts its blocks with and the flag of waits that gave up.
 __global__ void __launch_bounds__(kRThreads)
 ridge_means_kernel(const float* __restrict__ F, const float* __restrict__ y, int N, int P, double* __restrict__ mu,
-                   double* __restrict__ ybar, unsigned* __restrict__ ticket) {
+                   double* __restrict__ ybar, unsigned* __restrict__ ticket, int* __restrict__ failed) {
     __shared__ double red[kRWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool targets = (int)blockIdx.x * 32 >= P;
@@ -55,7 +56,7 @@ ridge_means_kernel(const float* __restrict__ F, const float* __restrict__ y, int
         if (targets) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) { *ybar = s / (double)N; *ticket = 0u; }
+            if (lane == 0) { *ybar = s / (double)N; *ticket = 0u; *failed = 0; }
         } else if (p < P) {
             mu[p] = s / (double)N;
         }
@@ -486,7 +487,7 @@ int status_of(cudaError_t e) {
 // per device, of at most kKeepBytes, outlives the call: a fit takes it while nobody else has it and puts it back after its
 // stream has finished; a larger or a concurrent fit allocates and frees its own.  The buffer is given back when a handle
 // of the library is destroyed and when a device allocation of the library fails (release_cached_workspaces).
-constexpr size_t kKeepBytes = (size_t)64 << 20;
+constexpr size_t kKeepBytes = (size_t)128 << 20;
 constexpr int kMaxDevices = 64;
 struct Kept { void* ptr = nullptr; size_t bytes = 0; bool taken = false; };
 std::mutex g_kept_mu;
@@ -568,39 +569,48 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     // than 40 MB of partial tiles (or one slice, 65 MB at the most examples).
     const int nt = (N + kGT - 1) / kGT, tiles = nt * (nt + 1) / 2;
     const size_t tile_bytes = (size_t)kGT * kGT * sizeof(double);
+    // Integers on the tensor cores from about 100 examples of 20,000 features on (us, FP64 and integers: 24 x 20,000 99 and 113, 97 x 3,001
+    // 111 and 121, 300 x 600 207 and 212, 100 x 20,000 166 and 155, 300 x 5,000 238 and 225, 677 x 20,000 931 and 632).
+    const bool integers = (double)N * N * P >= 1.2e8;
+    const GramPlan gram = gram_plan(N, P, sms);
     int slices = std::max(1, std::min({8 * sms / tiles, P / 128, (int)(((size_t)40 << 20) / (tile_bytes * tiles))}));
     const int slice = ((P + slices - 1) / slices + kGP - 1) / kGP * kGP;
-    slices = (P + slice - 1) / slice;
+    slices = integers ? gram.slices : (P + slice - 1) / slice;
     const int nb = (N + 1 + kCB - 1) / kCB, Np = nb * kCB;
     // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Ld[nb][32][32], partial Gram tiles, ticket, status
     size_t off = 0;
     auto take = [&](size_t doubles) { const size_t o = off; off += (doubles + 31) / 32 * 32; return o; };
     const size_t o_mu = take(P), o_a = take(N), o_part = take(col_blocks), o_ybar = take(1), o_G = take((size_t)Np * Np);
     const size_t o_Ld = take((size_t)nb * kCB * kCB), o_gram = take((size_t)slices * tiles * kGT * kGT), o_int = take(2);
+    const size_t o_up = take(integers ? N : 0), o_down = take(integers ? N : 0), o_digits = take(integers ? gram.digit_bytes / sizeof(double) : 0);
     const size_t bytes = off * sizeof(double);
     FitWorkspace ws;
     if ((e = ws.take(bytes)) != cudaSuccess) return status_of(e);
     double* d = static_cast<double*>(ws.ptr);
     unsigned* ticket = reinterpret_cast<unsigned*>(d + o_int);
     int* status = reinterpret_cast<int*>(d + o_int + 1);
-    ridge_means_kernel<<<col_blocks + 1, kRThreads, 0, stream>>>(feat_dev, y_dev, N, P, d + o_mu, d + o_ybar, ticket);
-    ridge_gram_kernel<<<dim3(tiles, slices), kGThreads, gram_smem, stream>>>(feat_dev, N, P, d + o_mu, slice, d + o_gram);
+    ridge_means_kernel<<<col_blocks + 1, kRThreads, 0, stream>>>(feat_dev, y_dev, N, P, d + o_mu, d + o_ybar, ticket, status + 1);
+    if (integers)
+        e = launch_gram(gram, feat_dev, N, P, d + o_mu, d + o_up, d + o_down, reinterpret_cast<uint8_t*>(d + o_digits), d + o_gram, status + 1, stream);
+    else
+        ridge_gram_kernel<<<dim3(tiles, slices), kGThreads, gram_smem, stream>>>(feat_dev, N, P, d + o_mu, slice, d + o_gram);
     CholArgs q{d + o_gram, slices, tiles, (double)alpha, y_dev, d + o_ybar, d + o_G, d + o_Ld, d + o_a, status, N, Np};
     void* args[] = {&q};
     // one block per SM: more would lengthen the grid barriers without shortening the chain
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(ridge_cholesky_solve_kernel),
+    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(ridge_cholesky_solve_kernel),
                                     dim3((unsigned)std::max(1, std::min(sms, nb * (nb + 1) / 2))), dim3(kCThreads), args, 0, stream);
     ridge_weights_kernel<<<col_blocks, kRThreads, 0, stream>>>(feat_dev, N, P, d + o_mu, d + o_a, d + o_ybar, w_dev, b_dev,
                                                                d + o_part, ticket);
     count_launch(4);
-    int host_status = 0;
+    int host_status[2] = {0, 0};
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&host_status, status, sizeof(int), cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(host_status, status, sizeof(host_status), cudaMemcpyDeviceToHost, stream);
     const cudaError_t done = cudaStreamSynchronize(stream);
     ws.put_back(bytes);
     if (e == cudaSuccess) e = done;
     if (e != cudaSuccess) return status_of(e);
-    return host_status == 0 ? ROCKET_OK : ROCKET_EINVAL;
+    if (host_status[1] != 0) return ROCKET_ECUDA;
+    return host_status[0] == 0 ? ROCKET_OK : ROCKET_EINVAL;
 }
 
 extern "C" int rocket_ridge_predict(const float* feat_dev, int N, int P, const float* w_dev, const float* b_dev,
