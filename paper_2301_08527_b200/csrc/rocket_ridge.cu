@@ -9,7 +9,7 @@
 // of the same data are bitwise identical.
 //
 // Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights take
-// 18 / 193 (in FP64 496) / 381 / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
+// 18 / 193 (in FP64 496) / 240 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
 // 55 / 2,607 / 20,270 / 174.
 #include <cooperative_groups.h>
 
@@ -144,12 +144,12 @@ ridge_gram_kernel(const float* __restrict__ F, int N, int P, const double* __res
 
 // ---- Cholesky factor and solves -------------------------------------------------------------------------------
 // G [Np][Np] (Np a multiple of 32 above N) holds the lower triangle of Fc Fc^T + alpha I, row N holds yc^T, rows below are
-// zero: the factorisation then leaves z = L^-1 yc in row N by itself.  Blocks of 32 x 32, right-looking: at step kb every
-// block of the grid factors the diagonal block for itself (one warp, a row per lane), solves the two panel blocks its
-// tile needs and updates the tile, so that a step takes one grid-wide barrier and no panel travels between barriers.
-// Solved panel blocks go transposed into the upper triangle, diagonal factors into Ld.  Bound: the chain of steps (22 of
-// them at N = 677; a diagonal block is 32 dependent pivots), not arithmetic.
-constexpr int kCB = 32, kCThreads = 256, kCPitch = kCB + 1, kDPitch = kCB + 2;
+// zero: the factorisation then leaves z = L^-1 yc in row N by itself.  Blocks of 32 x 32, right-looking, one grid-wide barrier per
+// step: block 0 updates the next diagonal block first and factors it while the others update the rest, and what it passes on is the
+// inverse of the factor, so that the panel blocks a tile needs are products that 256 threads share.  Solved panel blocks go transposed
+// into the upper triangle, inverse factors into Mi.  Bound: block 0's chain of 32 dependent pivots per step (22 steps at N = 677).
+constexpr int kCB = 32, kCThreads = 256, kCPitch = kCB + 4, kDPitch = kCB + 2;
+constexpr int kCSmem = kCB * kDPitch + 4 * kCB * kCPitch;              // doubles: a factor and four blocks; in the end the solution besides
 
 struct CholArgs {
     const double* part;       // partial Gram tiles [slices][tiles][64][64]
@@ -158,70 +158,105 @@ struct CholArgs {
     const float* y;
     const double* ybar;
     double* G;
-    double* Ld;               // diagonal factors [nb][32][32]
+    double* Mi;               // inverse factors of the diagonal blocks, transposed [nb][32][32]
+    double* z;                // row N of the factor, by blocks
     double* a;                // solution [N]
     int* status;              // 0 = ok, 1 = a pivot was not positive
     int N, Np;
 };
 
-// Factors the leading `ncols` columns of the block whose rows are held by the lanes (s[lane][0 .. lane]); the factor's
-// transpose goes to t (t[j][c] = L[c][j]), the reciprocal pivots to rinv.  One warp.
-__device__ __forceinline__ bool chol_factor_block(const double (*s)[kCPitch], double (*t)[kDPitch], double* rinv, int ncols,
-                                                  int lane) {
-    double a[kCB];
+// 1 / sqrt(d) for a normal d > 0: an approximation with about 20 good bits and one step of Householder's third-order method,
+// y (1 + e / 2 + 3 e^2 / 8) with e = 1 - d y^2, whose error is of the order of e^3.
+__device__ __forceinline__ double inverse_root(double d) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// Factors the leading `ncols` columns of the block whose rows are held by the lanes (s[lane][0 .. lane]) and inverts the factor: row r
+// of the inverse's transpose goes to m[r]; lane j returns in root the reciprocal of the factor's diagonal j, and t[j] holds column j of
+// the factor times that diagonal.  One warp.
+//
+// A double-precision operation takes some 40 clocks here, so what counts is how many of them lie between a pivot and the next.  The
+// elimination is square-root free (a_ik -= c_ij c_kj / d_j with unscaled columns c), 1 / d_j is y (1 + e + e^2) for an approximation y
+// of 20 bits and e = 1 - d_j y, and the next pivot's column takes a - g - g (e + e^2) with g = c_ij c_kj y ready by then: three operations after the approximation.
+// With the factor's own columns and 1 / sqrt(d_j) they were six: 10,800 clocks for a block, 8,400 now.  (One body for all pivots, the rows
+// moving down by a column each time, has twice the multiply-adds: 13,700.)
+__device__ __forceinline__ bool chol_factor_block(const double (*s)[kCPitch], double (*t)[kDPitch], double (*m)[kCPitch], int ncols, int lane, double& root) {
+    double a[kCB], x[kCB], mine = 1.0;
     bool good = true;
 #pragma unroll
-    for (int c = 0; c < kCB; ++c) a[c] = s[lane][c];
+    for (int c = 0; c < kCB; ++c) {
+        a[c] = s[lane][c];
+        x[c] = c == lane ? 1.0 : 0.0;
+    }
+    __syncwarp();
 #pragma unroll
     for (int j = 0; j < kCB; ++j) {
-        if (j < ncols) {
-            double d = __shfl_sync(0xffffffffu, a[j], j);
-            if (!(d > 0.0)) { good = false; d = 1.0; }
-            const double r = rsqrt(d);
-            const double l = lane == j ? d * r : a[j] * r;
-            t[j][lane] = lane >= j ? l : 0.0;
-            if (lane == 0) rinv[j] = r;
-            __syncwarp();
+        const bool there = j < ncols;
+        double d = __shfl_sync(0xffffffffu, a[j], j), y;
+        good = good && (!there || d >= 2.2250738585072014e-308);
+        d = there && d >= 2.2250738585072014e-308 ? d : 1.0;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+        const double col = there && lane >= j ? a[j] : 0.0;
+        if (lane == j) mine = d;
+        t[j][lane] = col;
+        const double e = fma(-d, y, 1.0), p = fma(e, e, e), cy = col * y;
+        if (j + 1 < kCB) {                             // what the next pivot waits for
+            const double next = __shfl_sync(0xffffffffu, col, j + 1), g = cy * next;
+            a[j + 1] = fma(-g, p, a[j + 1] - g);
+        }
+        __syncwarp();
+        const double f = fma(cy, p, cy), xy = x[j] * y, xs = there ? fma(xy, p, xy) : 0.0;
+        if (j + 1 < kCB) x[j + 1] = fma(-xs, t[j][j + 1], x[j + 1]);
 #pragma unroll
-            for (int c = j + 1; c < kCB; ++c) a[c] -= l * t[j][c];
+        for (int c = j + 2; c < kCB; ++c) {
+            const double lc = t[j][c];
+            a[c] = fma(-f, lc, a[c]);
+            x[c] = fma(-xs, lc, x[c]);
         }
     }
+    root = inverse_root(mine);
+#pragma unroll
+    for (int c = 0; c < kCB; ++c) m[lane][c] = x[c] * __shfl_sync(0xffffffffu, root, c);
     __syncwarp();
     return good;
 }
 
-// Row `lane` of a panel block: x L^T = g, in place.  One warp.
-__device__ __forceinline__ void chol_solve_row(double (*p)[kCPitch], const double (*t)[kDPitch], const double* rinv, int lane) {
-    double g[kCB];
-#pragma unroll
-    for (int c = 0; c < kCB; ++c) g[c] = p[lane][c];
-#pragma unroll
-    for (int j = 0; j < kCB; ++j) {
-        const double x = g[j] * rinv[j];
-        g[j] = x;
-#pragma unroll
-        for (int c = j + 1; c < kCB; ++c) g[c] -= x * t[j][c];
-    }
-#pragma unroll
-    for (int c = 0; c < kCB; ++c) p[lane][c] = g[c];
+__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
 }
 
 __global__ void __launch_bounds__(kCThreads)
 ridge_cholesky_solve_kernel(CholArgs q) {
-    __shared__ double s_t[kCB][kDPitch];
-    __shared__ double s_rinv[kCB];
-    __shared__ double s_raw[ROCKET_RIDGE_MAX_EXAMPLES];      // the panel blocks; in the end the solution
-    static_assert(2 * kCB * kCPitch <= ROCKET_RIDGE_MAX_EXAMPLES, "two panel blocks fit");
-    double (*s_pi)[kCPitch] = reinterpret_cast<double (*)[kCPitch]>(s_raw);
-    double (*s_pj)[kCPitch] = s_pi + kCB;
+    extern __shared__ double smem[];
+    double (*s_t)[kDPitch] = reinterpret_cast<double (*)[kDPitch]>(smem);
+    double (*s_m)[kCPitch] = reinterpret_cast<double (*)[kCPitch]>(smem + kCB * kDPitch), (*s_pi)[kCPitch] = s_m + kCB, (*s_pj)[kCPitch] = s_pi + kCB;
     cg::grid_group grid = cg::this_grid();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = q.N, Np = q.Np, nb = Np / kCB;
+    const int fr = lane >> 2, fk = lane & 3, br = warp >> 1, bc = (warp & 1) * 2;   // a warp's two 8 x 8 fragments of a block
     double* __restrict__ G = q.G;
+    bool good = true;
 
-    // lower blocks of G from the partial tiles, in slice order
-    const int blocks = nb * (nb + 1) / 2;
-    for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
+    // the inverse factor of diagonal block kb, whose elements are in s_pi (block 0)
+    auto factor = [&](int kb) {
+        const int ncols = min(kCB, N - kb * kCB);
+        double root = 0.0;
+        if (ncols > 0 && warp == 0) good = chol_factor_block(s_pi, s_t, s_m, ncols, lane, root) && good;
+        __syncthreads();
+        if (ncols > 0)
+            for (int e = tid; e < kCB * kCB; e += kCThreads) q.Mi[(size_t)kb * kCB * kCB + e] = s_m[e / kCB][e % kCB];
+        // row N of the factor: within its own diagonal block the factor's rows are not kept elsewhere
+        if (kb == N / kCB && tid < ncols) q.z[kb * kCB + tid] = s_t[tid][N - kb * kCB] * root;
+        __syncthreads();
+    };
+
+    // lower blocks of G from the partial tiles, in slice order; block 0 takes the first diagonal block only, and factors it meanwhile (the
+    // first run through that code takes 20,000 clocks longer than the others)
+    const int blocks = nb * (nb + 1) / 2, helpers = (int)gridDim.x - 1;
+    for (int b = blockIdx.x; b < (blockIdx.x == 0 && helpers > 0 ? 1 : blocks); b += max(1, helpers)) {
         int ib = (int)((sqrtf(8.0f * (float)b + 1.0f) - 1.0f) * 0.5f);
         while (ib * (ib + 1) / 2 > b) --ib;
         while ((ib + 1) * (ib + 2) / 2 <= b) ++ib;
@@ -239,101 +274,181 @@ ridge_cholesky_solve_kernel(CholArgs q) {
                 g = (double)q.y[j] - *q.ybar;
             }
             G[(size_t)i * Np + j] = g;
+            if (b == 0) s_pi[e / kCB][e % kCB] = g;
         }
     }
     if (blockIdx.x == 0 && tid == 0) *q.status = 0;
-    grid.sync();
+    __syncthreads();
 
-    bool good = true;
-    for (int kb = 0; kb < nb; ++kb) {
-        const int k0 = kb * kCB, ncols = min(kCB, N - k0);
-        const int rest = nb - kb - 1, tiles = rest * (rest + 1) / 2;
-        if (ncols > 0 && ((int)blockIdx.x < tiles || blockIdx.x == 0)) {
-            for (int e = tid; e < kCB * kCB; e += kCThreads) s_pi[e / kCB][e % kCB] = G[(size_t)(k0 + e / kCB) * Np + k0 + e % kCB];
-            __syncthreads();
-            if (warp == 0) good = chol_factor_block(s_pi, s_t, s_rinv, ncols, lane) && good;
-            __syncthreads();
-            if (blockIdx.x == 0)
-                for (int e = tid; e < kCB * kCB; e += kCThreads)
-                    q.Ld[(size_t)kb * kCB * kCB + e] = s_t[e % kCB][e / kCB];    // Ld[r][c] = L[r][c], read below r's diagonal only
-            for (int b = blockIdx.x; b < tiles; b += gridDim.x) {
+    // step -1 only factors the first diagonal block, so that there is one copy of that code: the first run through a second one took
+    // 40,000 clocks
+    for (int kb = -1; kb + 1 < nb; ++kb) {
+        const int k0 = kb * kCB, rest = nb - kb - 1, tiles = rest * (rest + 1) / 2;
+        // block 0 takes the next diagonal block, which is tile 0, and no other unless it is alone; the others share the rest
+        const int step = gridDim.x > 1 ? (int)gridDim.x - 1 : 1;
+        const int first = blockIdx.x, limit = kb < 0 ? (blockIdx.x == 0 ? 1 : 0) : blockIdx.x == 0 && gridDim.x > 1 ? 1 : tiles;
+        for (int b = first; b < limit; b += step) {
+            if (kb >= 0) {
                 // tile (ib, jb) of the trailing blocks, column by column so that the first ones are the panel's own
                 int x = (int)((sqrtf(8.0f * (float)(tiles - 1 - b) + 1.0f) - 1.0f) * 0.5f);
                 while (x * (x + 1) / 2 > tiles - 1 - b) --x;
                 while ((x + 1) * (x + 2) / 2 <= tiles - 1 - b) ++x;
                 const int jb = nb - 1 - x, ib = nb - 1 - ((tiles - 1 - b) - x * (x + 1) / 2);
                 const int i0 = ib * kCB, j0 = jb * kCB;
-                for (int e = tid; e < kCB * kCB; e += kCThreads) {
-                    const int r = e / kCB, c = e % kCB;
-                    s_pi[r][c] = G[(size_t)(i0 + r) * Np + k0 + c];
-                    if (ib != jb) s_pj[r][c] = G[(size_t)(j0 + r) * Np + k0 + c];
-                }
-                const int ty = tid / 16, tx = tid % 16;
-                double g[2][2];
+                const bool two = ib != jb;
+                // all loads of the tile at once: inverse factor, panel blocks, the warp's fragments of the tile (rows fr of row block 8 br,
+                // columns 2 fk, 2 fk + 1 of column blocks 8 bc and 8 (bc + 1))
+                constexpr int kEach = kCB * kCB / kCThreads;
+                double lm[kEach], li[kEach], lj[kEach], g[2][2];
 #pragma unroll
-                for (int u = 0; u < 2; ++u)
-#pragma unroll
-                    for (int v = 0; v < 2; ++v) g[u][v] = G[(size_t)(i0 + ty + 16 * u) * Np + j0 + tx + 16 * v];
-                __syncthreads();
-                if (warp == 0) chol_solve_row(s_pi, s_t, s_rinv, lane);
-                else if (warp == 1 && ib != jb) chol_solve_row(s_pj, s_t, s_rinv, lane);
-                __syncthreads();
-                const double (*pj)[kCPitch] = ib != jb ? s_pj : s_pi;
-#pragma unroll 8
-                for (int k = 0; k < kCB; ++k) {
-                    const double a0 = s_pi[ty][k], a1 = s_pi[ty + 16][k], b0 = pj[tx][k], b1 = pj[tx + 16][k];
-                    g[0][0] -= a0 * b0; g[0][1] -= a0 * b1; g[1][0] -= a1 * b0; g[1][1] -= a1 * b1;
+                for (int u = 0; u < kEach; ++u) {
+                    const int e = tid + u * kCThreads, r = e / kCB, c = e % kCB;
+                    lm[u] = __ldcg(q.Mi + (size_t)kb * kCB * kCB + e);
+                    li[u] = __ldcg(G + (size_t)(i0 + r) * Np + k0 + c);
+                    lj[u] = two ? __ldcg(G + (size_t)(j0 + r) * Np + k0 + c) : 0.0;
                 }
 #pragma unroll
-                for (int u = 0; u < 2; ++u)
+                for (int v = 0; v < 2; ++v) {
+                    const double2 w = __ldcg(reinterpret_cast<const double2*>(G + (size_t)(i0 + 8 * br + fr) * Np + j0 + 8 * (bc + v) + 2 * fk));
+                    g[v][0] = w.x; g[v][1] = w.y;
+                }
 #pragma unroll
-                    for (int v = 0; v < 2; ++v) G[(size_t)(i0 + ty + 16 * u) * Np + j0 + tx + 16 * v] = g[u][v];
-                if (jb == kb + 1)
+                for (int u = 0; u < kEach; ++u) {
+                    const int e = tid + u * kCThreads, r = e / kCB, c = e % kCB;
+                    s_m[r][c] = lm[u];
+                    s_pi[r][c] = li[u];
+                    if (two) s_pj[r][c] = lj[u];
+                }
+                double pi[2][2] = {}, pj[2][2] = {}, h0[2][2] = {}, h1[2][2] = {};   // a matrix instruction takes long, too: two sums for every fragment
+                __syncthreads();
+                // the solved panel blocks: rows of G times the inverse factor's transpose
+#pragma unroll
+                for (int k = 0; k < kCB; k += 4) {
+                    const double x = s_pi[8 * br + fr][k + fk], y = two ? s_pj[8 * br + fr][k + fk] : 0.0;
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) {
+                        const double m = s_m[k + fk][8 * (bc + v) + fr];
+                        dmma(k & 4 ? h0[v] : pi[v], x, m);
+                        if (two) dmma(k & 4 ? h1[v] : pj[v], y, m);
+                    }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int v = 0; v < 2; ++v)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        s_pi[8 * br + fr][8 * (bc + v) + 2 * fk + h] = pi[v][h] + h0[v][h];
+                        if (two) s_pj[8 * br + fr][8 * (bc + v) + 2 * fk + h] = pj[v][h] + h1[v][h];
+                        h0[v][h] = 0.0;
+                    }
+                __syncthreads();
+                const double (*sj)[kCPitch] = two ? s_pj : s_pi;
+#pragma unroll
+                for (int k = 0; k < kCB; k += 4) {
+                    const double x = -s_pi[8 * br + fr][k + fk];
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) dmma(k & 4 ? h0[v] : g[v], x, sj[8 * (bc + v) + fr][k + fk]);
+                }
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    g[v][0] += h0[v][0];
+                    g[v][1] += h0[v][1];
+                    *reinterpret_cast<double2*>(G + (size_t)(i0 + 8 * br + fr) * Np + j0 + 8 * (bc + v) + 2 * fk) = make_double2(g[v][0], g[v][1]);
+                }
+                if (jb == kb + 1) {
                     for (int e = tid; e < kCB * kCB; e += kCThreads) G[(size_t)(k0 + e / kCB) * Np + i0 + e % kCB] = s_pi[e % kCB][e / kCB];
+                    if (i0 <= N && N < i0 + kCB && tid < kCB) q.z[k0 + tid] = s_pi[N - i0][tid];
+                }
                 __syncthreads();
+                if (b == 0) {                                // the next diagonal block, whole
+#pragma unroll
+                    for (int v = 0; v < 2; ++v)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) s_pi[8 * br + fr][8 * (bc + v) + 2 * fk + h] = g[v][h];
+                    __syncthreads();
+                }
             }
+            if (b == 0) factor(kb + 1);                      // before the barrier
         }
-        if (rest > 0) grid.sync();
+        grid.sync();
     }
     if (blockIdx.x != 0) return;
 
-    // L^T a = z, from the last block up.  Row k0 + j of the upper triangle holds L's column: a warp per row takes the
-    // part below the diagonal block, one warp solves the diagonal block.
+    // L^T a = z, from the last block up: a_kb = M_kb (z_kb - sum of L_i,kb^T a_i over the blocks i below).  Row k0 + j of the upper
+    // triangle holds L's column.  The first warp finishes a block from what the others brought in and summed a phase earlier: the inverse factor, the
+    // block of L next to the diagonal, and the part of the sums whose a_i were known then.
     if (warp == 0 && lane == 0 && !good) *q.status = 1;
-    __syncthreads();
-    double* s_a = s_raw;
+    __shared__ double s_sum[2][kCB];
+    double (*s_inv)[kCPitch] = s_m, (*s_next)[kCPitch] = s_m + 2 * kCB;   // two of each
+    double* s_a = reinterpret_cast<double*>(s_m + 4 * kCB);
     const int nblk = (N + kCB - 1) / kCB;
-    for (int kb = nblk - 1; kb >= 0; --kb) {
-        const int k0 = kb * kCB, ncols = min(kCB, N - k0);
-        for (int e = tid; e < kCB * kCB; e += kCThreads) s_t[e / kCB][e % kCB] = q.Ld[(size_t)kb * kCB * kCB + e];   // s_t[r][c] = L[r][c]
-        double sum[kCB / (kCThreads / 32)];
+    constexpr int kHelpers = kCThreads / 32 - 1;
+    auto bring = [&](int kb) {                               // for block kb, by warps 1 .. 7, while a of blocks above kb + 1 is known
+        const int k0 = kb * kCB, buf = kb & 1, w = warp - 1;
+        constexpr int kEach = (kCB * kCB + kCThreads - 33) / (kCThreads - 32);
+        double inv[kEach], next[kEach];
 #pragma unroll
-        for (int u = 0; u < kCB / (kCThreads / 32); ++u) sum[u] = 0.0;
-        for (int i = k0 + kCB + lane; i < N; i += 32) {
+        for (int u = 0; u < kEach; ++u) {
+            const int e = min(tid - 32 + u * (kCThreads - 32), kCB * kCB - 1), r = e / kCB, c = e % kCB;
+            inv[u] = __ldcg(q.Mi + (size_t)kb * kCB * kCB + e);
+            next[u] = __ldcg(G + (size_t)(k0 + r) * Np + min(k0 + kCB + c, Np - 1));   // past column N: not used
+        }
+        // five rows a warp, side by side: what counts is how many loads are on their way
+        constexpr int kRows = (kCB + kHelpers - 1) / kHelpers;
+        double sum[kRows];
+        const double* row[kRows];
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+            sum[u] = 0.0;
+            row[u] = G + (size_t)min(k0 + w + kHelpers * u, N - 1) * Np;   // rows past the last are not used
+        }
+#pragma unroll 4
+        for (int i = k0 + 2 * kCB + lane; i < N; i += 32) {
             const double ai = s_a[i];
 #pragma unroll
-            for (int u = 0; u < kCB / (kCThreads / 32); ++u)
-                sum[u] += G[(size_t)(k0 + warp + (kCThreads / 32) * u) * Np + i] * ai;
+            for (int u = 0; u < kRows; ++u) sum[u] += __ldcg(row[u] + i) * ai;
         }
 #pragma unroll
-        for (int u = 0; u < kCB / (kCThreads / 32); ++u) {
+        for (int u = 0; u < kRows; ++u) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], o);
-            if (lane == 0) s_rinv[warp + (kCThreads / 32) * u] = sum[u];
+            if (lane == 0 && w + kHelpers * u < kCB) s_sum[buf][w + kHelpers * u] = sum[u];
         }
-        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) {
+            const int e = min(tid - 32 + u * (kCThreads - 32), kCB * kCB - 1), r = e / kCB, c = e % kCB;
+            s_inv[buf * kCB + r][c] = inv[u];
+            s_next[buf * kCB + r][c] = next[u];
+        }
+    };
+    __syncthreads();
+    if (warp > 0) bring(nblk - 1);
+    __syncthreads();
+    for (int kb = nblk - 1; kb >= 0; --kb) {
+        const int k0 = kb * kCB, ncols = min(kCB, N - k0), buf = kb & 1;
         if (warp == 0) {
-            double z = 0.0;
-            if (lane < ncols) z = (N / kCB == kb ? q.Ld[(size_t)kb * kCB * kCB + (N - k0) * kCB + lane] : G[(size_t)(k0 + lane) * Np + N]);
-            double v = lane < ncols ? z - s_rinv[lane] : 0.0;
-            const double inv = lane < ncols ? 1.0 / s_t[lane][lane] : 0.0;
+            double v = 0.0;
+            if (lane < ncols) {
+                v = __ldcg(q.z + k0 + lane) - s_sum[buf][lane];
+                const int below = min(kCB, N - k0 - kCB);
+                double u[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 4
-            for (int j = ncols - 1; j >= 0; --j) {
-                const double aj = __shfl_sync(0xffffffffu, v * inv, j);
-                if (lane == j) v = aj;
-                else if (lane < j) v -= s_t[j][lane] * aj;
+                for (int c = 0; c < below; ++c) u[c & 3] += s_next[buf * kCB + lane][c] * s_a[k0 + kCB + c];
+                v -= (u[0] + u[1]) + (u[2] + u[3]);
             }
-            if (lane < ncols) { s_a[k0 + lane] = v; q.a[k0 + lane] = v; }
+            __syncwarp();
+            s_t[0][lane] = v;
+            __syncwarp();
+            double u[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int c = 0; c < kCB; ++c) u[c & 3] += s_inv[buf * kCB + lane][c] * s_t[0][c];
+            if (lane < ncols) {
+                const double a = (u[0] + u[1]) + (u[2] + u[3]);
+                s_a[k0 + lane] = a;
+                q.a[k0 + lane] = a;
+            }
+        } else if (kb > 0) {
+            bring(kb - 1);
         }
         __syncthreads();
     }
@@ -563,6 +678,8 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t gram_smem = (size_t)2 * kGT * kGPitch * sizeof(double);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(ridge_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem);
+    const size_t chol_smem = (size_t)(kCSmem + N) * sizeof(double);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ridge_cholesky_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)((kCSmem + ROCKET_RIDGE_MAX_EXAMPLES) * sizeof(double)));
     if (e != cudaSuccess) return status_of(e);
     const int col_blocks = (P + 31) / 32;
     // Slices of the feature axis: about two waves of the four blocks an SM holds, at least 128 columns each, and no more
@@ -577,11 +694,11 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     const int slice = ((P + slices - 1) / slices + kGP - 1) / kGP * kGP;
     slices = integers ? gram.slices : (P + slice - 1) / slice;
     const int nb = (N + 1 + kCB - 1) / kCB, Np = nb * kCB;
-    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Ld[nb][32][32], partial Gram tiles, ticket, status
+    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Mi[nb][32][32], z[Np], partial Gram tiles, ticket, status
     size_t off = 0;
     auto take = [&](size_t doubles) { const size_t o = off; off += (doubles + 31) / 32 * 32; return o; };
     const size_t o_mu = take(P), o_a = take(N), o_part = take(col_blocks), o_ybar = take(1), o_G = take((size_t)Np * Np);
-    const size_t o_Ld = take((size_t)nb * kCB * kCB), o_gram = take((size_t)slices * tiles * kGT * kGT), o_int = take(2);
+    const size_t o_Mi = take((size_t)nb * kCB * kCB), o_z = take(Np), o_gram = take((size_t)slices * tiles * kGT * kGT), o_int = take(2);
     const size_t o_up = take(integers ? N : 0), o_down = take(integers ? N : 0), o_digits = take(integers ? gram.digit_bytes / sizeof(double) : 0);
     const size_t bytes = off * sizeof(double);
     FitWorkspace ws;
@@ -594,11 +711,11 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
         e = launch_gram(gram, feat_dev, N, P, d + o_mu, d + o_up, d + o_down, reinterpret_cast<uint8_t*>(d + o_digits), d + o_gram, status + 1, stream);
     else
         ridge_gram_kernel<<<dim3(tiles, slices), kGThreads, gram_smem, stream>>>(feat_dev, N, P, d + o_mu, slice, d + o_gram);
-    CholArgs q{d + o_gram, slices, tiles, (double)alpha, y_dev, d + o_ybar, d + o_G, d + o_Ld, d + o_a, status, N, Np};
+    CholArgs q{d + o_gram, slices, tiles, (double)alpha, y_dev, d + o_ybar, d + o_G, d + o_Mi, d + o_z, d + o_a, status, N, Np};
     void* args[] = {&q};
     // one block per SM: more would lengthen the grid barriers without shortening the chain
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(ridge_cholesky_solve_kernel),
-                                    dim3((unsigned)std::max(1, std::min(sms, nb * (nb + 1) / 2))), dim3(kCThreads), args, 0, stream);
+                                    dim3((unsigned)std::max(1, std::min(sms, nb * (nb + 1) / 2))), dim3(kCThreads), args, chol_smem, stream);
     ridge_weights_kernel<<<col_blocks, kRThreads, 0, stream>>>(feat_dev, N, P, d + o_mu, d + o_a, d + o_ybar, w_dev, b_dev,
                                                                d + o_part, ticket);
     count_launch(4);
