@@ -145,17 +145,23 @@ bool no_room(cudaError_t e) {
     return true;
 }
 
+// Whether every fused call of the handle is a matter of one kernel, or of tiles of at most kSMaxPlanes channels: no call of such a handle is
+// better served by the generic kernels.
+bool always_fused(const rocket_params* p, bool backward) {
+    return p->host.C <= fast::kSMaxPlanes || (backward ? fast::resident_backward(p->fast->host) : p->fast->host.resident);
+}
+
 // Whether the fused kernels serve a call of N examples (with the handle's kernels that they take).
-bool fused_call(const rocket_params* p, bool aligned, int N, bool soft) {
+bool fused_call(const rocket_params* p, bool aligned, int N, bool soft, bool backward = false) {
     if (p->path != 0 || !p->fast->host.enabled || !aligned) return false;
-    if (p->host.C <= fast::kSMaxPlanes || N == 0) return true;
+    if (always_fused(p, backward) || N == 0) return true;
     return !fast::generic_pays(p->fast->host, N, p->fast->sms, soft);
 }
 
 // A call covers every smaller one of its kind, also those that take the other kernels: their workspace is made with it.  Without room
 // for it they find that out themselves.
 void cover_smaller_calls(const rocket_params* p, int N, bool soft, bool backward, bool fused) {
-    if (p->path != 0 || !p->fast->host.enabled || p->host.C <= fast::kSMaxPlanes || N < 2) return;
+    if (p->path != 0 || !p->fast->host.enabled || always_fused(p, backward) || N < 2) return;
     const int n = fast::pays_up_to(p->fast->host, N - 1, p->fast->sms, soft || backward, fused);
     if (n == 0) return;
     const int64_t nW = n_weights_of(p);
@@ -395,7 +401,7 @@ int rocket_params_reserve(rocket_params_t* p, int max_N, int passes) {
     // kernels outside the fused path: the backward's per-example partial sums; 8-bit input: its fp32 copy
     const bool some_generic = !fused || !p->fast->host.generic_list.empty() || p->path == 1;
     int generic_N = some_generic ? max_N : 0;
-    if (!some_generic && p->host.C > fast::kSMaxPlanes) generic_N = fast::pays_up_to(p->fast->host, max_N, p->fast->sms, true, true);
+    if (!some_generic && !always_fused(p, backward)) generic_N = fast::pays_up_to(p->fast->host, max_N, p->fast->sms, true, true);
     if (backward && generic_N > 0) {
         cudaError_t e = p->scratch.reserve(generic_backward_scratch_floats(generic_N, nW, p->host.K) * sizeof(float));
         if (e != cudaSuccess) return cuda_status(e);
@@ -547,7 +553,7 @@ int rocket_transform_soft_backward(const rocket_params_t* p, const float* X_dev,
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const int64_t nW = n_weights_of(p);
     const bool aligned = (reinterpret_cast<uintptr_t>(X_dev) & 3u) == 0;
-    bool use_fast = fused_call(p, aligned || N == 0, N, true);
+    bool use_fast = fused_call(p, aligned || N == 0, N, true, true);
     cover_smaller_calls(p, N, false, true, use_fast);
     if (use_fast) {   // the fused kernels assign dW / db of the kernels they serve
         cudaError_t e = fast::launch_fast_backward(*p->fast, p->dp, nW, X_dev, N, lambda, shift, dfeat_dev, argmax_dev,

@@ -228,8 +228,49 @@ ROCKET_CX int w_rows_per_y(int d) { return d % 4 == 0 ? 1 : d % 4 == 2 ? 2 : 4; 
 // One tensor map: boxes of box_cols x box_rows floats over runs of 4 * d floats.
 struct TMapSpec { int32_t d, box_cols, box_rows; };
 
+// ---- resident regime (rocket_resident.cu): short series, whole examples in shared memory ------
+// Heights of its bands.  Odd: neighbouring columns of a band row lie side by side and those of the next band an odd number of rows further on, so
+// that a warp's loads meet few times in a shared-memory bank, at dilation 1 too, where 16 rows would meet sixteen times.  The low ones (small)
+// where series are too short for the others' 64 columns.  Measured, hard, us: 100 x 1 x 64 and 5,000 kernels 329 with 17 and 11 rows, 289
+// with 15 and 9; 100 x 6 x 1,251 1,261 and 1,274 (17 and 9: 1,322).
+ROCKET_CX int resident_high(bool small) { return small ? 9 : 17; }
+ROCKET_CX int resident_low(bool small) { return small ? 5 : 11; }
+// Warps of a block (mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half precision).
+ROCKET_CX int resident_warps(int mode, bool small) { return mode == 2 ? 16 : mode == 1 ? 20 : small ? 28 : 24; }
+constexpr int kRMostFloats = 57600;                                // what shared memory holds: examples, rows padded to 16 bytes
+// The longest series: beyond, a pair is a warp's for too long where there are few, and the other kernels' larger tiles are as good where there
+// are many (us, before and with this kernel: 1 x 3 x 5,000, 10,000 kernels 192 and 97, 100 x 3 x 5,000, 5,000 kernels 2,825 and 2,842; 8 x 3 x
+// 18,000, 1,000 kernels 205 and 257).  The second where tiles test their reads (24 x 32 x 1,751, 2,000 kernels 477 and 218; 8 x 9 x 6,000,
+// 1,000 kernels 142 and 240).
+constexpr int kRMostSteps = 5000, kRMostStepsTested = 2048, kRMostStepsBackward = 1000;
+constexpr int kRSmallSteps = 1024;                                 // series to be short for the low bands
+constexpr int kRMostOutputs = 1 << 20;                             // outputs and dilation up to which columns are counted exactly in FP32
+
+// One kernel (32 words).  Its outputs, counted from the first one, are t d + r for t < nq + (r < nr); the input rows of column r that
+// are samples, or zeros next to them in shared memory, are t from pq + (r < pr) to lq + (r < lr), exclusive.
+struct alignas(16) RUnit {
+    int32_t krec, k, len, d;
+    int32_t m, nout, p, high;             // high, low: bands of the greater height, then bands of the lesser
+    int32_t low, nq, nr, pq;
+    int32_t pr, lq, lr;
+    float inv_d;
+    uint8_t ch[12];
+    int32_t woff, pad_[12];
+};
+static_assert(sizeof(RUnit) == 128, "RUnit must be 32 words");
+// How a call of N examples is dealt to the blocks: tasks of `examples` examples and every parts-th kernel, of which a warp takes one for
+// `run` of the examples at a time, or for one of them every split-th tile.
+struct ResidentSplit { int examples, groups, parts, run, split; unsigned grid; };
+
 struct PlanHost {
     bool enabled = false;
+    bool resident = false;                // the examples fit the resident kernel's shared memory
+    bool r_small = false;                 // its bands are the low ones
+    bool r_zeros = false;                 // and so do zeros around every row, as far as any tile reads
+    std::vector<RUnit> runits;
+    int r_front = 0, r_pitch = 0;         // floats of zeros in front of the first channel row in shared memory; from row to row
+    int r_tiles = 0;                      // most tiles of a kernel
+    double r_clocks = 0.0, r_longest = 0.0;   // resident kernel: clocks of an SM for one example, and of a warp for its longest pair
     int split = kSplitDefault;
     std::vector<KRec> krec;
     std::vector<SBucket> sb;
@@ -263,8 +304,21 @@ int pays_up_to(const PlanHost& plan, int max_N, int sms, bool soft, bool generic
 struct SGroups { int end[3], examples[3], groups[3]; unsigned grid; };
 SGroups s_groups(const PlanHost& plan, int N, int sms);
 
+ResidentSplit resident_split(const PlanHost& plan, int N, int C, int sms, int mode);
+// And for the pairs of a task whose tiles several warps share (all modes but the backward, which adds up in global memory anyway).
+constexpr int kRMergeFloats = 8;
+inline int64_t resident_merge_floats(const PlanHost& plan, int64_t n, int parts, int split, int mode) {
+    return split > 1 && mode != 2 ? kRMergeFloats * n * ((int64_t)plan.runits.size() / parts + 1) : 0;
+}
+// The backward, whose code is twice as long and whose sums leave the warp once per tile, only where no tile has to test its reads and series
+// are short (us, before and with this kernel: 100 x 6 x 600, 2,000 kernels 1,106 and 855; 100 x 6 x 1,251 1,308 and 1,790).
+bool resident_backward(const PlanHost& plan);
+// Floats of shared memory for n examples.
+inline int64_t resident_floats(const PlanHost& plan, int64_t n, int C) { return plan.r_front + n * C * plan.r_pitch; }
+
 struct PlanDevice {
     const KRec* krec = nullptr;
+    const RUnit* runits = nullptr;
     const SBucket* sb = nullptr;
     const SItem* sitems = nullptr;
     const TItem* titems = nullptr;

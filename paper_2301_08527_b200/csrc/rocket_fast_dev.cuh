@@ -36,6 +36,29 @@ struct FwdArgs {
 void launch_stream(const FwdArgs& f, int mode, int sms, int64_t l2_bytes, bool after_s, cudaStream_t stream);   // after_s: directly behind the S kernel
 cudaError_t set_stream_attributes();   // opts the kernel into its shared-memory size
 
+// The resident kernel over N examples (rocket_resident.cu), modes as above.
+struct ResidentArgs {
+    const RUnit* units;
+    const KRec* krec;
+    const float* X;
+    const uint8_t* X8;       // or raw 8-bit samples, scaled with norm
+    NormArgs norm;
+    float* feat;
+    int32_t* argmax;         // soft: where the maxima are (or null)
+    float c1, c0, lambda;
+    int N, C, L, K, n_units;
+    int examples, groups, parts, run, split_bits;
+    int front, pitch;        // floats in front of the first channel row in shared memory, and from row to row
+    bool aligned;            // the rows of X start at 16-byte boundaries
+    const float* dfeat;      // backward
+    const int32_t* argmax_in;
+    long long* accfix;
+    const double* scale;
+    long long n_weights;
+};
+void launch_resident(ResidentArgs& a, const PlanHost& plan, int mode, int sms, cudaStream_t stream);
+cudaError_t set_resident_attributes();
+
 // A launch that may begin while its predecessor in the stream ends (programmatic dependent launch): the kernel itself waits for the
 // predecessor with dependency_wait() before it touches anything, or states why it need not.
 template <typename... P, typename... A>

@@ -845,6 +845,8 @@ cudaError_t set_kernel_attributes(int dev) {
         if (e != cudaSuccess) return e;
         e = set_stream_attributes();
         if (e != cudaSuccess) return e;
+        e = set_resident_attributes();
+        if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(fast_t_forward<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
         attr_done = true;
@@ -973,11 +975,11 @@ cudaError_t upload_plan(FastState& fs) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&fs.l2_bytes, cudaDevAttrL2CacheSize, dev);
     if (e != cudaSuccess) return e;
     struct Part { const void* src; size_t bytes; size_t off; };
-    Part parts[8] = {
+    Part parts[9] = {
         {h.krec.data(), h.krec.size() * sizeof(KRec), 0},   {h.sb.data(), h.sb.size() * sizeof(SBucket), 0},
         {h.sitems.data(), h.sitems.size() * sizeof(SItem), 0}, {h.titems.data(), h.titems.size() * sizeof(TItem), 0},
         {h.generic_list.data(), h.generic_list.size() * 4, 0}, {nullptr, 256, 0}, {nullptr, 256, 0},
-        {h.wunits.data(), h.wunits.size() * sizeof(WUnit), 0}};
+        {h.wunits.data(), h.wunits.size() * sizeof(WUnit), 0}, {h.runits.data(), h.runits.size() * sizeof(RUnit), 0}};
     size_t total = 0;
     for (auto& pt : parts) { pt.off = total; total += align256(pt.bytes); }
     e = device_malloc(&fs.plan_blob, std::max<size_t>(total, 256));
@@ -995,6 +997,7 @@ cudaError_t upload_plan(FastState& fs) {
     d.counters = reinterpret_cast<unsigned*>(base + parts[5].off);
     d.error_flag = reinterpret_cast<int*>(base + parts[6].off);
     d.wunits = reinterpret_cast<const WUnit*>(base + parts[7].off);
+    d.runits = reinterpret_cast<const RUnit*>(base + parts[8].off);
     d.n_wunits = (int)h.wunits.size();
     d.w_visits = h.w_visits;
     d.n_krec = (int)h.krec.size(); d.n_sitems = (int)h.sitems.size(); d.n_titems = (int)h.titems.size();
@@ -1182,6 +1185,8 @@ cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N,
     if (e != cudaSuccess) return e;
     if ((e = set_kernel_attributes(dev)) != cudaSuccess) return e;
     if (again) fs.most_examples = 1 << 30;
+    if (fs.host.resident && (!backward || resident_backward(fs.host)))
+        return backward ? ensure_bwd_ws(fs, dp, n_weights) : cudaSuccess;   // no copies, no sums but the backward's
     const bool stream = fs.dev.n_wunits > 0, copies = fs.dev.n_titems > 0 || u8;
     const int chunk = std::min(max_N, chunk_examples(fs, dp.C, stream, copies));
     if (stream && (e = ensure_stream_capacity(fs, chunk, dp.C, dp.L)) != cudaSuccess) return e;
@@ -1189,6 +1194,18 @@ cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N,
     if (soft && (e = ensure_soft_ws(fs, (int64_t)max_N * dp.K)) != cudaSuccess) return e;
     if (backward && (e = ensure_bwd_ws(fs, dp, n_weights)) != cudaSuccess) return e;
     return cudaSuccess;
+}
+
+// What the resident kernel's modes have in common.
+static ResidentArgs resident_args(const FastState& fs, const DeviceParams& dp, const float* X, int N, float lambda, float shift) {
+    ResidentArgs a{};
+    a.units = fs.dev.runits;
+    a.n_units = (int)fs.host.runits.size();
+    a.krec = fs.dev.krec;
+    a.X = X;
+    a.c1 = lambda * 1.4426950408889634f; a.c0 = -shift * 1.4426950408889634f; a.lambda = lambda;
+    a.N = N; a.C = dp.C; a.L = dp.L; a.K = dp.K;
+    return a;
 }
 
 cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const float* X, int N, float* feat,
@@ -1202,6 +1219,28 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev);
     if (e != cudaSuccess) return e;
+    if (fs.host.resident) {
+        ResidentArgs r = resident_args(fs, dp, X, N, lambda, shift);
+        r.feat = feat;
+        r.argmax = argmax;
+        r.X8 = X_u8;
+        if (X_u8) r.norm = *norm;
+        if (fs.profile) {                                  // one kernel, reported as the small dilations'
+            while (fs.evs.size() < 3) {
+                cudaEvent_t ev = nullptr;
+                if ((e = cudaEventCreate(&ev)) != cudaSuccess) return e;
+                fs.evs.push_back(ev);
+            }
+            cudaEventRecord(fs.evs[0], stream);
+        }
+        launch_resident(r, fs.host, soft ? 1 : half ? 3 : 0, sms, stream);
+        if (fs.profile) {
+            cudaEventRecord(fs.evs[1], stream);
+            cudaEventRecord(fs.evs[2], stream);
+            fs.ev_chunks = 1;
+        }
+        return cudaGetLastError();
+    }
     const size_t t_bytes = t_smem_bytes();
     const PlanDevice& pd = fs.dev;
     // the stream kernel takes the dilations the S kernel leaves; the T kernel where the stream kernel's copies have no room
@@ -1311,7 +1350,8 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     unsigned* absmax = reinterpret_cast<unsigned*>(static_cast<char*>(fs.bwd_ws) + acc_bytes + scale_bytes);
     const bool streamed = pd.n_wunits > 0, copied = pd.n_titems > 0;
     int chunk = chunk_examples(fs, dp.C, streamed, copied);
-    if (N > 0) {
+    const bool resident = resident_backward(fs.host);
+    if (N > 0 && !resident) {
         if (streamed) e = ensure_stream_capacity(fs, std::min(N, chunk), dp.C, dp.L);
         else if (copied) e = ensure_pad_capacity(fs, std::min(N, chunk), dp.C, dp.L);
         if (e != cudaSuccess) return e;
@@ -1340,7 +1380,12 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     a.C = dp.C; a.L = dp.L; a.K = dp.K;
     a.accfix = accfix; a.scale = scale; a.n_weights = n_weights; a.lambda = lambda;
     a.x_row_stride = dp.L;
-    for (int n0 = 0; n0 < N; n0 += std::min(chunk, N - n0)) {
+    if (resident && N > 0) {
+        ResidentArgs r = resident_args(fs, dp, X, N, lambda, shift);
+        r.dfeat = dfeat; r.argmax_in = argmax; r.accfix = accfix; r.scale = scale; r.n_weights = n_weights;
+        launch_resident(r, fs.host, 2, sms, stream);
+    }
+    for (int n0 = 0; n0 < N && !resident; n0 += std::min(chunk, N - n0)) {
         const int nc = std::min(chunk, N - n0);
         a.X = X + (size_t)n0 * dp.C * dp.L;
         a.dfeat = dfeat + (size_t)n0 * 2 * dp.K;

@@ -61,6 +61,27 @@ ROCKET_HD bool tile_interior(int trow, int c0, int span, int d, int lo_u, int hi
     return c0 + kWarpCols <= d && u >= lo_u && hi_u - kWarpCols - u >= span;
 }
 
+// Resident regime.  Column c of the bands of R rows that begin at row `base` of a kernel's outputs: band and column of A, the first row and
+// its output index, how many of its rows are outputs, and which of its input rows are samples.  c is below 2^22 (kRMostOutputs), so that
+// the quotient by way of the rounded reciprocal is exact.
+struct ResidentColumn { int band, r, row, i0, out, in_lo, in_hi; };
+ROCKET_HD ResidentColumn resident_column(int c, int base, int R, int len, int d, float inv_d, int nq, int nr, int pq, int pr, int lq, int lr) {
+    ResidentColumn at;
+    at.band = (int)(((float)c + 0.5f) * inv_d);
+    at.r = c - at.band * d;
+    at.row = base + at.band * R;
+    at.i0 = at.row * d + at.r;
+    const int out = nq + (at.r < nr ? 1 : 0) - at.row, lo = pq + (at.r < pr ? 1 : 0) - at.row, hi = lq + (at.r < lr ? 1 : 0) - at.row;
+    const int rows = R + len - 1;
+    at.out = out < 0 ? 0 : imin(out, R);
+    at.in_lo = lo < 0 ? 0 : imin(lo, rows);
+    at.in_hi = hi < 0 ? 0 : imin(hi, rows);
+    return at;
+}
+ROCKET_HD ResidentColumn resident_column(const RUnit& u, int c, int base, int R) {
+    return resident_column(c, base, R, u.len, u.d, u.inv_d, u.nq, u.nr, u.pq, u.pr, u.lq, u.lr);
+}
+
 // T regime.  A tile starts at A-row t0 and residue r0 (a multiple of 64).  Row s of the tile
 // (A-row t0 + s) arrives with the box of phase s & 3, as that box's row s >> 2.  In the
 // zero-margined copy the element (A-row t, residue r) of a channel row sits at float

@@ -14,6 +14,10 @@ namespace rocket {
 namespace fast {
 namespace {
 
+// Clocks of a scheduler: an input row of a tile and channel besides its multiply-adds, a channel, an output row, a tile, a pair, an item;
+// clocks of a block: a task.
+constexpr double kRRowClocks = 3.0, kRVisitClocks = 30.0, kRPoolClocks = 8.0, kRTileClocks = 120.0, kRPairClocks = 250.0, kRItemClocks = 500.0, kRTaskClocks = 3000.0;
+
 inline int64_t floor_div(int64_t a, int64_t b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
 
 // Units of the stream kernel for the kernels whose records start at `first`.  The output rows of a kernel (their count rounded
@@ -102,7 +106,122 @@ void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost&
     for (auto& kv : by_shape) out.wunits.insert(out.wunits.end(), kv.second.begin(), kv.second.end());
 }
 
+// The kernels of a handle whose examples fit shared memory.
+struct ResidentUnits {
+    struct Cost { double c; RUnit u; };
+    std::vector<Cost> units;
+    double clocks = 0.0, longest = 0.0;
+    int tiles = 0;
+    int64_t reach = 0;                                 // how far before the first and behind the last sample a tile reads
+};
+
+ResidentUnits resident_units(const HostParams& hp, const PlanHost& plan, bool small) {
+    const int kHigh = resident_high(small), kLow = resident_low(small);
+    ResidentUnits out;
+    out.units.reserve(plan.krec.size());
+    for (size_t i = 0; i < plan.krec.size(); ++i) {
+        const KRec& f = plan.krec[i];
+        RUnit u{};
+        u.krec = (int32_t)i; u.k = f.k; u.len = f.len; u.d = f.d; u.m = f.m; u.nout = f.nout; u.p = f.p; u.woff = f.woff;
+        u.nq = f.nout / f.d; u.nr = f.nout % f.d;
+        u.inv_d = 1.0f / (float)f.d;
+        const int32_t* S = hp.channel_idx.data() + hp.channel_offset[f.k];
+        for (int q = 0; q < f.m; ++q) u.ch[q] = (uint8_t)S[q];
+        // bands: all of one height, or as many high ones as fill whole tiles and low ones for the rest, whichever takes least
+        const int rows = u.nq + (u.nr > 0 ? 1 : 0);
+        auto tiles = [&](int bands) { return ((int64_t)bands * f.d + kWarpCols - 1) / kWarpCols; };
+        auto tile_clocks = [&](int R) { return f.m * ((R + f.len - 1) * kRRowClocks + 2.0 * R * f.len + kRVisitClocks) + R * kRPoolClocks + kRTileClocks; };
+        const double high = tile_clocks(kHigh), low = tile_clocks(kLow);
+        double best = 1e300;
+        auto consider = [&](int n) {
+            if (n < 0) return;
+            const int rest = std::max(0, rows - n * kHigh), n_low = (rest + kLow - 1) / kLow;
+            const double c = tiles(n) * high + tiles(n_low) * low;
+            if (c < best) { best = c; u.high = n; u.low = n_low; }
+        };
+        consider((rows + kHigh - 1) / kHigh);
+        consider(0);
+        for (int64_t t = (int64_t)(rows / kHigh) * f.d / kWarpCols, n = 0; t >= 0 && n < 2; --t, ++n) consider((int)(t * kWarpCols / f.d));
+        consider(rows / kHigh);
+        const int64_t last_row = (int64_t)u.high * kHigh + u.low * kLow - 1 + f.len - 1;
+        out.reach = std::max<int64_t>({out.reach, f.p, last_row * f.d + f.d - f.p - hp.L});
+        out.tiles = (int)std::max<int64_t>(out.tiles, tiles(u.high) + tiles(u.low));
+        best += kRPairClocks;
+        out.clocks += best / 4.0;
+        out.longest = std::max(out.longest, best);
+        out.units.push_back({best, u});
+    }
+    return out;
+}
+
+void build_resident_units(const HostParams& hp, PlanHost& out) {
+    const int64_t row = (hp.L + 3ll) / 4 * 4;
+    if (hp.C * row > kRMostFloats) return;
+    for (const KRec& f : out.krec)
+        if (f.nout > kRMostOutputs || f.d > kRMostOutputs) return;
+    ResidentUnits r = resident_units(hp, out, false);
+    if (hp.L < kRSmallSteps) {
+        ResidentUnits s = resident_units(hp, out, true);
+        out.r_small = s.clocks < r.clocks;
+        if (out.r_small) r = std::move(s);
+    }
+    out.r_clocks = r.clocks;
+    out.r_longest = r.longest;
+    out.r_tiles = r.tiles;
+    // Zeros around the rows make all reads alike; where they would not fit, or take more than twice the samples, some tiles test theirs.
+    const int64_t room = (kRMostFloats - hp.C * row) / (hp.C + 1) / 4 * 4;
+    const int zeros = (int)std::min<int64_t>({(r.reach + 3) / 4 * 4, room, 2 * row});
+    out.r_front = zeros;
+    out.r_pitch = (int)row + zeros;
+    out.r_zeros = zeros >= r.reach;
+    for (auto& c : r.units) {
+        RUnit& u = c.u;
+        const int before = std::max(0, u.p - zeros), end = hp.L + u.p + zeros;
+        u.pq = before / u.d; u.pr = before % u.d;
+        u.lq = end / u.d; u.lr = end % u.d;
+    }
+    // Kernels of a length follow one another, so that the warps of a block share inner loops; the longest pairs of a length first.  The
+    // instruction caches decide here: the longest pairs first throughout took 846 us where this order takes 410 (100 x 20 x 2,800, 400 kernels).
+    std::stable_sort(r.units.begin(), r.units.end(), [](const auto& a, const auto& b) { return a.u.len != b.u.len ? a.u.len > b.u.len : a.c > b.c; });
+    for (const auto& c : r.units) out.runits.push_back(c.u);
+    out.resident = !out.runits.empty() && hp.L <= (out.r_zeros ? kRMostSteps : kRMostStepsTested);
+}
+
 }  // namespace
+
+bool resident_backward(const PlanHost& plan) { return plan.resident && plan.r_zeros && plan.r_pitch - plan.r_front <= kRMostStepsBackward; }
+
+// Blocks take tasks of a few examples and a part of the kernels: as few copies of an example as leave every SM its share.
+ResidentSplit resident_split(const PlanHost& plan, int N, int C, int sms, int mode) {
+    const double work = plan.r_clocks * (mode == 1 ? 1.4 : mode == 2 ? 2.6 : 1.0);
+    const int64_t n_units = (int64_t)plan.runits.size();
+    const int warps = resident_warps(mode, plan.r_small);
+    // eight items per warp and task, if that many there are
+    auto run_of = [&](int64_t kernels, int64_t e) { return std::max<int64_t>(1, std::min<int64_t>(e, kernels * e / (8 * warps))); };
+    ResidentSplit best{1, N, 1, 1, 1, 1u};
+    double least = 1e300;
+    for (int64_t e = 1; e <= N && resident_floats(plan, e, C) <= kRMostFloats; e *= 2) {
+        const int64_t groups = (N + e - 1) / e;
+        int64_t last = 0;
+        for (int64_t rounds = 1; rounds <= 64; ++rounds) {
+            const int64_t parts = std::min(n_units, rounds * sms / groups);
+            if (parts < 1 || parts == last) continue;
+            last = parts;
+            const int64_t kernels = (n_units + parts - 1) / parts, run = run_of(kernels, e);
+            for (int split = 1; split <= 4 && (split == 1 || (run == 1 && split < 2 * plan.r_tiles)); split *= 2) {
+                if (resident_floats(plan, e, C) + resident_merge_floats(plan, e, (int)parts, split, mode) > kRMostFloats) continue;
+                const double items = (double)kernels * (double)((e + run - 1) / run) * split;
+                // a warp's last item runs beside those of the five other warps of its scheduler
+                const double task = kRTaskClocks + 4.0 * e * C * plan.r_pitch / 30.0 + e * work / parts + items * kRItemClocks / 4.0 +
+                                    2.0 * plan.r_longest * (double)run / std::min(split, plan.r_tiles);
+                const double t = (double)((groups * parts + sms - 1) / sms) * task;
+                if (t < least) { least = t; best = {(int)e, (int)groups, (int)parts, (int)run, split, 1u}; }
+            }
+        }
+    }
+    best.grid = (unsigned)std::min<int64_t>((int64_t)best.groups * best.parts, sms);
+    return best;
+}
 
 // One example where a bucket has many kernels, up to 4 and up to 16 where it has some or few (64 to 256 pairs per tile for its 16
 // warps), as far as the planes hold them and the launch keeps two tiles per SM.
@@ -518,6 +637,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
     const int64_t pitch = (int64_t)kTPadFront + hp.L + 4ll * d_max + kTXExtra + t_box_cols(4);
     out.pad_pitch = (pitch + 31) / 32 * 32;
     if (hp.C > kSMaxPlanes) estimate_costs(hp, out);
+    build_resident_units(hp, out);
 }
 
 }  // namespace fast
