@@ -857,20 +857,21 @@ cudaError_t set_kernel_attributes(int dev) {
 // ---- backward helpers ----------------------------------------------------------------------------
 // Largest |x| of the batch, as the bit pattern of a non-negative float (integer order = float order).  One atomic per block of 256
 // threads: one per warp, all to the same word, took 8 us of a minibatch.
-__device__ __forceinline__ void block_max(float m, unsigned* __restrict__ out) {
+__device__ __forceinline__ unsigned block_max(float m) {
     __shared__ unsigned s_max;
     if (threadIdx.x == 0) s_max = 0u;
     __syncthreads();
     const unsigned b = __reduce_max_sync(kFull, __float_as_uint(m));
     if ((threadIdx.x & 31) == 0) atomicMax(&s_max, b);
     __syncthreads();
-    if (threadIdx.x == 0) atomicMax(out, s_max);
+    return s_max;
 }
 __global__ void fast_absmax_scalar_kernel(const float* __restrict__ X, int64_t n, unsigned* __restrict__ out) {
     float m = 0.0f;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
         m = fmaxf(m, fabsf(__ldg(X + e)));
-    block_max(m, out);
+    const unsigned b = block_max(m);
+    if (threadIdx.x == 0) atomicMax(out, b);
 }
 
 __global__ void fast_absmax_kernel(const float4* __restrict__ X, int64_t n4, unsigned* __restrict__ out) {
@@ -879,16 +880,26 @@ __global__ void fast_absmax_kernel(const float4* __restrict__ X, int64_t n4, uns
         const float4 v = __ldg(X + e);
         m = fmaxf(fmaxf(m, fabsf(v.x)), fmaxf(fabsf(v.y), fmaxf(fabsf(v.z), fabsf(v.w))));
     }
-    block_max(m, out);
+    const unsigned b = block_max(m);
+    if (threadIdx.x == 0) atomicMax(out, b);
 }
 
 // Per kernel: a bound on sum |gz| |x| over the batch gives the fixed-point scale of its sums
 // (|sum_i gz_i| <= |gP| lambda / 4 + |gM| per example since h (1 - h) <= 1/4), and its sums are cleared.  A warp per kernel here
 // and in the finalise kernel: a thread per kernel went through up to 121 weights one by one (8 and 13 us of a minibatch).
+// Of a batch of at most kSmallBatch samples every block takes the maximum itself (small: the batch), which spares clearing the word and a launch.
+constexpr int64_t kSmallBatch = 4096;
 __global__ void fast_bwd_prepare_kernel(const float* __restrict__ dfeat, const KRec* __restrict__ krec, int n_krec, int N,
-                                        int K, float lambda, const unsigned* __restrict__ absmax_bits,
+                                        int K, float lambda, const unsigned* __restrict__ absmax_bits, const float* __restrict__ small, int n_small,
                                         double* __restrict__ scale, long long* __restrict__ accfix, long long n_weights,
                                         unsigned* __restrict__ counters) {
+    unsigned most = 0u;
+    if (small) {
+        float m = 0.0f;
+#pragma unroll 8
+        for (int e = threadIdx.x; e < n_small; e += blockDim.x) m = fmaxf(m, fabsf(__ldg(small + e)));
+        most = block_max(m);
+    }
     dependency_wait();
     const int f = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (f >= n_krec) return;
@@ -903,7 +914,7 @@ __global__ void fast_bwd_prepare_kernel(const float* __restrict__ dfeat, const K
     for (int sh = 16; sh > 0; sh >>= 1) bound += __shfl_xor_sync(kFull, bound, sh);
     for (int t = lane; t < taps; t += 32) accfix[r.woff + t] = 0;
     if (lane > 0) return;
-    const double xmax = fmax((double)__uint_as_float(*absmax_bits), 1.0);
+    const double xmax = fmax((double)__uint_as_float(small ? most : *absmax_bits), 1.0);
     bound *= xmax * 1.01;
     scale[k] = (bound > 0.0 && bound < 1e300) ? 1152921504606846976.0 / bound : 0.0;  // 2^60 / bound
     accfix[n_weights + k] = 0;
@@ -1357,22 +1368,23 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
         if (e != cudaSuccess) return e;
         if (streamed || copied) chunk = std::min(chunk, fs.most_examples);
     }
-    e = cudaMemsetAsync(absmax, 0, 256, stream);
-    if (e != cudaSuccess) return e;
     const int64_t n_x = (int64_t)N * dp.C * dp.L;
-    if (n_x > 0) {
+    const bool small = n_x > 0 && n_x <= kSmallBatch;
+    if (!small && (e = cudaMemsetAsync(absmax, 0, 256, stream)) != cudaSuccess) return e;
+    if (n_x > 0 && !small) {
         auto blocks = [&](int64_t loads) { return (unsigned)std::min<int64_t>(sms * 8, (loads + 1023) / 1024); };   // four loads per thread
         if (dp.L % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0)
             fast_absmax_kernel<<<blocks(n_x / 4), 256, 0, stream>>>(reinterpret_cast<const float4*>(X), n_x / 4, absmax);
         else fast_absmax_scalar_kernel<<<blocks(n_x), 256, 0, stream>>>(X, n_x, absmax);
         count_launch();
     }
-    if (n_x > 0)
-        launch_dependent(fast_bwd_prepare_kernel, (pd.n_krec + 7) / 8, 256, 0, stream, dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale,
+    const float* none = nullptr;
+    if (n_x > 0 && !small)
+        launch_dependent(fast_bwd_prepare_kernel, (pd.n_krec + 7) / 8, 256, 0, stream, dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, none, 0, scale,
                          accfix, n_weights, pd.counters);
     else
-        fast_bwd_prepare_kernel<<<(pd.n_krec + 7) / 8, 256, 0, stream>>>(dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, scale, accfix,
-                                                                         n_weights, pd.counters);
+        fast_bwd_prepare_kernel<<<(pd.n_krec + 7) / 8, 256, 0, stream>>>(dfeat, pd.krec, pd.n_krec, N, dp.K, lambda, absmax, small ? X : none,
+                                                                         (int)(small ? n_x : 0), scale, accfix, n_weights, pd.counters);
     count_launch();
     FwdArgs a;
     a.plan = fs.dev; a.feat_i = nullptr; a.ws = nullptr;
