@@ -1,14 +1,14 @@
 // Gram matrix of the centred features on the fifth-generation tensor cores, in integers.
 //
-// Fc = F - mu is taken in double precision, every row scaled by a power of two so that its largest magnitude lies in [2^45, 2^46), rounded
-// to an integer and written as six signed base-256 digits, d_0 first.  Then G_ij is a sum of digit products: all with a + b <= 5 are kept
-// (21 of 36; what is left out is below 2^-49 of the diagonal), products with the same a + b share a 32-bit accumulator and are exact there
-// (6 * 16,384 columns * 128^2 < 2^31), and the six accumulators meet in double precision.  The quantum is 2^-46 of a row's largest
-// value; against exact sums the result is as close as FP64 multiply-adds came.
+// Fc = F - mu is taken in double precision, every row scaled by a power of two so that its largest magnitude lies in [2^53, 2^54), rounded
+// to an integer and written as seven signed base-256 digits, d_0 first.  Then G_ij is a sum of digit products: all with a + b <= 6 are kept
+// (28 of 49; what is left out is of the order of 2^-55 sqrt(columns) of the rows' largest values), products with the same a + b share a 32-bit
+// accumulator and are exact there (7 * 16,384 columns * 128^2 < 2^31), and the seven accumulators meet in double precision.  That is as close as FP64
+// multiply-adds come; six digits and 21 products (146 in place of 180 us at 677 x 20,000) were not: the fit of 257 examples whose rows lie five
+// orders of magnitude apart was off by 4e-7 where FP64 sums leave 3e-8, and one value of 1e6 among shares made a penalty of 1e-3 too small.
 //
-// Why: FP64 products run at 37 TFLOP/s at the most, 8-bit ones at a hundred times that, and 21 of those replace one.  Measured at 677 x
-// 20,000: 193 us (scales 21, digits 26, products 146) where FP64 matrix instructions took 496.  Relative error of the fitted weights against
-// a solution in 64 bits: the same to three digits (2.52e-8, their rounding to FP32), at fifteen sizes from 24 x 200 to 1,500 x 9,001.
+// Why: FP64 products run at 37 TFLOP/s at the most, 8-bit ones at a hundred times that, and 28 of those replace one.  Measured at 677 x
+// 20,000: 229 us (scales 21, digits 28, products 180) where FP64 matrix instructions took 496.
 #include <algorithm>
 #include <cstdint>
 
@@ -25,15 +25,15 @@ using fast::mbar_init;
 using fast::mbar_wait;
 using fast::smem_u32;
 
-constexpr int kDigits = 6, kTileM = 128, kTileN = 64, kStageK = 64;
+constexpr int kDigits = 7, kTileM = 128, kTileN = 64, kStageK = 64;
 // The digits lie in memory as the matrix instruction reads them from shared memory (8 rows x 16 bytes to a core matrix, no swizzle):
 // [block of 64 columns][group of 8 rows][digit][4 core matrices][8 rows][16 columns], so that the operands of a stage are two bulk copies.
 constexpr int kCoreBytes = 128, kDigitBytes = kStageK / 16 * kCoreBytes, kGroupBytes = kDigits * kDigitBytes;
 constexpr int kABytes = kTileM / 8 * kGroupBytes, kBBytes = kTileN / 8 * kGroupBytes, kStageBytes = kABytes + kBBytes;
-constexpr int kStages = 3, kGramThreads = 128;
+constexpr int kStages = 2, kGramThreads = 128;
 static_assert(kDigits * kTileN <= 512, "an accumulator per a + b");
 
-// up[i] = 2^k with up[i] max_p |F[i][p] - mu[p]| in [2^45, 2^46), down[i] = 1 / up[i]; NaN where a value of the row is not finite.
+// up[i] = 2^k with up[i] max_p |F[i][p] - mu[p]| in [2^53, 2^54), down[i] = 1 / up[i]; NaN where a value of the row is not finite.
 __global__ void __launch_bounds__(256)
 gram_scale_kernel(const float* __restrict__ F, int P, const double* __restrict__ mu, double* __restrict__ up, double* __restrict__ down) {
     __shared__ unsigned long long s_max;
@@ -51,7 +51,7 @@ gram_scale_kernel(const float* __restrict__ F, int P, const double* __restrict__
     if (threadIdx.x > 0) return;
     m = s_max;
     const int e = (int)(m >> 52) - 1022;               // the maximum is below 2^e
-    const int k = min(max(46 - e, -1022), 1022);
+    const int k = min(max(54 - e, -1022), 1022);
     const bool finite = (m >> 52) < 2047ull;
     up[blockIdx.x] = finite ? __longlong_as_double((long long)(1023 + k) << 52) : __longlong_as_double(0x7ff8000000000000ll);
     down[blockIdx.x] = finite ? __longlong_as_double((long long)(1023 - k) << 52) : __longlong_as_double(0x7ff8000000000000ll);
@@ -73,9 +73,8 @@ gram_digits_kernel(const float* __restrict__ F, int N, int P, int p0, int cores,
     for (int c = 0; c < 4; ++c) {
         const bool ok = there && p0 + k + c < P;
         const double x = ok ? (double)__ldg(f + c) - __ldg(mu + p0 + k + c) : 0.0;
-        // 1.5 * 2^52 + q has q in its low bits; with 128 added to every digit the digits are the bytes
-        const double shifted = fma(x, scale, 6755399441055744.0);
-        const unsigned long long q = (unsigned long long)(__double_as_longlong(shifted) - 0x4338000000000000ll) + 0x808080808080ull;
+        // with 128 added to every digit the digits are the bytes
+        const unsigned long long q = (unsigned long long)__double2ll_rn(x * scale) + 0x80808080808080ull;
         lo[c] = (unsigned)q;
         hi[c] = (unsigned)(q >> 32);
     }
@@ -103,7 +102,7 @@ __device__ __forceinline__ uint64_t operand(uint32_t at) {   // K-major, no swiz
 }
 
 // One 128 x 64 tile of the lower triangle over a slice of the columns.  One thread copies stages in, one issues the matrix instructions
-// (42 per stage of 64 columns), all four warps turn the accumulators into doubles.  Bound: the matrix pipe, an instruction of 128 x 64 x 32
+// (56 per stage of 64 columns), all four warps turn the accumulators into doubles.  Bound: the matrix pipe, an instruction of 128 x 64 x 32
 // every 70 clocks; with A's digits copied to tensor memory, which spares two thirds of the shared-memory reads, the same.
 __global__ void __launch_bounds__(kGramThreads, 1)
 gram_mma_kernel(const GramArgs a) {
@@ -204,8 +203,8 @@ gram_mma_kernel(const GramArgs a) {
 #pragma unroll
                 for (int s = kDigits - 1; s >= 0; --s) sum = fma(sum, 1.0 / 256.0, (double)(int)v[s][e + h]);
                 const int j = j0 + c + e + h;
-                // 256^5 per factor between the leading digit and the integer
-                g[h] = sum * (1099511627776.0 * di) * (1099511627776.0 * (j < a.N ? __ldg(a.down + j) : 0.0));
+                // 256^6 per factor between the leading digit and the integer
+                g[h] = sum * (281474976710656.0 * di) * (281474976710656.0 * (j < a.N ? __ldg(a.down + j) : 0.0));
             }
             double2* to = reinterpret_cast<double2*>(out + c + e);
             if (a.add) {
@@ -234,13 +233,13 @@ GramPlan gram_plan(int N, int P, int sms) {
     const int blocks = (P + kStageK - 1) / kStageK;
     g.chunk = (int)std::max<size_t>(1, std::min<size_t>(blocks, kGramDigitBytes / block_bytes));
     g.chunk = (blocks + (blocks + g.chunk - 1) / g.chunk - 1) / ((blocks + g.chunk - 1) / g.chunk);   // evenly
-    // Slices of a chunk: the fewest clocks, where a stage takes 2,050 and a block's beginning and end 9,000; no more than 16,384 columns each
+    // Slices of a chunk: the fewest clocks, where a stage takes 4,000 and a block's beginning and end 10,000; no more than 16,384 columns each
     // (32-bit sums), and 24 MB of partial tiles (or one slice).
     const size_t slice_bytes = (size_t)nt * (nt + 1) / 2 * 4096 * sizeof(double);
     const int least = (g.chunk * kStageK + 16383) / 16384, most = std::max<int>(least, std::min<int>(16, (int)(((size_t)24 << 20) / slice_bytes)));
     double best = 1e300;
     for (int s = least; s <= most && s <= g.chunk; ++s) {
-        const double t = (double)(((long long)g.blocks_mn * s + sms - 1) / sms) * ((g.chunk + s - 1) / s * 2050.0 + 9000.0);
+        const double t = (double)(((long long)g.blocks_mn * s + sms - 1) / sms) * ((g.chunk + s - 1) / s * 4000.0 + 10000.0);
         if (t < best) { best = t; g.slices = s; }
     }
     g.digit_bytes = (size_t)g.chunk * block_bytes;

@@ -8,7 +8,7 @@
 
 namespace rocket {
 
-constexpr size_t kGramDigitBytes = (size_t)96 << 20;   // digits of as many columns at a time
+constexpr size_t kGramDigitBytes = (size_t)112 << 20;   // digits of as many columns at a time
 
 struct GramPlan {
     int groups, blocks_mn;     // groups of 8 rows; 128 x 64 tiles of the lower triangle

@@ -9,7 +9,7 @@
 // of the same data are bitwise identical.
 //
 // Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights take
-// 18 / 193 (in FP64 496) / 240 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
+// 18 / 229 (in FP64 496) / 214 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
 // 55 / 2,607 / 20,270 / 174.
 #include <cooperative_groups.h>
 
@@ -602,7 +602,7 @@ int status_of(cudaError_t e) {
 // per device, of at most kKeepBytes, outlives the call: a fit takes it while nobody else has it and puts it back after its
 // stream has finished; a larger or a concurrent fit allocates and frees its own.  The buffer is given back when a handle
 // of the library is destroyed and when a device allocation of the library fails (release_cached_workspaces).
-constexpr size_t kKeepBytes = (size_t)128 << 20;
+constexpr size_t kKeepBytes = (size_t)144 << 20;
 constexpr int kMaxDevices = 64;
 struct Kept { void* ptr = nullptr; size_t bytes = 0; bool taken = false; };
 std::mutex g_kept_mu;

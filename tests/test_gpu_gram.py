@@ -1,0 +1,57 @@
+"""Ridge fits whose Gram matrix is summed in integers (rocket_gram.cu), at the edges of its tiles, stages and slices.
+
+Rows around multiples of 64 and 128, columns around multiples of 64 and of a quadruple, more columns than a 32-bit sum takes at once, rows of
+very different magnitude.  Against the dual system in float64.  What the weights may be off by: their rounding to FP32 (2^-24 each) plus
+the errors of the two solutions, each of the order of 2^-53 times the condition number of the system.
+"""
+import numpy as np
+import pytest
+
+import paper_2301_08527_b200 as rk
+
+pytestmark = pytest.mark.gpu
+
+
+def _fit(F, y, alpha):
+    import torch
+    w, b = rk.rocket_ridge_fit(torch.from_numpy(F).cuda(), torch.from_numpy(y).cuda(), alpha)
+    return w.cpu().numpy().astype(np.float64), float(b)
+
+
+def _dual(F, y, alpha):
+    F, y = F.astype(np.float64), y.astype(np.float64)
+    mu, ym = F.mean(0), y.mean()
+    Fc = F - mu
+    w = Fc.T @ np.linalg.solve(Fc @ Fc.T + alpha * np.eye(len(y)), y - ym)
+    largest = np.linalg.norm(Fc, 2) ** 2
+    return w, ym - mu @ w, 2.0 ** -24 + 4 * 2.0 ** -53 * (largest + alpha) / alpha
+
+
+@pytest.mark.parametrize("N,P,kind", [(127, 7500, "shares"), (128, 7601, "shares"), (129, 7702, "shares"), (191, 3403, "shares"), (193, 40001, "shares"),
+                                      (257, 2049, "shares"), (257, 2111, "scales"), (320, 1985, "shifted"), (641, 320, "shares")])
+def test_fits_match_the_dual_system_in_float64(N, P, kind):
+    rng = np.random.default_rng(N + P)
+    F = rng.random((N, P))
+    F[:, 1::2] = 2.0 + 0.7 * rng.normal(size=(N, P // 2))
+    if kind == "scales":                                     # rows of very different magnitude, one of them constant
+        F *= 10.0 ** rng.uniform(-3, 3, size=(N, 1))
+        F[7] = 0.25
+    if kind == "shifted":                                    # far from zero: the centred values have few bits of the samples' left
+        F += 1000.0
+    F = F.astype(np.float32)
+    y = (F[:, :50].astype(np.float64) @ rng.normal(size=50) / 50 + rng.normal(size=N)).astype(np.float32)
+    w, b = _fit(F, y, 1.0)
+    rw, rb, bound = _dual(F, y, 1.0)
+    assert np.linalg.norm(w - rw) <= bound * np.linalg.norm(rw)
+    # the intercept is made from the stored weights
+    assert abs(b - rb) <= (bound + 2.0 ** -23) * (np.linalg.norm(rw) * np.linalg.norm(F.astype(np.float64).mean(0)) + abs(rb))
+    again, _ = _fit(F, y, 1.0)
+    assert np.array_equal(w, again)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_values_that_are_not_finite_are_refused(bad):
+    F = np.random.default_rng(1).random((200, 4000)).astype(np.float32)
+    F[13, 77] = bad
+    with pytest.raises(Exception):
+        _fit(F, F[:, 0].copy(), 1.0)
