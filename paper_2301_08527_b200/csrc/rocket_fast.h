@@ -92,6 +92,8 @@ constexpr int kMaxChannels = 255;                                  // channels o
 constexpr int kRS = ROCKET_S_ROWS;
 static_assert(kRS >= 8 && kRS <= 32, "the row masks of the pooling hold at most 32 rows");
 constexpr int kSRowsMax = kRS + ROCKET_MAX_LENGTH - 1;             // staged rows an S warp tile reads
+// Handles whose columns fill their last tiles badly at that height take a lower one (the planner's estimate decides; wide handles don't).
+constexpr int kSLowRows[2] = {21, 18};
 constexpr int kSThreads = ROCKET_S_THREADS, kSWarps = kSThreads / 32;   // one block per SM
 constexpr int kSPlaneFloats = kSRowsMax * kWarpCols;               // one channel of an S tile
 // Wide handles: the kernels of some dilation use more than kSMaxPlanes channels, none more than kSWidePlanes.  Their tiles are staged in two halves of kRS / 2
@@ -107,7 +109,7 @@ constexpr int kSLengthOrderMin = 100;                              // buckets fr
 // dilation use more, they are several buckets.  Their records hold positions in the bucket's channel list.
 struct SBucket {
     int32_t d, tmin, nbands, raster_len;  // raster_len = nbands * d
-    int32_t kbeg, kend, rows, nch;        // kernels [kbeg, kend) of krec; rows = kRS + max len - 1; channels used
+    int32_t kbeg, kend, rows, nch;        // kernels [kbeg, kend) of krec; rows = s_rows + max len - 1; channels used
     uint8_t ch[40];                       // the channels (at most kSWidePlanes)
     int32_t pad_[2];
 };
@@ -285,6 +287,7 @@ struct PlanHost {
     int64_t pad_pitch = 0;                // floats per channel row of the zero-margined copy
     int s_max_nch = 0;                    // most channels of any S bucket
     bool s_wide = false;                  // the S tiles are staged in halves of up to kSWidePlanes planes
+    int s_rows = kRS;                     // rows of a band of the S tiles
     int s_class_end[3] = {0, 0, 0};       // S tiles by kernels in their bucket: at least kSManyKernels, kSSomeKernels, fewer
     double flops_s = 0.0, flops_t = 0.0;  // conv flop of one example in either regime
     // What generic_pays compares, in us: work of one example for one SM (small dilations) and for the GPU (large dilations and their
@@ -340,7 +343,7 @@ void fill_record_weights(const HostParams& hp, KRec& f);
 cudaError_t upload_records(FastState& fs);
 
 // Builds the launch plan for the kernels in hp (host side, once per handle).  all_tiles: also the T tiles of kernels that have
-// stream units, which no launch uses.
+// stream units, which no launch uses, and S bands of kRS rows.
 void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles = true);
 
 // Device-side state of the fast path owned by a handle.

@@ -96,13 +96,13 @@ __device__ __forceinline__ void s_kernel_tile_h(const float* planes, const KRec*
 // at dilations 32 to 63, 11,400 are work.  Measured at 60 x 20 x 50,000, hard: 24.1 ms with weights read by every lane, 22.6 now.
 // Tried and not kept: two half tiles in flight behind producer warps (22.9 ms; 22 input rows for 12 rows of outputs make the
 // shared memory the limit), drawing the next tile during the copies (22.5 to 22.6, and late draws matter for small batches).
-template <int MODE, bool HALF = false>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision; HALF: a wide handle
+template <int MODE, int ROWS = kRS, bool HALF = false>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision; ROWS: of a band; HALF: a wide handle
 __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
     dependency_wait();
     // The stream kernel needs what came before this one, not this one: it may begin on the SMs that run out of tiles (8 x 20 x 10,001:
     // 1.52 -> 1.45 ms; 10 x 6 x 1,251, 1,000 kernels: soft transform 88 -> 72 us).
     dependency_release();
-    constexpr int R = HALF ? kSHalfRows : kRS, kPlanes = HALF ? kSWidePlanes : kSMaxPlanes, kPlaneFloats = s_plane_floats(R);
+    constexpr int R = HALF ? kSHalfRows : ROWS, kPlanes = HALF ? kSWidePlanes : kSMaxPlanes, kPlaneFloats = s_plane_floats(R);
     float* planes = reinterpret_cast<float*>(smem_raw);                               // [kPlanes][rows][64]
     KRec* recs = reinterpret_cast<KRec*>(planes + kPlanes * kPlaneFloats);             // [warps][2]
     __shared__ unsigned s_item;
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
             const int col = threadIdx.x & (kWarpCols - 1), rg = threadIdx.x / kWarpCols;
             const int cg = item.c0 + col;
             const bool col_ok = cg < b.raster_len;
-            const int fu0 = s_column_u0(b, cg) + half_row * d, n_planes = nch * ne, rows = b.rows - (kRS - R);
+            const int fu0 = s_column_u0(b, cg, ROWS) + half_row * d, n_planes = nch * ne, rows = b.rows - (ROWS - R);
             int xi[kRows], bytes[kRows];
 #pragma unroll
             for (int i = 0; i < kRows; ++i) {
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kSThreads, 1) fast_s_forward(FwdArgs a) {
         const bool ok0 = cg0 < b.raster_len, ok1 = cg0 + 1 < b.raster_len;
         const int band0 = cg0 / d, c0 = cg0 - band0 * d;          // (first A-row, residue) of the two columns
         const int band1 = c0 + 1 < d ? band0 : band0 + 1, c1 = c0 + 1 < d ? c0 + 1 : 0;
-        const int trow0 = b.tmin + band0 * kRS + half_row, trow1 = b.tmin + band1 * kRS + half_row;
+        const int trow0 = b.tmin + band0 * ROWS + half_row, trow1 = b.tmin + band1 * ROWS + half_row;
         cp_async_wait<0>();
         __syncthreads();
 
@@ -823,31 +823,23 @@ cudaError_t set_kernel_attributes(int dev) {
     bool& attr_done = attr_done_for[dev & 63];
     const size_t t_bytes = t_smem_bytes();
     if (!attr_done) {
-        e = cudaFuncSetAttribute(fast_s_forward<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_t_forward<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_t_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_t_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(true));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(true));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_s_forward<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(true));
-        if (e != cudaSuccess) return e;
+        for (auto kernel : {fast_s_forward<0>, fast_s_forward<1>, fast_s_forward<2>, fast_s_forward<3>,
+                            fast_s_forward<0, kSLowRows[0]>, fast_s_forward<1, kSLowRows[0]>, fast_s_forward<2, kSLowRows[0]>, fast_s_forward<3, kSLowRows[0]>,
+                            fast_s_forward<0, kSLowRows[1]>, fast_s_forward<1, kSLowRows[1]>, fast_s_forward<2, kSLowRows[1]>, fast_s_forward<3, kSLowRows[1]>}) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
+            if (e != cudaSuccess) return e;
+        }
+        for (auto kernel : {fast_s_forward<0, kRS, true>, fast_s_forward<1, kRS, true>, fast_s_forward<2, kRS, true>}) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(true));
+            if (e != cudaSuccess) return e;
+        }
+        for (auto kernel : {fast_t_forward<0>, fast_t_forward<1>, fast_t_forward<2>, fast_t_forward<3>}) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
+            if (e != cudaSuccess) return e;
+        }
         e = set_stream_attributes();
         if (e != cudaSuccess) return e;
         e = set_resident_attributes();
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fast_t_forward<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
@@ -960,13 +952,17 @@ static void launch_s(FwdArgs& a, const FastState& fs, int mode, int sms, bool af
         if (after_kernel) launch_dependent(kernel, grid, kSThreads, bytes, stream, a);
         else kernel<<<grid, kSThreads, bytes, stream>>>(a);
     };
-    if (mode == 3) launch(fast_s_forward<3>);
-    else if (mode == 0 && wide) launch(fast_s_forward<0, true>);
-    else if (mode == 0) launch(fast_s_forward<0>);
-    else if (mode == 1 && wide) launch(fast_s_forward<1, true>);
-    else if (mode == 1) launch(fast_s_forward<1>);
-    else if (wide) launch(fast_s_forward<2, true>);
-    else launch(fast_s_forward<2>);
+    auto rows = [&](auto mode_tag) {
+        constexpr int MODE = decltype(mode_tag)::value;
+        if (wide && MODE != 3) launch(fast_s_forward<MODE, kRS, MODE != 3>);
+        else if (fs.host.s_rows == kSLowRows[0]) launch(fast_s_forward<MODE, kSLowRows[0]>);
+        else if (fs.host.s_rows == kSLowRows[1]) launch(fast_s_forward<MODE, kSLowRows[1]>);
+        else launch(fast_s_forward<MODE>);
+    };
+    if (mode == 0) rows(std::integral_constant<int, 0>{});
+    else if (mode == 1) rows(std::integral_constant<int, 1>{});
+    else if (mode == 2) rows(std::integral_constant<int, 2>{});
+    else rows(std::integral_constant<int, 3>{});
     count_launch();
 }
 

@@ -43,10 +43,10 @@ ROCKET_HD void rows_in_series(int t0, int r, int th, int rh, int rows, int& lo, 
     hi = left < (unsigned)rows ? (int)left : rows;
 }
 
-// S regime: the u of the first output row of raster column cg of a bucket.
-ROCKET_HD int s_column_u0(const SBucket& b, int cg) {
+// S regime: the u of the first output row of raster column cg of a bucket whose bands have `rows` rows.
+ROCKET_HD int s_column_u0(const SBucket& b, int cg, int rows = kRS) {
     const int band = cg / b.d, r = cg - band * b.d;
-    return (b.tmin + band * kRS) * b.d + r;
+    return (b.tmin + band * rows) * b.d + r;
 }
 
 // Stream regime: every one of the rows x 64 columns from (row trow, column c0) is an output of a kernel of dilation d.  span is

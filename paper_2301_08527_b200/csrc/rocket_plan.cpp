@@ -307,6 +307,38 @@ void estimate_costs(const HostParams& hp, PlanHost& p) {
     }
 }
 
+// Rows of the S bands: the height that takes the fewest clocks over all tiles.  A tile costs 3,000 clocks and its copies (24 B/clk) besides the
+// work of its kernels; a low band reads more rows per row of outputs, a high one may leave a dilation's last tile half empty (20 x 5,000: 81 % of the
+// positions of tiles of 24 rows are outputs, 89 % of 21).  Measured (us, 24 rows and the chosen height): 64 x 20 x 5,000 and 10,000 kernels 6,173
+// and 5,923, 1 x 20 x 5,000 322 and 289, backward of 24 x 20 x 5,000 and 3,000 kernels 2,087 and 1,948.
+int s_band_rows(const HostParams& hp, const std::vector<std::pair<int, std::vector<int>>>& groups) {
+    int best_rows = kRS;
+    double best = 1e300;
+    for (int R : {kRS, kSLowRows[0], kSLowRows[1]}) {
+        double clocks = 0.0;
+        for (const auto& kv : groups) {
+            const int64_t d = kv.first;
+            int64_t tmin = INT64_MAX, tmax = INT64_MIN;
+            double work = 0.0;
+            std::vector<char> used(hp.C, 0);
+            int nch = 0;
+            for (int k : kv.second) {
+                const int len = hp.length[k], m = hp.num_channels[k];
+                const int64_t lo = -(int64_t)hp.padding[k], hi = (int64_t)hp.L + hp.padding[k] - (len - 1) * d;
+                tmin = std::min(tmin, floor_div(lo, d));
+                tmax = std::max(tmax, floor_div(hi - 1, d));
+                work += m * (2.0 * R * len + 1.5 * (R + len) + 40.0) + 8.0 * R + 120.0;
+                for (int q = hp.channel_offset[k]; q < hp.channel_offset[k] + m; ++q)
+                    if (!used[hp.channel_idx[q]]) { used[hp.channel_idx[q]] = 1; ++nch; }
+            }
+            const int64_t bands = (tmax - tmin + R) / R, tiles = (bands * d + kWarpCols - 1) / kWarpCols;
+            clocks += (double)tiles * (work / 4.0 + 3000.0 + nch * (R + 10) * kWarpCols * 4 / 24.0);
+        }
+        if (clocks < 0.99 * best) { best = clocks; best_rows = R; }
+    }
+    return best_rows;
+}
+
 }  // namespace
 
 // A series of more channels than a tile has planes for needs buckets and copies that few or short kernels do not pay for: the generic
@@ -428,6 +460,8 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
         }
         for (Group& g : gs) groups.emplace_back(kv.first, std::move(g.ks));
     }
+    if (!all_tiles && hp.C <= kSMaxPlanes) out.s_rows = s_band_rows(hp, groups);
+    const int band_rows = out.s_rows;
     for (auto& kv : groups) {
         const int d = kv.first;
         auto& ks = kv.second;
@@ -461,9 +495,9 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
             out.s_max_nch = std::max(out.s_max_nch, b.nch);
         }
         b.tmin = (int32_t)tmin;
-        b.nbands = (int32_t)((tmax - tmin + 1 + kRS - 1) / kRS);
+        b.nbands = (int32_t)((tmax - tmin + 1 + band_rows - 1) / band_rows);
         b.raster_len = b.nbands * d;
-        b.rows = kRS + maxlen - 1;
+        b.rows = band_rows + maxlen - 1;
         const int bi = (int)out.sb.size();
         out.sb.push_back(b);
         // a tile is interior when its 64 raster positions exist and the u of every (row, column) lies inside
@@ -476,8 +510,8 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
         for (int c0 = 0; c0 < b.raster_len; c0 += kWarpCols) {
             bool interior = c0 + kWarpCols <= b.raster_len;
             for (int c = c0; interior && c < c0 + kWarpCols; ++c) {
-                const int64_t u0 = s_column_u0(b, c);
-                interior = u0 >= lo_max && u0 + (int64_t)(kRS - 1) * d < hi_min;
+                const int64_t u0 = s_column_u0(b, c, band_rows);
+                interior = u0 >= lo_max && u0 + (int64_t)(band_rows - 1) * d < hi_min;
             }
             s_cost.push_back({work + 0.3 * b.nch * b.rows, (int)out.sitems.size()});
             out.sitems.push_back({bi, c0, interior ? 1 : 0, 0});
