@@ -114,7 +114,7 @@ int finish_handle(rocket_params* p, rocket_params_t** out) {
     if (st == ROCKET_OK) {
         try {
             p->fast = new fast::FastState();
-            fast::build_plan(p->host, fast::kSplitDefault, p->fast->host, false);
+            fast::build_plan(p->host, fast::kSplitDefault, p->fast->host, false, true);
         } catch (const std::bad_alloc&) {
             st = ROCKET_ENOMEM;
         }

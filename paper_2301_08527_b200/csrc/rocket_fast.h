@@ -343,8 +343,9 @@ void fill_record_weights(const HostParams& hp, KRec& f);
 cudaError_t upload_records(FastState& fs);
 
 // Builds the launch plan for the kernels in hp (host side, once per handle).  all_tiles: also the T tiles of kernels that have
-// stream units, which no launch uses, and S bands of kRS rows.
-void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles = true);
+// stream units, which no launch uses, and S bands of kRS rows.  only_used: no tiles and units at all where the resident kernel serves every
+// pass of the handle.
+void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles = true, bool only_used = false);
 
 // Device-side state of the fast path owned by a handle.
 struct FastState {

@@ -814,36 +814,38 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-// Opts every fused kernel into its dynamic shared memory size, once per device.
-cudaError_t set_kernel_attributes(int dev) {
+template <typename... K>
+cudaError_t allow_smem(size_t bytes, K... kernels) {
     cudaError_t e = cudaSuccess;
+    ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : e), ...);
+    return e;
+}
+template <int ROWS>
+cudaError_t allow_s() {
+    return allow_smem(s_smem_bytes(false), fast_s_forward<0, ROWS>, fast_s_forward<1, ROWS>, fast_s_forward<2, ROWS>, fast_s_forward<3, ROWS>);
+}
+// Opts the fused kernels that a handle's calls may launch into their dynamic shared memory sizes, once per device and kind of kernel (which
+// also loads them: all kinds take milliseconds).
+cudaError_t set_kernel_attributes(int dev, const PlanHost& h) {
     static std::mutex attr_mu;
     std::lock_guard<std::mutex> attr_lock(attr_mu);
-    static bool attr_done_for[64] = {};
-    bool& attr_done = attr_done_for[dev & 63];
-    const size_t t_bytes = t_smem_bytes();
-    if (!attr_done) {
-        for (auto kernel : {fast_s_forward<0>, fast_s_forward<1>, fast_s_forward<2>, fast_s_forward<3>,
-                            fast_s_forward<0, kSLowRows[0]>, fast_s_forward<1, kSLowRows[0]>, fast_s_forward<2, kSLowRows[0]>, fast_s_forward<3, kSLowRows[0]>,
-                            fast_s_forward<0, kSLowRows[1]>, fast_s_forward<1, kSLowRows[1]>, fast_s_forward<2, kSLowRows[1]>, fast_s_forward<3, kSLowRows[1]>}) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(false));
-            if (e != cudaSuccess) return e;
-        }
-        for (auto kernel : {fast_s_forward<0, kRS, true>, fast_s_forward<1, kRS, true>, fast_s_forward<2, kRS, true>}) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem_bytes(true));
-            if (e != cudaSuccess) return e;
-        }
-        for (auto kernel : {fast_t_forward<0>, fast_t_forward<1>, fast_t_forward<2>, fast_t_forward<3>}) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t_bytes);
-            if (e != cudaSuccess) return e;
-        }
-        e = set_stream_attributes();
-        if (e != cudaSuccess) return e;
-        e = set_resident_attributes();
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
-    return cudaSuccess;
+    static bool done_for[64][8] = {};
+    bool* done = done_for[dev & 63];
+    cudaError_t e = cudaSuccess;
+    auto once = [&](int kind, bool needed, auto&& set) {
+        if (e != cudaSuccess || done[kind] || !needed) return;
+        e = set();
+        done[kind] = e == cudaSuccess;
+    };
+    once(0, h.resident && !h.r_small, [] { return set_resident_attributes(false); });
+    once(1, h.resident && h.r_small, [] { return set_resident_attributes(true); });
+    once(2, !h.sitems.empty() && !h.s_wide && h.s_rows == kRS, allow_s<kRS>);
+    once(3, !h.sitems.empty() && h.s_rows == kSLowRows[0], allow_s<kSLowRows[0]>);
+    once(4, !h.sitems.empty() && h.s_rows == kSLowRows[1], allow_s<kSLowRows[1]>);
+    once(5, h.s_wide, [] { return allow_smem(s_smem_bytes(true), fast_s_forward<0, kRS, true>, fast_s_forward<1, kRS, true>, fast_s_forward<2, kRS, true>); });
+    once(6, !h.wunits.empty(), [] { return set_stream_attributes(); });
+    once(7, !h.titems.empty(), [] { return allow_smem(t_smem_bytes(), fast_t_forward<0>, fast_t_forward<1>, fast_t_forward<2>, fast_t_forward<3>); });
+    return e;
 }
 
 // ---- backward helpers ----------------------------------------------------------------------------
@@ -1190,7 +1192,7 @@ cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N,
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if ((e = set_kernel_attributes(dev)) != cudaSuccess) return e;
+    if ((e = set_kernel_attributes(dev, fs.host)) != cudaSuccess) return e;
     if (again) fs.most_examples = 1 << 30;
     if (fs.host.resident && (!backward || resident_backward(fs.host)))
         return backward ? ensure_bwd_ws(fs, dp, n_weights) : cudaSuccess;   // no copies, no sums but the backward's
@@ -1224,7 +1226,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    e = set_kernel_attributes(dev);
+    e = set_kernel_attributes(dev, fs.host);
     if (e != cudaSuccess) return e;
     if (fs.host.resident) {
         ResidentArgs r = resident_args(fs, dp, X, N, lambda, shift);
@@ -1345,7 +1347,7 @@ cudaError_t launch_fast_backward(FastState& fs, const DeviceParams& dp, int64_t 
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    e = set_kernel_attributes(dev);
+    e = set_kernel_attributes(dev, fs.host);
     if (e != cudaSuccess) return e;
     const size_t t_bytes = t_smem_bytes();
     const PlanDevice& pd = fs.dev;

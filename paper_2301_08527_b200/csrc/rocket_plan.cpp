@@ -108,8 +108,8 @@ void build_stream_units(const HostParams& hp, size_t first, int d_max, PlanHost&
 
 // The kernels of a handle whose examples fit shared memory.
 struct ResidentUnits {
-    struct Cost { double c; RUnit u; };
-    std::vector<Cost> units;
+    std::vector<RUnit> units;
+    std::vector<double> cost;                          // of a pair, clocks of a scheduler
     double clocks = 0.0, longest = 0.0;
     int tiles = 0;
     int64_t reach = 0;                                 // how far before the first and behind the last sample a tile reads
@@ -119,6 +119,7 @@ ResidentUnits resident_units(const HostParams& hp, const PlanHost& plan, bool sm
     const int kHigh = resident_high(small), kLow = resident_low(small);
     ResidentUnits out;
     out.units.reserve(plan.krec.size());
+    out.cost.reserve(plan.krec.size());
     for (size_t i = 0; i < plan.krec.size(); ++i) {
         const KRec& f = plan.krec[i];
         RUnit u{};
@@ -149,16 +150,22 @@ ResidentUnits resident_units(const HostParams& hp, const PlanHost& plan, bool sm
         best += kRPairClocks;
         out.clocks += best / 4.0;
         out.longest = std::max(out.longest, best);
-        out.units.push_back({best, u});
+        out.units.push_back(u);
+        out.cost.push_back(best);
     }
     return out;
 }
 
 void build_resident_units(const HostParams& hp, PlanHost& out) {
     const int64_t row = (hp.L + 3ll) / 4 * 4;
-    if (hp.C * row > kRMostFloats) return;
-    for (const KRec& f : out.krec)
+    if (hp.C * row > kRMostFloats || hp.L > kRMostSteps) return;
+    const int64_t room = (kRMostFloats - hp.C * row) / (hp.C + 1) / 4 * 4;   // for zeros around the rows
+    int32_t most_padding = 0;
+    for (const KRec& f : out.krec) {
         if (f.nout > kRMostOutputs || f.d > kRMostOutputs) return;
+        most_padding = std::max(most_padding, f.p);
+    }
+    if (hp.L > kRMostStepsTested && room < most_padding) return;
     ResidentUnits r = resident_units(hp, out, false);
     if (hp.L < kRSmallSteps) {
         ResidentUnits s = resident_units(hp, out, true);
@@ -169,22 +176,26 @@ void build_resident_units(const HostParams& hp, PlanHost& out) {
     out.r_longest = r.longest;
     out.r_tiles = r.tiles;
     // Zeros around the rows make all reads alike; where they would not fit, or take more than twice the samples, some tiles test theirs.
-    const int64_t room = (kRMostFloats - hp.C * row) / (hp.C + 1) / 4 * 4;
     const int zeros = (int)std::min<int64_t>({(r.reach + 3) / 4 * 4, room, 2 * row});
     out.r_front = zeros;
     out.r_pitch = (int)row + zeros;
     out.r_zeros = zeros >= r.reach;
-    for (auto& c : r.units) {
-        RUnit& u = c.u;
+    out.resident = !r.units.empty() && hp.L <= (out.r_zeros ? kRMostSteps : kRMostStepsTested);
+    if (!out.resident) return;
+    for (RUnit& u : r.units) {
         const int before = std::max(0, u.p - zeros), end = hp.L + u.p + zeros;
         u.pq = before / u.d; u.pr = before % u.d;
         u.lq = end / u.d; u.lr = end % u.d;
     }
     // Kernels of a length follow one another, so that the warps of a block share inner loops; the longest pairs of a length first.  The
     // instruction caches decide here: the longest pairs first throughout took 846 us where this order takes 410 (100 x 20 x 2,800, 400 kernels).
-    std::stable_sort(r.units.begin(), r.units.end(), [](const auto& a, const auto& b) { return a.u.len != b.u.len ? a.u.len > b.u.len : a.c > b.c; });
-    for (const auto& c : r.units) out.runits.push_back(c.u);
-    out.resident = !out.runits.empty() && hp.L <= (out.r_zeros ? kRMostSteps : kRMostStepsTested);
+    std::vector<int> order(r.units.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return r.units[a].len != r.units[b].len ? r.units[a].len > r.units[b].len : r.cost[a] > r.cost[b];
+    });
+    out.runits.reserve(order.size());
+    for (int i : order) out.runits.push_back(r.units[i]);
 }
 
 }  // namespace
@@ -312,27 +323,33 @@ void estimate_costs(const HostParams& hp, PlanHost& p) {
 // positions of tiles of 24 rows are outputs, 89 % of 21).  Measured (us, 24 rows and the chosen height): 64 x 20 x 5,000 and 10,000 kernels 6,173
 // and 5,923, 1 x 20 x 5,000 322 and 289, backward of 24 x 20 x 5,000 and 3,000 kernels 2,087 and 1,948.
 int s_band_rows(const HostParams& hp, const std::vector<std::pair<int, std::vector<int>>>& groups) {
+    struct Sums { int64_t d, tmin, tmax; double taps, visits, kernels; int nch; };   // taps: products per output; visits: (kernel, channel) pairs
+    std::vector<Sums> sums;
+    for (const auto& kv : groups) {
+        Sums g{kv.first, INT64_MAX, INT64_MIN, 0.0, 0.0, (double)kv.second.size(), 0};
+        std::vector<char> used(hp.C, 0);
+        int64_t lo = INT64_MAX, hi = INT64_MIN;
+        for (int k : kv.second) {
+            const int len = hp.length[k], m = hp.num_channels[k];
+            lo = std::min<int64_t>(lo, -(int64_t)hp.padding[k]);
+            hi = std::max<int64_t>(hi, (int64_t)hp.L + hp.padding[k] - (len - 1) * g.d);
+            g.taps += (double)m * len;
+            g.visits += m;
+            for (int q = hp.channel_offset[k]; q < hp.channel_offset[k] + m; ++q)
+                if (!used[hp.channel_idx[q]]) { used[hp.channel_idx[q]] = 1; ++g.nch; }
+        }
+        g.tmin = floor_div(lo, g.d);
+        g.tmax = floor_div(hi - 1, g.d);
+        sums.push_back(g);
+    }
     int best_rows = kRS;
     double best = 1e300;
     for (int R : {kRS, kSLowRows[0], kSLowRows[1]}) {
         double clocks = 0.0;
-        for (const auto& kv : groups) {
-            const int64_t d = kv.first;
-            int64_t tmin = INT64_MAX, tmax = INT64_MIN;
-            double work = 0.0;
-            std::vector<char> used(hp.C, 0);
-            int nch = 0;
-            for (int k : kv.second) {
-                const int len = hp.length[k], m = hp.num_channels[k];
-                const int64_t lo = -(int64_t)hp.padding[k], hi = (int64_t)hp.L + hp.padding[k] - (len - 1) * d;
-                tmin = std::min(tmin, floor_div(lo, d));
-                tmax = std::max(tmax, floor_div(hi - 1, d));
-                work += m * (2.0 * R * len + 1.5 * (R + len) + 40.0) + 8.0 * R + 120.0;
-                for (int q = hp.channel_offset[k]; q < hp.channel_offset[k] + m; ++q)
-                    if (!used[hp.channel_idx[q]]) { used[hp.channel_idx[q]] = 1; ++nch; }
-            }
-            const int64_t bands = (tmax - tmin + R) / R, tiles = (bands * d + kWarpCols - 1) / kWarpCols;
-            clocks += (double)tiles * (work / 4.0 + 3000.0 + nch * (R + 10) * kWarpCols * 4 / 24.0);
+        for (const Sums& g : sums) {
+            const double work = (2.0 * R + 1.5) * g.taps + (1.5 * R + 40.0) * g.visits + (8.0 * R + 120.0) * g.kernels;
+            const int64_t bands = (g.tmax - g.tmin + R) / R, tiles = (bands * g.d + kWarpCols - 1) / kWarpCols;
+            clocks += (double)tiles * (work / 4.0 + 3000.0 + g.nch * (R + 10) * kWarpCols * 4 / 24.0);
         }
         if (clocks < 0.99 * best) { best = clocks; best_rows = R; }
     }
@@ -368,7 +385,7 @@ void fill_record_weights(const HostParams& hp, KRec& f) {
         for (int j = 0; j < f.len; ++j) f.w2[q][2 * j] = f.w2[q][2 * j + 1] = 0.0f - W[q * f.len + j];
 }
 
-void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) {
+void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles, bool only_used) {
     out = PlanHost();
     out.flops_s = out.flops_t = 0.0;
     if (split < kTMinDilation) split = kTMinDilation;
@@ -409,6 +426,22 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles) 
         for (int q = 0; q < f.m; ++q) f.ch[q] = S[q];
         fill_record_weights(hp, f);
     };
+
+    if (only_used && (int64_t)hp.C * hp.L <= kRMostFloats && hp.L <= kRMostStepsBackward) {
+        // series for which the resident kernel most likely serves every pass: then nothing else is needed
+        for (const auto* list : {&s_kernels, &t_kernels})
+            for (int k : *list) {
+                add_kernel(k);
+                const KRec& f = out.krec.back();
+                (list == &s_kernels ? out.flops_s : out.flops_t) += 2.0 * f.len * f.m * (double)f.nout;
+            }
+        build_resident_units(hp, out);
+        if (resident_backward(out)) return;
+        out.krec.clear();
+        out.runits.clear();
+        out.resident = false;
+        out.flops_s = out.flops_t = 0.0;
+    }
 
     // ---- S regime: one bucket per dilation, kernels inside ordered by cost (largest first: the warps of a
     // block pull them one by one, so the cheap ones fill the end of a tile evenly).  Buckets with many

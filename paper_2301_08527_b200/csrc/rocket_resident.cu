@@ -490,14 +490,14 @@ __global__ void __launch_bounds__(32 * resident_warps(MODE, SMALL), 1) fast_resi
 
 }  // namespace
 
-cudaError_t set_resident_attributes() {
-    constexpr int bytes = kRMostFloats * (int)sizeof(float);
+template <bool SMALL>
+static cudaError_t allow_smem() {
     cudaError_t e = cudaSuccess;
-    for (auto kernel : {fast_resident<0, false>, fast_resident<1, false>, fast_resident<2, false>, fast_resident<3, false>, fast_resident<0, true>,
-                        fast_resident<1, true>, fast_resident<2, true>, fast_resident<3, true>})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    for (auto kernel : {fast_resident<0, SMALL>, fast_resident<1, SMALL>, fast_resident<2, SMALL>, fast_resident<3, SMALL>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRMostFloats * (int)sizeof(float));
     return e;
 }
+cudaError_t set_resident_attributes(bool small) { return small ? allow_smem<true>() : allow_smem<false>(); }
 
 void launch_resident(ResidentArgs& a, const PlanHost& plan, int mode, int sms, cudaStream_t stream) {
     const ResidentSplit s = resident_split(plan, a.N, a.C, sms, mode);
