@@ -232,20 +232,28 @@ struct TMapSpec { int32_t d, box_cols, box_rows; };
 
 // ---- resident regime (rocket_resident.cu): short series, whole examples in shared memory ------
 // Heights of its bands.  Odd: neighbouring columns of a band row lie side by side and those of the next band an odd number of rows further on, so
-// that a warp's loads meet few times in a shared-memory bank, at dilation 1 too, where 16 rows would meet sixteen times.  The low ones (small)
-// where series are too short for the others' 64 columns.  Measured, hard, us: 100 x 1 x 64 and 5,000 kernels 329 with 17 and 11 rows, 289
-// with 15 and 9; 100 x 6 x 1,251 1,261 and 1,274 (17 and 9: 1,322).
-ROCKET_CX int resident_high(bool small) { return small ? 9 : 17; }
-ROCKET_CX int resident_low(bool small) { return small ? 5 : 11; }
+// that a warp's loads meet few times in a shared-memory bank, at dilation 1 too, where 16 rows would meet sixteen times.  A tile is 64
+// columns, so that what decides is how many tiles a series fills.
+// Forward: 17 and 11 rows (bands = 0), 9 and 5 (1) where series are too short for those 64 columns, 21 and 11 (2) just beyond what one tile of
+// 17 rows holds.  Hard, us: 100 x 1 x 64 and 5,000 kernels 329 with 17 and 11 rows, 289 with 15 and 9; 120 x 1 x 1,180 and 10,000 kernels 1,626
+// with 17 and 11, 1,379 with 21 and 11 (20 warps; 18: 1,414).
+// Backward: one height, 5, 7, 9 or 11 (3 to 6).  It runs a convolution and a gradient per length and height, more code than the instruction
+// caches hold (at 17 and 11 rows 40 % of the issue slots were used, with more than half of a warp's stalls for instructions): less code
+// is worth more than the reads that higher bands save.  24 x 6 x 900 and 2,000 kernels 312 us before, 360 at 17 and 11 rows, 233 at 9; 100 x 6 x
+// 640 and 5,000 kernels 2,480, 1,915, 1,475 (11; 13: 1,970); 100 x 6 x 1,900 and 5,000 4,560, 3,840 (tile kernels), 3,647; 100 x 6 x 200 and
+// 5,000 2,527, 905 (9 and 5 rows, 16 warps), 812 (5 rows).
+ROCKET_CX int resident_high(int bands) { return bands >= 3 ? 2 * bands - 1 : bands == 2 ? 21 : bands == 1 ? 9 : 17; }
+ROCKET_CX int resident_low(int bands) { return bands >= 3 ? 2 * bands - 1 : bands == 1 ? 5 : 11; }
+constexpr int kRBackBands[4] = {3, 4, 5, 6};
 // Warps of a block (mode: 0 = hard, 1 = soft, 2 = backward, 3 = hard in half precision).
-ROCKET_CX int resident_warps(int mode, bool small) { return mode == 2 ? 16 : mode == 1 ? 20 : small ? 28 : 24; }
+ROCKET_CX int resident_warps(int mode, int bands) { return mode == 2 || mode == 1 || bands == 2 ? 20 : bands == 1 ? 28 : 24; }
 constexpr int kRMostFloats = 57600;                                // what shared memory holds: examples, rows padded to 16 bytes
 // The longest series: beyond, a pair is a warp's for too long where there are few, and the other kernels' larger tiles are as good where there
 // are many (us, before and with this kernel: 1 x 3 x 5,000, 10,000 kernels 192 and 97, 100 x 3 x 5,000, 5,000 kernels 2,825 and 2,842; 8 x 3 x
 // 18,000, 1,000 kernels 205 and 257).  The second where tiles test their reads (24 x 32 x 1,751, 2,000 kernels 477 and 218; 8 x 9 x 6,000,
 // 1,000 kernels 142 and 240).
-constexpr int kRMostSteps = 5000, kRMostStepsTested = 2048, kRMostStepsBackward = 1000;
-constexpr int kRSmallSteps = 1024;                                 // series to be short for the low bands
+constexpr int kRMostSteps = 5000, kRMostStepsTested = 2048;
+constexpr int kRSmallSteps = 1024, kRTallSteps = 1600;             // steps up to which the low bands are considered, and from there the tallest
 constexpr int kRMostOutputs = 1 << 20;                             // outputs and dilation up to which columns are counted exactly in FP32
 
 // One kernel (32 words).  Its outputs, counted from the first one, are t d + r for t < nq + (r < nr); the input rows of column r that
@@ -267,7 +275,7 @@ struct ResidentSplit { int examples, groups, parts, run, split; unsigned grid; }
 struct PlanHost {
     bool enabled = false;
     bool resident = false;                // the examples fit the resident kernel's shared memory
-    bool r_small = false;                 // its bands are the low ones
+    int r_bands = 0, r_back = 0;          // the heights of its bands; those of the backward's, 0 if it does not serve it
     bool r_zeros = false;                 // and so do zeros around every row, as far as any tile reads
     std::vector<RUnit> runits;
     int r_front = 0, r_pitch = 0;         // floats of zeros in front of the first channel row in shared memory; from row to row
@@ -315,7 +323,7 @@ inline int64_t resident_merge_floats(const PlanHost& plan, int64_t n, int parts,
 }
 // The backward, whose code is twice as long and whose sums leave the warp once per tile, only where no tile has to test its reads and series
 // are short (us, before and with this kernel: 100 x 6 x 600, 2,000 kernels 1,106 and 855; 100 x 6 x 1,251 1,308 and 1,790).
-bool resident_backward(const PlanHost& plan);
+inline bool resident_backward(const PlanHost& plan) { return plan.r_back != 0; }
 // Floats of shared memory for n examples.
 inline int64_t resident_floats(const PlanHost& plan, int64_t n, int C) { return plan.r_front + n * C * plan.r_pitch; }
 

@@ -57,7 +57,7 @@ struct ResidentArgs {
     long long n_weights;
 };
 void launch_resident(ResidentArgs& a, const PlanHost& plan, int mode, int sms, cudaStream_t stream);
-cudaError_t set_resident_attributes(bool small);
+cudaError_t set_resident_attributes(int bands, bool backward);
 
 // A launch that may begin while its predecessor in the stream ends (programmatic dependent launch): the kernel itself waits for the
 // predecessor with dependency_wait() before it touches anything, or states why it need not.

@@ -829,7 +829,7 @@ cudaError_t allow_s() {
 cudaError_t set_kernel_attributes(int dev, const PlanHost& h) {
     static std::mutex attr_mu;
     std::lock_guard<std::mutex> attr_lock(attr_mu);
-    static bool done_for[64][8] = {};
+    static bool done_for[64][13] = {};
     bool* done = done_for[dev & 63];
     cudaError_t e = cudaSuccess;
     auto once = [&](int kind, bool needed, auto&& set) {
@@ -837,14 +837,14 @@ cudaError_t set_kernel_attributes(int dev, const PlanHost& h) {
         e = set();
         done[kind] = e == cudaSuccess;
     };
-    once(0, h.resident && !h.r_small, [] { return set_resident_attributes(false); });
-    once(1, h.resident && h.r_small, [] { return set_resident_attributes(true); });
-    once(2, !h.sitems.empty() && !h.s_wide && h.s_rows == kRS, allow_s<kRS>);
-    once(3, !h.sitems.empty() && h.s_rows == kSLowRows[0], allow_s<kSLowRows[0]>);
-    once(4, !h.sitems.empty() && h.s_rows == kSLowRows[1], allow_s<kSLowRows[1]>);
-    once(5, h.s_wide, [] { return allow_smem(s_smem_bytes(true), fast_s_forward<0, kRS, true>, fast_s_forward<1, kRS, true>, fast_s_forward<2, kRS, true>); });
-    once(6, !h.wunits.empty(), [] { return set_stream_attributes(); });
-    once(7, !h.titems.empty(), [] { return allow_smem(t_smem_bytes(), fast_t_forward<0>, fast_t_forward<1>, fast_t_forward<2>, fast_t_forward<3>); });
+    for (int bands = 0; bands < 3; ++bands) once(6 + bands, h.resident && h.r_bands == bands, [bands] { return set_resident_attributes(bands, false); });
+    for (int bands : kRBackBands) once(6 + bands, h.r_back == bands, [bands] { return set_resident_attributes(bands, true); });
+    once(0, !h.sitems.empty() && !h.s_wide && h.s_rows == kRS, allow_s<kRS>);
+    once(1, !h.sitems.empty() && h.s_rows == kSLowRows[0], allow_s<kSLowRows[0]>);
+    once(2, !h.sitems.empty() && h.s_rows == kSLowRows[1], allow_s<kSLowRows[1]>);
+    once(3, h.s_wide, [] { return allow_smem(s_smem_bytes(true), fast_s_forward<0, kRS, true>, fast_s_forward<1, kRS, true>, fast_s_forward<2, kRS, true>); });
+    once(4, !h.wunits.empty(), [] { return set_stream_attributes(); });
+    once(5, !h.titems.empty(), [] { return allow_smem(t_smem_bytes(), fast_t_forward<0>, fast_t_forward<1>, fast_t_forward<2>, fast_t_forward<3>); });
     return e;
 }
 

@@ -113,10 +113,12 @@ struct ResidentUnits {
     double clocks = 0.0, longest = 0.0;
     int tiles = 0;
     int64_t reach = 0;                                 // how far before the first and behind the last sample a tile reads
+    double clocks_back[4] = {};                        // the same for each height of the backward
+    int64_t reach_back[4] = {};
 };
 
-ResidentUnits resident_units(const HostParams& hp, const PlanHost& plan, bool small) {
-    const int kHigh = resident_high(small), kLow = resident_low(small);
+ResidentUnits resident_units(const HostParams& hp, const PlanHost& plan, int kind) {
+    const int kHigh = resident_high(kind), kLow = resident_low(kind);
     ResidentUnits out;
     out.units.reserve(plan.krec.size());
     out.cost.reserve(plan.krec.size());
@@ -146,6 +148,11 @@ ResidentUnits resident_units(const HostParams& hp, const PlanHost& plan, bool sm
         consider(rows / kHigh);
         const int64_t last_row = (int64_t)u.high * kHigh + u.low * kLow - 1 + f.len - 1;
         out.reach = std::max<int64_t>({out.reach, f.p, last_row * f.d + f.d - f.p - hp.L});
+        for (int h = 0; h < 4; ++h) {
+            const int R = resident_high(kRBackBands[h]), bands = (rows + R - 1) / R;
+            out.clocks_back[h] += tiles(bands) * tile_clocks(R);
+            out.reach_back[h] = std::max<int64_t>({out.reach_back[h], f.p, (int64_t)(bands * R + f.len - 2) * f.d + f.d - f.p - hp.L});
+        }
         out.tiles = (int)std::max<int64_t>(out.tiles, tiles(u.high) + tiles(u.low));
         best += kRPairClocks;
         out.clocks += best / 4.0;
@@ -166,22 +173,31 @@ void build_resident_units(const HostParams& hp, PlanHost& out) {
         most_padding = std::max(most_padding, f.p);
     }
     if (hp.L > kRMostStepsTested && room < most_padding) return;
-    ResidentUnits r = resident_units(hp, out, false);
-    if (hp.L < kRSmallSteps) {
-        ResidentUnits s = resident_units(hp, out, true);
-        out.r_small = s.clocks < r.clocks;
-        if (out.r_small) r = std::move(s);
+    ResidentUnits r = resident_units(hp, out, 0);
+    if (hp.L <= kRTallSteps) {
+        const int other = hp.L < kRSmallSteps ? 1 : 2;
+        ResidentUnits s = resident_units(hp, out, other);
+        if (s.clocks < r.clocks) {
+            out.r_bands = other;
+            r = std::move(s);
+        }
     }
     out.r_clocks = r.clocks;
     out.r_longest = r.longest;
     out.r_tiles = r.tiles;
+    const int64_t most_zeros = std::min(room, 2 * row);
+    int h = 0;
+    for (int other = 1; other < 4; ++other)
+        if (r.reach_back[h] > most_zeros || (r.reach_back[other] <= most_zeros && r.clocks_back[other] < r.clocks_back[h])) h = other;
+    const bool back = r.reach_back[h] <= most_zeros;
     // Zeros around the rows make all reads alike; where they would not fit, or take more than twice the samples, some tiles test theirs.
-    const int zeros = (int)std::min<int64_t>({(r.reach + 3) / 4 * 4, room, 2 * row});
+    const int zeros = (int)std::min((std::max(r.reach, back ? r.reach_back[h] : 0) + 3) / 4 * 4, most_zeros);
     out.r_front = zeros;
     out.r_pitch = (int)row + zeros;
     out.r_zeros = zeros >= r.reach;
     out.resident = !r.units.empty() && hp.L <= (out.r_zeros ? kRMostSteps : kRMostStepsTested);
     if (!out.resident) return;
+    out.r_back = back ? kRBackBands[h] : 0;
     for (RUnit& u : r.units) {
         const int before = std::max(0, u.p - zeros), end = hp.L + u.p + zeros;
         u.pq = before / u.d; u.pr = before % u.d;
@@ -200,13 +216,11 @@ void build_resident_units(const HostParams& hp, PlanHost& out) {
 
 }  // namespace
 
-bool resident_backward(const PlanHost& plan) { return plan.resident && plan.r_zeros && plan.r_pitch - plan.r_front <= kRMostStepsBackward; }
-
 // Blocks take tasks of a few examples and a part of the kernels: as few copies of an example as leave every SM its share.
 ResidentSplit resident_split(const PlanHost& plan, int N, int C, int sms, int mode) {
     const double work = plan.r_clocks * (mode == 1 ? 1.4 : mode == 2 ? 2.6 : 1.0);
     const int64_t n_units = (int64_t)plan.runits.size();
-    const int warps = resident_warps(mode, plan.r_small);
+    const int warps = resident_warps(mode, mode == 2 ? plan.r_back : plan.r_bands);
     // eight items per warp and task, if that many there are
     auto run_of = [&](int64_t kernels, int64_t e) { return std::max<int64_t>(1, std::min<int64_t>(e, kernels * e / (8 * warps))); };
     ResidentSplit best{1, N, 1, 1, 1, 1u};
@@ -427,7 +441,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles, 
         fill_record_weights(hp, f);
     };
 
-    if (only_used && (int64_t)hp.C * hp.L <= kRMostFloats && hp.L <= kRMostStepsBackward) {
+    if (only_used && (int64_t)hp.C * hp.L <= kRMostFloats && hp.L <= kRMostSteps) {
         // series for which the resident kernel most likely serves every pass: then nothing else is needed
         for (const auto* list : {&s_kernels, &t_kernels})
             for (int k : *list) {
@@ -440,6 +454,7 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles, 
         out.krec.clear();
         out.runits.clear();
         out.resident = false;
+        out.r_back = 0;
         out.flops_s = out.flops_t = 0.0;
     }
 

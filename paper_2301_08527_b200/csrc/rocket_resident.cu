@@ -3,8 +3,8 @@
 // With u = t d + r a dilated convolution is a dense filter down the columns of A[t][r] = x[t d + r].  A block brings one or more whole
 // examples (all channels, zeros between the rows as far as there is room) into shared memory and its warps take (kernel, example) pairs one by
 // one, or parts of them where there are few; the parts of a pair meet in shared memory, so that features are written once and finally: no
-// initialising and finalising kernels, no staging copies, no workspace.  A pair's outputs are cut into bands of two heights (17 and 11 rows, 9
-// and 5 for the shortest series) from its own first output on; a warp tile is 64 neighbouring columns of the bands strung together, a lane
+// initialising and finalising kernels, no staging copies, no workspace.  A pair's outputs are cut into bands of two heights, in the
+// backward of one (see resident_high), from its own first output on; a warp tile is 64 neighbouring columns of the bands strung together, a lane
 // owns columns lane and lane + 32 as packed pairs.
 //
 // Why: the other kernels copy a tile per dilation (or per kernel) to use it for a handful of kernels, in bands of at least 8 rows that
@@ -15,7 +15,8 @@
 // that addresses are no immediate offsets); what else counts is code, of which the warps of an SM should share as little as possible at a
 // time: with zeros beside the rows in place of tests a backward of 24 x 6 x 1,251 went from 960 to 540 us, with kernels ordered by length and
 // not by work 100 x 20 x 2,800 from 846 to 410.  Measured (us, before and now): 24 x 32 x 1,751 with 2,000 kernels 476 and 222, 16 x 1 x 512 with 1,000
-// 35 and 22, 100 x 20 x 600 with 4,000 1,283 and 717, soft 1,167 and 445 (2,000 kernels).
+// 35 and 22, 100 x 20 x 600 with 4,000 1,283 and 717, soft 1,167 and 445 (2,000
+// kernels), backward of 24 x 9 x 700 with 2,000 373 and 200.
 #include <algorithm>
 
 #include "rocket_fast.h"
@@ -28,7 +29,7 @@ namespace {
 
 extern __shared__ __align__(128) unsigned char smem_raw[];
 
-static_assert(resident_high(false) + ROCKET_MAX_LENGTH - 1 <= 31, "the row masks hold the input rows of a tile");
+static_assert(resident_high(2) + ROCKET_MAX_LENGTH - 1 <= 31, "the row masks hold the input rows of a tile");
 
 __device__ __forceinline__ void copy4(uint32_t dst, const void* src) { asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory"); }
 __device__ __forceinline__ void copy16(uint32_t dst, const void* src) { asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory"); }
@@ -81,9 +82,9 @@ struct Pair {
 };
 
 // What depends on the heights of the bands.
-template <bool SMALL>
+template <int HIGH, int LOW>
 struct Bands {
-static constexpr int kHigh = resident_high(SMALL), kLow = resident_low(SMALL);
+static constexpr int kHigh = HIGH, kLow = LOW;
 
 template <int ELL, int R, bool INSIDE>
 static __device__ __forceinline__ void resident_conv(const Columns& at, float mine, u64 (&acc)[kHigh]) {
@@ -251,10 +252,11 @@ static __device__ __forceinline__ float make_gz_rows(u64 (&acc)[kHigh], bool hig
 }
 };
 
-template <int MODE, bool SMALL>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision; SMALL: low bands
-__global__ void __launch_bounds__(32 * resident_warps(MODE, SMALL), 1) fast_resident(const __grid_constant__ ResidentArgs a) {
-    using B = Bands<SMALL>;
-    constexpr int kWarps = resident_warps(MODE, SMALL), kHigh = B::kHigh, kLow = B::kLow;
+template <int MODE, int BANDS>  // 0 = hard, 1 = soft, 2 = backward of soft, 3 = hard in half precision; BANDS: their heights
+__global__ void __launch_bounds__(32 * resident_warps(MODE, BANDS), 1) fast_resident(const __grid_constant__ ResidentArgs a) {
+    using B = Bands<resident_high(BANDS), resident_low(BANDS)>;
+    constexpr bool kOneHeight = B::kHigh == B::kLow;
+    constexpr int kWarps = resident_warps(MODE, BANDS), kHigh = B::kHigh, kLow = B::kLow;
     __shared__ int s_next;
     float* xs = reinterpret_cast<float*>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -318,10 +320,10 @@ __global__ void __launch_bounds__(32 * resident_warps(MODE, SMALL), 1) fast_resi
             const float w_first_n = first_weight(v1), negb_n = bias_of(v1);   // what the next item needs first
             auto field = [&](int f) { return __shfl_sync(kFull, v, f); };
             const int krec = field(0), k = field(1), len = field(2), d = field(3), m = field(4), nout = field(5), p = field(6);
-            const int high_bands = field(7), low_bands = field(8);
             const float* __restrict__ wl = &a.krec[krec].w2[0][0] + weight_lane;
             const int nq = field(9), nr = field(10), pq = field(11), pr = field(12), lq = field(13), lr = field(14);
             const float inv_d = __int_as_float(field(15));
+            const int high_bands = kOneHeight ? (nq + (nr > 0) + kHigh - 1) / kHigh : field(7), low_bands = kOneHeight ? 0 : field(8);
             const unsigned row_bytes = 4u * (unsigned)a.pitch;
             const int e_end = min(ne, e0 + a.run);
             const double scale = MODE == 2 ? __ldg(a.scale + k) : 0.0;
@@ -345,7 +347,7 @@ __global__ void __launch_bounds__(32 * resident_warps(MODE, SMALL), 1) fast_resi
                     tA = at / d;
                     rA = at - tA * d;
                 }
-                for (int half = 0; half < 2; ++half) {
+                for (int half = 0; half < (kOneHeight ? 1 : 2); ++half) {
                     const bool high = half == 0;
                     const int R = high ? kHigh : kLow, ncols = (high ? high_bands : low_bands) * d;
                     for (int c0 = 0; c0 < ncols; c0 += kWarpCols) {
@@ -394,7 +396,7 @@ __global__ void __launch_bounds__(32 * resident_warps(MODE, SMALL), 1) fast_resi
                             if (q + 1 < m) wn += kPairRow;
                             const float mine_next = __ldg(wn);
                             const Columns at = columns(q);
-                            B::by_form(len, high, inside, [&](auto len_tag, auto r_tag, auto inside_tag) {
+                            B::by_form(len, high, MODE == 2 || inside, [&](auto len_tag, auto r_tag, auto inside_tag) {
                                 if constexpr (MODE == 3) B::template resident_conv<decltype(len_tag)::value, decltype(r_tag)::value, decltype(inside_tag)::value>(at, mine, acch);
                                 else B::template resident_conv<decltype(len_tag)::value, decltype(r_tag)::value, decltype(inside_tag)::value>(at, mine, acc);
                             });
@@ -412,7 +414,7 @@ __global__ void __launch_bounds__(32 * resident_warps(MODE, SMALL), 1) fast_resi
 #pragma unroll
                                 for (int j = 0; j < ROCKET_MAX_LENGTH; ++j) dw[j] = 0ull;
                                 const Columns at = columns(q);
-                                B::by_form(len, high, inside, [&](auto len_tag, auto r_tag, auto inside_tag) {
+                                B::by_form(len, high, MODE == 2 || inside, [&](auto len_tag, auto r_tag, auto inside_tag) {
                                     B::template resident_grad<decltype(len_tag)::value, decltype(r_tag)::value, decltype(inside_tag)::value>(at, acc, dw);
                                 });
                                 reduce_publish_dw<ROCKET_MAX_LENGTH>(dw, dst, scale, lane, len);
@@ -490,14 +492,18 @@ __global__ void __launch_bounds__(32 * resident_warps(MODE, SMALL), 1) fast_resi
 
 }  // namespace
 
-template <bool SMALL>
-static cudaError_t allow_smem() {
+static cudaError_t allow_smem(std::initializer_list<void (*)(ResidentArgs)> kernels) {
     cudaError_t e = cudaSuccess;
-    for (auto kernel : {fast_resident<0, SMALL>, fast_resident<1, SMALL>, fast_resident<2, SMALL>, fast_resident<3, SMALL>})
+    for (auto kernel : kernels)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRMostFloats * (int)sizeof(float));
     return e;
 }
-cudaError_t set_resident_attributes(bool small) { return small ? allow_smem<true>() : allow_smem<false>(); }
+cudaError_t set_resident_attributes(int bands, bool backward) {
+    if (backward) return allow_smem({bands == 3 ? fast_resident<2, 3> : bands == 4 ? fast_resident<2, 4> : bands == 5 ? fast_resident<2, 5> : fast_resident<2, 6>});
+    return bands == 0   ? allow_smem({fast_resident<0, 0>, fast_resident<1, 0>, fast_resident<3, 0>})
+           : bands == 1 ? allow_smem({fast_resident<0, 1>, fast_resident<1, 1>, fast_resident<3, 1>})
+                        : allow_smem({fast_resident<0, 2>, fast_resident<1, 2>, fast_resident<3, 2>});
+}
 
 void launch_resident(ResidentArgs& a, const PlanHost& plan, int mode, int sms, cudaStream_t stream) {
     const ResidentSplit s = resident_split(plan, a.N, a.C, sms, mode);
@@ -510,12 +516,13 @@ void launch_resident(ResidentArgs& a, const PlanHost& plan, int mode, int sms, c
     a.pitch = plan.r_pitch;
     a.aligned = a.L % 4 == 0 && (reinterpret_cast<uintptr_t>(a.X) & 15u) == 0;
     const size_t bytes = (size_t)(resident_floats(plan, s.examples, a.C) + resident_merge_floats(plan, s.examples, s.parts, s.split, mode)) * sizeof(float);
-    const bool small = plan.r_small;
-    auto kernel = mode == 0   ? (small ? fast_resident<0, true> : fast_resident<0, false>)
-                  : mode == 1 ? (small ? fast_resident<1, true> : fast_resident<1, false>)
-                  : mode == 2 ? (small ? fast_resident<2, true> : fast_resident<2, false>)
-                              : (small ? fast_resident<3, true> : fast_resident<3, false>);
-    kernel<<<s.grid, 32 * resident_warps(mode, small), bytes, stream>>>(a);
+    const int bands = mode == 2 ? plan.r_back : plan.r_bands;
+    auto of = [bands](auto k0, auto k1, auto k2) { return bands == 0 ? k0 : bands == 1 ? k1 : k2; };
+    auto kernel = mode == 0   ? of(fast_resident<0, 0>, fast_resident<0, 1>, fast_resident<0, 2>)
+                  : mode == 1 ? of(fast_resident<1, 0>, fast_resident<1, 1>, fast_resident<1, 2>)
+                  : mode == 3 ? of(fast_resident<3, 0>, fast_resident<3, 1>, fast_resident<3, 2>)
+                              : bands == 3 ? fast_resident<2, 3> : bands == 4 ? fast_resident<2, 4> : bands == 5 ? fast_resident<2, 5> : fast_resident<2, 6>;
+    kernel<<<s.grid, 32 * resident_warps(mode, bands), bytes, stream>>>(a);
     count_launch();
 }
 

@@ -24,12 +24,16 @@ namespace rocket { std::atomic<int64_t> g_launch_count{0}; }
         }                                                         \
     } while (0)
 
-static void check_units(const PlanHost& plan, int L) {
+// backward: in the bands of its own, all of whose reads are samples or zeros
+static void check_units(const PlanHost& plan, int L, bool backward) {
+    const int bands = backward ? plan.r_back : plan.r_bands;
+    const bool one_height = resident_high(bands) == resident_low(bands);
     for (const RUnit& u : plan.runits) {
         std::vector<int> owned(u.nout, 0);
         for (int half = 0; half < 2; ++half) {
-            const int high = resident_high(plan.r_small), R = half ? resident_low(plan.r_small) : high;
-            const int ncols = (half ? u.low : u.high) * u.d, base = half ? high * u.high : 0;
+            const int high = resident_high(bands), R = half ? resident_low(bands) : high;
+            const int high_bands = one_height ? (u.nq + (u.nr > 0) + high - 1) / high : u.high, low_bands = one_height ? 0 : u.low;
+            const int ncols = (half ? low_bands : high_bands) * u.d, base = half ? high * high_bands : 0;
             for (int c0 = 0; c0 < ncols; c0 += kWarpCols)
                 for (int l = 0; l < kWarpCols; ++l) {
                     const int c = std::min(c0 + l, ncols - 1);
@@ -44,6 +48,7 @@ static void check_units(const PlanHost& plan, int L) {
                     if (out < R && c0 + l < ncols) REQUIRE(at.i0 + (int64_t)out * u.d >= u.nout, "an output is left out");
                     for (int s = 0; s < rows; ++s) {
                         const int64_t x = at.i0 - (int64_t)u.p + (int64_t)s * u.d;
+                        if (backward) REQUIRE(s >= at.in_lo && s < at.in_hi, "a read of the backward outside the zeros");
                         REQUIRE((s >= at.in_lo && s < at.in_hi) == (x >= -plan.r_front && x < L + plan.r_front), "input row %d of column %d (d %d, p %d)", s, c, u.d, u.p);
                     }
                 }
@@ -53,7 +58,8 @@ static void check_units(const PlanHost& plan, int L) {
 }
 
 static void check_split(const PlanHost& plan, int C) {
-    for (int mode = 0; mode < 4; ++mode)
+    for (int mode = 0; mode < 4; ++mode) {
+        if (mode == 2 && !resident_backward(plan)) continue;
         for (int N : {1, 2, 3, 7, 24, 100, 149, 1000, 20000, 300000}) {
             const ResidentSplit s = resident_split(plan, N, C, 148, mode);
             REQUIRE(s.examples >= 1 && resident_floats(plan, s.examples, C) <= kRMostFloats, "examples %d", s.examples);
@@ -63,24 +69,25 @@ static void check_split(const PlanHost& plan, int C) {
             REQUIRE(s.split == 1 || (s.run == 1 && resident_floats(plan, s.examples, C) + resident_merge_floats(plan, s.examples, s.parts, s.split, mode) <= kRMostFloats), "room to merge");
             REQUIRE(s.grid >= 1 && s.grid <= 148 && (int64_t)s.groups * s.parts <= 0x7fffffff, "grid");
         }
+    }
 }
 
 int main() {
     std::mt19937 rng(5);
-    int resident = 0, others = 0, small = 0;
-    for (int round = 0; round < 60; ++round) {
+    int resident = 0, others = 0, bands[7] = {};
+    for (int round = 0; round < 90; ++round) {
         HostParams hp;
-        const int Ls[] = {16, 64, 65, 301, 512, 1025, 1251, 1800, 2047, 2880, 9001};
-        const int L = Ls[rng() % 11], C = std::max(1, std::min<int>(255, round % 3 ? (int)(rng() % 40) + 1 : 57600 / L + (int)(rng() % 2)));
+        const int Ls[] = {16, 64, 65, 301, 512, 700, 900, 1025, 1100, 1251, 1800, 2047, 2880, 9001};
+        const int L = Ls[rng() % 14], C = std::max(1, std::min<int>(255, round % 3 ? (int)(rng() % 40) + 1 : 57600 / L + (int)(rng() % 2)));
         hp.C = C; hp.L = L; hp.K = 40;
         for (int k = 0; k < hp.K; ++k) {
             const int len = (int)(rng() % 3) * 2 + 7, dmax = std::max(1, (L - 1) / (len - 1));
             int d = 1 + (int)(rng() % dmax), p = 0;
             if (k % 3 == 0) d = 1 + (int)(rng() % std::min(dmax, 9));
-            if (k % 7 == 0) d = L / 3 + (int)(rng() % L);                            // beyond what random kernels have
+            if (k % 7 == 0 && round % 2) d = L / 3 + (int)(rng() % L);                            // beyond what random kernels have
             const int span = (len - 1) * d;
             const int lowest = std::max(0, (span - L) / 2 + 1), choices[] = {lowest, std::max(lowest, span / 2), std::max(lowest, (int)(rng() % (span + 3))), std::max(lowest, span + 5)};
-            p = choices[rng() % 4];
+            p = choices[round % 2 ? rng() % 4 : rng() % 2];
             const int m = 1 + (int)(rng() % std::min(C, len));
             hp.length.push_back(len); hp.dilation.push_back(d); hp.padding.push_back(p); hp.num_channels.push_back(m);
             hp.bias.push_back(0.5f);
@@ -98,7 +105,6 @@ int main() {
         if (!fits || L > kRMostSteps) REQUIRE(!plan.resident, "%d x %d is too long", C, L);
         if (fits && L <= kRMostStepsTested) REQUIRE(plan.resident, "%d x %d fits", C, L);
         ++(plan.resident ? resident : others);
-        small += plan.r_small;
         if (!plan.resident) continue;
         REQUIRE(L <= kRMostStepsTested || plan.r_zeros, "%d steps test their reads", L);
         REQUIRE((int)plan.runits.size() == hp.K, "a kernel is missing");
@@ -109,11 +115,15 @@ int main() {
             for (int k = 0; k < hp.K; ++k) REQUIRE(alone.krec[alone.runits[k].krec].k == alone.runits[k].k, "record of a unit");
             REQUIRE(alone.flops_s + alone.flops_t > 0.999 * (plan.flops_s + plan.flops_t), "work of a pass");
         }
-        check_units(plan, L);
+        check_units(plan, L, false);
+        if (resident_backward(plan)) check_units(plan, L, true);
+        ++bands[plan.r_bands];
+        ++bands[plan.r_back];
         check_split(plan, C);
         REQUIRE(plan.r_pitch >= L + plan.r_front && plan.r_front % 4 == 0 && plan.r_pitch % 4 == 0, "zeros between the rows");
     }
-    REQUIRE(resident - small > 8 && small > 8 && others > 3, "%d handles with units, %d of them of low bands, %d without", resident, small, others);
+    REQUIRE(resident > 16 && others > 3, "%d handles with units, %d without", resident, others);
+    for (int b = 0; b < 7; ++b) REQUIRE(bands[b] > 0, "%d handles with bands %d", bands[b], b);
     std::printf("ok\n");
     return 0;
 }

@@ -1,6 +1,6 @@
 """The kernel that holds whole examples in shared memory, at the edges of its tiles and of its range, against the oracles (every mode).
 
-Rows of a dilation around multiples of its bands of 17 and 9, columns around the 64 of a tile, examples that fill shared memory with no room
+Rows of a dilation around multiples of its bands of 5 to 21 rows (one height or two), columns around the 64 of a tile, examples that fill shared memory with no room
 for zeros between the rows, samples at odd addresses, one more step than it serves, more examples than blocks, one kernel.  Tiles shared
 among examples (small dilations of the other kernels) at a length beyond this kernel's.
 """
@@ -20,7 +20,8 @@ pytestmark = pytest.mark.gpu
 # channels, steps, examples, kernels, dilations
 CASES = [(1, 64, 3, 24, (1, 2, 3, 5, 7)), (2, 152, 5, 30, (8, 9, 15, 16, 17)), (3, 153, 4, 30, (1, 2, 4, 8, 9, 17)), (5, 1088, 2, 40, (1, 3, 31, 32, 33, 63, 64, 65)),
          (1, 1089, 149, 12, (1, 2, 100)), (32, 1800, 2, 30, (1, 2, 7, 40, 128, 179)), (28, 2047, 2, 24, (1, 6, 65, 200)), (7, 301, 300, 1, (4,)),
-         (1, 5000, 2, 24, (1, 2, 9, 70, 400)), (1, 5001, 2, 24, (1, 2, 9, 70, 400)), (2, 6001, 41, 20, (1, 2, 3, 11))]
+         (6, 640, 3, 30, (1, 2, 5, 11, 60, 106)), (4, 900, 3, 30, (1, 3, 14, 15, 16, 149)), (3, 1344, 4, 30, (1, 2, 21, 63, 64, 223)),
+         (2, 1409, 3, 30, (1, 2, 11, 64, 65, 234)), (20, 1251, 2, 24, (1, 2, 30, 208)), (1, 5000, 2, 24, (1, 2, 9, 70, 400)), (1, 5001, 2, 24, (1, 2, 9, 70, 400)), (2, 6001, 41, 20, (1, 2, 3, 11))]
 
 
 @pytest.mark.parametrize("shift", [0, 1])
