@@ -1,4 +1,4 @@
-// Host-side checker of the small-dilation tiles whose bands have fewer rows than 24 (no GPU needed): replays, with the kernel's own index
+// Host-side check of the small-dilation tiles whose bands have fewer rows than 24 (no GPU needed): replays, with the kernel's own index
 // arithmetic, which outputs the threads of every tile own.  Every output of every kernel of a small dilation is owned once, tiles marked as
 // interior need no tests, and every height there is gets chosen.  With arguments C, L and kernels from standard input (K, then per kernel length,
 // dilation, padding and its channels): prints the rows of a band.

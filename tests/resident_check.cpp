@@ -1,4 +1,4 @@
-// Host-side checker of the resident kernel's plan (no GPU needed): replays, with the kernel's own column arithmetic, which outputs the
+// Host-side check of the resident kernel's plan (no GPU needed): replays, with the kernel's own column arithmetic, which outputs the
 // lanes of every tile own and which samples (or zeros around them) they read, and how calls are dealt to blocks.  Every output of every kernel is owned once,
 // every input row counted as a sample lies in the series (and no other one does), every example and kernel is dealt once.
 #include <cstdio>
