@@ -1,14 +1,17 @@
 // Gram matrix of the centred features on the fifth-generation tensor cores, in integers.
 //
-// Fc = F - mu is taken in double precision, every row scaled by a power of two so that its largest magnitude lies in [2^53, 2^54), rounded
-// to an integer and written as seven signed base-256 digits, d_0 first.  Then G_ij is a sum of digit products: all with a + b <= 6 are kept
-// (28 of 49; what is left out is of the order of 2^-55 sqrt(columns) of the rows' largest values), products with the same a + b share a 32-bit
-// accumulator and are exact there (7 * 16,384 columns * 128^2 < 2^31), and the seven accumulators meet in double precision.  That is as close as FP64
-// multiply-adds come; six digits and 21 products (146 in place of 180 us at 677 x 20,000) were not: the fit of 257 examples whose rows lie five
-// orders of magnitude apart was off by 4e-7 where FP64 sums leave 3e-8, and one value of 1e6 among shares made a penalty of 1e-3 too small.
+// Fc = F - mu is taken in double precision, every row scaled by a power of two so that its largest magnitude lies in [63/64 2^54, 63/64 2^55),
+// rounded to an integer and written as seven signed base-256 digits, d_0 first.  Then G_ij is a sum of digit products: all with a + b <= 7 are kept
+// (34 of 49), products with the same a + b share a 32-bit accumulator and are exact there (7 * 16,384 columns * 128^2 < 2^31), and the eight
+// accumulators meet in double precision.
 //
-// Why: FP64 products run at 37 TFLOP/s at the most, 8-bit ones at a hundred times that, and 28 of those replace one.  Measured at 677 x
-// 20,000: 229 us (scales 21, digits 28, products 180) where FP64 matrix instructions took 496.
+// How close: what is left out and the rounding to integers together are of the order of 2^-54 |x_i| |x_j| for rows x_i, x_j of Fc, below the 2^-53 that
+// the factorisation rounds its own terms by.  With a + b <= 6 (28 products) 2^-47 max|x_i| max|x_j| was left out: no matter among values of one
+// size, but the weights of 120 examples of 10,000 shares and maxima, one column of them 10^6 times as large, were off by 1.0e-5 where sums in FP64
+// leave 1.2e-6; they are off by 3.0e-7 now.
+//
+// Why: FP64 products run at 37 TFLOP/s at the most, 8-bit ones at a hundred times that, and 34 of those replace one.  Measured at 677 x
+// 20,000: 254 us (scales 21, digits 28, products 205; 28 products took 180) where FP64 matrix instructions took 496.
 #include <algorithm>
 #include <cstdint>
 
@@ -25,15 +28,16 @@ using fast::mbar_init;
 using fast::mbar_wait;
 using fast::smem_u32;
 
-constexpr int kDigits = 7, kTileM = 128, kTileN = 64, kStageK = 64;
+constexpr int kDigits = 7, kSums = 8, kTileM = 128, kTileN = 64, kStageK = 64;
 // The digits lie in memory as the matrix instruction reads them from shared memory (8 rows x 16 bytes to a core matrix, no swizzle):
 // [block of 64 columns][group of 8 rows][digit][4 core matrices][8 rows][16 columns], so that the operands of a stage are two bulk copies.
 constexpr int kCoreBytes = 128, kDigitBytes = kStageK / 16 * kCoreBytes, kGroupBytes = kDigits * kDigitBytes;
 constexpr int kABytes = kTileM / 8 * kGroupBytes, kBBytes = kTileN / 8 * kGroupBytes, kStageBytes = kABytes + kBBytes;
 constexpr int kStages = 2, kGramThreads = 128;
-static_assert(kDigits * kTileN <= 512, "an accumulator per a + b");
+static_assert(kSums * kTileN <= 512, "an accumulator per a + b");
 
-// up[i] = 2^k with up[i] max_p |F[i][p] - mu[p]| in [2^53, 2^54), down[i] = 1 / up[i]; NaN where a value of the row is not finite.
+// up[i] = 2^k with up[i] max_p |F[i][p] - mu[p]| in [63/64 2^54, 63/64 2^55), as large as seven signed digits hold; down[i] = 1 / up[i]; NaN where
+// a value of the row is not finite.
 __global__ void __launch_bounds__(256)
 gram_scale_kernel(const float* __restrict__ F, int P, const double* __restrict__ mu, double* __restrict__ up, double* __restrict__ down) {
     __shared__ unsigned long long s_max;
@@ -50,8 +54,8 @@ gram_scale_kernel(const float* __restrict__ F, int P, const double* __restrict__
     __syncthreads();
     if (threadIdx.x > 0) return;
     m = s_max;
-    const int e = (int)(m >> 52) - 1022;               // the maximum is below 2^e
-    const int k = min(max(54 - e, -1022), 1022);
+    const int e = (int)(m >> 52) - 1022 + ((m >> 46 & 63ull) == 63ull ? 1 : 0);   // the maximum is below 63/64 2^e
+    const int k = min(max(55 - e, -1022), 1022);
     const bool finite = (m >> 52) < 2047ull;
     up[blockIdx.x] = finite ? __longlong_as_double((long long)(1023 + k) << 52) : __longlong_as_double(0x7ff8000000000000ll);
     down[blockIdx.x] = finite ? __longlong_as_double((long long)(1023 - k) << 52) : __longlong_as_double(0x7ff8000000000000ll);
@@ -102,7 +106,7 @@ __device__ __forceinline__ uint64_t operand(uint32_t at) {   // K-major, no swiz
 }
 
 // One 128 x 64 tile of the lower triangle over a slice of the columns.  One thread copies stages in, one issues the matrix instructions
-// (56 per stage of 64 columns), all four warps turn the accumulators into doubles.  Bound: the matrix pipe, an instruction of 128 x 64 x 32
+// (68 per stage of 64 columns), all four warps turn the accumulators into doubles.  Bound: the matrix pipe, an instruction of 128 x 64 x 32
 // every 70 clocks; with A's digits copied to tensor memory, which spares two thirds of the shared-memory reads, the same.
 __global__ void __launch_bounds__(kGramThreads, 1)
 gram_mma_kernel(const GramArgs a) {
@@ -161,8 +165,9 @@ gram_mma_kernel(const GramArgs a) {
 #pragma unroll
                 for (int da = 0; da < kDigits; ++da)
 #pragma unroll
-                    for (int db = 0; db + da < kDigits; ++db) {
-                        const uint32_t fresh = da == 0 && k == 0 && st == 0 ? 0u : 1u;   // the first product of an accumulator assigns it
+                    for (int db = 0; db < kDigits && db + da < kSums; ++db) {
+                        // the first product of an accumulator assigns it
+                        const uint32_t fresh = (da == 0 || db == kDigits - 1) && k == 0 && st == 0 ? 0u : 1u;
                         asm volatile(
                             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                             "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
@@ -186,9 +191,9 @@ gram_mma_kernel(const GramArgs a) {
     const bool lower = bj <= ti && i < (a.N + 63) / 64 * 64;
 #pragma unroll 1
     for (int c = 0; c < kTileN; c += 8) {
-        uint32_t v[kDigits][8];
+        uint32_t v[kSums][8];
 #pragma unroll
-        for (int s = 0; s < kDigits; ++s)
+        for (int s = 0; s < kSums; ++s)
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                          : "=r"(v[s][0]), "=r"(v[s][1]), "=r"(v[s][2]), "=r"(v[s][3]), "=r"(v[s][4]), "=r"(v[s][5]), "=r"(v[s][6]), "=r"(v[s][7])
                          : "r"(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(s * kTileN + c)));
@@ -201,7 +206,7 @@ gram_mma_kernel(const GramArgs a) {
             for (int h = 0; h < 2; ++h) {
                 double sum = 0.0;                      // smallest first
 #pragma unroll
-                for (int s = kDigits - 1; s >= 0; --s) sum = fma(sum, 1.0 / 256.0, (double)(int)v[s][e + h]);
+                for (int s = kSums - 1; s >= 0; --s) sum = fma(sum, 1.0 / 256.0, (double)(int)v[s][e + h]);
                 const int j = j0 + c + e + h;
                 // 256^6 per factor between the leading digit and the integer
                 g[h] = sum * (281474976710656.0 * di) * (281474976710656.0 * (j < a.N ? __ldg(a.down + j) : 0.0));

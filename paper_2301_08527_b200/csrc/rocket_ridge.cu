@@ -9,7 +9,7 @@
 // of the same data are bitwise identical.
 //
 // Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights take
-// 18 / 229 (in FP64 496) / 214 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
+// 18 / 254 (in FP64 496) / 214 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
 // 55 / 2,607 / 20,270 / 174.
 #include <cooperative_groups.h>
 

@@ -3,6 +3,9 @@
 Rows around multiples of 64 and 128, columns around multiples of 64 and of a quadruple, more columns than a 32-bit sum takes at once, rows of
 very different magnitude.  Against the dual system in float64.  What the weights may be off by: their rounding to FP32 (2^-24 each) plus
 the errors of the two solutions, each of the order of 2^-53 times the condition number of the system.
+
+Features one column or value of which is far larger than the others, against the dual system in 80 bits: the weights may be off by their
+rounding and twice what the same system summed and solved in float64 is off by (another order of its sums changes that by less).
 """
 import numpy as np
 import pytest
@@ -47,6 +50,53 @@ def test_fits_match_the_dual_system_in_float64(N, P, kind):
     assert abs(b - rb) <= (bound + 2.0 ** -23) * (np.linalg.norm(rw) * np.linalg.norm(F.astype(np.float64).mean(0)) + abs(rb))
     again, _ = _fit(F, y, 1.0)
     assert np.array_equal(w, again)
+
+
+def _weights_in_80_bits(F, y, alpha):
+    Fc = F.astype(np.longdouble)
+    Fc -= Fc.mean(0)
+    x = y.astype(np.longdouble)
+    x -= x.mean()
+    A = Fc @ Fc.T + np.longdouble(alpha) * np.eye(len(y), dtype=np.longdouble)
+    for j in range(len(y)):                                  # L D L^T
+        A[j + 1:, j] /= A[j, j]
+        A[j + 1:, j + 1:] -= np.outer(A[j + 1:, j] * A[j, j], A[j + 1:, j])
+        x[j + 1:] -= A[j + 1:, j] * x[j]
+    x /= np.diag(A)
+    for j in range(len(y) - 1, -1, -1):
+        x[j] -= A[j + 1:, j] @ x[j + 1:]
+    return Fc.T @ x
+
+
+def _weights_in_64_bits(F, y, alpha):
+    Fc, yc = F.astype(np.float64), y.astype(np.float64)
+    Fc, yc = Fc - Fc.mean(0), yc - yc.mean()
+    G = alpha * np.eye(len(y))
+    for p in range(0, F.shape[1], 128):
+        G += Fc[:, p:p + 128] @ Fc[:, p:p + 128].T
+    return Fc.T @ np.linalg.solve(G, yc)
+
+
+def _no_further_off_than_64_bits(F, y, alpha):
+    w, _ = _fit(F, y, alpha)
+    exact = _weights_in_80_bits(F, y, alpha)
+    size = np.linalg.norm(exact)
+    err, err64 = (float(np.linalg.norm(v - exact) / size) for v in (w, _weights_in_64_bits(F, y, alpha)))
+    assert err <= 2.0 ** -24 + 2.0 * err64, (err, err64)
+
+
+@pytest.mark.parametrize("kind,size,alpha", [("column", 1e5, 1e-3), ("column", 1e6, 1e-3), ("column", 1e6, 1.0), ("column", 1e7, 1.0), ("value", 1e7, 1.0), ("value", 1e8, 1.0)])
+def test_one_large_column_or_value(kind, size, alpha):
+    N, P = 160, 12001
+    rng = np.random.default_rng(int(np.log10(size)))
+    F = rng.random((N, P))
+    F[:, 1::2] = 2.0 + 0.7 * rng.normal(size=(N, P // 2))
+    y = (F[:, :50] @ rng.normal(size=50) / 50 + rng.normal(size=N)).astype(np.float32)
+    if kind == "column":
+        F[:, 1] *= size
+    else:
+        F[3, 5] = size
+    _no_further_off_than_64_bits(F.astype(np.float32), y, alpha)
 
 
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
