@@ -9,7 +9,7 @@
 // of the same data are bitwise identical.
 //
 // Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights take
-// 18 / 254 (in FP64 496) / 214 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
+// 18 / 254 (in FP64 496) / 229 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
 // 55 / 2,607 / 20,270 / 174.
 #include <cooperative_groups.h>
 
@@ -146,10 +146,15 @@ ridge_gram_kernel(const float* __restrict__ F, int N, int P, const double* __res
 // G [Np][Np] (Np a multiple of 32 above N) holds the lower triangle of Fc Fc^T + alpha I, row N holds yc^T, rows below are
 // zero: the factorisation then leaves z = L^-1 yc in row N by itself.  Blocks of 32 x 32, right-looking, one grid-wide barrier per
 // step: block 0 updates the next diagonal block first and factors it while the others update the rest, and what it passes on is the
-// inverse of the factor, so that the panel blocks a tile needs are products that 256 threads share.  Solved panel blocks go transposed
-// into the upper triangle, inverse factors into Mi.  Bound: block 0's chain of 32 dependent pivots per step (22 steps at N = 677).
+// factor and its inverse, so that the panel blocks a tile needs are products that 256 threads share.  Solved panel blocks go transposed
+// into the upper triangle, factors and inverses into Li and Mi.  Bound: block 0's chain of 32 dependent pivots per step (22 steps at N = 677).
+//
+// A product with an explicit inverse is off by 2^-53 times the condition of the diagonal block, where a substitution is off by 2^-53 of its own
+// terms: X = A M alone left rows of 10^-4 to 10^4 with errors 10 to 400 times as large, or refused them for a pivot that was not positive.  So every
+// product takes one step of iterative refinement, X + (A - X L^T) M, which leaves the square of that error: the same as a substitution's up to
+// conditions of 10^8 of a factor, which is as far as any factorisation in double precision goes.
 constexpr int kCB = 32, kCThreads = 256, kCPitch = kCB + 4, kDPitch = kCB + 2;
-constexpr int kCSmem = kCB * kDPitch + 4 * kCB * kCPitch;              // doubles: a factor and four blocks; in the end the solution besides
+constexpr int kCSmem = kCB * kDPitch + 6 * kCB * kCPitch;              // doubles: a factor and six blocks; in the end the solution besides
 
 struct CholArgs {
     const double* part;       // partial Gram tiles [slices][tiles][64][64]
@@ -159,6 +164,7 @@ struct CholArgs {
     const double* ybar;
     double* G;
     double* Mi;               // inverse factors of the diagonal blocks, transposed [nb][32][32]
+    double* Li;               // the factors, transposed [nb][32][32]
     double* z;                // row N of the factor, by blocks
     double* a;                // solution [N]
     int* status;              // 0 = ok, 1 = a pivot was not positive
@@ -175,8 +181,8 @@ __device__ __forceinline__ double inverse_root(double d) {
 }
 
 // Factors the leading `ncols` columns of the block whose rows are held by the lanes (s[lane][0 .. lane]) and inverts the factor: row r
-// of the inverse's transpose goes to m[r]; lane j returns in root the reciprocal of the factor's diagonal j, and t[j] holds column j of
-// the factor times that diagonal.  One warp.
+// of the inverse's transpose goes to m[r]; lane j returns in root the reciprocal of the factor's diagonal j, which is in t[j][32] as well, and t[j]
+// holds column j of the factor times that diagonal.  One warp.
 //
 // A double-precision operation takes some 40 clocks here, so what counts is how many of them lie between a pivot and the next.  The
 // elimination is square-root free (a_ik -= c_ij c_kj / d_j with unscaled columns c), 1 / d_j is y (1 + e + e^2) for an approximation y
@@ -218,6 +224,7 @@ __device__ __forceinline__ bool chol_factor_block(const double (*s)[kCPitch], do
         }
     }
     root = inverse_root(mine);
+    t[lane][kCB] = root;
 #pragma unroll
     for (int c = 0; c < kCB; ++c) m[lane][c] = x[c] * __shfl_sync(0xffffffffu, root, c);
     __syncwarp();
@@ -233,21 +240,26 @@ ridge_cholesky_solve_kernel(CholArgs q) {
     extern __shared__ double smem[];
     double (*s_t)[kDPitch] = reinterpret_cast<double (*)[kDPitch]>(smem);
     double (*s_m)[kCPitch] = reinterpret_cast<double (*)[kCPitch]>(smem + kCB * kDPitch), (*s_pi)[kCPitch] = s_m + kCB, (*s_pj)[kCPitch] = s_pi + kCB;
+    double (*s_l)[kCPitch] = s_pj + kCB, (*s_xi)[kCPitch] = s_l + kCB, (*s_xj)[kCPitch] = s_xi + kCB;
     cg::grid_group grid = cg::this_grid();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = q.N, Np = q.Np, nb = Np / kCB;
-    const int fr = lane >> 2, fk = lane & 3, br = warp >> 1, bc = (warp & 1) * 2;   // a warp's two 8 x 8 fragments of a block
+    // a warp's two 8 x 8 fragments of a block: those columns of a triangular factor that have as many products together for every warp
+    const int fr = lane >> 2, fk = lane & 3, br = warp >> 1, bc[2] = {warp & 1, 3 - (warp & 1)};
     double* __restrict__ G = q.G;
     bool good = true;
 
-    // the inverse factor of diagonal block kb, whose elements are in s_pi (block 0)
+    // the factor of diagonal block kb, whose elements are in s_pi, and its inverse (block 0)
     auto factor = [&](int kb) {
         const int ncols = min(kCB, N - kb * kCB);
         double root = 0.0;
         if (ncols > 0 && warp == 0) good = chol_factor_block(s_pi, s_t, s_m, ncols, lane, root) && good;
         __syncthreads();
         if (ncols > 0)
-            for (int e = tid; e < kCB * kCB; e += kCThreads) q.Mi[(size_t)kb * kCB * kCB + e] = s_m[e / kCB][e % kCB];
+            for (int e = tid; e < kCB * kCB; e += kCThreads) {
+                q.Mi[(size_t)kb * kCB * kCB + e] = s_m[e / kCB][e % kCB];
+                q.Li[(size_t)kb * kCB * kCB + e] = s_t[e / kCB][e % kCB] * s_t[e / kCB][kCB];
+            }
         // row N of the factor: within its own diagonal block the factor's rows are not kept elsewhere
         if (kb == N / kCB && tid < ncols) q.z[kb * kCB + tid] = s_t[tid][N - kb * kCB] * root;
         __syncthreads();
@@ -296,64 +308,98 @@ ridge_cholesky_solve_kernel(CholArgs q) {
                 const int jb = nb - 1 - x, ib = nb - 1 - ((tiles - 1 - b) - x * (x + 1) / 2);
                 const int i0 = ib * kCB, j0 = jb * kCB;
                 const bool two = ib != jb;
-                // all loads of the tile at once: inverse factor, panel blocks, the warp's fragments of the tile (rows fr of row block 8 br,
-                // columns 2 fk, 2 fk + 1 of column blocks 8 bc and 8 (bc + 1))
+                // all loads of the tile at once: factor and inverse, panel blocks, the warp's fragments of the tile (rows fr of row block 8 br,
+                // columns 2 fk, 2 fk + 1 of column blocks bc)
                 constexpr int kEach = kCB * kCB / kCThreads;
-                double lm[kEach], li[kEach], lj[kEach], g[2][2];
+                double lm[kEach], ll[kEach], li[kEach], lj[kEach], g[2][2];
 #pragma unroll
                 for (int u = 0; u < kEach; ++u) {
                     const int e = tid + u * kCThreads, r = e / kCB, c = e % kCB;
                     lm[u] = __ldcg(q.Mi + (size_t)kb * kCB * kCB + e);
+                    ll[u] = __ldcg(q.Li + (size_t)kb * kCB * kCB + e);
                     li[u] = __ldcg(G + (size_t)(i0 + r) * Np + k0 + c);
                     lj[u] = two ? __ldcg(G + (size_t)(j0 + r) * Np + k0 + c) : 0.0;
                 }
 #pragma unroll
                 for (int v = 0; v < 2; ++v) {
-                    const double2 w = __ldcg(reinterpret_cast<const double2*>(G + (size_t)(i0 + 8 * br + fr) * Np + j0 + 8 * (bc + v) + 2 * fk));
+                    const double2 w = __ldcg(reinterpret_cast<const double2*>(G + (size_t)(i0 + 8 * br + fr) * Np + j0 + 8 * bc[v] + 2 * fk));
                     g[v][0] = w.x; g[v][1] = w.y;
                 }
 #pragma unroll
                 for (int u = 0; u < kEach; ++u) {
                     const int e = tid + u * kCThreads, r = e / kCB, c = e % kCB;
                     s_m[r][c] = lm[u];
+                    s_l[r][c] = ll[u];
                     s_pi[r][c] = li[u];
                     if (two) s_pj[r][c] = lj[u];
                 }
-                double pi[2][2] = {}, pj[2][2] = {}, h0[2][2] = {}, h1[2][2] = {};   // a matrix instruction takes long, too: two sums for every fragment
-                __syncthreads();
-                // the solved panel blocks: rows of G times the inverse factor's transpose
+                // a matrix instruction takes long, too: two sums for every fragment
+                double xi[2][2] = {}, xj[2][2] = {};
+                // times an upper triangle, onto xi, xj
+                auto multiply = [&](const double (*pi)[kCPitch], const double (*pj)[kCPitch], const double (*by)[kCPitch], double sign) {
+                    double h0[2][2] = {}, h1[2][2] = {};
 #pragma unroll
-                for (int k = 0; k < kCB; k += 4) {
-                    const double x = s_pi[8 * br + fr][k + fk], y = two ? s_pj[8 * br + fr][k + fk] : 0.0;
+                    for (int k = 0; k < kCB; k += 4) {
+                        const double x = sign * pi[8 * br + fr][k + fk], y = two ? sign * pj[8 * br + fr][k + fk] : 0.0;
 #pragma unroll
-                    for (int v = 0; v < 2; ++v) {
-                        const double m = s_m[k + fk][8 * (bc + v) + fr];
-                        dmma(k & 4 ? h0[v] : pi[v], x, m);
-                        if (two) dmma(k & 4 ? h1[v] : pj[v], y, m);
+                        for (int v = 0; v < 2; ++v) {
+                            if (k >= 8 * bc[v] + 8) continue;      // zeros
+                            const double m = by[k + fk][8 * bc[v] + fr];
+                            dmma(k & 4 ? h0[v] : xi[v], x, m);
+                            if (two) dmma(k & 4 ? h1[v] : xj[v], y, m);
+                        }
                     }
-                }
-                __syncthreads();
 #pragma unroll
-                for (int v = 0; v < 2; ++v)
+                    for (int v = 0; v < 2; ++v)
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        s_pi[8 * br + fr][8 * (bc + v) + 2 * fk + h] = pi[v][h] + h0[v][h];
-                        if (two) s_pj[8 * br + fr][8 * (bc + v) + 2 * fk + h] = pj[v][h] + h1[v][h];
-                        h0[v][h] = 0.0;
-                    }
+                        for (int h = 0; h < 2; ++h) {
+                            xi[v][h] += h0[v][h];
+                            xj[v][h] += h1[v][h];
+                        }
+                };
+                auto fetch = [&](const double (*pi)[kCPitch], const double (*pj)[kCPitch]) {
+#pragma unroll
+                    for (int v = 0; v < 2; ++v)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            xi[v][h] = pi[8 * br + fr][8 * bc[v] + 2 * fk + h];
+                            xj[v][h] = two ? pj[8 * br + fr][8 * bc[v] + 2 * fk + h] : 0.0;
+                        }
+                };
+                auto keep = [&](double (*pi)[kCPitch], double (*pj)[kCPitch]) {
+#pragma unroll
+                    for (int v = 0; v < 2; ++v)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            pi[8 * br + fr][8 * bc[v] + 2 * fk + h] = xi[v][h];
+                            if (two) pj[8 * br + fr][8 * bc[v] + 2 * fk + h] = xj[v][h];
+                        }
+                    __syncthreads();
+                };
                 __syncthreads();
+                // the solved panel blocks: X = A M, R = A - X L^T, X + R M
+                multiply(s_pi, s_pj, s_m, 1.0);
+                keep(s_xi, s_xj);
+                fetch(s_pi, s_pj);
+                multiply(s_xi, s_xj, s_l, -1.0);
+                keep(s_pi, s_pj);
+                fetch(s_xi, s_xj);
+                multiply(s_pi, s_pj, s_m, 1.0);
+                __syncthreads();
+                keep(s_pi, s_pj);
+                double h0[2][2] = {};
                 const double (*sj)[kCPitch] = two ? s_pj : s_pi;
 #pragma unroll
                 for (int k = 0; k < kCB; k += 4) {
                     const double x = -s_pi[8 * br + fr][k + fk];
 #pragma unroll
-                    for (int v = 0; v < 2; ++v) dmma(k & 4 ? h0[v] : g[v], x, sj[8 * (bc + v) + fr][k + fk]);
+                    for (int v = 0; v < 2; ++v) dmma(k & 4 ? h0[v] : g[v], x, sj[8 * bc[v] + fr][k + fk]);
                 }
 #pragma unroll
                 for (int v = 0; v < 2; ++v) {
                     g[v][0] += h0[v][0];
                     g[v][1] += h0[v][1];
-                    *reinterpret_cast<double2*>(G + (size_t)(i0 + 8 * br + fr) * Np + j0 + 8 * (bc + v) + 2 * fk) = make_double2(g[v][0], g[v][1]);
+                    *reinterpret_cast<double2*>(G + (size_t)(i0 + 8 * br + fr) * Np + j0 + 8 * bc[v] + 2 * fk) = make_double2(g[v][0], g[v][1]);
                 }
                 if (jb == kb + 1) {
                     for (int e = tid; e < kCB * kCB; e += kCThreads) G[(size_t)(k0 + e / kCB) * Np + i0 + e % kCB] = s_pi[e % kCB][e / kCB];
@@ -364,7 +410,7 @@ ridge_cholesky_solve_kernel(CholArgs q) {
 #pragma unroll
                     for (int v = 0; v < 2; ++v)
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) s_pi[8 * br + fr][8 * (bc + v) + 2 * fk + h] = g[v][h];
+                        for (int h = 0; h < 2; ++h) s_pi[8 * br + fr][8 * bc[v] + 2 * fk + h] = g[v][h];
                     __syncthreads();
                 }
             }
@@ -375,22 +421,23 @@ ridge_cholesky_solve_kernel(CholArgs q) {
     if (blockIdx.x != 0) return;
 
     // L^T a = z, from the last block up: a_kb = M_kb (z_kb - sum of L_i,kb^T a_i over the blocks i below).  Row k0 + j of the upper
-    // triangle holds L's column.  The first warp finishes a block from what the others brought in and summed a phase earlier: the inverse factor, the
-    // block of L next to the diagonal, and the part of the sums whose a_i were known then.
+    // triangle holds L's column.  The first warp finishes a block from what the others brought in and summed a phase earlier: the factor and its
+    // inverse, the block of L next to the diagonal, and the part of the sums whose a_i were known then.
     if (warp == 0 && lane == 0 && !good) *q.status = 1;
     __shared__ double s_sum[2][kCB];
-    double (*s_inv)[kCPitch] = s_m, (*s_next)[kCPitch] = s_m + 2 * kCB;   // two of each
-    double* s_a = reinterpret_cast<double*>(s_m + 4 * kCB);
+    double (*s_inv)[kCPitch] = s_m, (*s_next)[kCPitch] = s_m + 2 * kCB, (*s_own)[kCPitch] = s_m + 4 * kCB;   // two of each
+    double* s_a = reinterpret_cast<double*>(s_m + 6 * kCB);
     const int nblk = (N + kCB - 1) / kCB;
     constexpr int kHelpers = kCThreads / 32 - 1;
     auto bring = [&](int kb) {                               // for block kb, by warps 1 .. 7, while a of blocks above kb + 1 is known
         const int k0 = kb * kCB, buf = kb & 1, w = warp - 1;
         constexpr int kEach = (kCB * kCB + kCThreads - 33) / (kCThreads - 32);
-        double inv[kEach], next[kEach];
+        double inv[kEach], own[kEach], next[kEach];
 #pragma unroll
         for (int u = 0; u < kEach; ++u) {
             const int e = min(tid - 32 + u * (kCThreads - 32), kCB * kCB - 1), r = e / kCB, c = e % kCB;
             inv[u] = __ldcg(q.Mi + (size_t)kb * kCB * kCB + e);
+            own[u] = __ldcg(q.Li + (size_t)kb * kCB * kCB + e);
             next[u] = __ldcg(G + (size_t)(k0 + r) * Np + min(k0 + kCB + c, Np - 1));   // past column N: not used
         }
         // five rows a warp, side by side: what counts is how many loads are on their way
@@ -418,6 +465,7 @@ ridge_cholesky_solve_kernel(CholArgs q) {
         for (int u = 0; u < kEach; ++u) {
             const int e = min(tid - 32 + u * (kCThreads - 32), kCB * kCB - 1), r = e / kCB, c = e % kCB;
             s_inv[buf * kCB + r][c] = inv[u];
+            s_own[buf * kCB + r][c] = own[u];
             s_next[buf * kCB + r][c] = next[u];
         }
     };
@@ -436,14 +484,19 @@ ridge_cholesky_solve_kernel(CholArgs q) {
                 for (int c = 0; c < below; ++c) u[c & 3] += s_next[buf * kCB + lane][c] * s_a[k0 + kCB + c];
                 v -= (u[0] + u[1]) + (u[2] + u[3]);
             }
-            __syncwarp();
-            s_t[0][lane] = v;
-            __syncwarp();
-            double u[4] = {0.0, 0.0, 0.0, 0.0};
+            // row `lane` of a block of the buffer times a vector in s_t
+            auto times = [&](const double (*m)[kCPitch], int at, double x) {
+                __syncwarp();
+                s_t[at][lane] = x;
+                __syncwarp();
+                double u[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-            for (int c = 0; c < kCB; ++c) u[c & 3] += s_inv[buf * kCB + lane][c] * s_t[0][c];
+                for (int c = 0; c < kCB; ++c) u[c & 3] += m[buf * kCB + lane][c] * s_t[at][c];
+                return lane < ncols ? (u[0] + u[1]) + (u[2] + u[3]) : 0.0;
+            };
+            double a = times(s_inv, 0, v);
+            a += times(s_inv, 2, v - times(s_own, 1, a));
             if (lane < ncols) {
-                const double a = (u[0] + u[1]) + (u[2] + u[3]);
                 s_a[k0 + lane] = a;
                 q.a[k0 + lane] = a;
             }
@@ -694,11 +747,11 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     const int slice = ((P + slices - 1) / slices + kGP - 1) / kGP * kGP;
     slices = integers ? gram.slices : (P + slice - 1) / slice;
     const int nb = (N + 1 + kCB - 1) / kCB, Np = nb * kCB;
-    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Mi[nb][32][32], z[Np], partial Gram tiles, ticket, status
+    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Mi[nb][32][32], Li[nb][32][32], z[Np], partial Gram tiles, ticket, status
     size_t off = 0;
     auto take = [&](size_t doubles) { const size_t o = off; off += (doubles + 31) / 32 * 32; return o; };
     const size_t o_mu = take(P), o_a = take(N), o_part = take(col_blocks), o_ybar = take(1), o_G = take((size_t)Np * Np);
-    const size_t o_Mi = take((size_t)nb * kCB * kCB), o_z = take(Np), o_gram = take((size_t)slices * tiles * kGT * kGT), o_int = take(2);
+    const size_t o_Mi = take((size_t)nb * kCB * kCB), o_Li = take((size_t)nb * kCB * kCB), o_z = take(Np), o_gram = take((size_t)slices * tiles * kGT * kGT), o_int = take(2);
     const size_t o_up = take(integers ? N : 0), o_down = take(integers ? N : 0), o_digits = take(integers ? gram.digit_bytes / sizeof(double) : 0);
     const size_t bytes = off * sizeof(double);
     FitWorkspace ws;
@@ -711,7 +764,7 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
         e = launch_gram(gram, feat_dev, N, P, d + o_mu, d + o_up, d + o_down, reinterpret_cast<uint8_t*>(d + o_digits), d + o_gram, status + 1, stream);
     else
         ridge_gram_kernel<<<dim3(tiles, slices), kGThreads, gram_smem, stream>>>(feat_dev, N, P, d + o_mu, slice, d + o_gram);
-    CholArgs q{d + o_gram, slices, tiles, (double)alpha, y_dev, d + o_ybar, d + o_G, d + o_Mi, d + o_z, d + o_a, status, N, Np};
+    CholArgs q{d + o_gram, slices, tiles, (double)alpha, y_dev, d + o_ybar, d + o_G, d + o_Mi, d + o_Li, d + o_z, d + o_a, status, N, Np};
     void* args[] = {&q};
     // one block per SM: more would lengthen the grid barriers without shortening the chain
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(ridge_cholesky_solve_kernel),

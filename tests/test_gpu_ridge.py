@@ -14,6 +14,8 @@ import oracle
 import paper_2301_08527_b200 as rk
 from rocket_inputs import ar1_spike_series, generate_kernels
 
+from test_gpu_gram import _no_further_off_than_64_bits
+
 pytestmark = pytest.mark.gpu
 
 
@@ -66,6 +68,17 @@ def test_fit_at_paper_size_satisfies_the_conditions_of_the_minimiser():
     assert torch.equal(w, w2) and torch.equal(b, b2)
     yhat = rk.rocket_ridge_predict(_dev(F[:60]), w, b).cpu().numpy()
     assert np.abs(yhat - (F64[:60] @ w64 + b64)).max() <= 1e-5 * max(1.0, float(np.abs(y).max()))
+
+
+@pytest.mark.parametrize("N,P,seed", [(33, 700, 0), (97, 1500, 1), (97, 1500, 2), (160, 12001, 3)])
+def test_rows_of_very_different_size_and_a_small_penalty(N, P, seed):
+    # diagonal blocks of the factor with conditions up to some 10^8 (FP64 sums up to N N P of 3e8, integers beyond)
+    rng = np.random.default_rng(seed)
+    F = rng.random((N, P))
+    F[:, 1::2] = 2.0 + 0.7 * rng.normal(size=(N, P // 2))
+    y = (F[:, :50] @ rng.normal(size=50) / 50 + rng.normal(size=N)).astype(np.float32)
+    F *= 10.0 ** rng.uniform(-4, 4, size=(N, 1))
+    _no_further_off_than_64_bits(F.astype(np.float32), y, 1e-2)
 
 
 def test_transform_features_feed_the_regressor_without_leaving_the_device():
