@@ -12,7 +12,6 @@
 //
 // Why: FP64 products run at 37 TFLOP/s at the most, 8-bit ones at a hundred times that, and 34 of those replace one.  Measured at 677 x
 // 20,000: 254 us (scales 21, digits 28, products 205; 28 products took 180) where FP64 matrix instructions took 496.
-#include <algorithm>
 #include <cstdint>
 
 #include "rocket_fast_dev.cuh"
@@ -28,10 +27,11 @@ using fast::mbar_init;
 using fast::mbar_wait;
 using fast::smem_u32;
 
-constexpr int kDigits = 7, kSums = 8, kTileM = 128, kTileN = 64, kStageK = 64;
+constexpr int kDigits = kGramDigits, kSums = 8, kTileM = kGramTileM, kTileN = kGramTileN, kStageK = kGramStageK;
 // The digits lie in memory as the matrix instruction reads them from shared memory (8 rows x 16 bytes to a core matrix, no swizzle):
 // [block of 64 columns][group of 8 rows][digit][4 core matrices][8 rows][16 columns], so that the operands of a stage are two bulk copies.
-constexpr int kCoreBytes = 128, kDigitBytes = kStageK / 16 * kCoreBytes, kGroupBytes = kDigits * kDigitBytes;
+constexpr int kCoreBytes = 128, kDigitBytes = kStageK / 16 * kCoreBytes, kGroupBytes = kGramGroupBytes;
+static_assert(kGroupBytes == kDigits * kDigitBytes, "a group's digits");
 constexpr int kABytes = kTileM / 8 * kGroupBytes, kBBytes = kTileN / 8 * kGroupBytes, kStageBytes = kABytes + kBBytes;
 constexpr int kStages = 2, kGramThreads = 128;
 static_assert(kSums * kTileN <= 512, "an accumulator per a + b");
@@ -98,7 +98,7 @@ struct GramArgs {
     const double* down;
     double* part;             // [slices][tiles of 64 x 64][64][64]
     int* failed;
-    int N, groups, blocks, tiles, slices, add;   // groups: of 8 rows; blocks: of 64 columns; tiles: 64 x 64 ones of a slice; add: onto what part holds
+    int N, groups, blocks, tiles, slices, add;   // groups: of 8 rows; blocks: of 64 columns, no fewer than slices; tiles: 64 x 64 ones of a slice; add: onto what part holds
 };
 
 __device__ __forceinline__ uint64_t operand(uint32_t at) {   // K-major, no swizzle: core matrices along K, groups of 8 rows
@@ -229,28 +229,6 @@ constexpr size_t kGramSmem = (size_t)kStages * kStageBytes + 128;
 
 }  // namespace
 
-GramPlan gram_plan(int N, int P, int sms) {
-    GramPlan g{};
-    g.groups = (N + kTileM - 1) / kTileM * (kTileM / 8);
-    const int nt = (N + 63) / 64, last = (N + kTileM - 1) / kTileM - 1;
-    g.blocks_mn = last * (last + 1) + std::min(2 * last + 2, nt);
-    const size_t block_bytes = (size_t)g.groups * kGroupBytes;
-    const int blocks = (P + kStageK - 1) / kStageK;
-    g.chunk = (int)std::max<size_t>(1, std::min<size_t>(blocks, kGramDigitBytes / block_bytes));
-    g.chunk = (blocks + (blocks + g.chunk - 1) / g.chunk - 1) / ((blocks + g.chunk - 1) / g.chunk);   // evenly
-    // Slices of a chunk: the fewest clocks, where a stage takes 4,000 and a block's beginning and end 10,000; no more than 16,384 columns each
-    // (32-bit sums), and 24 MB of partial tiles (or one slice).
-    const size_t slice_bytes = (size_t)nt * (nt + 1) / 2 * 4096 * sizeof(double);
-    const int least = (g.chunk * kStageK + 16383) / 16384, most = std::max<int>(least, std::min<int>(16, (int)(((size_t)24 << 20) / slice_bytes)));
-    double best = 1e300;
-    for (int s = least; s <= most && s <= g.chunk; ++s) {
-        const double t = (double)(((long long)g.blocks_mn * s + sms - 1) / sms) * ((g.chunk + s - 1) / s * 4000.0 + 10000.0);
-        if (t < best) { best = t; g.slices = s; }
-    }
-    g.digit_bytes = (size_t)g.chunk * block_bytes;
-    return g;
-}
-
 cudaError_t launch_gram(const GramPlan& g, const float* F, int N, int P, const double* mu, double* up, double* down, uint8_t* digits, double* part,
                         int* failed, cudaStream_t stream) {
     cudaError_t e = cudaFuncSetAttribute(gram_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmem);
@@ -261,8 +239,9 @@ cudaError_t launch_gram(const GramPlan& g, const float* F, int N, int P, const d
     for (int b0 = 0; b0 < blocks; b0 += g.chunk) {
         const int nb = std::min(g.chunk, blocks - b0);
         gram_digits_kernel<<<dim3((nb * 4 + 7) / 8, g.groups), 256, 0, stream>>>(F, N, P, b0 * kStageK, nb * 4, mu, up, g.groups, digits);
-        const GramArgs a{digits, down, part, failed, N, g.groups, nb, nt * (nt + 1) / 2, g.slices, b0 > 0 ? 1 : 0};
-        gram_mma_kernel<<<dim3(g.blocks_mn, g.slices), kGramThreads, kGramSmem, stream>>>(a);
+        const int slices = gram_slices(g, nb);
+        const GramArgs a{digits, down, part, failed, N, g.groups, nb, nt * (nt + 1) / 2, slices, b0 > 0 ? 1 : 0};
+        gram_mma_kernel<<<dim3(g.blocks_mn, slices), kGramThreads, kGramSmem, stream>>>(a);
         count_launch(2);
     }
     return cudaGetLastError();

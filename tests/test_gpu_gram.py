@@ -52,6 +52,23 @@ def test_fits_match_the_dual_system_in_float64(N, P, kind):
     assert np.array_equal(w, again)
 
 
+@pytest.mark.parametrize("N,P", [(897, 19003), (2305, 17001)])
+def test_digits_of_several_chunks_of_columns(N, P):
+    # two and three chunks, the last one shorter; the dual system on the device
+    import torch
+    rng = np.random.default_rng(N)
+    F = rng.random((N, P), dtype=np.float32)
+    F[:, 1::2] = 2.0 + 0.7 * rng.normal(size=(N, P // 2)).astype(np.float32)
+    y = rng.normal(size=N).astype(np.float32)
+    w, _ = _fit(F, y, 1.0)
+    Fc, yc = torch.from_numpy(F).cuda().double(), torch.from_numpy(y).cuda().double()
+    Fc, yc = Fc - Fc.mean(0), yc - yc.mean()
+    G = Fc @ Fc.T
+    rw = (Fc.T @ torch.linalg.solve(G + torch.eye(N, dtype=torch.float64, device="cuda"), yc)).cpu().numpy()
+    bound = 2.0 ** -24 + 4 * 2.0 ** -53 * (float(G.trace()) + 1.0)   # the trace is more than the largest eigenvalue
+    assert np.linalg.norm(w - rw) <= bound * np.linalg.norm(rw)
+
+
 def _weights_in_80_bits(F, y, alpha):
     Fc = F.astype(np.longdouble)
     Fc -= Fc.mean(0)
