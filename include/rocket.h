@@ -244,9 +244,10 @@ int rocket_transform_u8_host(rocket_params_t* p, const uint8_t* X_u8_host, int N
  * with Fc, yc the column-centred features and targets, w minimises |Fc w - yc|^2 + alpha |w|^2 and
  * b = mean(y) - mean(F) . w.  Solved in its dual form (an N x N system, N <= ROCKET_RIDGE_MAX_EXAMPLES)
  * in double precision; w_dev [P] and b_dev [1] receive the result as fp32.  The call returns after the
- * work on cuda_stream has finished.  Its workspace (about P + N*N doubles, and partial sums of up to 40 MB, or of one slice of the
- * features where that is more: 65 MB at 4,096 examples) is
- * allocated with cudaMalloc; one buffer of up to 64 MiB per device is kept for the next fit until a parameter
+ * work on cuda_stream has finished.  Its workspace is about P + N*N doubles, partial sums of up to 40 MB, or of one slice of the
+ * features where that is more (65 MB at 4,096 examples), and for larger fits up to 112 MiB for the features as integers; where
+ * there is no room for those, the fit goes on without.  It is
+ * allocated with cudaMalloc; one buffer of up to 144 MiB per device is kept for the next fit until a parameter
  * handle is destroyed or the library runs short of memory, anything else is freed before the call returns.  Errors: ROCKET_EINVAL for NULL pointers, N < 1, P < 1, a negative or
  * non-finite alpha, or a system that is not positive definite (alpha = 0 with dependent rows);
  * ROCKET_EUNSUPPORTED beyond the size limit; ROCKET_ENOMEM / ROCKET_ECUDA from the runtime.

@@ -11,7 +11,7 @@ namespace rocket {
 
 constexpr int kGramDigits = 7, kGramTileM = 128, kGramTileN = 64, kGramStageK = 64;   // of a row; rows and columns of a tile; columns of a stage
 constexpr int kGramGroupBytes = kGramDigits * 8 * kGramStageK;      // digits of eight rows and a stage
-constexpr size_t kGramDigitBytes = (size_t)112 << 20;   // digits of as many columns at a time
+constexpr size_t kGramDigitBytes = (size_t)112 << 20;   // digits of as many columns at a time, unless that is too much memory
 constexpr int kGramSliceStages = 16384 / kGramStageK;   // of a slice: a 32-bit sum holds as many columns
 
 struct GramPlan {
@@ -20,14 +20,14 @@ struct GramPlan {
     size_t digit_bytes;
 };
 
-inline GramPlan gram_plan(int N, int P, int sms) {
+inline GramPlan gram_plan(int N, int P, int sms, size_t most_digit_bytes = kGramDigitBytes) {
     GramPlan g{};
     g.groups = (N + kGramTileM - 1) / kGramTileM * (kGramTileM / 8);
     const int nt = (N + 63) / 64, last = (N + kGramTileM - 1) / kGramTileM - 1;
     g.blocks_mn = last * (last + 1) + std::min(2 * last + 2, nt);
     const size_t block_bytes = (size_t)g.groups * kGramGroupBytes;
     const int blocks = (P + kGramStageK - 1) / kGramStageK;
-    g.chunk = (int)std::max<size_t>(1, std::min<size_t>(blocks, kGramDigitBytes / block_bytes));
+    g.chunk = (int)std::max<size_t>(1, std::min<size_t>(blocks, most_digit_bytes / block_bytes));
     g.chunk = (blocks + (blocks + g.chunk - 1) / g.chunk - 1) / ((blocks + g.chunk - 1) / g.chunk);   // evenly
     // Slices of a chunk: the fewest clocks, where a stage takes 4,800 and a block's beginning and end 10,000; no more columns than 32-bit sums
     // hold each, and 24 MB of partial tiles (or one slice).

@@ -656,6 +656,7 @@ int status_of(cudaError_t e) {
 // stream has finished; a larger or a concurrent fit allocates and frees its own.  The buffer is given back when a handle
 // of the library is destroyed and when a device allocation of the library fails (release_cached_workspaces).
 constexpr size_t kKeepBytes = (size_t)144 << 20;
+constexpr size_t kLeastDigitBytes = (size_t)32 << 20;   // digits are not divided further for that
 constexpr int kMaxDevices = 64;
 struct Kept { void* ptr = nullptr; size_t bytes = 0; bool taken = false; };
 std::mutex g_kept_mu;
@@ -735,27 +736,52 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     if (e == cudaSuccess) e = cudaFuncSetAttribute(ridge_cholesky_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)((kCSmem + ROCKET_RIDGE_MAX_EXAMPLES) * sizeof(double)));
     if (e != cudaSuccess) return status_of(e);
     const int col_blocks = (P + 31) / 32;
-    // Slices of the feature axis: about two waves of the four blocks an SM holds, at least 128 columns each, and no more
-    // than 40 MB of partial tiles (or one slice, 65 MB at the most examples).
     const int nt = (N + kGT - 1) / kGT, tiles = nt * (nt + 1) / 2;
-    const size_t tile_bytes = (size_t)kGT * kGT * sizeof(double);
+    const int nb = (N + 1 + kCB - 1) / kCB, Np = nb * kCB;
     // Integers on the tensor cores from about 100 examples of 20,000 features on (us, FP64 and integers: 24 x 20,000 99 and 113, 97 x 3,001
     // 111 and 121, 300 x 600 207 and 212, 100 x 20,000 166 and 155, 300 x 5,000 238 and 225, 677 x 20,000 931 and 632).
-    const bool integers = (double)N * N * P >= 1.2e8;
-    const GramPlan gram = gram_plan(N, P, sms);
-    int slices = std::max(1, std::min({8 * sms / tiles, P / 128, (int)(((size_t)40 << 20) / (tile_bytes * tiles))}));
-    const int slice = ((P + slices - 1) / slices + kGP - 1) / kGP * kGP;
-    slices = integers ? gram.slices : (P + slice - 1) / slice;
-    const int nb = (N + 1 + kCB - 1) / kCB, Np = nb * kCB;
-    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Mi[nb][32][32], Li[nb][32][32], z[Np], partial Gram tiles, ticket, status
-    size_t off = 0;
-    auto take = [&](size_t doubles) { const size_t o = off; off += (doubles + 31) / 32 * 32; return o; };
-    const size_t o_mu = take(P), o_a = take(N), o_part = take(col_blocks), o_ybar = take(1), o_G = take((size_t)Np * Np);
-    const size_t o_Mi = take((size_t)nb * kCB * kCB), o_Li = take((size_t)nb * kCB * kCB), o_z = take(Np), o_gram = take((size_t)slices * tiles * kGT * kGT), o_int = take(2);
-    const size_t o_up = take(integers ? N : 0), o_down = take(integers ? N : 0), o_digits = take(integers ? gram.digit_bytes / sizeof(double) : 0);
-    const size_t bytes = off * sizeof(double);
+    bool integers = (double)N * N * P >= 1.2e8;
+    GramPlan gram{};
+    int slices = 0, slice = 0;
+    size_t o_mu, o_a, o_part, o_ybar, o_G, o_Mi, o_Li, o_z, o_gram, o_int, o_up, o_down, o_digits, bytes;
+    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Mi[nb][32][32], Li[nb][32][32], z[Np], partial Gram tiles, ticket, status; for
+    // integers the rows' scales and digits
+    auto lay_out = [&]() {
+        size_t off = 0;
+        auto take = [&](size_t doubles) { const size_t o = off; off += (doubles + 31) / 32 * 32; return o; };
+        o_mu = take(P); o_a = take(N); o_part = take(col_blocks); o_ybar = take(1); o_G = take((size_t)Np * Np);
+        o_Mi = take((size_t)nb * kCB * kCB); o_Li = take((size_t)nb * kCB * kCB); o_z = take(Np); o_gram = take((size_t)slices * tiles * kGT * kGT); o_int = take(2);
+        o_up = take(integers ? N : 0); o_down = take(integers ? N : 0); o_digits = take(integers ? gram.digit_bytes / sizeof(double) : 0);
+        bytes = off * sizeof(double);
+    };
     FitWorkspace ws;
-    if ((e = ws.take(bytes)) != cudaSuccess) return status_of(e);
+    if (integers) {
+        auto plan = [&](size_t digits) {
+            gram = gram_plan(N, P, sms, digits);
+            slices = gram.slices;
+            lay_out();
+        };
+        plan(kGramDigitBytes);
+        // Digits of fewer columns at a time where that lets the workspace be the one that is kept: two or three chunks cost little, allocations a
+        // millisecond (1,600 x 20,000).
+        const bool could = bytes <= kKeepBytes + gram.digit_bytes - std::min(gram.digit_bytes, kLeastDigitBytes);
+        while (could && bytes > kKeepBytes && gram.digit_bytes > kLeastDigitBytes) plan(gram.digit_bytes / 4 * 3);
+        if ((e = ws.take(bytes)) == cudaErrorMemoryAllocation) {   // no room for the digits: the FP64 kernel, which needs none
+            cudaGetLastError();
+            integers = false;
+        }
+    }
+    if (!integers) {
+        // Slices of the feature axis: about two waves of the four blocks an SM holds, at least 128 columns each, and no more
+        // than 40 MB of partial tiles (or one slice, 65 MB at the most examples).
+        const size_t tile_bytes = (size_t)kGT * kGT * sizeof(double);
+        slices = std::max(1, std::min({8 * sms / tiles, P / 128, (int)(((size_t)40 << 20) / (tile_bytes * tiles))}));
+        slice = ((P + slices - 1) / slices + kGP - 1) / kGP * kGP;
+        slices = (P + slice - 1) / slice;
+        lay_out();
+        e = ws.take(bytes);
+    }
+    if (e != cudaSuccess) return status_of(e);
     double* d = static_cast<double*>(ws.ptr);
     unsigned* ticket = reinterpret_cast<unsigned*>(d + o_int);
     int* status = reinterpret_cast<int*>(d + o_int + 1);

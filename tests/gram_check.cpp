@@ -22,12 +22,13 @@ int main() {
     for (int N : rows)
         for (long long P = 1; P < 40000000ll; P += 1 + P / 7) {
             for (int p : {(int)P, N == 1728 ? 1354944 : (int)P / 64 * 64 + 1}) {
-                const GramPlan g = gram_plan(N, p, 148);
+                const size_t most = P % 3 == 0 ? kGramDigitBytes / 5 : kGramDigitBytes;
+                const GramPlan g = gram_plan(N, p, 148, most);
                 const int blocks = (p + kGramStageK - 1) / kGramStageK;
                 REQUIRE(g.chunk >= 1 && g.slices >= 1 && g.slices <= g.chunk, "%d x %d: %d slices of %d blocks", N, p, g.slices, g.chunk);
                 REQUIRE(g.groups * 8 >= N && g.groups % (kGramTileM / 8) == 0, "%d x %d: %d groups", N, p, g.groups);
                 const size_t block = (size_t)g.groups * kGramGroupBytes;
-                REQUIRE(g.digit_bytes == g.chunk * block && (g.chunk == 1 || g.digit_bytes <= kGramDigitBytes), "%d x %d: digits", N, p);
+                REQUIRE(g.digit_bytes == g.chunk * block && (g.chunk == 1 || g.digit_bytes <= most), "%d x %d: digits", N, p);
                 for (int b0 = 0; b0 < blocks; b0 += g.chunk) {
                     const int nb = blocks - b0 < g.chunk ? blocks - b0 : g.chunk, slices = gram_slices(g, nb);
                     REQUIRE(slices >= 1 && slices <= g.slices, "%d x %d: %d slices where there is room for %d", N, p, slices, g.slices);

@@ -67,3 +67,41 @@ def test_less_memory_than_the_copies_take(C):
         for name in ("hard", "soft", "arg"):
             assert torch.equal(want[name], full[name]), name
         p.close()
+
+
+def _fit_problem(N, P):
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+    F = torch.rand((N, P), generator=g, device="cuda")
+    return F, torch.randn((N,), generator=g, device="cuda")
+
+
+def _give_back():
+    """The regressor's workspace goes when a handle does."""
+    p = rk.RocketParams.generate(1, 1, 1, 64)
+    p.bind_device()
+    p.close()
+
+
+def test_a_fit_goes_on_without_room_for_the_features_as_integers():
+    import torch
+    F, y = _fit_problem(677, 20000)
+    want, _ = rk.rocket_ridge_fit(F, y, 1.0)
+    _give_back()
+    held = _leave(64 << 20)                                # the digits alone take 107 MB, all the rest 45
+    got, _ = rk.rocket_ridge_fit(F, y, 1.0)
+    del held
+    torch.cuda.empty_cache()
+    # both as close as double precision goes: rounded to FP32 each
+    assert (got.double() - want.double()).norm() <= 2.0 ** -23 * want.double().norm()
+    _give_back()
+
+
+def test_larger_fits_keep_their_workspace_too():
+    F, y = _fit_problem(1600, 20000)
+    rk.rocket_ridge_fit(F, y, 1.0)
+    before = rk.device_alloc_count()
+    rk.rocket_ridge_fit(F, y, 1.0)
+    assert rk.device_alloc_count() == before
+    _give_back()
