@@ -797,7 +797,7 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
                                     dim3((unsigned)std::max(1, std::min(sms, nb * (nb + 1) / 2))), dim3(kCThreads), args, chol_smem, stream);
     ridge_weights_kernel<<<col_blocks, kRThreads, 0, stream>>>(feat_dev, N, P, d + o_mu, d + o_a, d + o_ybar, w_dev, b_dev,
                                                                d + o_part, ticket);
-    count_launch(4);
+    count_launch(integers ? 3 : 4);                        // launch_gram counts its own
     int host_status[2] = {0, 0};
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_status, status, sizeof(host_status), cudaMemcpyDeviceToHost, stream);

@@ -69,6 +69,16 @@ def test_digits_of_several_chunks_of_columns(N, P):
     assert np.linalg.norm(w - rw) <= bound * np.linalg.norm(rw)
 
 
+@pytest.mark.parametrize("N,P,launches", [(33, 500, 4), (193, 40001, 6), (897, 19003, 8)])
+def test_every_kernel_of_a_fit_is_counted_once(N, P, launches):
+    # means, Gram matrix, factorisation and weights; integers: the scales, and digits and their products per chunk
+    import torch
+    F, y = torch.rand((N, P), device="cuda"), torch.rand(N, device="cuda")
+    before = rk.kernel_launch_count()
+    rk.rocket_ridge_fit(F, y, 1.0)
+    assert rk.kernel_launch_count() - before == launches
+
+
 def _weights_in_80_bits(F, y, alpha):
     Fc = F.astype(np.longdouble)
     Fc -= Fc.mean(0)
