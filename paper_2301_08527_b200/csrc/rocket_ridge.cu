@@ -738,9 +738,11 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     const int col_blocks = (P + 31) / 32;
     const int nt = (N + kGT - 1) / kGT, tiles = nt * (nt + 1) / 2;
     const int nb = (N + 1 + kCB - 1) / kCB, Np = nb * kCB;
-    // Integers on the tensor cores from about 100 examples of 20,000 features on (us, FP64 and integers: 24 x 20,000 99 and 113, 97 x 3,001
-    // 111 and 121, 300 x 600 207 and 212, 100 x 20,000 166 and 155, 300 x 5,000 238 and 225, 677 x 20,000 931 and 632).
-    bool integers = (double)N * N * P >= 1.2e8;
+    // Integers on the tensor cores beyond N N P = 3e8 (us, FP64 and integers: 200 x 4,000 143 and 148, 300 x 3,000 171 and 175, 677 x 300 293 and 298;
+    // 677 x 800 306 and 308; 200 x 8,000 168 and 154, 100 x 40,000 217 and 209, 300 x 5,000 193 and 186, 677 x 20,000 784 and 546).  Their tiles are 128
+    // rows high: up to 64 rows are half empty, and the digits of as many columns take longer than the products (64 x 120,000 364 and 398,
+    // 24 x 300,000 474 and 878).
+    bool integers = N > 64 && (double)N * N * P >= 3e8;
     GramPlan gram{};
     int slices = 0, slice = 0;
     size_t o_mu, o_a, o_part, o_ybar, o_G, o_Mi, o_Li, o_z, o_gram, o_int, o_up, o_down, o_digits, bytes;

@@ -1,6 +1,6 @@
 """Ridge fits whose Gram matrix is summed in integers (rocket_gram.cu), at the edges of its tiles, stages and slices.
 
-Rows around multiples of 64 and 128, columns around multiples of 64 and of a quadruple, more columns than a 32-bit sum takes at once, rows of
+From N N P = 3e8 on (smaller fits, among them the first nine here, take the FP64 kernel).  Rows around multiples of 64 and 128, columns around multiples of 64 and of a quadruple, more columns than a 32-bit sum takes at once, rows of
 very different magnitude.  Against the dual system in float64.  What the weights may be off by: their rounding to FP32 (2^-24 each) plus
 the errors of the two solutions, each of the order of 2^-53 times the condition number of the system.
 
@@ -31,7 +31,9 @@ def _dual(F, y, alpha):
 
 
 @pytest.mark.parametrize("N,P,kind", [(127, 7500, "shares"), (128, 7601, "shares"), (129, 7702, "shares"), (191, 3403, "shares"), (193, 40001, "shares"),
-                                      (257, 2049, "shares"), (257, 2111, "scales"), (320, 1985, "shifted"), (641, 320, "shares")])
+                                      (257, 2049, "shares"), (257, 2111, "scales"), (320, 1985, "shifted"), (641, 320, "shares"),
+                                      (127, 18700, "shares"), (128, 18353, "shares"), (129, 18070, "shares"), (191, 8331, "shares"), (257, 4609, "shares"),
+                                      (257, 4607, "scales"), (320, 2945, "shifted"), (641, 768, "shares")])
 def test_fits_match_the_dual_system_in_float64(N, P, kind):
     rng = np.random.default_rng(N + P)
     F = rng.random((N, P))
@@ -69,7 +71,7 @@ def test_digits_of_several_chunks_of_columns(N, P):
     assert np.linalg.norm(w - rw) <= bound * np.linalg.norm(rw)
 
 
-@pytest.mark.parametrize("N,P,launches", [(33, 500, 4), (193, 40001, 6), (897, 19003, 8)])
+@pytest.mark.parametrize("N,P,launches", [(33, 500, 4), (200, 7499, 4), (200, 7500, 6), (64, 120000, 4), (897, 19003, 8)])
 def test_every_kernel_of_a_fit_is_counted_once(N, P, launches):
     # means, Gram matrix, factorisation and weights; integers: the scales, and digits and their products per chunk
     import torch
@@ -128,7 +130,8 @@ def test_one_large_column_or_value(kind, size, alpha):
 
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_values_that_are_not_finite_are_refused(bad):
-    F = np.random.default_rng(1).random((200, 4000)).astype(np.float32)
+    F = np.random.default_rng(1).random((200, 8000)).astype(np.float32)
     F[13, 77] = bad
-    with pytest.raises(Exception):
+    with pytest.raises(rk.RocketError) as refused:
         _fit(F, F[:, 0].copy(), 1.0)
+    assert refused.value.status == -1                        # invalid argument
