@@ -19,6 +19,7 @@
 
 #include "rocket_gram.h"
 #include "rocket_internal.h"
+#include "rocket_pivot.cuh"
 
 namespace rocket {
 namespace {
@@ -171,22 +172,13 @@ struct CholArgs {
     int N, Np;
 };
 
-// 1 / sqrt(d) for a normal d > 0: an approximation with about 20 good bits and one step of Householder's third-order method,
-// y (1 + e / 2 + 3 e^2 / 8) with e = 1 - d y^2, whose error is of the order of e^3.
-__device__ __forceinline__ double inverse_root(double d) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    const double e = fma(-d * y, y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 // Factors the leading `ncols` columns of the block whose rows are held by the lanes (s[lane][0 .. lane]) and inverts the factor: row r
 // of the inverse's transpose goes to m[r]; lane j returns in root the reciprocal of the factor's diagonal j, which is in t[j][32] as well, and t[j]
 // holds column j of the factor times that diagonal.  One warp.
 //
 // A double-precision operation takes some 40 clocks here, so what counts is how many of them lie between a pivot and the next.  The
-// elimination is square-root free (a_ik -= c_ij c_kj / d_j with unscaled columns c), 1 / d_j is y (1 + e + e^2) for an approximation y
-// of 20 bits and e = 1 - d_j y, and the next pivot's column takes a - g - g (e + e^2) with g = c_ij c_kj y ready by then: three operations after the approximation.
+// elimination is square-root free (a_ik -= c_ij c_kj / d_j with unscaled columns c), 1 / d_j is y (1 + p) with a p that is ready one operation after y
+// (pivot_reciprocal), and the next pivot's column takes a - g - g p with g = c_ij c_kj y ready by then: three operations after the approximation.
 // With the factor's own columns and 1 / sqrt(d_j) they were six: 10,800 clocks for a block, 8,400 now.  (One body for all pivots, the rows
 // moving down by a column each time, has twice the multiply-adds: 13,700.)
 __device__ __forceinline__ bool chol_factor_block(const double (*s)[kCPitch], double (*t)[kDPitch], double (*m)[kCPitch], int ncols, int lane, double& root) {
@@ -201,20 +193,20 @@ __device__ __forceinline__ bool chol_factor_block(const double (*s)[kCPitch], do
 #pragma unroll
     for (int j = 0; j < kCB; ++j) {
         const bool there = j < ncols;
-        double d = __shfl_sync(0xffffffffu, a[j], j), y;
+        double d = __shfl_sync(0xffffffffu, a[j], j), y, p;
         good = good && (!there || d >= 2.2250738585072014e-308);
         d = there && d >= 2.2250738585072014e-308 ? d : 1.0;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+        pivot_reciprocal(d, y, p);
         const double col = there && lane >= j ? a[j] : 0.0;
         if (lane == j) mine = d;
         t[j][lane] = col;
-        const double e = fma(-d, y, 1.0), p = fma(e, e, e), cy = col * y;
+        const double cy = col * y;
         if (j + 1 < kCB) {                             // what the next pivot waits for
             const double next = __shfl_sync(0xffffffffu, col, j + 1), g = cy * next;
             a[j + 1] = fma(-g, p, a[j + 1] - g);
         }
         __syncwarp();
-        const double f = fma(cy, p, cy), xy = x[j] * y, xs = there ? fma(xy, p, xy) : 0.0;
+        const double f = fma(cy, p, cy), xs = there ? times_reciprocal(x[j], y, p) : 0.0;
         if (j + 1 < kCB) x[j + 1] = fma(-xs, t[j][j + 1], x[j + 1]);
 #pragma unroll
         for (int c = j + 2; c < kCB; ++c) {
@@ -223,7 +215,7 @@ __device__ __forceinline__ bool chol_factor_block(const double (*s)[kCPitch], do
             x[c] = fma(-xs, lc, x[c]);
         }
     }
-    root = inverse_root(mine);
+    root = rsqrt(mine);
     t[lane][kCB] = root;
 #pragma unroll
     for (int c = 0; c < kCB; ++c) m[lane][c] = x[c] * __shfl_sync(0xffffffffu, root, c);
