@@ -166,7 +166,7 @@ void cover_smaller_calls(const rocket_params* p, int N, bool soft, bool backward
     if (n == 0) return;
     const int64_t nW = n_weights_of(p);
     if (!fused) {
-        no_room(fast::reserve_fast_state(*p->fast, p->dp, n, soft, backward, false, nW, false));
+        no_room(fast::reserve_fast_state(*p->fast, p->dp, n, !soft && !backward, soft, backward, false, nW, false));
     } else if (backward) {
         std::lock_guard<std::mutex> lk(p->mu);
         no_room(p->scratch.reserve(generic_backward_scratch_floats(n, nW, p->host.K) * sizeof(float)));
@@ -393,7 +393,7 @@ int rocket_params_reserve(rocket_params_t* p, int max_N, int passes) {
     const int64_t nW = n_weights_of(p);
     bool fused = p->fast->host.enabled;
     if (fused) {
-        cudaError_t e = fast::reserve_fast_state(*p->fast, p->dp, max_N, soft, backward, u8, nW);
+        cudaError_t e = fast::reserve_fast_state(*p->fast, p->dp, max_N, (passes & ROCKET_PASS_HARD) != 0, soft, backward, u8, nW);
         if (no_room(e)) fused = false;
         else if (e != cudaSuccess) return cuda_status(e);
     }

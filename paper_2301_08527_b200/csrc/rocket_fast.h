@@ -281,6 +281,7 @@ struct PlanHost {
     int r_front = 0, r_pitch = 0;         // floats of zeros in front of the first channel row in shared memory; from row to row
     int r_tiles = 0;                      // most tiles of a kernel
     double r_clocks = 0.0, r_longest = 0.0;   // resident kernel: clocks of an SM for one example, and of a warp for its longest pair
+    int r_tiles_from = 0;                 // examples from which a hard transform goes to the tile kernels all the same; 0: never
     int split = kSplitDefault;
     std::vector<KRec> krec;
     std::vector<SBucket> sb;
@@ -324,6 +325,15 @@ inline int64_t resident_merge_floats(const PlanHost& plan, int64_t n, int parts,
 // The backward, whose code is twice as long and whose sums leave the warp once per tile, only where no tile has to test its reads and series
 // are short (us, before and with this kernel: 100 x 6 x 600, 2,000 kernels 1,106 and 855; 100 x 6 x 1,251 1,308 and 1,790).
 inline bool resident_backward(const PlanHost& plan) { return plan.r_back != 0; }
+// Hard transforms of many kernels on many examples, from 1,345 steps on: copying a tile per dilation is then spread over hundreds of kernels,
+// and the tile kernels' inner loops, whose addresses are constants, are the faster ones.  Measured (us, tile kernels and resident, 20,000
+// kernels): 100 x 6 x 1,400 4,738 and 5,100, 100 x 20 x 1,400 5,984 and 6,374, 100 x 6 x 2,300 6,925 and 7,821; on the other side of the lines
+// 24 x 6 x 1,400 1,390 and 1,230, 60 x 6 x 1,400 and 3,000 kernels 528 and 506, 128 x 3 x 1,560 2.5 % and 60 x 1 x 1,700 and 10,000 11 % in the
+// resident kernel's favour.  One size behind them is slower, 60 x 2 x 3,200 and 10,000 kernels by 2 %.  The soft modes and half precision are
+// faster with the resident kernel throughout.  Handles of such sizes hold both plans (20,000 kernels: created in 48 ms where 32 do).
+constexpr int kRTilesSteps = 1345, kRTilesMidSteps = 1500, kRTilesFarSteps = 2048, kRTilesKernels = 10000;
+constexpr double kRTilesPairs = 1.2e6, kRTilesFarPairs = 6e5;      // (kernel, example) pairs; beyond kRTilesFarSteps steps
+inline bool resident_forward(const PlanHost& plan, int N, bool hard) { return plan.resident && !(hard && plan.r_tiles_from > 0 && N >= plan.r_tiles_from); }
 // Floats of shared memory for n examples.
 inline int64_t resident_floats(const PlanHost& plan, int64_t n, int C) { return plan.r_front + n * C * plan.r_pitch; }
 
@@ -392,7 +402,7 @@ cudaError_t ensure_pad_capacity(FastState& fs, int N, int C, int L, bool without
 // copies and their tensor maps, the soft transform's and the backward's workspaces) and opts the kernels
 // into their shared-memory sizes; later calls within that size allocate nothing.
 // again: the full size, where there was no room for it before.
-cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N, bool soft, bool backward, bool u8,
+cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N, bool hard, bool soft, bool backward, bool u8,
                                int64_t n_weights, bool again = true);
 
 // Backward of the soft transform through the fast path (every kernel must be a fast-path kernel):

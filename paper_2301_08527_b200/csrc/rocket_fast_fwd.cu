@@ -1186,7 +1186,21 @@ static cudaError_t ensure_bwd_ws(FastState& fs, const DeviceParams& dp, int64_t 
     return e;
 }
 
-cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N, bool soft, bool backward, bool u8,
+// Room for the copies of a hard transform of N examples that the resident kernel could serve as well; that one does where there is none,
+// or where making it would end a capture.
+static bool tiles_have_room(FastState& fs, const DeviceParams& dp, int N, bool u8, cudaStream_t stream = nullptr) {
+    const bool streamed = fs.dev.n_wunits > 0, copies = fs.dev.n_titems > 0 || u8;
+    const int n = std::min({N, chunk_examples(fs, dp.C, streamed, copies), fs.most_examples});
+    if ((!streamed && !copies) || (n > 0 && n <= (streamed ? fs.wpad_examples : fs.pad_examples))) return true;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = stream ? cudaStreamIsCapturing(stream, &capture) : cudaSuccess;
+    if (e == cudaSuccess && capture == cudaStreamCaptureStatusNone)
+        e = streamed ? ensure_stream_capacity(fs, n, dp.C, dp.L) : ensure_pad_capacity(fs, n, dp.C, dp.L, u8 && fs.dev.n_titems == 0);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+}
+
+cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N, bool hard, bool soft, bool backward, bool u8,
                                int64_t n_weights, bool again) {
     std::lock_guard<std::mutex> lk(fs.mu);
     int dev = 0;
@@ -1194,8 +1208,10 @@ cudaError_t reserve_fast_state(FastState& fs, const DeviceParams& dp, int max_N,
     if (e != cudaSuccess) return e;
     if ((e = set_kernel_attributes(dev, fs.host)) != cudaSuccess) return e;
     if (again) fs.most_examples = 1 << 30;
-    if (fs.host.resident && (!backward || resident_backward(fs.host)))
-        return backward ? ensure_bwd_ws(fs, dp, n_weights) : cudaSuccess;   // no copies, no sums but the backward's
+    if (fs.host.resident && (!backward || resident_backward(fs.host))) {   // no copies, no sums but the backward's
+        if (!resident_forward(fs.host, max_N, hard)) tiles_have_room(fs, dp, max_N, u8);
+        return backward ? ensure_bwd_ws(fs, dp, n_weights) : cudaSuccess;
+    }
     const bool stream = fs.dev.n_wunits > 0, copies = fs.dev.n_titems > 0 || u8;
     const int chunk = std::min(max_N, chunk_examples(fs, dp.C, stream, copies));
     if (stream && (e = ensure_stream_capacity(fs, chunk, dp.C, dp.L)) != cudaSuccess) return e;
@@ -1228,7 +1244,7 @@ cudaError_t launch_fast_forward(FastState& fs, const DeviceParams& dp, const flo
     if (e != cudaSuccess) return e;
     e = set_kernel_attributes(dev, fs.host);
     if (e != cudaSuccess) return e;
-    if (fs.host.resident) {
+    if (resident_forward(fs.host, N, !soft && !half) || (fs.host.resident && !tiles_have_room(fs, dp, N, X_u8 != nullptr, stream))) {
         ResidentArgs r = resident_args(fs, dp, X, N, lambda, shift);
         r.feat = feat;
         r.argmax = argmax;

@@ -198,6 +198,9 @@ void build_resident_units(const HostParams& hp, PlanHost& out) {
     out.resident = !r.units.empty() && hp.L <= (out.r_zeros ? kRMostSteps : kRMostStepsTested);
     if (!out.resident) return;
     out.r_back = back ? kRBackBands[h] : 0;
+    const bool far = hp.L > kRTilesFarSteps;
+    if (hp.L >= kRTilesSteps && hp.C >= (far ? 2 : hp.L <= kRTilesMidSteps ? 3 : 6) && hp.C <= kSMaxPlanes && (int)out.krec.size() >= kRTilesKernels)
+        out.r_tiles_from = (int)std::ceil((far ? kRTilesFarPairs : kRTilesPairs) / (double)out.krec.size());
     for (RUnit& u : r.units) {
         const int before = std::max(0, u.p - zeros), end = hp.L + u.p + zeros;
         u.pq = before / u.d; u.pr = before % u.d;
@@ -207,6 +210,7 @@ void build_resident_units(const HostParams& hp, PlanHost& out) {
     // instruction caches decide here: the longest pairs first throughout took 846 us where this order takes 410 (100 x 20 x 2,800, 400 kernels).
     std::vector<int> order(r.units.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+    std::sort(order.begin(), order.end(), [&](int a, int b) { return r.units[a].k < r.units[b].k; });
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
         return r.units[a].len != r.units[b].len ? r.units[a].len > r.units[b].len : r.cost[a] > r.cost[b];
     });
@@ -450,11 +454,11 @@ void build_plan(const HostParams& hp, int split, PlanHost& out, bool all_tiles, 
                 (list == &s_kernels ? out.flops_s : out.flops_t) += 2.0 * f.len * f.m * (double)f.nout;
             }
         build_resident_units(hp, out);
-        if (resident_backward(out)) return;
+        if (resident_backward(out) && out.r_tiles_from == 0) return;
         out.krec.clear();
         out.runits.clear();
         out.resident = false;
-        out.r_back = 0;
+        out.r_back = out.r_tiles_from = 0;
         out.flops_s = out.flops_t = 0.0;
     }
 

@@ -133,6 +133,34 @@ static void check_generic() {
     }
 }
 
+static PlanHost plan_of(int C, int L, int K) {
+    HostParams hp;
+    generate_host_params(8527, K, C, L, hp);
+    hp.channel_offset.assign(hp.K + 1, 0);
+    hp.weight_offset.assign(hp.K + 1, 0);
+    for (int k = 0; k < hp.K; ++k) {
+        hp.channel_offset[k + 1] = hp.channel_offset[k] + hp.num_channels[k];
+        hp.weight_offset[k + 1] = hp.weight_offset[k] + hp.num_channels[k] * hp.length[k];
+    }
+    PlanHost plan;
+    build_plan(hp, kSplitDefault, plan, false, true);
+    return plan;
+}
+
+// Hard transforms of short series that go to the tile kernels: their handles hold both plans, others what their calls use.
+static void check_tiles_from() {
+    struct Case { int C, L, K, from; };
+    for (const Case& c : {Case{6, 1400, 20000, 60}, Case{6, 1344, 20000, 0}, Case{6, 1400, 9999, 0}, Case{2, 1400, 20000, 0}, Case{2, 2100, 10000, 60},
+                          Case{3, 2049, 30000, 20}, Case{6, 2048, 30000, 40}, Case{5, 1501, 20000, 0}, Case{3, 1500, 20000, 60}, Case{1, 2100, 20000, 0}, Case{20, 1345, 20000, 60}, Case{32, 1700, 20000, 0}, Case{3, 6000, 20000, 0}}) {
+        const PlanHost plan = plan_of(c.C, c.L, c.K);
+        REQUIRE(plan.r_tiles_from == c.from, "%d x %d, %d kernels: from %d examples", c.C, c.L, c.K, plan.r_tiles_from);
+        REQUIRE(c.from == 0 || (plan.resident && !plan.sitems.empty() && !plan.wunits.empty()), "%d x %d: both plans", c.C, c.L);
+        REQUIRE(c.from == 0 || (resident_forward(plan, c.from - 1, true) && !resident_forward(plan, c.from, true) && resident_forward(plan, c.from, false)), "%d x %d", c.C, c.L);
+        REQUIRE(c.from != 0 || resident_forward(plan, 1 << 20, true) == plan.resident, "%d x %d", c.C, c.L);
+    }
+    REQUIRE(plan_of(6, 1400, 9999).sitems.empty(), "tiles that no call uses");
+}
+
 // Kernels from standard input (C, L, K, then per kernel length, dilation, padding and its channels): prints, for N examples, how many
 // examples the tiles of each class share and how many tiles there are of each, and whether the generic kernels serve the call.
 static int print_sharing(int N) {
@@ -165,6 +193,7 @@ int main(int argc, char** argv) {
     check_rows_in_series();
     check_stream_items();
     check_generic();
+    check_tiles_from();
     if (failures == 0) std::printf("ok\n");
     return failures ? 1 : 0;
 }

@@ -66,3 +66,73 @@ def test_bytes_give_the_bits_of_their_samples():
     want = rk.rocket_transform(p, scaled.contiguous())
     assert torch.equal(got, want)
     p.close()
+
+
+def _many_kernels(C, L, K):
+    import torch
+    p = rk.RocketParams.generate(8527, K, C, L)
+    return p, lambda N: torch.from_numpy(np.tile(ar1_spike_series(C, 8, C, L), (-(-N // 8), 1, 1))[:N].copy()).cuda()
+
+
+def _launches(call):
+    before = rk.kernel_launch_count()
+    out = call()
+    return rk.kernel_launch_count() - before, out
+
+
+def test_large_hard_transforms_take_the_tile_kernels():
+    # from 6e5 (kernel, example) pairs on beyond 2,048 steps; the same bits, one example more or less, and the other modes stay
+    import torch
+    C, L, K = 3, 2100, 10000
+    p, series = _many_kernels(C, L, K)
+    X = series(60)
+    n, large = _launches(lambda: rk.rocket_transform(p, X))
+    assert n > 1
+    n, small = _launches(lambda: rk.rocket_transform(p, X[:59].contiguous()))
+    assert n == 1
+    assert torch.equal(large[:59], small)
+    assert _launches(lambda: rk.rocket_transform_f16(p, X))[0] == 1
+    assert _launches(lambda: rk.rocket_transform_soft(p, X, 10.0, 3.0))[0] == 1
+    v = ((X - X.min()) * (255 / (X.max() - X.min()))).to(torch.uint8)
+    mean, inv_std = np.full(C, 100.0, np.float32), np.full(C, 1 / 40.0, np.float32)
+    n, large = _launches(lambda: rk.rocket_transform_u8(p, v, mean, inv_std))
+    assert n > 1
+    assert torch.equal(large[:59], rk.rocket_transform_u8(p, v[:59].contiguous(), mean, inv_std))
+    assert p.device_status() == 0
+    p.close()
+
+
+def test_large_hard_transforms_after_reserve_and_without_it():
+    import torch
+    C, L, K = 3, 2100, 10000
+    p, series = _many_kernels(C, L, K)
+    X = series(64)
+    p.reserve(64, rk.PASS_HARD)
+    before = rk.device_alloc_count()
+    n, want = _launches(lambda: rk.rocket_transform(p, X))
+    assert n > 1 and rk.device_alloc_count() == before
+    p.close()
+    # nothing reserved: a capture goes on, with the kernel that needs no workspace
+    p, _ = _many_kernels(C, L, K)
+    rk.rocket_transform(p, X[:1].contiguous())
+    out = torch.zeros_like(want)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        rk.rocket_transform(p, X, out=out)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    del graph
+    p.close()
+    # next to no room: fewer examples at a time, or that kernel
+    p, _ = _many_kernels(C, L, K)
+    p.bind_device()
+    torch.cuda.empty_cache()
+    held = torch.empty(max(0, torch.cuda.mem_get_info()[0] - (4 << 20)), dtype=torch.uint8, device="cuda")
+    rk.rocket_transform(p, X, out=out.zero_())
+    torch.cuda.synchronize()
+    del held
+    torch.cuda.empty_cache()
+    assert torch.equal(out, want)
+    p.close()
