@@ -145,11 +145,7 @@ bool no_room(cudaError_t e) {
     return true;
 }
 
-// Whether every fused call of the handle is a matter of one kernel, or of tiles of at most kSMaxPlanes channels: no call of such a handle is
-// better served by the generic kernels.
-bool always_fused(const rocket_params* p, bool backward) {
-    return p->host.C <= fast::kSMaxPlanes || (backward ? fast::resident_backward(p->fast->host) : p->fast->host.resident);
-}
+bool always_fused(const rocket_params* p, bool backward) { return fast::always_fused(p->fast->host, p->host.C, backward); }
 
 // Whether the fused kernels serve a call of N examples (with the handle's kernels that they take).
 bool fused_call(const rocket_params* p, bool aligned, int N, bool soft, bool backward = false) {

@@ -325,6 +325,11 @@ inline int64_t resident_merge_floats(const PlanHost& plan, int64_t n, int parts,
 // The backward, whose code is twice as long and whose sums leave the warp once per tile, only where no tile has to test its reads and series
 // are short (us, before and with this kernel: 100 x 6 x 600, 2,000 kernels 1,106 and 855; 100 x 6 x 1,251 1,308 and 1,790).
 inline bool resident_backward(const PlanHost& plan) { return plan.r_back != 0; }
+// Whether every fused call of the handle is a matter of one kernel, or of tiles of at most kSMaxPlanes channels: no call of such a handle is
+// better served by the generic kernels, and generic_pays is not asked.
+inline bool always_fused(const PlanHost& plan, int C, bool backward) {
+    return C <= kSMaxPlanes || (backward ? resident_backward(plan) : plan.resident);
+}
 // Hard transforms of many kernels on many examples, from 1,345 steps on: copying a tile per dilation is then spread over hundreds of kernels,
 // and the tile kernels' inner loops, whose addresses are constants, are the faster ones.  Measured (us, tile kernels and resident, 20,000
 // kernels): 100 x 6 x 1,400 4,738 and 5,100, 100 x 20 x 1,400 5,984 and 6,374, 100 x 6 x 2,300 6,925 and 7,821; on the other side of the lines

@@ -106,34 +106,7 @@ static void check_copies() {
     }
 }
 
-// Many channels: the generic kernels where they were measured to be faster, the fused ones where those were.
-static void check_generic() {
-    struct Case { int N, C, L, K, generic; };
-    for (const Case& c : {Case{1, 32, 32, 1500, 1}, Case{1, 21, 100, 300, 1}, Case{32, 255, 102, 1500, 1}, Case{32, 255, 1002, 60, 1}, Case{1, 64, 31, 300, 1},
-                          Case{6, 32, 102, 1500, 1}, Case{24, 32, 1751, 2000, 0}, Case{1, 32, 4000, 300, 0}, Case{32, 255, 4002, 1500, 0}, Case{6, 64, 4000, 60, 0},
-                          Case{32, 21, 300, 1500, 0}, Case{1, 30, 100000, 100, 0}, Case{4, 100, 20000, 500, 0}, Case{32, 64, 4003, 60, 0}, Case{32, 32, 4000, 60, 0}}) {
-        HostParams hp;
-        generate_host_params(8527, c.K, c.C, c.L, hp);
-        hp.channel_offset.assign(hp.K + 1, 0);
-        hp.weight_offset.assign(hp.K + 1, 0);
-        for (int k = 0; k < hp.K; ++k) {
-            hp.channel_offset[k + 1] = hp.channel_offset[k] + hp.num_channels[k];
-            hp.weight_offset[k + 1] = hp.weight_offset[k] + hp.num_channels[k] * hp.length[k];
-        }
-        PlanHost plan;
-        build_plan(hp, kSplitDefault, plan, false);
-        REQUIRE(generic_pays(plan, c.N, kSms, false) == (c.generic != 0), "%d x %d x %d, %d kernels", c.N, c.C, c.L, c.K);
-        for (int way = 0; way < 4; ++way)
-            for (int most : {1, 7, 32, 300}) {
-                const bool generic = (way & 1) != 0, soft = (way & 2) != 0;
-                const int up_to = pays_up_to(plan, most, kSms, soft, generic);
-                for (int n = 1; n <= most; ++n)
-                    REQUIRE(n <= up_to || generic_pays(plan, n, kSms, soft) != generic, "%d of at most %d examples", n, up_to);
-            }
-    }
-}
-
-static PlanHost plan_of(int C, int L, int K) {
+static PlanHost plan_of(int C, int L, int K, bool only_used = true) {
     HostParams hp;
     generate_host_params(8527, K, C, L, hp);
     hp.channel_offset.assign(hp.K + 1, 0);
@@ -143,8 +116,29 @@ static PlanHost plan_of(int C, int L, int K) {
         hp.weight_offset[k + 1] = hp.weight_offset[k] + hp.num_channels[k] * hp.length[k];
     }
     PlanHost plan;
-    build_plan(hp, kSplitDefault, plan, false, true);
+    build_plan(hp, kSplitDefault, plan, false, only_used);
     return plan;
+}
+
+// Many channels: the generic kernels where they were measured to be faster, the fused ones where those were; handles whose examples the resident
+// kernel holds are not asked.
+static void check_generic() {
+    struct Case { int N, C, L, K, generic, asked; };
+    for (const Case& c : {Case{1, 32, 32, 1500, 1, 0}, Case{1, 21, 100, 300, 1, 0}, Case{32, 255, 102, 1500, 1, 0}, Case{32, 255, 1002, 60, 1, 1}, Case{1, 64, 31, 300, 1, 0},
+                          Case{6, 32, 102, 1500, 1, 0}, Case{24, 32, 1751, 2000, 0, 0}, Case{1, 32, 4000, 300, 0, 1}, Case{32, 255, 4002, 1500, 0, 1}, Case{6, 64, 4000, 60, 0, 1},
+                          Case{32, 21, 300, 1500, 0, 0}, Case{1, 30, 100000, 100, 0, 1}, Case{4, 100, 20000, 500, 0, 1}, Case{32, 64, 4003, 60, 0, 1}, Case{32, 32, 4000, 60, 0, 1}}) {
+        // as a handle has it, and with every plan: the rule is asked for backwards that the resident kernel does not serve
+        REQUIRE(always_fused(plan_of(c.C, c.L, c.K), c.C, false) == (c.asked == 0), "%d x %d x %d, %d kernels", c.N, c.C, c.L, c.K);
+        const PlanHost plan = plan_of(c.C, c.L, c.K, false);
+        REQUIRE(generic_pays(plan, c.N, kSms, false) == (c.generic != 0), "%d x %d x %d, %d kernels", c.N, c.C, c.L, c.K);
+        for (int way = 0; way < 4; ++way)
+            for (int most : {1, 7, 32, 300}) {
+                const bool generic = (way & 1) != 0, soft = (way & 2) != 0;
+                const int up_to = pays_up_to(plan, most, kSms, soft, generic);
+                for (int n = 1; n <= most; ++n)
+                    REQUIRE(n <= up_to || generic_pays(plan, n, kSms, soft) != generic, "%d of at most %d examples", n, up_to);
+            }
+    }
 }
 
 // Hard transforms of short series that go to the tile kernels: their handles hold both plans, others what their calls use.
@@ -161,8 +155,9 @@ static void check_tiles_from() {
     REQUIRE(plan_of(6, 1400, 9999).sitems.empty(), "tiles that no call uses");
 }
 
-// Kernels from standard input (C, L, K, then per kernel length, dilation, padding and its channels): prints, for N examples, how many
-// examples the tiles of each class share and how many tiles there are of each, and whether the generic kernels serve the call.
+// Kernels from standard input (C, L, K, then per kernel length, dilation, padding and its channels): prints, for N examples and the plan a handle
+// has, how many examples the small-dilation tiles of each class share and how many tiles there are of each, and which kernels serve the
+// forward modes and the backward: g(eneric), r(esident) or t(iles).
 static int print_sharing(int N) {
     HostParams hp;
     if (std::scanf("%d %d %d", &hp.C, &hp.L, &hp.K) != 3) return 2;
@@ -179,10 +174,14 @@ static int print_sharing(int N) {
     }
     hp.weights.assign(hp.weight_offset.back(), 1.0f);
     PlanHost plan;
-    build_plan(hp, kSplitDefault, plan, false);
+    build_plan(hp, kSplitDefault, plan, false, true);
     const SGroups s = s_groups(plan, N, kSms);
     for (int i = 0; i < 3; ++i) std::printf("%d %d ", s.examples[i], s.end[i] - (i ? s.end[i - 1] : 0));
-    std::printf("%d\n", hp.C > kSMaxPlanes && generic_pays(plan, N, kSms, false) && generic_pays(plan, N, kSms, true) ? 1 : 0);
+    auto served = [&](bool hard, bool soft, bool backward) {
+        if (!always_fused(plan, hp.C, backward) && generic_pays(plan, N, kSms, soft)) return 'g';
+        return (backward ? resident_backward(plan) : resident_forward(plan, N, hard)) ? 'r' : 't';
+    };
+    std::printf("%c%c%c\n", served(true, false, false), served(false, true, false), served(false, true, true));
     return 0;
 }
 

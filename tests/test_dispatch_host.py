@@ -4,7 +4,7 @@ import subprocess
 
 import pytest
 
-from test_gpu_sharing import CASES, WIDE_CASES, kernels
+from test_gpu_sharing import CASES, SHORT_CASES, WIDE_CASES, kernels
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -25,24 +25,25 @@ def test_dispatch_rules(check):
 
 
 def _dispatch(check, C, L, N, kp):
-    """(examples that share a tile, tiles) per class, and whether the generic kernels serve the call."""
+    """(examples that share a tile, tiles) per class, and which kernels serve the call in each mode."""
     text = "%d %d %d\n" % (C, L, kp.K)
     for k in range(kp.K):
         ch = kp.channel_idx[kp.channel_offset[k]:kp.channel_offset[k + 1]]
         text += " ".join(map(str, [kp.length[k], kp.dilation[k], kp.padding[k], len(ch), *ch])) + "\n"
-    out = list(map(int, subprocess.run([check, str(N)], input=text, capture_output=True, text=True, check=True).stdout.split()))
-    return out[0:6:2], out[1:6:2], out[6] != 0
+    out = subprocess.run([check, str(N)], input=text, capture_output=True, text=True, check=True).stdout.split()
+    return list(map(int, out[0:6:2])), list(map(int, out[1:6:2])), out[6]
 
 
 @pytest.mark.parametrize("case", CASES)
 def test_the_sharing_cases_share_tiles(check, case):
     C, L, N, K, dilations, classes = case
-    examples, tiles, _ = _dispatch(check, C, L, N, kernels(C, L, K, dilations))
+    examples, tiles, served = _dispatch(check, C, L, N, kernels(C, L, K, dilations))
+    assert served == "ttt"
     for cls in classes:
         assert tiles[cls] > 0 and examples[cls] > 1 and N % examples[cls] != 0, (examples, tiles)
 
 
-@pytest.mark.parametrize("case", WIDE_CASES)
-def test_the_wide_cases_take_the_kernels_they_name(check, case):
-    C, L, N, K, dilations, generic = case
-    assert _dispatch(check, C, L, N, kernels(C, L, K, dilations))[2] == generic
+@pytest.mark.parametrize("case", SHORT_CASES + WIDE_CASES)
+def test_the_other_cases_take_the_kernels_they_name(check, case):
+    C, L, N, K, dilations, served = case
+    assert _dispatch(check, C, L, N, kernels(C, L, K, dilations))[2] == served

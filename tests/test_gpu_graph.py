@@ -25,10 +25,11 @@ def _handle(C, L, small, large):
     return rk.RocketParams.from_kernel_params(kernels_from_lists(C, L, ks))
 
 
-@pytest.mark.parametrize("small,large", [(400, 2), (3, 200), (50, 0)])
-def test_captured_calls_give_the_bits_of_plain_calls(small, large):
+# 6,001 steps: the tile kernels; 2,001: the kernel that holds whole examples, which has no neighbour but in the backward
+@pytest.mark.parametrize("L,small,large", [(6001, 400, 2), (6001, 3, 200), (6001, 50, 0), (2001, 40, 30)])
+def test_captured_calls_give_the_bits_of_plain_calls(L, small, large):
     import torch
-    C, L, N = 6, 6001, 5
+    C, N = 6, 5
     p = _handle(C, L, small, large)
     K = small + large
     X = torch.from_numpy(ar1_spike_series(3, N, C, L)).cuda()

@@ -1,8 +1,9 @@
 """Small-dilation tiles shared among examples, with a last group that is not full, and series of more than 20 channels on either side of
 the line between the fused and the generic kernels, against the oracles (every mode).
 
-Which tiles are shared, and by how many examples, and which kernels serve the wide series, test_dispatch_host.py checks on the host
-for the cases below (buckets of 8 to 31 kernels are class 1, of fewer class 2; 148 SMs).
+Which tiles are shared, and by how many examples, and which kernels serve the series, test_dispatch_host.py checks on the host
+for the cases below (buckets of 8 to 31 kernels are class 1, of fewer class 2; 148 SMs).  Served by, for hard, soft and backward: t the tile
+kernels, r the one that holds whole examples, g the generic ones.
 """
 import numpy as np
 import pytest
@@ -16,11 +17,15 @@ from test_gpu_edges import _kernels
 from test_gpu_f16 import _check_bitwise
 
 # channels, steps, examples, kernels, dilations; classes whose tiles are shared
-CASES = [(1, 65, 401, 60, (1, 2, 9), (1,)), (3, 207, 233, 40, (1, 2, 3, 5, 6, 7, 11, 13), (2,)),
-         (2, 120, 401, 52, (1, 1, 1, 1, 1, 1, 1, 2, 3, 4, 5, 6, 7), (1, 2)), (4, 99, 403, 30, (1, 2, 3, 4, 5), (2,))]
-# channels, steps, examples, kernels, dilations; served by the generic kernels
-WIDE_CASES = [(21, 1501, 9, 120, (1, 5, 40), False), (34, 1701, 8, 160, (1, 3, 63, 90), False), (35, 1500, 8, 160, (2, 9, 130), False),
-              (48, 2003, 6, 90, (1, 2, 7, 66, 160), False), (25, 86, 3, 60, (1, 2, 5), True), (255, 130, 5, 40, (1, 4, 9), True)]
+CASES = [(1, 5003, 103, 60, (1, 2, 9), (1,)), (3, 5002, 83, 40, (1, 2, 3, 5, 6, 7, 11, 13), (2,)),
+         (2, 5001, 107, 52, (1, 1, 1, 1, 1, 1, 1, 2, 3, 4, 5, 6, 7), (1, 2)), (4, 5001, 103, 30, (1, 2, 3, 4, 5), (2,))]
+# short ones, which share no tiles; served by
+SHORT_CASES = [(1, 65, 401, 60, (1, 2, 9), "rrr"), (3, 207, 233, 40, (1, 2, 3, 5, 6, 7, 11, 13), "rrr"),
+               (2, 120, 401, 52, (1, 1, 1, 1, 1, 1, 1, 2, 3, 4, 5, 6, 7), "rrr"), (4, 99, 403, 30, (1, 2, 3, 4, 5), "rrr")]
+# more than 20 channels; served by
+WIDE_CASES = [(21, 1501, 9, 120, (1, 5, 40), "rrr"), (34, 1701, 8, 160, (1, 3, 63, 90), "ttt"), (35, 1500, 8, 160, (2, 9, 130), "rrt"),
+              (48, 2003, 6, 90, (1, 2, 7, 66, 160), "ttt"), (25, 86, 3, 60, (1, 2, 5), "rrr"), (255, 130, 5, 40, (1, 4, 9), "rrr"),
+              (255, 229, 2, 12, (1, 2, 5, 20), "ggg"), (255, 220, 2, 12, (1, 2, 5, 20), "rrg"), (255, 331, 5, 40, (1, 4, 9), "ttt")]
 
 
 def kernels(C, L, K, dilations):
@@ -28,7 +33,7 @@ def kernels(C, L, K, dilations):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("case", CASES + WIDE_CASES)
+@pytest.mark.parametrize("case", CASES + SHORT_CASES + WIDE_CASES)
 def test_every_mode(case):
     import torch
     C, L, N, K, dilations, _ = case
