@@ -9,7 +9,7 @@
 // of the same data are bitwise identical.
 //
 // Measured at 677 x 20,000 (B200): column means, Gram matrix, factorisation with solves and weights take
-// 18 / 254 (in FP64 496) / 229 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
+// 18 / 255 (in FP64 496) / 228 (381 before) / 21 us; as one thread per column, 2 x 2 outputs per thread, one block and one thread per column they took
 // 55 / 2,607 / 20,270 / 174.
 #include <cooperative_groups.h>
 
@@ -151,10 +151,13 @@ ridge_gram_kernel(const float* __restrict__ F, int N, int P, const double* __res
 // into the upper triangle, factors and inverses into Li and Mi.  Bound: block 0's chain of 32 dependent pivots per step (22 steps at N = 677).
 //
 // A product with an explicit inverse is off by 2^-53 times the condition of the diagonal block, where a substitution is off by 2^-53 of its own
-// terms: X = A M alone left rows of 10^-4 to 10^4 with errors 10 to 400 times as large, or refused them for a pivot that was not positive.  So every
-// product takes one step of iterative refinement, X + (A - X L^T) M, which leaves the square of that error: the same as a substitution's up to
-// conditions of 10^8 of a factor, which is as far as any factorisation in double precision goes.
+// terms: X = A M alone left rows of 10^-4 to 10^4 with errors 10 to 400 times as large, or refused them for a pivot that was not positive.  So
+// where the factor or its inverse has an element far beyond the others (kCLarge) a product takes one step of iterative refinement,
+// X + (A - X L^T) M, which leaves the square of that error: the same as a substitution's up to conditions of 10^8 of a factor, which is as far
+// as any factorisation in double precision goes.  In every block it takes 26 us at 677 x 20,000; left out where no element is beyond 2, 8 or 32
+// times the others, the errors of sixty fits of twelve kinds were the same to three digits.  It takes 1 us where no block does.
 constexpr int kCB = 32, kCThreads = 256, kCPitch = kCB + 4, kDPitch = kCB + 2;
+constexpr double kCLarge = 8.0;                                       // times the largest diagonal of the factor or the least of its inverse
 constexpr int kCSmem = kCB * kDPitch + 6 * kCB * kCPitch;              // doubles: a factor and six blocks; in the end the solution besides
 
 struct CholArgs {
@@ -166,6 +169,7 @@ struct CholArgs {
     double* G;
     double* Mi;               // inverse factors of the diagonal blocks, transposed [nb][32][32]
     double* Li;               // the factors, transposed [nb][32][32]
+    int* refine;              // whether products with the inverse take a refinement step [nb]
     double* z;                // row N of the factor, by blocks
     double* a;                // solution [N]
     int* status;              // 0 = ok, 1 = a pivot was not positive
@@ -173,8 +177,8 @@ struct CholArgs {
 };
 
 // Factors the leading `ncols` columns of the block whose rows are held by the lanes (s[lane][0 .. lane]) and inverts the factor: row r
-// of the inverse's transpose goes to m[r]; lane j returns in root the reciprocal of the factor's diagonal j, which is in t[j][32] as well, and t[j]
-// holds column j of the factor times that diagonal.  One warp.
+// of the inverse's transpose goes to m[r]; lane j returns in root the reciprocal of the factor's diagonal j, which is in t[j][32] as well (their
+// least in t[0][33]), and t[j] holds column j of the factor times that diagonal.  One warp.
 //
 // A double-precision operation takes some 40 clocks here, so what counts is how many of them lie between a pivot and the next.  The
 // elimination is square-root free (a_ik -= c_ij c_kj / d_j with unscaled columns c), 1 / d_j is y (1 + p) with a p that is ready one operation after y
@@ -217,6 +221,8 @@ __device__ __forceinline__ bool chol_factor_block(const double (*s)[kCPitch], do
     }
     root = rsqrt(mine);
     t[lane][kCB] = root;
+    const int least = __reduce_min_sync(0xffffffffu, __double2hiint(root));   // positive: the high words are in their order
+    if (lane == 0) t[0][kCB + 1] = __hiloint2double(least, 0);
 #pragma unroll
     for (int c = 0; c < kCB; ++c) m[lane][c] = x[c] * __shfl_sync(0xffffffffu, root, c);
     __syncwarp();
@@ -245,15 +251,21 @@ ridge_cholesky_solve_kernel(CholArgs q) {
     auto factor = [&](int kb) {
         const int ncols = min(kCB, N - kb * kCB);
         double root = 0.0;
+        bool large = false;
         if (ncols > 0 && warp == 0) good = chol_factor_block(s_pi, s_t, s_m, ncols, lane, root) && good;
         __syncthreads();
         if (ncols > 0)
             for (int e = tid; e < kCB * kCB; e += kCThreads) {
-                q.Mi[(size_t)kb * kCB * kCB + e] = s_m[e / kCB][e % kCB];
-                q.Li[(size_t)kb * kCB * kCB + e] = s_t[e / kCB][e % kCB] * s_t[e / kCB][kCB];
+                const double m = s_m[e / kCB][e % kCB], l = s_t[e / kCB][e % kCB] * s_t[e / kCB][kCB];
+                q.Mi[(size_t)kb * kCB * kCB + e] = m;
+                large = large || fabs(m) > kCLarge * s_t[0][kCB + 1] || fabs(l) * s_t[0][kCB + 1] > kCLarge;
             }
         // row N of the factor: within its own diagonal block the factor's rows are not kept elsewhere
         if (kb == N / kCB && tid < ncols) q.z[kb * kCB + tid] = s_t[tid][N - kb * kCB] * root;
+        large = __syncthreads_or(large);
+        if (large)
+            for (int e = tid; e < kCB * kCB; e += kCThreads) q.Li[(size_t)kb * kCB * kCB + e] = s_t[e / kCB][e % kCB] * s_t[e / kCB][kCB];
+        if (tid == 0) q.refine[kb] = large ? 1 : 0;
         __syncthreads();
     };
 
@@ -300,15 +312,15 @@ ridge_cholesky_solve_kernel(CholArgs q) {
                 const int jb = nb - 1 - x, ib = nb - 1 - ((tiles - 1 - b) - x * (x + 1) / 2);
                 const int i0 = ib * kCB, j0 = jb * kCB;
                 const bool two = ib != jb;
-                // all loads of the tile at once: factor and inverse, panel blocks, the warp's fragments of the tile (rows fr of row block 8 br,
+                // all loads of the tile at once: inverse factor, panel blocks, the warp's fragments of the tile (rows fr of row block 8 br,
                 // columns 2 fk, 2 fk + 1 of column blocks bc)
                 constexpr int kEach = kCB * kCB / kCThreads;
-                double lm[kEach], ll[kEach], li[kEach], lj[kEach], g[2][2];
+                const bool refine = __ldcg(q.refine + kb) != 0;
+                double lm[kEach], li[kEach], lj[kEach], g[2][2];
 #pragma unroll
                 for (int u = 0; u < kEach; ++u) {
                     const int e = tid + u * kCThreads, r = e / kCB, c = e % kCB;
                     lm[u] = __ldcg(q.Mi + (size_t)kb * kCB * kCB + e);
-                    ll[u] = __ldcg(q.Li + (size_t)kb * kCB * kCB + e);
                     li[u] = __ldcg(G + (size_t)(i0 + r) * Np + k0 + c);
                     lj[u] = two ? __ldcg(G + (size_t)(j0 + r) * Np + k0 + c) : 0.0;
                 }
@@ -321,7 +333,6 @@ ridge_cholesky_solve_kernel(CholArgs q) {
                 for (int u = 0; u < kEach; ++u) {
                     const int e = tid + u * kCThreads, r = e / kCB, c = e % kCB;
                     s_m[r][c] = lm[u];
-                    s_l[r][c] = ll[u];
                     s_pi[r][c] = li[u];
                     if (two) s_pj[r][c] = lj[u];
                 }
@@ -369,14 +380,17 @@ ridge_cholesky_solve_kernel(CholArgs q) {
                     __syncthreads();
                 };
                 __syncthreads();
-                // the solved panel blocks: X = A M, R = A - X L^T, X + R M
+                // the solved panel blocks: X = A M, and to refine them R = A - X L^T, X + R M
                 multiply(s_pi, s_pj, s_m, 1.0);
-                keep(s_xi, s_xj);
-                fetch(s_pi, s_pj);
-                multiply(s_xi, s_xj, s_l, -1.0);
-                keep(s_pi, s_pj);
-                fetch(s_xi, s_xj);
-                multiply(s_pi, s_pj, s_m, 1.0);
+                if (refine) {
+                    for (int e = tid; e < kCB * kCB; e += kCThreads) s_l[e / kCB][e % kCB] = __ldcg(q.Li + (size_t)kb * kCB * kCB + e);
+                    keep(s_xi, s_xj);
+                    fetch(s_pi, s_pj);
+                    multiply(s_xi, s_xj, s_l, -1.0);
+                    keep(s_pi, s_pj);
+                    fetch(s_xi, s_xj);
+                    multiply(s_pi, s_pj, s_m, 1.0);
+                }
                 __syncthreads();
                 keep(s_pi, s_pj);
                 double h0[2][2] = {};
@@ -417,6 +431,7 @@ ridge_cholesky_solve_kernel(CholArgs q) {
     // inverse, the block of L next to the diagonal, and the part of the sums whose a_i were known then.
     if (warp == 0 && lane == 0 && !good) *q.status = 1;
     __shared__ double s_sum[2][kCB];
+    __shared__ bool s_refine[2];
     double (*s_inv)[kCPitch] = s_m, (*s_next)[kCPitch] = s_m + 2 * kCB, (*s_own)[kCPitch] = s_m + 4 * kCB;   // two of each
     double* s_a = reinterpret_cast<double*>(s_m + 6 * kCB);
     const int nblk = (N + kCB - 1) / kCB;
@@ -424,12 +439,12 @@ ridge_cholesky_solve_kernel(CholArgs q) {
     auto bring = [&](int kb) {                               // for block kb, by warps 1 .. 7, while a of blocks above kb + 1 is known
         const int k0 = kb * kCB, buf = kb & 1, w = warp - 1;
         constexpr int kEach = (kCB * kCB + kCThreads - 33) / (kCThreads - 32);
-        double inv[kEach], own[kEach], next[kEach];
+        const bool refine = __ldcg(q.refine + kb) != 0;
+        double inv[kEach], next[kEach];
 #pragma unroll
         for (int u = 0; u < kEach; ++u) {
             const int e = min(tid - 32 + u * (kCThreads - 32), kCB * kCB - 1), r = e / kCB, c = e % kCB;
             inv[u] = __ldcg(q.Mi + (size_t)kb * kCB * kCB + e);
-            own[u] = __ldcg(q.Li + (size_t)kb * kCB * kCB + e);
             next[u] = __ldcg(G + (size_t)(k0 + r) * Np + min(k0 + kCB + c, Np - 1));   // past column N: not used
         }
         // five rows a warp, side by side: what counts is how many loads are on their way
@@ -457,9 +472,10 @@ ridge_cholesky_solve_kernel(CholArgs q) {
         for (int u = 0; u < kEach; ++u) {
             const int e = min(tid - 32 + u * (kCThreads - 32), kCB * kCB - 1), r = e / kCB, c = e % kCB;
             s_inv[buf * kCB + r][c] = inv[u];
-            s_own[buf * kCB + r][c] = own[u];
+            if (refine) s_own[buf * kCB + r][c] = __ldcg(q.Li + (size_t)kb * kCB * kCB + e);
             s_next[buf * kCB + r][c] = next[u];
         }
+        if (tid == 32) s_refine[buf] = refine;
     };
     __syncthreads();
     if (warp > 0) bring(nblk - 1);
@@ -487,7 +503,7 @@ ridge_cholesky_solve_kernel(CholArgs q) {
                 return lane < ncols ? (u[0] + u[1]) + (u[2] + u[3]) : 0.0;
             };
             double a = times(s_inv, 0, v);
-            a += times(s_inv, 2, v - times(s_own, 1, a));
+            if (s_refine[buf]) a += times(s_inv, 2, v - times(s_own, 1, a));
             if (lane < ncols) {
                 s_a[k0 + lane] = a;
                 q.a[k0 + lane] = a;
@@ -737,14 +753,14 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
     bool integers = N > 64 && (double)N * N * P >= 3e8;
     GramPlan gram{};
     int slices = 0, slice = 0;
-    size_t o_mu, o_a, o_part, o_ybar, o_G, o_Mi, o_Li, o_z, o_gram, o_int, o_up, o_down, o_digits, bytes;
-    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Mi[nb][32][32], Li[nb][32][32], z[Np], partial Gram tiles, ticket, status; for
+    size_t o_mu, o_a, o_part, o_ybar, o_G, o_Mi, o_Li, o_refine, o_z, o_gram, o_int, o_up, o_down, o_digits, bytes;
+    // workspace: mu[P], a[N], part[col_blocks], ybar, G[Np][Np], Mi[nb][32][32], Li[nb][32][32], refine[nb], z[Np], partial Gram tiles, ticket, status; for
     // integers the rows' scales and digits
     auto lay_out = [&]() {
         size_t off = 0;
         auto take = [&](size_t doubles) { const size_t o = off; off += (doubles + 31) / 32 * 32; return o; };
         o_mu = take(P); o_a = take(N); o_part = take(col_blocks); o_ybar = take(1); o_G = take((size_t)Np * Np);
-        o_Mi = take((size_t)nb * kCB * kCB); o_Li = take((size_t)nb * kCB * kCB); o_z = take(Np); o_gram = take((size_t)slices * tiles * kGT * kGT); o_int = take(2);
+        o_Mi = take((size_t)nb * kCB * kCB); o_Li = take((size_t)nb * kCB * kCB); o_refine = take((nb + 1) / 2); o_z = take(Np); o_gram = take((size_t)slices * tiles * kGT * kGT); o_int = take(2);
         o_up = take(integers ? N : 0); o_down = take(integers ? N : 0); o_digits = take(integers ? gram.digit_bytes / sizeof(double) : 0);
         bytes = off * sizeof(double);
     };
@@ -784,7 +800,7 @@ extern "C" int rocket_ridge_fit(const float* feat_dev, int N, int P, const float
         e = launch_gram(gram, feat_dev, N, P, d + o_mu, d + o_up, d + o_down, reinterpret_cast<uint8_t*>(d + o_digits), d + o_gram, status + 1, stream);
     else
         ridge_gram_kernel<<<dim3(tiles, slices), kGThreads, gram_smem, stream>>>(feat_dev, N, P, d + o_mu, slice, d + o_gram);
-    CholArgs q{d + o_gram, slices, tiles, (double)alpha, y_dev, d + o_ybar, d + o_G, d + o_Mi, d + o_Li, d + o_z, d + o_a, status, N, Np};
+    CholArgs q{d + o_gram, slices, tiles, (double)alpha, y_dev, d + o_ybar, d + o_G, d + o_Mi, d + o_Li, reinterpret_cast<int*>(d + o_refine), d + o_z, d + o_a, status, N, Np};
     void* args[] = {&q};
     // one block per SM: more would lengthen the grid barriers without shortening the chain
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(ridge_cholesky_solve_kernel),
