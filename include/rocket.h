@@ -295,7 +295,9 @@ int rocket_params_device_status(const rocket_params_t* p, int* wait_timeouts);
  * The batch goes through both kernels in chunks of a few examples; rocket_params_last_profile waits
  * for the last such call and returns the two durations, summed over the chunks, in milliseconds
  * (0 when nothing was recorded), and the convolution work of one example in either
- * kernel under the count 2*len*channels*L_out (flop).  Any output pointer may be NULL.
+ * kernel under the count 2*len*channels*L_out (flop).  Short series are served by one kernel for all
+ * dilations: its time is reported as the small dilations', the large ones' is 0, and the work is divided
+ * between the two as if two kernels did it.  Any output pointer may be NULL.
  */
 int rocket_params_set_profiling(rocket_params_t* p, int enable);
 int rocket_params_last_profile(const rocket_params_t* p, double* ms_small_dilations, double* ms_large_dilations,

@@ -322,8 +322,8 @@ constexpr int kRMergeFloats = 8;
 inline int64_t resident_merge_floats(const PlanHost& plan, int64_t n, int parts, int split, int mode) {
     return split > 1 && mode != 2 ? kRMergeFloats * n * ((int64_t)plan.runits.size() / parts + 1) : 0;
 }
-// The backward, whose code is twice as long and whose sums leave the warp once per tile, only where no tile has to test its reads and series
-// are short (us, before and with this kernel: 100 x 6 x 600, 2,000 kernels 1,106 and 855; 100 x 6 x 1,251 1,308 and 1,790).
+// The backward, whose code is twice as long and whose sums leave the warp once per tile, only where no tile has to test its reads: handles with room
+// for the zeros of its height (us, before and with this kernel, 2,000 kernels: 100 x 6 x 1,251 1,307 and 1,124, 60 x 3 x 5,000 1,850 and 1,615).
 inline bool resident_backward(const PlanHost& plan) { return plan.r_back != 0; }
 // Whether every fused call of the handle is a matter of one kernel, or of tiles of at most kSMaxPlanes channels: no call of such a handle is
 // better served by the generic kernels, and generic_pays is not asked.

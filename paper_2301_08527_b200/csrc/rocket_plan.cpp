@@ -207,7 +207,7 @@ void build_resident_units(const HostParams& hp, PlanHost& out) {
         u.lq = end / u.d; u.lr = end % u.d;
     }
     // Kernels of a length follow one another, so that the warps of a block share inner loops; the longest pairs of a length first.  The
-    // instruction caches decide here: the longest pairs first throughout took 846 us where this order takes 410 (100 x 20 x 2,800, 400 kernels).
+    // instruction caches decide here: the longest pairs first throughout take 548 us where this order takes 222 (24 x 32 x 1,751, 2,000 kernels).
     std::vector<int> order(r.units.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     std::sort(order.begin(), order.end(), [&](int a, int b) { return r.units[a].k < r.units[b].k; });
@@ -240,7 +240,7 @@ ResidentSplit resident_split(const PlanHost& plan, int N, int C, int sms, int mo
             for (int split = 1; split <= 4 && (split == 1 || (run == 1 && split < 2 * plan.r_tiles)); split *= 2) {
                 if (resident_floats(plan, e, C) + resident_merge_floats(plan, e, (int)parts, split, mode) > kRMostFloats) continue;
                 const double items = (double)kernels * (double)((e + run - 1) / run) * split;
-                // a warp's last item runs beside those of the five other warps of its scheduler
+                // a warp's last item runs beside those of the four to six other warps of its scheduler
                 const double task = kRTaskClocks + 4.0 * e * C * plan.r_pitch / 30.0 + e * work / parts + items * kRItemClocks / 4.0 +
                                     2.0 * plan.r_longest * (double)run / std::min(split, plan.r_tiles);
                 const double t = (double)((groups * parts + sms - 1) / sms) * task;

@@ -12,11 +12,11 @@
 // 250 kernels shared; here an example is copied once for all of them.
 //
 // Bound: issue slots.  A row of a tile is two loads, two address steps and 7 to 11 packed multiply-adds (the dilation is no constant, so
-// that addresses are no immediate offsets); what else counts is code, of which the warps of an SM should share as little as possible at a
-// time: with zeros beside the rows in place of tests a backward of 24 x 6 x 1,251 went from 960 to 540 us, with kernels ordered by length and
-// not by work 100 x 20 x 2,800 from 846 to 410.  Measured (us, before and now): 24 x 32 x 1,751 with 2,000 kernels 476 and 222, 16 x 1 x 512 with 1,000
-// 35 and 22, 100 x 20 x 600 with 4,000 1,283 and 717, soft 1,167 and 445 (2,000
-// kernels), backward of 24 x 9 x 700 with 2,000 373 and 200.
+// that addresses are no immediate offsets); what else counts is code, of which the warps of an SM should use as little as possible at a
+// time: hence zeros beside the rows in place of tests, and kernels ordered by length and not by work (24 x 32 x 1,751 with 2,000 kernels 222 and
+// 548 us, 100 x 20 x 1,400 with 4,000 1,339 and 1,577).  Measured (us, before and now): 24 x 32 x 1,751 with 2,000 kernels 476 and 222, 16 x 1 x 512
+// with 1,000 36 and 18.5, 100 x 20 x 600 with 4,000 1,283 and 715, soft 1,166 and 444 (2,000
+// kernels), backward of 24 x 9 x 700 with 2,000 374 and 229.
 #include <algorithm>
 
 #include "rocket_fast.h"
