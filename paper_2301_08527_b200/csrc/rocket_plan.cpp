@@ -210,7 +210,6 @@ void build_resident_units(const HostParams& hp, PlanHost& out) {
     // instruction caches decide here: the longest pairs first throughout take 548 us where this order takes 222 (24 x 32 x 1,751, 2,000 kernels).
     std::vector<int> order(r.units.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
-    std::sort(order.begin(), order.end(), [&](int a, int b) { return r.units[a].k < r.units[b].k; });
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
         return r.units[a].len != r.units[b].len ? r.units[a].len > r.units[b].len : r.cost[a] > r.cost[b];
     });
